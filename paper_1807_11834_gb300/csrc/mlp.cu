@@ -13,9 +13,11 @@
 // wait), and each thread reads back its row with tcgen05.ld.  The biases
 // b1 and b2 ride in the products: three operand columns of ones meet the
 // bias split into three BF16 terms whose sum is the FP32 bias exactly, so
-// the epilogue between the products is the activation alone.  The small
-// weight-gradient products (A^T dZ) run in FP32 on the CUDA cores in a
-// fixed order, so training is deterministic.
+// the epilogue between the products is the activation alone.  The
+// weight-gradient products (dZ^T A over a tile's rows) also run on the tensor
+// cores: A is BF16 already, and each FP32 dZ is split into three BF16 terms
+// whose sum is dZ exactly, so no operand is rounded.  Every sum has a fixed
+// order, so training is deterministic.
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -48,7 +50,7 @@ constexpr int NPARAM = OFF_B3 + 1;     // 5313
 constexpr int TILE = 128;              // rows per CTA tile
 constexpr uint32_t kSpinLimit = 1u << 22;
 constexpr uint32_t kInferCols = 64;     // TMEM columns of a forward-only CTA (Z1, then Z2 in the same columns)
-constexpr uint32_t kTrainCols = 256;    // Z1 (0..63), Z2 (64..127), dA1 (128..191)
+constexpr uint32_t kTrainCols = 512;    // Z1 (0..63), Z2 then dA1 (64..127), weight gradients of four groups of 32 rows (128..511)
 
 // ---------------------------------------------------------------------------
 // tcgen05 / TMEM / mbarrier primitives (inline PTX)
@@ -85,9 +87,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
     return done != 0;
 }
 
-// Shared-memory matrix descriptor: no swizzle, K-major core matrices of
-// 8 rows x 16 bytes; lbo = byte step between core matrices along K, sbo =
-// byte step between 8-row groups along M (or N).
+// Shared-memory matrix descriptor: no swizzle, core matrices of 8 x 16 bytes
+// (K-major: 8 rows of M or N with 8 values of K each; MN-major: 8 rows of K
+// with 8 values of M or N each); lbo = byte step between core matrices along
+// K, sbo = byte step between them along M (or N).
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
     uint64_t d = 0;
     d |= (uint64_t)((addr >> 4) & 0x3FFFu);
@@ -97,10 +100,11 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
     return d;                 // base offset 0, layout type 0 (no swizzle)
 }
 
-// Instruction descriptor, kind::f16: BF16 A and B, FP32 accumulate, both
-// operands K-major, shape M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor, kind::f16: BF16 A and B, FP32 accumulate, shape
+// M x N; both operands K-major, or both MN-major (mn).
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool mn = false) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -254,47 +258,71 @@ struct Smem {
     uint32_t tmem;
     int fail;
 };
+// Training: the A operands of a tile in one 96-column tile (0..63 act(Z1),
+// 64..66 ones, 67..79 zeros, 80..95 the network input), so that it is the A
+// of both forward products (K-major) and the B of the gradient product
+// (rows as K, MN-major) from the same bytes; and the three BF16 terms of
+// (dZ2 | dZ1), 128 columns, whose first half is also the A of dA1.
+constexpr int KX = 96;                 // columns of the training tile
+constexpr int XCOL = 80;               // its first input column
+constexpr int KD = 2 * H;              // columns of a dZ tile
+constexpr int TRAIN_THREADS = 512;     // four threads per row, 16 hidden columns each
 struct SmemTrain {
-    Smem s;
+    Smem s;                                        // w, bar, tmem and fail are used
+    alignas(128) unsigned char AX[TILE * KX * 2];
+    alignas(128) unsigned char D[3][TILE * KD * 2];
     alignas(128) unsigned char W2b[H * H * 2];     // B of the dA1 product: (n = in, k = out)
-    alignas(128) unsigned char dZ2b[TILE * H * 2]; // A of the dA1 product (BF16 dZ2)
-    float dZ2[TILE][H + 1];   // FP32 dZ2 (padded against bank conflicts)
-    float dZ1[TILE][H + 1];   // FP32 dZ1
-    float A2dc[TILE][H + 1];  // A2 * dc, for the w3 gradient
-    float dc[TILE];
-    float r2[TILE];
+    float c4[4][TILE];                             // a row's output, per 16-column quarter
+    float w3part[4][H];                            // w3 gradient per group of 32 rows
+    float red[2][4];                               // output bias gradient and loss per group of 32 rows
+    uint64_t bar2;                                 // completions of the gradient product
 };
 
-// The weight image from the FP32 parameters: BF16 operand copies of the
-// weights with the split biases, and the FP32 vectors.  One CTA.
+// The image entries that come from parameter i (of value w): the BF16
+// operand copy of a weight, the three split terms of a bias, or the FP32
+// entry of the output layer.  Entries without a parameter stay zero.
+__device__ __forceinline__ void image_put(WeightImage* __restrict__ img, int i, float w) {
+    auto put = [](unsigned char* t, uint32_t off, float x) { *reinterpret_cast<uint16_t*>(t + off) = bf16_bits(x); };
+    if (i < OFF_B1) {
+        const int k = i / H, n = i % H;   // W1[k][n] as (n = hidden, k); inputs past NFEAT are zero
+        if (k < NFEAT) put(img->W1t, koff(n, k, K0), w);
+    } else if (i < OFF_W2) {
+        for (int j = 0; j < 3; ++j) put(img->W1t, koff(i - OFF_B1, NFEAT + j, K0), bias_term(w, j));
+    } else if (i < OFF_B2) {
+        const int in = (i - OFF_W2) / H, out = (i - OFF_W2) % H;   // W2[in][out] as (n = out, k = in)
+        put(img->W2t, koff(out, in, KA), w);
+    } else if (i < OFF_W3) {
+        for (int j = 0; j < 3; ++j) put(img->W2t, koff(i - OFF_B2, H + j, KA), bias_term(w, j));
+    } else if (i < OFF_B3) {
+        img->w3[i - OFF_W3] = w;
+    } else {
+        img->b3 = w;
+    }
+}
+
+// The whole weight image from the FP32 parameters (an image of zeros
+// beforehand); a training step writes only the entries it changes.
 __global__ void __launch_bounds__(256)
 k_mlp_image(const float* __restrict__ P, const float* __restrict__ scale, WeightImage* __restrict__ img) {
-    for (int e = threadIdx.x; e < H * K0; e += blockDim.x) {
-        const int n = e / K0, k = e % K0;   // W1t(n, k) = W1[k][n]; inputs past NFEAT are zero
-        const float w = k < NFEAT ? P[OFF_W1 + k * H + n] : k < NFEAT + 3 ? bias_term(P[OFF_B1 + n], k - NFEAT) : 0.f;
-        *reinterpret_cast<uint16_t*>(img->W1t + koff(n, k, K0)) = bf16_bits(w);
-    }
-    for (int e = threadIdx.x; e < H * KA; e += blockDim.x) {
-        const int i = e / H, o = e % H;     // W2[i][o] as (n = out, k = in)
-        const float w = i < H ? P[OFF_W2 + i * H + o] : i < H + 3 ? bias_term(P[OFF_B2 + o], i - H) : 0.f;
-        *reinterpret_cast<uint16_t*>(img->W2t + koff(o, i, KA)) = bf16_bits(w);
-    }
-    for (int j = threadIdx.x; j < H; j += blockDim.x) img->w3[j] = P[OFF_W3 + j];
-    if (threadIdx.x < FEAT_STRIDE) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NPARAM; i += gridDim.x * blockDim.x)
+        image_put(img, i, P[i]);
+    if (blockIdx.x == 0 && threadIdx.x < FEAT_STRIDE) {
         img->lo[threadIdx.x] = scale[threadIdx.x];
         img->inv[threadIdx.x] = scale[FEAT_STRIDE + threadIdx.x];
     }
-    if (threadIdx.x == 0) img->b3 = P[OFF_B3];
 }
 
 // A CTA's copy of the weight image (16-byte words, all in flight at once),
 // and the constant columns of the second product's A tile (ones at
 // 64..66, zeros up to KA), which no tile overwrites.
-__device__ void load_weights(Smem& s, const WeightImage* __restrict__ img) {
+__device__ void load_image(Smem& s, const WeightImage* __restrict__ img) {
     const uint4* src = reinterpret_cast<const uint4*>(img);
     uint4* dst = reinterpret_cast<uint4*>(&s.w);
     constexpr int words = (int)(sizeof(WeightImage) / 16);
     for (int e = threadIdx.x; e < words; e += blockDim.x) dst[e] = __ldg(src + e);
+}
+__device__ void load_weights(Smem& s, const WeightImage* __restrict__ img) {
+    load_image(s, img);
     for (int row = threadIdx.x; row < TILE; row += blockDim.x) {
         const float one[8] = {1.f, 1.f, 1.f, 0.f, 0.f, 0.f, 0.f, 0.f}, zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         st_row8(s.A1, row, H, KA, one);
@@ -438,7 +466,7 @@ __device__ __forceinline__ float act_grad(float x) {
 // BF16 act(z) of 16 consecutive columns into row `row` of the second
 // product's A tile.  ReLU: the clamp is part of the conversion, one
 // instruction per pair.
-template <int ACT>
+template <int ACT, int K = KA>
 __device__ __forceinline__ void act_store16(unsigned char* A1, int row, int k0, const float (&z)[16]) {
     uint32_t w[8];
     if (ACT == ACT_RELU) {
@@ -452,8 +480,8 @@ __device__ __forceinline__ void act_store16(unsigned char* A1, int row, int k0, 
             w[i] = bf16x2(a, b);
         }
     }
-    *reinterpret_cast<uint4*>(A1 + koff(row, k0, KA)) = make_uint4(w[0], w[1], w[2], w[3]);
-    *reinterpret_cast<uint4*>(A1 + koff(row, k0 + 8, KA)) = make_uint4(w[4], w[5], w[6], w[7]);
+    *reinterpret_cast<uint4*>(A1 + koff(row, k0, K)) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4*>(A1 + koff(row, k0 + 8, K)) = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
 // First epilogue: act(Z1) of this thread's row (TMEM columns col0..col0+63)
@@ -546,11 +574,83 @@ k_mlp_forward(const WeightImage* __restrict__ img, const float* __restrict__ fea
     cta_teardown(s, kInferCols);
 }
 
+// One product of the training kernel, issued by thread 0 after the CTA's
+// operand stores: D columns [dcol, dcol + N) (+)= A B^T over nk steps of K,
+// operand starts moving by astep / bstep bytes per step.
+__device__ void train_issue(Smem& s, uint64_t* bar, uint32_t dcol, uint32_t idesc, const unsigned char* A,
+                            uint32_t albo, uint32_t asbo, uint32_t astep, const unsigned char* B, uint32_t blbo,
+                            uint32_t bsbo, uint32_t bstep, int nk) {
+    fence_async_smem();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < nk; ++k)
+            umma(s.tmem + dcol, sdesc(saddr(A) + k * astep, albo, asbo), sdesc(saddr(B) + k * bstep, blbo, bsbo), idesc,
+                 k > 0);
+        umma_commit(bar);
+    }
+}
+
+// The three BF16 terms of 16 consecutive columns of a dZ row (see bias_term).
+__device__ __forceinline__ void split_store16(SmemTrain& st, int row, int col, const float (&d)[16]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float r[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = d[8 * h + i];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                w[i] = bf16x2(r[2 * i], r[2 * i + 1]);
+                // what the pair leaves, exactly (a BF16 is the upper half of its FP32)
+                r[2 * i] -= __uint_as_float(w[i] << 16);
+                r[2 * i + 1] -= __uint_as_float(w[i] & 0xffff0000u);
+            }
+            *reinterpret_cast<uint4*>(st.D[t] + koff(row, col + 8 * h, KD)) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+
+// Sums of 16 columns over the warp's 32 lanes in a fixed tree; lane l ends
+// with the sum of column l / 2 (both lanes of a pair alike).
+__device__ __forceinline__ float column_sums16(float (&v)[16]) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int w = 8; w >= 1; w >>= 1) {
+        const bool up = lane & (2 * w);
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const float send = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+            v[i] = keep + __shfl_xor_sync(full, send, 2 * w);
+        }
+    }
+    return v[0] + __shfl_xor_sync(full, v[0], 1);
+}
+
 // Loss and gradient partials of a batch: each CTA accumulates its tiles'
 // contributions in a fixed order and writes one partial per parameter.
 // Layout of part: [gridDim.x][NPARAM + 1] (the last entry: sum of residual^2).
+//
+// 512 threads share a tile of 128 rows, 16 hidden columns of a row each: the
+// kernel is bound by the activations and their derivatives (three passes of
+// 8192 per tile), so four warps per scheduler hide the TMEM and tensor-core
+// round trips of the tile's serial chain of products.  The gradients of W2,
+// b2, W1 and b1 of a tile are one product of M = 128 ((dZ2 | dZ1) columns) by
+// N = 96 (the training tile's columns) over K = 128 rows, three times for the
+// BF16 terms of dZ (half of the product is not read; it costs 0.3 us per
+// tile).  The tensor core truncates as it accumulates, so every group of 32
+// rows has its own accumulator, the small terms go in first, and the groups
+// are added up in rounded FP32: accumulated in TMEM over all of a CTA's tiles
+// the gradient was 1.3e-6 from a 64-bit sum of the same operands (65,536
+// rows, GELU, W2), the loop over the rows that this replaces 2.7e-7, this
+// 2.6e-7.  That loop on 128 threads took 201 us for 65,536 rows, this kernel
+// 40 us.
 template <int ACT>
-__global__ void __launch_bounds__(TILE, 1)
+__global__ void __launch_bounds__(TRAIN_THREADS, 1)
 k_mlp_grad(const float* __restrict__ P, const WeightImage* __restrict__ img, const float* __restrict__ feat,
            const float* __restrict__ target, long long n, float* __restrict__ part,
            unsigned long long* __restrict__ status) {
@@ -558,119 +658,187 @@ k_mlp_grad(const float* __restrict__ P, const WeightImage* __restrict__ img, con
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     SmemTrain& st = smem_as<SmemTrain>(smem_raw);
     Smem& s = st.s;
-    load_weights(s, img);
+    load_image(s, img);
     load_w2b(st, P);
+    const int tid = threadIdx.x, row = tid & (TILE - 1), q = tid >> 7, lane = tid & 31;
+    if (tid < TILE) {
+        const float one[8] = {1.f, 1.f, 1.f, 0.f, 0.f, 0.f, 0.f, 0.f}, zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        st_row8(st.AX, row, H, KX, one);
+        st_row8(st.AX, row, H + 8, KX, zero);
+    }
+    if (tid == 0) mbar_init(&st.bar2, 1);
     cta_setup(s, kTrainCols);
-    uint32_t phase = 0;
-    const int tid = threadIdx.x;
+    uint32_t phase = 0, phase2 = 0;
     const float inv_n = 1.0f / (float)n;
-    // this thread's gradient accumulators: W2 entries tid*32 .. +32 (flattened
-    // (in, out)), W1 entries tid*8 .. +8, bias / w3 entries for tid < 64
-    float gW2[32], gW1[8];
+    float gw3 = 0.f, gb3 = 0.f, loss = 0.f;   // gw3: of column 16 q + lane / 2, rows of this warp
+    // rows < 64: W2[16 q ..][row] and, for q = 0, b2[row]; rows >= 64, q = 0: W1 and b1 of column row - 64
+    float gw[16], gb2 = 0.f;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) gW2[i] = 0.f;
+    for (int i = 0; i < 16; ++i) gw[i] = 0.f;
+    auto collect = [&]() {   // the gradient product of a tile, complete in TMEM
+        if (row < H || q == 0)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) gW1[i] = 0.f;
-    float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, loss = 0.f;
+            for (int ch = 0; ch < 4; ++ch) {
+                float g[16];
+                tmem_ld16(lane_addr(s, 128 + KX * ch + (row < H ? 16 * q : XCOL)), g);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) gw[i] += g[i];
+                if (row < H && q == 0) {
+                    tmem_ld16(lane_addr(s, 128 + KX * ch + H), g);
+                    gb2 += g[0];
+                }
+            }
+    };
     const long long ntiles = (n + TILE - 1) / TILE;
+    bool ok = true, first = true;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const long long r = t * TILE + tid;
+        const long long r = t * TILE + row;
+        const float tg = r < n ? __ldg(target + r) : 0.f;
         float f[FEAT_STRIDE] = {0, 0, 0, 0, 0, 0, 0, 0};
-        float tg = 0.f;
-        if (r < n) {
-            const float4 a = reinterpret_cast<const float4*>(feat)[2 * r];
-            const float4 b = reinterpret_cast<const float4*>(feat)[2 * r + 1];
+        if (q == 0 && r < n) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(feat) + 2 * r);
+            const float4 b = __ldg(reinterpret_cast<const float4*>(feat) + 2 * r + 1);
             f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-            tg = target[r];
         }
-        float x[K0];
-        scale_row(s, f, x);
-        st_row8(s.X, tid, 0, K0, x);
-        st_row8(s.X, tid, 8, K0, x + 8);
-        float c = 0.f;
-        if (!tile_forward<ACT>(s, phase, status, c, 64)) break;
-        const float res = (r < n) ? (c - tg) : 0.f;
-        const float dc = 2.0f * res * inv_n;
-        st.dc[tid] = dc;
-        st.r2[tid] = res * res;
-        // dZ2 = dc w3 * act'(Z2); A2 dc for the w3 gradient
-#pragma unroll
-        for (int q = 0; q < H / 16; ++q) {
-            float z[16], d[16];
+        // the last tile's gradient product has read the operands this tile overwrites
+        if (!first) {
+            if (!(ok = gemm_wait(s, &st.bar2, phase2, status))) break;
+            collect();
+        }
+        if (q == 0) {
+            float x[K0];
+            scale_row(s, f, x);
+            st_row8(st.AX, row, XCOL, KX, x);
+            st_row8(st.AX, row, XCOL + 8, KX, x + 8);
+        }
+        // Z1 = X W1 + b1
+        train_issue(s, &s.bar, 0, idesc_bf16(TILE, H), st.AX + XCOL / 8 * 128, 128, KX * 16, 256, s.w.W1t, 128, 256, 256, 1);
+        if (!(ok = gemm_wait(s, &s.bar, phase, status))) break;
+        {
+            float z[16];
+            tmem_ld16(lane_addr(s, 16 * q), z);
+            act_store16<ACT, KX>(st.AX, row, 16 * q, z);
+        }
+        // Z2 = A1 W2 + b2
+        train_issue(s, &s.bar, 64, idesc_bf16(TILE, H), st.AX, 128, KX * 16, 256, s.w.W2t, 128, KA * 16, 256, KA / 16);
+        if (!(ok = gemm_wait(s, &s.bar, phase, status))) break;
+        {
+            float z[16], d[16], a2[16];
             tmem_ld16(lane_addr(s, 64 + 16 * q), z);
+            float acc = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+                if (ACT == ACT_RELU) {
+                    a2[i] = fmaxf(z[i], 0.f);
+                    a2[i + 1] = fmaxf(z[i + 1], 0.f);
+                } else {
+                    gelu2(z[i], z[i + 1], a2[i], a2[i + 1]);
+                }
+                acc = fmaf(a2[i], s.w.w3[16 * q + i], acc);
+                acc = fmaf(a2[i + 1], s.w.w3[16 * q + i + 1], acc);
+            }
+            st.c4[q][row] = acc;
+            __syncthreads();
+            const float c = ((st.c4[0][row] + st.c4[1][row]) + (st.c4[2][row] + st.c4[3][row])) + s.w.b3;
+            const float res = r < n ? c - tg : 0.f;
+            const float dc = 2.0f * res * inv_n;
+            if (q == 0) {
+                gb3 += dc;
+                loss = fmaf(res, res, loss);
+            }
+            // dZ2 = dc w3 act'(Z2); A2 dc for the w3 gradient
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const int j = 16 * q + i;
-                d[i] = dc * s.w.w3[j] * act_grad<ACT>(z[i]);
-                st.dZ2[tid][j] = d[i];
-                st.A2dc[tid][j] = act1<ACT>(z[i]) * dc;
+                d[i] = dc * s.w.w3[16 * q + i] * act_grad<ACT>(z[i]);
+                a2[i] *= dc;
             }
-            st_row8(st.dZ2b, tid, 16 * q, H, d);
-            st_row8(st.dZ2b, tid, 16 * q + 8, H, d + 8);
+            split_store16(st, row, 16 * q, d);
+            gw3 += column_sums16(a2);
         }
-        // dA1 = dZ2 W2^T on the tensor cores
-        if (!run_gemm(s, 128, st.dZ2b, st.W2b, H / 16, phase, status)) break;
+        // dA1 = dZ2 W2^T (dZ2 rounded to BF16: the first term), over Z2's columns, which every thread has read
+        train_issue(s, &s.bar, 64, idesc_bf16(TILE, H), st.D[0], 128, KD * 16, 256, st.W2b, 128, H * 16, 256, H / 16);
+        if (!(ok = gemm_wait(s, &s.bar, phase, status))) break;
+        {
+            float da[16], z[16];
+            tmem_ld16(lane_addr(s, 64 + 16 * q), da);
+            tmem_ld16(lane_addr(s, 16 * q), z);
 #pragma unroll
-        for (int q = 0; q < H / 16; ++q) {
-            float da[16], z1[16];
-            tmem_ld16(lane_addr(s, 128 + 16 * q), da);
-            tmem_ld16(lane_addr(s, 16 * q), z1);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) st.dZ1[tid][16 * q + i] = da[i] * act_grad<ACT>(z1[i]);
+            for (int i = 0; i < 16; ++i) da[i] *= act_grad<ACT>(z[i]);
+            split_store16(st, row, H + 16 * q, da);
         }
+        // the weight gradients, smallest terms first
+        fence_async_smem();
+        fence_before();
         __syncthreads();
-        // weight gradients, rows summed in increasing order
-#pragma unroll 1
-        for (int row = 0; row < TILE; ++row) {
-            // W2 (in, out): entries tid*32 + e -> in = (tid*32+e) / 64, out = (tid*32+e) % 64
-            const int in = (tid * 32) / H, out0 = (tid * 32) % H;
-            const float a1 = bf16_val(*reinterpret_cast<const uint16_t*>(s.A1 + koff(row, in, KA)));
-#pragma unroll
-            for (int e = 0; e < 32; ++e) gW2[e] = fmaf(a1, st.dZ2[row][out0 + e], gW2[e]);
-            // W1 (k, j): entries tid*8 + e -> k = (tid*8+e) / 64, j = (tid*8+e) % 64; the
-            // inputs past NFEAT are zero in the network (the tile's ones there meet b1)
-            const int k = (tid * 8) / H, j0 = (tid * 8) % H;
-            const float xk =
-                k < NFEAT ? bf16_val(*reinterpret_cast<const uint16_t*>(s.X + koff(row, k, K0))) : 0.f;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) gW1[e] = fmaf(xk, st.dZ1[row][j0 + e], gW1[e]);
-            if (tid < H) {
-                gb1 += st.dZ1[row][tid];
-                gb2 += st.dZ2[row][tid];
-                gw3 += st.A2dc[row][tid];
-            } else if (tid == H) {
-                gb3 += st.dc[row];
-                loss += st.r2[row];
-            }
+        fence_after();
+        if (tid == 0) {
+            for (int j = 2; j >= 0; --j)
+                for (int k = 0; k < TILE / 16; ++k)
+                    umma(s.tmem + 128 + KX * (k >> 1), sdesc(saddr(st.D[j]) + k * KD * 32, KD * 16, 128),
+                         sdesc(saddr(st.AX) + k * KX * 32, KX * 16, 128), idesc_bf16(TILE, KX, true),
+                         j < 2 || (k & 1));
+            umma_commit(&st.bar2);
         }
-        __syncthreads();
+        first = false;
     }
+    if (ok && !first && (ok = gemm_wait(s, &st.bar2, phase2, status))) collect();
+    // lanes 0..63 of the product's columns: dZ2's, lanes 64..127: dZ1's
     float* out = part + (long long)blockIdx.x * (NPARAM + 1);
+    if (row < H) {
 #pragma unroll
-    for (int e = 0; e < 32; ++e) out[OFF_W2 + tid * 32 + e] = gW2[e];
+        for (int i = 0; i < 16; ++i) out[OFF_W2 + (16 * q + i) * H + row] = gw[i];
+        if (q == 0) out[OFF_B2 + row] = gb2;
+    } else if (q == 0) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) out[OFF_W1 + tid * 8 + e] = gW1[e];
-    if (tid < H) {
-        out[OFF_B1 + tid] = gb1;
-        out[OFF_B2 + tid] = gb2;
-        out[OFF_W3 + tid] = gw3;
-    } else if (tid == H) {
-        out[OFF_B3] = gb3;
-        out[NPARAM] = loss;
+        for (int k = 0; k < K0; ++k) out[OFF_W1 + k * H + row - H] = k < NFEAT ? gw[k] : 0.f;
+        out[OFF_B1 + row - H] = gw[NFEAT];
     }
-    cta_teardown(s, kTrainCols);
+    // the output layer and the loss: over each warp's rows, then the four groups of rows in order
+    if (!(lane & 1)) st.w3part[row >> 5][16 * q + (lane >> 1)] = gw3;
+    if (q == 0) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            gb3 += __shfl_xor_sync(0xffffffffu, gb3, off);
+            loss += __shfl_xor_sync(0xffffffffu, loss, off);
+        }
+        if (lane == 0) {
+            st.red[0][row >> 5] = gb3;
+            st.red[1][row >> 5] = loss;
+        }
+    }
+    __syncthreads();
+    if (tid < H)
+        out[OFF_W3 + tid] = (st.w3part[0][tid] + st.w3part[1][tid]) + (st.w3part[2][tid] + st.w3part[3][tid]);
+    else if (tid < H + 2)
+        out[tid == H ? OFF_B3 : NPARAM] = (st.red[tid - H][0] + st.red[tid - H][1]) + (st.red[tid - H][2] + st.red[tid - H][3]);
+    cta_teardown(s, kTrainCols, &st.bar2);
 }
 
-// Sum the CTA partials (fixed order), optionally apply one Adam step.
-__global__ void __launch_bounds__(256)
+// Sum the CTA partials (fixed order), optionally apply one Adam step and
+// update the weight image.  A CTA takes 32 parameters, eight threads each
+// summing an eighth of the partials (7.0 us): with one thread per
+// parameter the 152 dependent additions took 10.4 us, and rebuilding the
+// image by a CTA of its own 15.2 us more.
+constexpr int kReduceParts = 8;
+__global__ void __launch_bounds__(32 * kReduceParts)
 k_mlp_reduce_adam(const float* __restrict__ part, int nparts, float* __restrict__ grads, float* __restrict__ P,
                   float* __restrict__ m, float* __restrict__ v, int t, float lr, int do_update,
-                  float* __restrict__ loss_out, long long n) {
+                  float* __restrict__ loss_out, long long n, WeightImage* __restrict__ img) {
+    __shared__ float sh[kReduceParts][32];
     pdl_wait();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > NPARAM) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
     float g = 0.f;
-    for (int b = 0; b < nparts; ++b) g += part[(long long)b * (NPARAM + 1) + i];
+    if (i <= NPARAM) {
+        const int per = (nparts + kReduceParts - 1) / kReduceParts;
+        const int b1 = min(nparts, (w + 1) * per);
+#pragma unroll 8
+        for (int b = w * per; b < b1; ++b) g += part[(long long)b * (NPARAM + 1) + i];
+    }
+    sh[w][lane] = g;
+    __syncthreads();
+    if (w != 0 || i > NPARAM) return;
+    g = ((sh[0][lane] + sh[1][lane]) + (sh[2][lane] + sh[3][lane])) + ((sh[4][lane] + sh[5][lane]) + (sh[6][lane] + sh[7][lane]));
     if (i == NPARAM) {
         if (loss_out) loss_out[0] = g / (float)n;
         return;
@@ -684,7 +852,9 @@ k_mlp_reduce_adam(const float* __restrict__ part, int nparts, float* __restrict_
         v[i] = vi;
         const float mh = mi / (1.f - powf(b1, (float)t));
         const float vh = vi / (1.f - powf(b2, (float)t));
-        P[i] -= lr * mh / (sqrtf(vh) + eps);
+        const float p = P[i] - lr * mh / (sqrtf(vh) + eps);
+        P[i] = p;
+        image_put(img, i, p);
     }
 }
 
@@ -1002,10 +1172,10 @@ cg_status mlp_attrs() {
     });
 }
 
-// Rebuild the weight image from P on the closure's stream (after every
-// change of P, in the same stream order).
+// Rebuild the weight image from P on the closure's stream (a training step
+// updates its entries with the parameters).
 cg_status rebuild_image(cg_mlp* m) {
-    k_mlp_image<<<1, 256, 0, m->stream>>>(m->P, m->scale, m->img);
+    k_mlp_image<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->P, m->scale, m->img);
     CG_CUDA(cudaGetLastError());
     return CG_OK;
 }
@@ -1063,6 +1233,25 @@ cg_status mlp_feature_box(const cg_mlp* m, float* lo, float* hi) {
     return CG_OK;
 }
 }  // namespace cg
+
+// A programmatic dependent launch on the closure's stream (the kernels start
+// with pdl_wait, so only the launch latency overlaps).
+template <typename... KArgs, typename... Args>
+static cg_status mlp_launch(cg_mlp* m, void (*kernel)(KArgs...), int grid, int block, size_t smem, Args... args) {
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = m->stream;
+    c.attrs = a;
+    c.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&c, kernel, KArgs(args)...);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    return e == cudaSuccess ? CG_OK : CG_ERR_CUDA;
+}
 
 extern "C" {
 
@@ -1133,6 +1322,7 @@ cg_status cg_mlp_create(const float* params, const float* feat_lo, const float* 
               cudaMalloc(&m->status, sizeof(unsigned long long) * cg::kNumSlots) == cudaSuccess;
     ok = ok && cudaMemcpy(m->P, params, pb, cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(m->m, 0, pb) == cudaSuccess && cudaMemset(m->v, 0, pb) == cudaSuccess &&
+         cudaMemset(m->img, 0, sizeof(WeightImage)) == cudaSuccess &&
          cudaMemcpy(m->scale, sc, sizeof sc, cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(m->status, 0, sizeof(unsigned long long) * cg::kNumSlots) == cudaSuccess;
     ok = ok && mlp_attrs() == CG_OK && rebuild_image(m) == CG_OK && cudaStreamSynchronize(m->stream) == cudaSuccess;
@@ -1204,15 +1394,11 @@ static cg_status grad_impl(cg_mlp* m, int64_t n, const float* features, const fl
     CG_TRY(mlp_attrs());
     const long long ntiles = (n + TILE - 1) / TILE;
     const int grid = (int)std::min(ntiles, (long long)m->num_sms);
-    auto kern = m->act == CG_MLP_RELU ? k_mlp_grad<ACT_RELU> : k_mlp_grad<ACT_GELU>;
-    kern<<<grid, TILE, smem_train(), m->stream>>>(m->P, m->img, features, targets, n, m->part, m->status);
-    CG_CUDA(cudaGetLastError());
+    CG_TRY(mlp_launch(m, m->act == CG_MLP_RELU ? k_mlp_grad<ACT_RELU> : k_mlp_grad<ACT_GELU>, grid, TRAIN_THREADS,
+                      smem_train(), m->P, m->img, features, targets, n, m->part, m->status));
     if (do_update) m->t += 1;
-    k_mlp_reduce_adam<<<(NPARAM + 1 + 255) / 256, 256, 0, m->stream>>>(m->part, grid, m->grads, m->P, m->m, m->v,
-                                                                        m->t, lr, do_update, loss_out, n);
-    CG_CUDA(cudaGetLastError());
-    if (do_update) CG_TRY(rebuild_image(m));
-    return CG_OK;
+    return mlp_launch(m, k_mlp_reduce_adam, (NPARAM + 1 + 31) / 32, 32 * kReduceParts, 0, m->part, grid, m->grads,
+                      m->P, m->m, m->v, m->t, lr, do_update, loss_out, n, m->img);
 }
 
 cg_status cg_mlp_grads(cg_mlp* m, int64_t n, const float* features, const float* targets, float* loss_out) {
