@@ -132,9 +132,8 @@ void prof_end(cg_grids* g, int slot, int ev) {
 // ---------------------------------------------------------------------------
 cg_status ensure_partials(cg_grids* g, long long n) {
     const long long bulk_blk = (g->gd.nbulk + 7) / 8;   // cell kernels run 8 cells (warps) per block
-    const long long fine_blk = (g->gd.nfine + 255) / 256;
     (void)n;
-    const long long proj_blk = (g->gd.r == 2 || g->gd.r == 4 || g->gd.r == 8) ? bulk_blk : fine_blk;
+    const long long proj_blk = project_blocks(g->gd, 3, g->fp64);   // the projection of the source forms sums
     const long long part_blk = std::max(bulk_blk, (long long)g->num_sms * 8);
     const long long need = part_blk * (1 + kDragCellSums) + proj_blk * 6;
     if (need > g->part_cap) {

@@ -188,20 +188,23 @@ cg_status plan(cg_batch* b) {
         set(BP_PLACE, I.cellsort ? cdiv(n, 512LL * kPlaceItems) : 0);
         set(BP_SEGSORT, I.cellsort ? cdiv(nb, (long long)kGroupCells * kSegSortWarps) : 0);
         set(BP_DEPV, seg);
-        set(BP_AVG, std::max(1LL, cdiv(nb, 256LL * c.avg_items)));
+        set(BP_AVG, std::max(1LL, cdiv(nb * average_lanes(g->gd.r, false), 256LL * c.avg_items)));
         set(BP_PACK, cellb);
         set(BP_DRAG, std::max(1LL, cdiv(n, 256LL * c.drag_items)));
         set(BP_DEPM, seg);
-        set(BP_PROJ, cellb);
-        set(BP_PROJE, I.eps_fine ? cellb : 0);
+        I.depth = project_depth(g->gd, 3, false);
+        I.depth_eps = project_depth(g->gd, 1, false);
+        const long long projb = cdiv(project_threads(g->gd, I.depth), 256);
+        set(BP_PROJ, 3 * projb);
+        set(BP_PROJE, I.eps_fine ? cdiv(project_threads(g->gd, I.depth_eps), 256) : 0);
         set(BP_SUMS, CG_NSUMS);
         // partial regions (pairs): volume 1 column, projection 6 (S_f V_f, S_B V_B), drag 9
         I.part_blocks[PS_VOL] = seg;
-        I.part_blocks[PS_PROJ] = cellb;
+        I.part_blocks[PS_PROJ] = projb;
         I.part_blocks[PS_DRAG] = B[(size_t)BP_DRAG * ni];
         I.part_off[PS_VOL] = 0;
         I.part_off[PS_PROJ] = seg;
-        I.part_off[PS_DRAG] = seg + 6 * cellb;
+        I.part_off[PS_DRAG] = seg + 6 * projb;
         const long long pairs = I.part_off[PS_DRAG] + (long long)kDragSums * I.part_blocks[PS_DRAG];
         CG_TRY(dev_alloc(b, (void**)&I.part, sizeof(float) * 2 * pairs));
         I.smap = sums_map(I.part_off, I.part_blocks);

@@ -24,6 +24,7 @@ struct BInst {
     long long n;
     int ntiles, b0, b1, npasses;
     int cellsort;          // per-cell sort (else the digit sort)
+    int depth, depth_eps;  // layers per thread of the projections (source, porosity)
     float* pos;
     float* vel;
     const float* u_fine;

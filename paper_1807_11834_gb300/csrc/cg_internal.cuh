@@ -267,7 +267,7 @@ void prof_end(cg_grids* g, int slot, int ev);
         a_[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;           \
         a_[0].val.programmaticStreamSerializationAllowed = 1;                    \
         cudaLaunchConfig_t c_ = {};                                              \
-        c_.gridDim = dim3((unsigned)(grid));                                     \
+        c_.gridDim = dim3(grid);                                                 \
         c_.blockDim = dim3((unsigned)(block));                                   \
         c_.dynamicSmemBytes = (size_t)(smem);                                    \
         c_.stream = (g)->stream;                                                 \
@@ -374,6 +374,18 @@ cg_status mlp_feature_box(const cg_mlp* m, float* lo, float* hi);
 // The stale variance field, fine velocity and record age bound to a closure by cg_mlp_bind.
 cg_status mlp_bound_inputs(const cg_mlp* m, const void** var_stale, const void** u_fine, int32_t* age);
 cg_status launch_project(cg_grids* g, int ncomp, const void* const* in, void* const* out, bool sums);
+// Lanes of a warp that share a bulk cell in the average: one per plane for
+// FP32 r = 2 and 4, fewer values per lane where a plane would not fit the
+// registers (r = 8, 64 values) or where FP64 doubles them; 1 otherwise.
+__host__ __device__ constexpr int average_lanes(int r, bool fp64) {
+    return r == 2 ? 2 : r == 4 ? (fp64 ? 8 : 4) : r == 8 ? (fp64 ? 32 : 16) : 1;
+}
+// Layers a thread of the projection walks, and its blocks of
+// project_block threads per component.
+int project_depth(const GridDev& g, int ncomp, bool fp64);
+int project_block(const GridDev& g, int ncomp, bool fp64);
+long long project_threads(const GridDev& g, int depth);
+long long project_blocks(const GridDev& g, int ncomp, bool fp64);
 cg_status launch_sums(cg_grids* g, double* sums);
 // Sum columns of the partial regions (offsets in pairs; blocks < 0: region not formed).
 SumsMap sums_map(const long long* part_off, const long long* part_blocks);
