@@ -681,19 +681,76 @@ __device__ __forceinline__ void seg_chunk_range(long long base, long long n, con
     if (s > last) t = s;   // the whole chunk lies inside a segment owned earlier
 }
 
-// Segmented sum of K values per slot over the slots [s, t) of one chunk,
-// 32 slots per round: a plain shuffle scan inside the round (at most five
-// roundings), compensated sums for the carry between rounds and for each
-// segment's total.  load(i, v) fills the K values of slot i; emit(key, tot)
-// receives each segment's compensated total on the lane of its last slot.
-// The next round's slots are loaded before the current one is reduced.
+// One round of the segmented sum of K (<= 4) values per slot over a chunk's
+// slots: 32 consecutive slots, one per lane (key -1: none), with `next31` the key
+// of the next round's first slot (-1 past the chunk's end).  A plain inclusive shuffle scan inside the round
+// (at most five roundings); the segment that goes on from round to round is a
+// compensated sum.  That sum is held once per warp, value k on lane k, so that
+// its additions cost one instruction for all K values (held by every lane,
+// they were 40% of the reaction's FP32 and two thirds of its FP64
+// instructions: FP64, 1M particles 137 -> 68 us; FP32, which the shuffles bound,
+// 4M particles 32 -> 29, 32M 190 -> 170).
+// emit(key, k, total) is called once per segment and value, each value by
+// one lane.
+template <typename T, int K>
+struct SegCarry {
+    CSum<T> a;      // lane k: value k of the segment of `key`
+    int key = -1;
+};
+template <typename T, int K, typename Emit>
+__device__ __forceinline__ void seg_round(T (&v)[K], int key, int next31, SegCarry<T, K>& carry, Emit emit) {
+    static_assert(K <= 4, "one lane per value");
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int prev = __shfl_up_sync(full, key, 1);
+    const unsigned heads = __ballot_sync(full, lane == 0 || prev != key);
+    const int head = 31 - __clz(heads & ((2u << lane) - 1u));   // first lane of this lane's segment
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const T o = __shfl_up_sync(full, v[k], off);
+            if (lane - off >= head) v[k] += o;
+        }
+    }
+    auto to_lanes = [&](int src) {   // value k of lane src, on lane k
+        T x = __shfl_sync(full, v[0], src);
+#pragma unroll
+        for (int k = 1; k < K; ++k) {
+            const T y = __shfl_sync(full, v[k], src);
+            if (lane == k) x = y;
+        }
+        return x;
+    };
+    const int first = __shfl_sync(full, key, 0), last = __shfl_sync(full, key, 31);
+    const unsigned endm = (heads >> 1) | (next31 != last ? 0x80000000u : 0u);   // last lanes of their segments
+    const bool ends = key >= 0 && (endm >> lane & 1u);
+    const bool cont = first >= 0 && first == carry.key;   // the round goes on with the carried segment
+    if (cont) {
+        const unsigned later = heads & ~1u;
+        const int e = later ? __ffs(later) - 2 : 31;      // its last lane in this round
+        carry.a.add(to_lanes(e));
+        if ((endm >> e & 1u) && lane < K) emit(first, lane, carry.a.get());
+    }
+    if (ends && !(cont && key == first))
+#pragma unroll
+        for (int k = 0; k < K; ++k) emit(key, k, v[k]);
+    if (last != carry.key) {
+        carry.a = CSum<T>();
+        carry.a.s = to_lanes(31);
+        carry.key = last;
+    }
+}
+
+// Segmented sum of K values per slot over the slots [s, t) of one chunk by
+// one warp, in rounds of 32 slots.  load(i, v) fills the K values of slot i.
+// Four rounds are loaded ahead of the reduction.
 template <typename T, int K, typename Load, typename Emit>
 __device__ __forceinline__ void seg_rounds(long long s, long long t, const int32_t* __restrict__ key_sorted,
                                            Load load, Emit emit) {
     constexpr int B = 4;   // rounds loaded ahead of the reduction
     const int lane = threadIdx.x & 31;
-    CSum<T> carry[K];
-    int carry_key = -1;
+    SegCarry<T, K> carry;
     for (long long r0 = s; r0 < t; r0 += 32 * B) {
         int key[B + 1];
         T v[B][K];
@@ -715,45 +772,7 @@ __device__ __forceinline__ void seg_rounds(long long s, long long t, const int32
 #pragma unroll
         for (int j = 0; j < B; ++j) {
             if (r0 + 32 * j >= t) break;   // warp-uniform
-            const long long i = r0 + 32 * j + lane;
-            const bool valid = i < t;
-            const int kj = key[j];
-            T* vj = v[j];
-            // plain inclusive segmented scan over the lanes
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int ko = __shfl_up_sync(0xffffffffu, kj, off);
-                const bool take = lane >= off && ko == kj;
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const T vo = __shfl_up_sync(0xffffffffu, vj[k], off);
-                    if (take) vj[k] += vo;
-                }
-            }
-            // every lane takes part in both shuffles; lane 31 looks at the next round
-            int next = __shfl_down_sync(0xffffffffu, kj, 1);
-            const int next31 = __shfl_sync(0xffffffffu, j + 1 < B ? key[j + 1] : key[B], 0);
-            if (lane == 31) next = next31;
-            const bool ends = valid && next != kj;
-            const bool cont = kj == carry_key;
-            if (ends) {
-                CSum<T> tot[K];
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    if (cont) tot[k] = carry[k];
-                    tot[k].add(vj[k]);
-                }
-                emit(kj, tot);
-            }
-            // carry: the segment of lane 31 if it goes on into the next round
-            const int k31 = __shfl_sync(0xffffffffu, kj, 31);
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const T v31 = __shfl_sync(0xffffffffu, vj[k], 31);
-                if (k31 != carry_key) carry[k] = CSum<T>();
-                carry[k].add(v31);
-            }
-            carry_key = k31;
+            seg_round<T, K>(v[j], key[j], __shfl_sync(0xffffffffu, key[j + 1], 0), carry, emit);
         }
     }
 }
@@ -882,19 +901,13 @@ __device__ __forceinline__ void seg_seq(long long s, long long t, const int32_t*
     }
 }
 
-// Reaction of one cell from its compensated force sum a: S_B = -(1/V_B) sum F
-// (Eq. UFP: F_fpi is the fluid-side reaction to F_drag), written to S
-// ([3][n_b]).  The conservation sum of S_B V_B is formed by the projection,
-// which reads every S_B.
+// Component k of the reaction of one cell from its force sum: S_B =
+// -(1/V_B) sum F (Eq. UFP: F_fpi is the fluid-side reaction to F_drag), written
+// to S ([3][n_b]).  The conservation sum of S_B V_B is formed by the
+// projection, which reads every S_B.
 template <typename T>
-__device__ __forceinline__ void reaction_emit(const GridDev& g, T* __restrict__ S, int key, const CSum<T> (&a)[3]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        T s_;
-        if (sizeof(T) == 4) s_ = -(a[k].get()) * (T)g.invVBf;
-        else s_ = -(a[k].get()) * (T)g.invVB;
-        S[k * g.nbulk + key] = s_;
-    }
+__device__ __forceinline__ void reaction_emit(const GridDev& g, T* __restrict__ S, int key, int k, T sum) {
+    S[k * g.nbulk + key] = -sum * (sizeof(T) == 4 ? (T)g.invVBf : (T)g.invVB);
 }
 
 // Sphere volume pi d^3 / 6 as an unevaluated pair hi + lo: exact products

@@ -147,7 +147,7 @@ __device__ __forceinline__ void deposit_sorted_force_body(const T* __restrict__ 
                 v[1] = f.y;
                 v[2] = f.z;
             },
-            [&](int key, CSum<T> (&a)[3]) { reaction_emit<T>(g, S, key, a); });
+            [&](int key, int k, T sum) { reaction_emit<T>(g, S, key, k, sum); });
     }
 }
 
@@ -173,16 +173,14 @@ __device__ __forceinline__ void deposit_implicit_body(const T* __restrict__ Bs, 
                 v[2] = r.z;
                 v[3] = r.w;
             },
-            [&](int key, CSum<T> (&a)[4]) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    coef[k * g.nbulk + key] = sizeof(T) == 4 ? a[k].get() * (T)g.invVBf : a[k].get() * (T)g.invVB;
+            [&](int key, int k, T sum) {
+                coef[k * g.nbulk + key] = sum * (sizeof(T) == 4 ? (T)g.invVBf : (T)g.invVB);
             });
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 k_deposit_implicit(const T* __restrict__ Bs, long long n, const int32_t* __restrict__ key_sorted,
                    const int32_t* __restrict__ cs, GridDev g, T* __restrict__ coef) {
     pdl_wait();
@@ -190,7 +188,7 @@ k_deposit_implicit(const T* __restrict__ Bs, long long n, const int32_t* __restr
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4)
 k_deposit_sorted_force(const T* __restrict__ Fs, long long n, const int32_t* __restrict__ key_sorted,
                        const int32_t* __restrict__ cs, GridDev g, T* __restrict__ S) {
     pdl_wait();
@@ -208,49 +206,19 @@ k_deposit_momentum(const T* __restrict__ F, long long n, const int32_t* __restri
                    const int32_t* __restrict__ key_sorted, const int32_t* __restrict__ cs, GridDev g,
                    T* __restrict__ S) {
     pdl_wait();
-    const int lane = threadIdx.x & 31;
     const long long wg = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long base = wg * kSegChunk; base < n; base += nw * kSegChunk) {
         long long s, t;
         seg_chunk_range(base, n, key_sorted, cs, s, t);
-        CSum<T> carry[3];
-        int carry_key = -1;
-        for (long long r = s; r < t; r += 32) {
-            const long long i = r + lane;
-            const bool valid = i < t;
-            int key = -1;
-            CSum<T> v[3];
-            if (valid) {
-                key = __ldg(key_sorted + i);
+        seg_rounds<T, 3>(
+            s, t, key_sorted,
+            [&](long long i, T (&v)[3]) {
                 const long long p = __ldg(perm + i);
-                v[0].s = __ldg(F + p);
-                v[1].s = __ldg(F + n + p);
-                v[2].s = __ldg(F + 2 * n + p);
-            }
-            if (lane == 0 && key == carry_key)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    CSum<T> c0 = carry[k];
-                    c0.merge(v[k]);
-                    v[k] = c0;
-                }
-            warp_seg_scan<T, 3>(v, key);
-            int next = __shfl_down_sync(0xffffffffu, key, 1);
-            if (lane == 31) next = (i + 1 < t) ? __ldg(key_sorted + i + 1) : -1;
-            if (valid && next != key)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    if (sizeof(T) == 4) S[k * g.nbulk + key] = -(v[k].get()) * (T)g.invVBf;
-                    else S[k * g.nbulk + key] = -(v[k].get()) * (T)g.invVB;
-                }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                carry[k].s = __shfl_sync(0xffffffffu, v[k].s, 31);
-                carry[k].c = __shfl_sync(0xffffffffu, v[k].c, 31);
-            }
-            carry_key = __shfl_sync(0xffffffffu, key, 31);
-        }
+                for (int k = 0; k < 3; ++k) v[k] = __ldg(F + k * n + p);
+            },
+            [&](int key, int k, T sum) { reaction_emit<T>(g, S, key, k, sum); });
     }
 }
 
@@ -397,11 +365,14 @@ int batch_deposit_occupancy(int phase) {
 static inline unsigned blocks_for(long long n, int per) { return (unsigned)((n + per - 1) / per); }
 
 // Grid of the segmented deposits: at most one chunk per warp, and no more
-// CTAs than are resident at once (4 per SM at their 64 registers), so the
-// grid-stride loop runs without a second, partial wave.
-static unsigned seg_blocks(cg_grids* g, long long n) {
-    const long long chunks = (n + kSegChunk - 1) / kSegChunk;
-    return (unsigned)std::max(1LL, std::min((chunks + 7) / 8, (long long)g->num_sms * 4));
+// CTAs than are resident at once (the reaction's 48 registers allow five per
+// SM, 64 four), so the grid-stride loop runs without a second, partial wave.  Few chunks take
+// blocks of one warp, so that they reach as many SMs as there are chunks
+// (10,000 particles, FP64: 40 chunks, 47 -> 19 us).
+static unsigned seg_threads(cg_grids* g, long long n) { return n <= (long long)g->num_sms * 8 * kSegChunk ? 32 : 256; }
+static unsigned seg_blocks(cg_grids* g, long long n, int per_sm = 4) {
+    const long long chunks = (n + kSegChunk - 1) / kSegChunk, per = seg_threads(g, n) / 32;
+    return (unsigned)std::max(1LL, std::min((chunks + per - 1) / per, (long long)g->num_sms * (per == 1 ? 8 : per_sm)));
 }
 
 cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, double* eps, bool sums,
@@ -421,20 +392,20 @@ cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, dou
     if (pos_d == nullptr) {
         // diameters already in sorted order from the binning of these positions
         if (g->fp64)
-            CG_LAUNCH(g, "deposit_volume", k_deposit_volume_sorted<double>, nblk, 256, 0,
+            CG_LAUNCH(g, "deposit_volume", k_deposit_volume_sorted<double>, nblk, seg_threads(g, n), 0,
                       (const double*)g->vol_sorted, n, g->key_sorted, g->cell_start, g->gd, eps, (double*)part,
                       (long long)nblk, (int)sums, (double*)rec, (double*)eps_t);
         else
-            CG_LAUNCH(g, "deposit_volume", k_deposit_volume_sorted<float>, nblk, 256, 0,
+            CG_LAUNCH(g, "deposit_volume", k_deposit_volume_sorted<float>, nblk, seg_threads(g, n), 0,
                       (const float*)g->vol_sorted, n, g->key_sorted, g->cell_start, g->gd, eps, (float*)part,
                       (long long)nblk, (int)sums, (float*)rec, (float*)eps_t);
         return CG_OK;
     }
     if (g->fp64)
-        CG_LAUNCH(g, "deposit_volume", k_deposit_volume<double>, nblk, 256, 0, (const double*)pos_d, n, g->perm,
+        CG_LAUNCH(g, "deposit_volume", k_deposit_volume<double>, nblk, seg_threads(g, n), 0, (const double*)pos_d, n, g->perm,
                   g->key_sorted, g->cell_start, g->gd, eps, (double*)part, (long long)nblk, (int)sums);
     else
-        CG_LAUNCH(g, "deposit_volume", k_deposit_volume<float>, nblk, 256, 0, (const float*)pos_d, n, g->perm,
+        CG_LAUNCH(g, "deposit_volume", k_deposit_volume<float>, nblk, seg_threads(g, n), 0, (const float*)pos_d, n, g->perm,
                   g->key_sorted, g->cell_start, g->gd, eps, (float*)part, (long long)nblk, (int)sums);
     return CG_OK;
 }
@@ -442,12 +413,12 @@ cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, dou
 cg_status launch_deposit_sorted_force(cg_grids* g, long long n, void* S_bulk) {
     CG_CUDA(cudaMemsetAsync(S_bulk, 0, 3 * g->tsize * (size_t)g->gd.nbulk, g->stream));
     if (n == 0) return CG_OK;
-    const unsigned nblk = seg_blocks(g, n);
+    const unsigned nblk = seg_blocks(g, n, 5);
     if (g->fp64)
-        CG_LAUNCH(g, "deposit_momentum", k_deposit_sorted_force<double>, nblk, 256, 0, (const double*)g->Fs, n,
+        CG_LAUNCH(g, "deposit_momentum", k_deposit_sorted_force<double>, nblk, seg_threads(g, n), 0, (const double*)g->Fs, n,
                   g->key_sorted, g->cell_start, g->gd, (double*)S_bulk);
     else
-        CG_LAUNCH(g, "deposit_momentum", k_deposit_sorted_force<float>, nblk, 256, 0, (const float*)g->Fs, n,
+        CG_LAUNCH(g, "deposit_momentum", k_deposit_sorted_force<float>, nblk, seg_threads(g, n), 0, (const float*)g->Fs, n,
                   g->key_sorted, g->cell_start, g->gd, (float*)S_bulk);
     return CG_OK;
 }
@@ -457,10 +428,10 @@ cg_status launch_deposit_implicit(cg_grids* g, long long n, void* coef_bulk) {
     if (n == 0) return CG_OK;
     const unsigned nblk = seg_blocks(g, n);
     if (g->fp64)
-        CG_LAUNCH(g, "deposit_implicit", k_deposit_implicit<double>, nblk, 256, 0, (const double*)g->Bs.p, n,
+        CG_LAUNCH(g, "deposit_implicit", k_deposit_implicit<double>, nblk, seg_threads(g, n), 0, (const double*)g->Bs.p, n,
                   g->key_sorted, g->cell_start, g->gd, (double*)coef_bulk);
     else
-        CG_LAUNCH(g, "deposit_implicit", k_deposit_implicit<float>, nblk, 256, 0, (const float*)g->Bs.p, n,
+        CG_LAUNCH(g, "deposit_implicit", k_deposit_implicit<float>, nblk, seg_threads(g, n), 0, (const float*)g->Bs.p, n,
                   g->key_sorted, g->cell_start, g->gd, (float*)coef_bulk);
     return CG_OK;
 }
@@ -470,10 +441,10 @@ cg_status launch_deposit_momentum(cg_grids* g, long long n, const void* force_so
     if (n == 0) return CG_OK;
     const unsigned nblk = seg_blocks(g, n);
     if (g->fp64)
-        CG_LAUNCH(g, "deposit_momentum", k_deposit_momentum<double>, nblk, 256, 0, (const double*)force_soa, n,
+        CG_LAUNCH(g, "deposit_momentum", k_deposit_momentum<double>, nblk, seg_threads(g, n), 0, (const double*)force_soa, n,
                   g->perm, g->key_sorted, g->cell_start, g->gd, (double*)S_bulk);
     else
-        CG_LAUNCH(g, "deposit_momentum", k_deposit_momentum<float>, nblk, 256, 0, (const float*)force_soa, n,
+        CG_LAUNCH(g, "deposit_momentum", k_deposit_momentum<float>, nblk, seg_threads(g, n), 0, (const float*)force_soa, n,
                   g->perm, g->key_sorted, g->cell_start, g->gd, (float*)S_bulk);
     return CG_OK;
 }
