@@ -239,7 +239,7 @@ cg_status cg_grid_dims(const cg_grids* g, int32_t bulk_n[3], int64_t* n_bulk, in
  * cg_step_sorted, the particle at its slot i).  The result is the same
  * stable order whatever the particles did (moved, resized or permuted);
  * any share of them may change cell, and when a cell receives more than
- * 256 in one call the device falls back to the per-cell sort.  When none
+ * 32 in one call the device falls back to the per-cell sort.  When none
  * changed cell the bins are kept and only the sorted diameters are read
  * afresh.  A descriptor with a digit width (6..11) always sorts from
  * scratch. */

@@ -168,7 +168,6 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     dfree(g->rb_rid);
     dfree(g->rb_rkn);
     dfree(g->rb_mov);
-    dfree(g->rb_arr);
     dfree(g->rb_small);
     g->cap = -1;
     g->n_binned = -1;
@@ -192,17 +191,15 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     g->hist_cap = std::max<long long>(ntiles << maxbits, cap / 256 + 2);
     CG_TRY(dalloc(&g->hist, sizeof(int32_t) * g->hist_cap));
     // incremental rebinning: records per old slot, room for every particle to
-    // move (each block of old slots has its own part of the mover list), the
-    // arrival lists, per-cell and per-block counts
+    // move (each block of old slots has its own part of the mover list),
+    // per-cell and per-block counts
     g->rb_nblk = (cap + kRebinTile - 1) / kRebinTile;
     CG_TRY(dalloc(&g->rb_rid, sizeof(int32_t) * cap));
     CG_TRY(dalloc(&g->rb_rkn, sizeof(int32_t) * cap));
-    CG_TRY(dalloc(&g->rb_mov, sizeof(int2) * g->rb_nblk * kRebinTile));
-    CG_TRY(dalloc(&g->rb_arr, sizeof(int2) * cap));
+    CG_TRY(dalloc(&g->rb_mov, sizeof(int4) * g->rb_nblk * kRebinTile));
     CG_TRY(dalloc(&g->rb_small, sizeof(int32_t) * rebin_small_ints(g->gd.nbulk, g->rb_nblk)));
     const long long cells_blk = (g->gd.nbulk + 1 + kScanItems - 1) / kScanItems;
-    g->scan_cap = std::max((g->hist_cap + kScanItems - 1) / kScanItems + cells_blk,
-                           2 * cells_blk + (g->rb_nblk + 1 + kScanItems - 1) / kScanItems);
+    g->scan_cap = (g->hist_cap + kScanItems - 1) / kScanItems + cells_blk;
     CG_TRY(dalloc(&g->scan_part, sizeof(int32_t) * g->scan_cap));
     g->cap = cap;
     return CG_OK;
@@ -246,11 +243,11 @@ static void free_all(cg_grids* g) {
     dfree(g->rb_rid);
     dfree(g->rb_rkn);
     dfree(g->rb_mov);
-    dfree(g->rb_arr);
     dfree(g->rb_small);
     dfree(g->cell_start);
     dfree(g->bulk4);
     dfree(g->eps_t);
+    dfree(g->vol_acc);
     dfree(g->partials);
     dfree(g->sums_scratch);
     dfree(g->status);
@@ -358,7 +355,9 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     gd.Vff = (float)gd.Vf;
     split_ff(gd.VB, gd.VBh, gd.VBl);
     split_ff(gd.Vf, gd.Vfh, gd.Vfl);
-    split_ff(gd.invVB, gd.ivBh, gd.ivBl);
+    const double vc = 0.52359877559829887308 * gd.invVB;
+    split_ff(vc, gd.vch, gd.vcl);
+    gd.vcd57 = ldexp(vc, 57);
     gd.law = d.law;
     gd.interp = d.interp;
     gd.rho_f = d.rho_f;
@@ -375,6 +374,9 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     if (st == CG_OK) st = dalloc(&g->cell_start, sizeof(int32_t) * (nbulk + 1));
     if (st == CG_OK) st = dalloc(&g->bulk4, 4 * g->tsize * nbulk);
     if (st == CG_OK) st = dalloc(&g->eps_t, g->tsize * nbulk);
+    if (st == CG_OK) st = dalloc(&g->vol_acc, 3 * sizeof(unsigned long long) * nbulk);
+    if (st == CG_OK && cudaMemsetAsync(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk, g->stream) != cudaSuccess)
+        st = CG_ERR_CUDA;
     if (st == CG_OK) st = dalloc(&g->sums_scratch, sizeof(double) * CG_NSUMS);
     if (st == CG_OK) st = dalloc(&g->status, sizeof(unsigned long long) * kNumSlots);
     if (st == CG_OK && cudaMemset(g->status, 0, sizeof(unsigned long long) * kNumSlots) != cudaSuccess)
@@ -426,9 +428,7 @@ cg_status cg_grid_dims(const cg_grids* g, int32_t bulk_n[3], int64_t* n_bulk, in
 static cg_status check_n(long long n) { return (n < 0 || n > 2147483647LL) ? CG_ERR_OUT_OF_RANGE : CG_OK; }
 
 static cg_status copy_bins(cg_grids* g, long long n, int32_t* cell_out, int32_t* perm_out, int32_t* cs_out) {
-    if (cell_out && n) CG_TRY(ensure_keys(g, n));
-    if (cell_out && n)
-        CG_CUDA(cudaMemcpyAsync(cell_out, g->key, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, g->stream));
+    if (cell_out) CG_TRY(copy_cells(g, n, cell_out));
     if (perm_out && n)
         CG_CUDA(cudaMemcpyAsync(perm_out, g->perm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, g->stream));
     if (cs_out)
@@ -473,7 +473,11 @@ cg_status cg_deposit(cg_grids* g, int32_t kind, int64_t n, const void* per_parti
     if (!bulk_out || (n > 0 && !per_particle)) return CG_ERR_INVALID_ARG;
     if (kind == CG_DEP_VOLUME && n > 0 && !aligned16(per_particle)) return CG_ERR_INVALID_ARG;
     if (g->n_binned != n) return CG_ERR_NOT_BINNED;
-    if (kind == CG_DEP_VOLUME) return launch_deposit_volume(g, n, per_particle, (double*)bulk_out, false);
+    if (kind == CG_DEP_VOLUME) {
+        StepEps e;
+        e.eps = (double*)bulk_out;
+        return launch_deposit_volume(g, n, per_particle, &e);
+    }
     return launch_deposit_momentum(g, n, per_particle, bulk_out);
 }
 
@@ -555,26 +559,30 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     CG_CUDA(cudaEventRecord(g->ev_fork, g->stream));
     CG_CUDA(cudaStreamWaitEvent(side, g->ev_fork, 0));
     // the drag's packed record (eps, u) is written by the kernels that form its
-    // parts: the average (u, on the side stream), the binning (eps = 1 in every
-    // cell) and the porosity deposit (eps of occupied cells); with a closure
-    // or no particles it is packed from the outputs instead
+    // parts: the average (u, on the side stream) and the porosity's pass over
+    // the cells (eps; while binning when that is incremental, else after it);
+    // with a closure or no particles it is packed from the outputs instead
     const bool fused = !mlp && n > 0;
-    void* eps_t = o->eps_fine ? g->eps_t : nullptr;
     if (!mlp)
         CG_TRY(on_aux(g, [&] { return launch_average(g, u_fine, o->u_bulk, o->var_bulk, fused ? g->bulk4 : nullptr); }));
     CG_CUDA(cudaEventRecord(g->ev_avg, side));
-    if (fused) CG_TRY(launch_bin(g, n, p->pos_d, o->eps_bulk, g->bulk4, eps_t));
-    else CG_TRY(launch_bin(g, n, p->pos_d, o->eps_bulk));
-    CG_TRY(copy_bins(g, n, o->cell, o->perm, o->cell_start));
+    StepEps eps;
+    eps.eps = o->eps_bulk;
+    eps.S = o->S_bulk;
+    eps.rec = fused ? g->bulk4 : nullptr;
+    eps.eps_t = fused && o->eps_fine ? g->eps_t : nullptr;
+    eps.sums = true;
+    eps.ready = eps.eps_t ? g->ev_pack : nullptr;
+    CG_TRY(launch_bin(g, n, p->pos_d, &eps));
     // sorted diameters of this binning
-    if (fused) CG_TRY(launch_deposit_volume(g, n, nullptr, o->eps_bulk, true, true, g->bulk4, eps_t));
-    else CG_TRY(launch_deposit_volume(g, n, nullptr, o->eps_bulk, true, true));
+    if (!eps.formed) CG_TRY(launch_deposit_volume(g, n, nullptr, &eps));
+    CG_TRY(copy_bins(g, n, o->cell, o->perm, o->cell_start));
     if (!fused) {
         CG_CUDA(cudaStreamWaitEvent(g->stream, g->ev_avg, 0));
         CG_TRY(launch_pack(g, o->eps_bulk, o->u_bulk, o->eps_fine != nullptr));
     }
     if (o->eps_fine) {
-        CG_CUDA(cudaEventRecord(g->ev_pack, g->stream));
+        if (!eps.ready) CG_CUDA(cudaEventRecord(g->ev_pack, g->stream));
         CG_CUDA(cudaStreamWaitEvent(side, g->ev_pack, 0));
         const void* ein[4] = {g->eps_t, nullptr, nullptr, nullptr};
         void* eout[4] = {o->eps_fine, nullptr, nullptr, nullptr};
@@ -584,9 +592,9 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     CG_CUDA(cudaEventRecord(g->ev_epsf, side));
     if (mlp)
         CG_TRY(launch_drag_learned(g, mlp, n, p->pos_d, p->vel, o->var_bulk, u_fine, age, o->force, o->S_bulk,
-                                   dt));
+                                   dt, true));
     else
-        CG_TRY(launch_drag(g, n, p->pos_d, p->vel, o->force, o->S_bulk, true, dt, o->implicit_bulk,
+        CG_TRY(launch_drag(g, n, p->pos_d, p->vel, o->force, o->S_bulk, true, dt, true, o->implicit_bulk,
                            sorted_out ? sorted_out->pos_d : nullptr, sorted_out ? sorted_out->vel : nullptr));
     // the binning above lists the sorted output's particle i at slot i
     if (sorted_out && g->n_binned == n) g->hint_ident = sorted_out->pos_d;

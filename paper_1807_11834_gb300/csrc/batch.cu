@@ -125,7 +125,6 @@ cg_status plan(cg_batch* b) {
         I.pos = (float*)it.particles.pos_d;
         I.vel = (float*)it.particles.vel;
         I.u_fine = (const float*)it.u_fine;
-        I.eps = it.out.eps_bulk;
         I.u_bulk = (float*)it.out.u_bulk;
         I.var = (float*)it.out.var_bulk;
         I.S_bulk = (float*)it.out.S_bulk;
@@ -147,6 +146,12 @@ cg_status plan(cg_batch* b) {
         I.bulk4 = (float*)g->bulk4;
         I.eps_t = (float*)g->eps_t;
         I.status = g->status;
+        StepEps se;
+        se.eps = it.out.eps_bulk;
+        se.rec = I.bulk4;
+        se.eps_t = I.eps_fine ? I.eps_t : nullptr;
+        se.S = I.S_bulk;
+        I.eps_out = eps_out<float>(g, &se);
         // batch-owned scratch: digit histograms, scan partials, sum partials
         const long long m0 = I.cellsort ? 0 : (long long)I.ntiles << I.b0;
         const long long m1 = (long long)I.ntiles << I.b1;
@@ -176,7 +181,7 @@ cg_status plan(cg_batch* b) {
         const long long chunks = cdiv(n, kSegChunk);
         const long long seg = std::max(1LL, cdiv(chunks, 8LL * c.seg_chunks));
         const long long cellb = cdiv(nb, 256);
-        set(BP_ZERO, cdiv(3 * nb, 1024));
+        set(BP_ZERO, cdiv(nb + 1, 1024));
         set(BP_KEY, I.cellsort ? cdiv(n, (long long)kSortThreads * kKeyItems) : I.ntiles);
         set(BP_SCAN0_R, I.scan0.nblk[0] + I.scan0.nblk[1]);
         set(BP_SCAN0_D, I.scan0.nblk[0] + I.scan0.nblk[1]);
@@ -187,7 +192,7 @@ cg_status plan(cg_batch* b) {
         set(BP_SCAT1, I.npasses == 2 ? I.ntiles : 0);
         set(BP_PLACE, I.cellsort ? cdiv(n, 512LL * kPlaceItems) : 0);
         set(BP_SEGSORT, I.cellsort ? cdiv(nb, (long long)kGroupCells * kSegSortWarps) : 0);
-        set(BP_DEPV, seg);
+        set(BP_DEPV, std::max(1LL, cdiv(n, 1024LL * c.seg_chunks)));
         set(BP_AVG, std::max(1LL, cdiv(nb * average_lanes(g->gd.r, false), 256LL * c.avg_items)));
         set(BP_PACK, cellb);
         set(BP_DRAG, std::max(1LL, cdiv(n, 256LL * c.drag_items)));
@@ -199,12 +204,12 @@ cg_status plan(cg_batch* b) {
         set(BP_PROJE, I.eps_fine ? cdiv(project_threads(g->gd, I.depth_eps), 256) : 0);
         set(BP_SUMS, CG_NSUMS);
         // partial regions (pairs): volume 1 column, projection 6 (S_f V_f, S_B V_B), drag 9
-        I.part_blocks[PS_VOL] = seg;
+        I.part_blocks[PS_VOL] = cellb;
         I.part_blocks[PS_PROJ] = projb;
         I.part_blocks[PS_DRAG] = B[(size_t)BP_DRAG * ni];
         I.part_off[PS_VOL] = 0;
-        I.part_off[PS_PROJ] = seg;
-        I.part_off[PS_DRAG] = seg + 6 * projb;
+        I.part_off[PS_PROJ] = cellb;
+        I.part_off[PS_DRAG] = cellb + 6 * projb;
         const long long pairs = I.part_off[PS_DRAG] + (long long)kDragSums * I.part_blocks[PS_DRAG];
         CG_TRY(dev_alloc(b, (void**)&I.part, sizeof(float) * 2 * pairs));
         I.smap = sums_map(I.part_off, I.part_blocks);

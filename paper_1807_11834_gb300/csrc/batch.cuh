@@ -29,7 +29,7 @@ struct BInst {
     float* vel;
     const float* u_fine;
     // outputs (cg_step_out of the instance)
-    double* eps;
+    EpsOut<float> eps_out;
     float* u_bulk;
     float* var;
     float* S_bulk;

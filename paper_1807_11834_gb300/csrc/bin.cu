@@ -53,9 +53,7 @@ template <typename T>
 __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long long n, const GridDev& g,
                                              int32_t* __restrict__ key, int32_t* __restrict__ count,
                                              int32_t* __restrict__ hist, int ntiles, int bits0, T* __restrict__ vol,
-                                             unsigned long long* __restrict__ status, int* sh, Blk blk,
-                                             double* __restrict__ eps_fill = nullptr, T* __restrict__ rec_fill = nullptr,
-                                             T* __restrict__ eps_t_fill = nullptr) {
+                                             unsigned long long* __restrict__ status, int* sh, Blk blk) {
     __shared__ int s_cnt[2];
     const int R = 1 << bits0;
     for (int i = threadIdx.x; i < R; i += blockDim.x) sh[i] = 0;
@@ -77,10 +75,10 @@ __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long lon
         int c = -1;
         if (valid) {
             const V4<T>& v = pv[k];
-            int outside = 0;
-            if (!(isfinite(v.x) && isfinite(v.y) && isfinite(v.z))) n_nf++;
-            c = cell_of(v, g, outside);
+            int outside = 0, nonfinite = 0;
+            c = cell_of(v, g, outside, nonfinite);
             n_out += outside;
+            n_nf += nonfinite;
             key[p] = c;
             vol[p] = v.w;   // the diameter: the porosity forms the volume as an exact pair
         }
@@ -97,31 +95,20 @@ __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long lon
     __syncthreads();
     for (int i = threadIdx.x; i < R; i += blockDim.x) hist[(long long)i * ntiles + blk.id] = sh[i];
     if (threadIdx.x == 0) add_status(status, s_cnt[0], s_cnt[1]);
-    // the porosity of cells without particles is 1: set every cell here (and
-    // the porosity of the drag record and of its path-precision copy), the
-    // deposit overwrites the occupied ones (saves launches in the step)
-    if (eps_fill)
-        for (long long c = blk.id * blockDim.x + threadIdx.x; c < g.nbulk; c += blk.n * blockDim.x) {
-            eps_fill[c] = 1.0;
-            if (rec_fill) rec_fill[4 * c] = T(1);
-            if (eps_t_fill) eps_t_fill[c] = T(1);
-        }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kSortThreads)
 k_bin_key(const T* __restrict__ pos, long long n, GridDev g, int32_t* __restrict__ key,
           int32_t* __restrict__ count, int32_t* __restrict__ hist, int ntiles, int bits0,
-          T* __restrict__ vol, unsigned long long* __restrict__ status, double* __restrict__ eps_fill,
-          T* __restrict__ rec_fill, T* __restrict__ eps_t_fill) {
+          T* __restrict__ vol, unsigned long long* __restrict__ status) {
     pdl_wait();
     extern __shared__ int sh[];
-    bin_key_body<T>(pos, n, g, key, count, hist, ntiles, bits0, vol, status, sh, launch_blk(), eps_fill, rec_fill,
-                    eps_t_fill);
+    bin_key_body<T>(pos, n, g, key, count, hist, ntiles, bits0, vol, status, sh, launch_blk());
 }
 
 // Key kernel of the per-cell sort: cell, diameter and arrival rank of every
-// particle, per-cell counts, porosity fill.  No shared memory and no block
+// particle, per-cell counts.  No shared memory and no block
 // barrier; a block takes 4 x (its threads) particles, four per thread,
 // consecutive lanes on consecutive particles (so runs of equal cells share
 // one count atomic), and the thread's count atomics are issued together so
@@ -131,8 +118,7 @@ template <typename T>
 __device__ __forceinline__ void bin_key_rank_body(const T* __restrict__ pos, long long n, const GridDev& g,
                                                   int32_t* __restrict__ key, int32_t* __restrict__ count,
                                                   T* __restrict__ vol, unsigned long long* __restrict__ status,
-                                                  double* __restrict__ eps_fill, T* __restrict__ rec_fill,
-                                                  T* __restrict__ eps_t_fill, int32_t* __restrict__ arrival, Blk blk) {
+                                                  int32_t* __restrict__ arrival, Blk blk) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const long long base = blk.id * (long long)(blockDim.x * kKeyItems);
@@ -151,10 +137,10 @@ __device__ __forceinline__ void bin_key_rank_body(const T* __restrict__ pos, lon
         int c = -1;
         if (valid) {
             const V4<T>& v = pv[k];
-            int outside = 0;
-            if (!(isfinite(v.x) && isfinite(v.y) && isfinite(v.z))) n_nf++;
-            c = cell_of(v, g, outside);
+            int outside = 0, nonfinite = 0;
+            c = cell_of(v, g, outside, nonfinite);
             n_out += outside;
+            n_nf += nonfinite;
             key[p] = c;
             vol[p] = v.w;   // the diameter: the porosity forms the volume as an exact pair
         }
@@ -176,25 +162,15 @@ __device__ __forceinline__ void bin_key_rank_body(const T* __restrict__ pos, lon
     n_out = __reduce_add_sync(full, n_out);
     n_nf = __reduce_add_sync(full, n_nf);
     if (lane == 0 && (n_out | n_nf)) add_status(status, n_out, n_nf);
-    // the porosity of cells without particles is 1: set every cell here (and
-    // the porosity of the drag record and of its path-precision copy), the
-    // deposit overwrites the occupied ones
-    if (eps_fill)
-        for (long long c = blk.id * blockDim.x + threadIdx.x; c < g.nbulk; c += blk.n * blockDim.x) {
-            eps_fill[c] = 1.0;
-            if (rec_fill) rec_fill[4 * c] = T(1);
-            if (eps_t_fill) eps_t_fill[c] = T(1);
-        }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kKeyThreads, 5)
 k_bin_key_rank(const T* __restrict__ pos, long long n, GridDev g, int32_t* __restrict__ key,
                int32_t* __restrict__ count, T* __restrict__ vol, unsigned long long* __restrict__ status,
-               double* __restrict__ eps_fill, T* __restrict__ rec_fill, T* __restrict__ eps_t_fill,
                int32_t* __restrict__ arrival) {
     pdl_wait();
-    bin_key_rank_body<T>(pos, n, g, key, count, vol, status, eps_fill, rec_fill, eps_t_fill, arrival, launch_blk());
+    bin_key_rank_body<T>(pos, n, g, key, count, vol, status, arrival, launch_blk());
 }
 
 // Tile histogram of a digit of already-computed keys (second pass).
@@ -407,8 +383,8 @@ __device__ __forceinline__ void scan_locate(const ScanJob& j, long long id, int&
     }
 }
 
-// Blocks of a job: [0, nblk[0]) over array 0, then nblk[1] over array 1,
-// then nblk[2] over array 2; part holds one total per block of the job.
+// Blocks of a job: [0, nblk[0]) over array 0, then nblk[1] over array 1; part
+// holds one total per block of the job.
 __device__ __forceinline__ void scan_reduce_body(const ScanJob& j, int32_t* __restrict__ part, Blk b) {
     __shared__ int shw[32];
     int which;
@@ -427,7 +403,6 @@ __device__ __forceinline__ void scan_reduce_body(const ScanJob& j, int32_t* __re
 
 __global__ void __launch_bounds__(256) k_scan_reduce(ScanJob j, int32_t* __restrict__ part) {
     pdl_wait();
-    if (j.skip && __ldg(j.skip) == 0) return;
     scan_reduce_body(j, part, launch_blk());
 }
 
@@ -465,24 +440,22 @@ __device__ __forceinline__ void scan_down_body(const ScanJob& j, const int32_t* 
 
 __global__ void __launch_bounds__(256) k_scan_down(ScanJob j, const int32_t* __restrict__ part) {
     pdl_wait();
-    if (j.skip && __ldg(j.skip) == 0) return;
     scan_down_body(j, part, launch_blk());
 }
 
-// Exclusive scans of up to three arrays by one pair of launches (out may
-// alias in; an array with in == nullptr is skipped).  skip (device, may be
-// null): when it reads 0 the launches return at once, the caller having
-// left the outputs in their scanned form.
-cg_status scan_exclusive(cg_grids* g, int count, const int32_t* const* in, int32_t* const* out, const long long* m,
-                         const int32_t* skip) {
+// Exclusive scans of up to two arrays by one pair of launches (out may alias
+// in; an array with inB == nullptr is skipped).
+static cg_status scan_exclusive2(cg_grids* g, const int32_t* inA, int32_t* outA, long long mA,
+                                 const int32_t* inB, int32_t* outB, long long mB) {
     ScanJob j;
-    j.skip = skip;
+    const int32_t* in[2] = {inA, inB};
+    int32_t* out[2] = {outA, outB};
+    const long long m[2] = {mA, mB};
     long long nblk = 0;
     for (int a = 0; a < kScanArrays; ++a) {
-        const bool use = a < count && in[a];
-        j.in[a] = use ? in[a] : nullptr;
-        j.out[a] = use ? out[a] : nullptr;
-        j.m[a] = use ? m[a] : 0;
+        j.in[a] = in[a];
+        j.out[a] = in[a] ? out[a] : nullptr;
+        j.m[a] = in[a] ? m[a] : 0;
         j.nblk[a] = (j.m[a] + kScanItems - 1) / kScanItems;
         nblk += j.nblk[a];
     }
@@ -492,15 +465,6 @@ cg_status scan_exclusive(cg_grids* g, int count, const int32_t* const* in, int32
     CG_LAUNCH(g, "bin_scan", k_scan_down, (unsigned)nblk, 256, 0, j, g->scan_part);
     return CG_OK;
 }
-
-static cg_status scan_exclusive2(cg_grids* g, const int32_t* inA, int32_t* outA, long long mA,
-                                 const int32_t* inB, int32_t* outB, long long mB) {
-    const int32_t* in[2] = {inA, inB};
-    int32_t* out[2] = {outA, outB};
-    const long long m[2] = {mA, mB};
-    return scan_exclusive(g, 2, in, out, m);
-}
-
 
 // ----------------------------------------------------------------------
 // Default sort: arrival rank, placement, and a sort of every cell's ids.
@@ -544,14 +508,11 @@ __device__ __forceinline__ void place_body(const int32_t* __restrict__ key, cons
     }
 }
 
-// run_if (nullable): the kernel does nothing unless *run_if is non-zero
-// (the fallback of the incremental rebinning, decided on the device).
 __global__ void __launch_bounds__(512) k_bin_place(const int32_t* __restrict__ key,
                                                    const int32_t* __restrict__ arrival,
                                                    const int32_t* __restrict__ cell_start, long long n,
-                                                   int32_t* __restrict__ tmp, const int32_t* __restrict__ run_if) {
+                                                   int32_t* __restrict__ tmp) {
     pdl_wait();
-    if (run_if && *run_if == 0) return;
     place_body(key, arrival, cell_start, n, tmp, launch_blk());
 }
 
@@ -590,15 +551,16 @@ __device__ __forceinline__ void warp_bitonic(int (&v)[K]) {
     }
 }
 
-// Outputs of one sorted slot: the id, its cell, its inverse, its diameter.
+// Outputs of one sorted slot: the id, its cell, and (nullable) its inverse and
+// its diameter.
 template <typename T>
 __device__ __forceinline__ void emit_slot(long long slot, int id, int cell, int32_t* __restrict__ perm,
                                           int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
                                           const T* __restrict__ vol, T* __restrict__ vol_sorted) {
     perm[slot] = id;
     key_sorted[slot] = cell;
-    inv_perm[id] = (int)slot;
-    vol_sorted[slot] = __ldg(vol + id);
+    if (inv_perm) inv_perm[id] = (int)slot;
+    if (vol_sorted) vol_sorted[slot] = __ldg(vol + id);
 }
 
 // Sort the c (<= 32 K) ids at src (shared memory when staged, else global)
@@ -792,15 +754,15 @@ __device__ __forceinline__ void seg_sort_body(const int32_t* __restrict__ cell_s
                     for (int u = 0; u < U; ++u) {
                         const int i = i0 + u * 32;
                         id[u] = i < m ? stage[i] : -1;
-                        if (id[u] >= 0) d[u] = __ldg(vol + id[u]);
+                        if (id[u] >= 0 && vol_sorted) d[u] = __ldg(vol + id[u]);
                     }
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const long long slot = (long long)s0 + i0 + u * 32;
                         if (id[u] >= 0) {
                             perm[slot] = id[u];
-                            inv_perm[id[u]] = (int)slot;
-                            vol_sorted[slot] = d[u];
+                            if (inv_perm) inv_perm[id[u]] = (int)slot;
+                            if (vol_sorted) vol_sorted[slot] = d[u];
                         }
                     }
                 }
@@ -821,10 +783,22 @@ template <typename T>
 __global__ void __launch_bounds__(kSegSortWarps * 32, 4)
 k_seg_sort(const int32_t* __restrict__ cell_start, long long nbulk, int32_t* tmp, int32_t* alt,
            int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-           const T* __restrict__ vol, T* __restrict__ vol_sorted, const int32_t* __restrict__ run_if) {
+           const T* __restrict__ vol, T* __restrict__ vol_sorted) {
     pdl_wait();
-    if (run_if && *run_if == 0) return;
     seg_sort_body<T>(cell_start, nbulk, tmp, alt, perm, key_sorted, inv_perm, vol, vol_sorted, launch_blk());
+}
+
+// The last kernel of an incremental rebinning: the new starts to their
+// place, and in the fallback (run_if) the sort of every cell.
+__global__ void __launch_bounds__(kSegSortWarps * 32, 4)
+k_seg_sort_fallback(const int32_t* __restrict__ cs, long long nbulk, int32_t* tmp, int32_t* alt,
+                    int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
+                    const int32_t* __restrict__ run_if, int32_t* __restrict__ cs_copy) {
+    pdl_wait();
+    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c <= nbulk; c += (long long)gridDim.x * blockDim.x)
+        cs_copy[c] = __ldg(cs + c);
+    if (*run_if == 0) return;
+    seg_sort_body<float>(cs, nbulk, tmp, alt, perm, key_sorted, inv_perm, nullptr, nullptr, launch_blk());
 }
 
 static PerDeviceOnce g_attr_once;
@@ -848,13 +822,12 @@ static cg_status set_attrs() {
 }
 
 template <typename T>
-static cg_status bin_passes(cg_grids* g, long long n, const T* pos, int ntiles, long long m0, double* eps_fill,
-                            T* rec_fill, T* eps_t_fill) {
+static cg_status bin_passes(cg_grids* g, long long n, const T* pos, int ntiles, long long m0) {
     const long long nbulk = g->gd.nbulk;
     const int np = g->npasses;
     const int b0 = g->pass_bits[0];
     CG_LAUNCH(g, "bin_key", k_bin_key<T>, ntiles, kSortThreads, sizeof(int) << b0, pos, n, g->gd, g->key,
-              g->cell_start, g->hist, ntiles, b0, (T*)g->vol, g->status, eps_fill, rec_fill, eps_t_fill);
+              g->cell_start, g->hist, ntiles, b0, (T*)g->vol, g->status);
     CG_TRY(scan_exclusive2(g, g->cell_start, g->cell_start, nbulk + 1, g->hist, g->hist, m0));
     // pass p reads (keys, ids) from in[p] and writes them to in[p + 1]; the
     // last pass writes the final order
@@ -895,34 +868,26 @@ static cg_status bin_passes(cg_grids* g, long long n, const T* pos, int ntiles, 
 // Default sort: key + arrival rank, scan of the counts (two launches),
 // placement, per-cell sort.
 template <typename T>
-static cg_status bin_rank(cg_grids* g, long long n, const T* pos, int ntiles, double* eps_fill, T* rec_fill,
-                          T* eps_t_fill) {
+static cg_status bin_rank(cg_grids* g, long long n, const T* pos) {
     const long long nbulk = g->gd.nbulk;
     const long long kb = (n + kKeyThreads * kKeyItems - 1) / (kKeyThreads * kKeyItems);
     CG_LAUNCH(g, "bin_key", k_bin_key_rank<T>, (unsigned)kb, kKeyThreads, 0, pos, n, g->gd, g->key, g->cell_start,
-              (T*)g->vol, g->status, eps_fill, rec_fill, eps_t_fill, g->key2);
+              (T*)g->vol, g->status, g->key2);
     CG_TRY(scan_exclusive2(g, g->cell_start, g->cell_start, nbulk + 1, nullptr, nullptr, 0));
-    return launch_cellsort_tail(g, n, g->cell_start, nullptr);
+    const long long pb = std::min<long long>((n + 512 * kPlaceItems - 1) / (512 * kPlaceItems), (long long)g->num_sms * 4);
+    CG_LAUNCH(g, "bin_place", k_bin_place, (unsigned)pb, 512, 0, g->key, g->key2, g->cell_start, n, g->val1);
+    const long long sb = std::min<long long>((nbulk + kGroupCells * kSegSortWarps - 1) / (kGroupCells * kSegSortWarps),
+                                             (long long)g->num_sms * 4);
+    CG_LAUNCH(g, "bin_seg_sort", k_seg_sort<T>, (unsigned)sb, kSegSortWarps * 32, 0, g->cell_start, nbulk, g->val1,
+              g->key1, g->perm, g->key_sorted, g->inv_perm, (const T*)g->vol, (T*)g->vol_sorted);
+    return CG_OK;
 }
 
-// Placement and per-cell sort of the per-cell sort, from the cell starts cs
-// and the arrival ranks in key2 (the keys in key, the diameters in vol).
-cg_status launch_cellsort_tail(cg_grids* g, long long n, const int32_t* cs, const int32_t* run_if) {
-    const long long nbulk = g->gd.nbulk;
-    // as the device's fallback (run_if set) the kernels are usually idle: one
-    // grid-stride CTA per SM keeps an idle launch short
-    const long long per_sm = run_if ? 1 : 4;
-    const long long pb = std::min<long long>((n + 512 * kPlaceItems - 1) / (512 * kPlaceItems),
-                                             (long long)g->num_sms * per_sm);
-    CG_LAUNCH(g, "bin_place", k_bin_place, (unsigned)pb, 512, 0, g->key, g->key2, cs, n, g->val1, run_if);
-    const long long sb = std::min<long long>((nbulk + kGroupCells * kSegSortWarps - 1) / (kGroupCells * kSegSortWarps),
-                                             (long long)g->num_sms * per_sm);
-    if (g->fp64)
-        CG_LAUNCH(g, "bin_seg_sort", k_seg_sort<double>, (unsigned)sb, kSegSortWarps * 32, 0, cs, nbulk, g->val1,
-                  g->key1, g->perm, g->key_sorted, g->inv_perm, (const double*)g->vol, (double*)g->vol_sorted, run_if);
-    else
-        CG_LAUNCH(g, "bin_seg_sort", k_seg_sort<float>, (unsigned)sb, kSegSortWarps * 32, 0, cs, nbulk, g->val1,
-                  g->key1, g->perm, g->key_sorted, g->inv_perm, (const float*)g->vol, (float*)g->vol_sorted, run_if);
+cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, const int32_t* run_if, int32_t* cs_copy,
+                                   int32_t* inv_perm) {
+    // usually only the copy: one grid-stride CTA per SM keeps the launch short
+    CG_LAUNCH(g, "rebin_starts", k_seg_sort_fallback, (unsigned)g->num_sms, kSegSortWarps * 32, 0, cs, g->gd.nbulk,
+              g->val1, g->key1, g->perm, g->key_sorted, inv_perm, run_if, cs_copy);
     return CG_OK;
 }
 
@@ -965,8 +930,7 @@ __global__ void __launch_bounds__(kSortThreads) kb_bin_key(BLaunch L) {
     extern __shared__ int sh[];
     batch_loop(L, [&](const BInst& I, Blk b) {
         if (I.cellsort)
-            bin_key_rank_body<float>(I.pos, I.n, I.gd, I.key, I.count, I.vol, I.status, nullptr, nullptr, nullptr,
-                                     I.arrival, b);
+            bin_key_rank_body<float>(I.pos, I.n, I.gd, I.key, I.count, I.vol, I.status, I.arrival, b);
         else
             bin_key_body<float>(I.pos, I.n, I.gd, I.key, I.count, I.hist, I.ntiles, I.b0, I.vol, I.status, sh, b);
     });
@@ -1070,60 +1034,46 @@ int batch_bin_occupancy(int phase, size_t smem) {
     return occ > 0 ? occ : 1;
 }
 
-cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, double* eps_fill, void* rec_fill,
-                     void* eps_t_fill) {
+cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps) {
     CG_TRY(set_attrs());
     const long long nbulk = g->gd.nbulk;
     // a binning of the same count held by the handle is the starting point
     // (rebin.cu), unless the descriptor asks for a digit sort
-    const bool rebin = n > 0 && g->rb_rkn && g->hint_n == n && n <= g->cap &&
+    const bool rebin = n > 0 && n < kRebinMaxParticles && g->rb_rkn && g->hint_n == n && n <= g->cap &&
                        (g->desc.sort_digits == CG_SORT_AUTO || g->desc.sort_digits == CG_SORT_CELLS);
     const bool ident = rebin && pos_d == g->hint_ident;
+    // a binning that finds no mover leaves perm and inv_perm as they are
+    if (rebin && !ident) CG_TRY(ensure_inverse(g, n));
     g->hint_n = -1;
     g->hint_ident = nullptr;
     g->n_binned = -1;
-    g->vol_valid = false;
-    g->key_valid = true;   // written by every path but the identity-hint rebinning
     if (rebin) {
-        CG_TRY(launch_rebin(g, n, pos_d, ident, eps_fill, rec_fill, eps_t_fill));
+        CG_TRY(launch_rebin(g, n, pos_d, ident, eps));
         g->n_binned = n;
-        g->vol_valid = true;
-        g->key_valid = !ident;
+        g->key_valid = false;
+        g->inv_valid = !ident;
         g->hint_n = n;
         return CG_OK;
     }
+    g->key_valid = g->inv_valid = true;
     // count[] lives in cell_start; the exclusive scan turns it into starts
     CG_CUDA(cudaMemsetAsync(g->cell_start, 0, sizeof(int32_t) * (nbulk + 1), g->stream));
     if (n == 0) {
         g->n_binned = 0;
-        g->vol_valid = true;
         return CG_OK;
     }
     const int ntiles = (int)((n + kSortTile - 1) / kSortTile);
     const long long m0 = (long long)ntiles << g->pass_bits[0];
     if (use_cell_sort(g->desc.sort_digits, n, nbulk)) {
-        if (g->fp64)
-            CG_TRY(bin_rank<double>(g, n, (const double*)pos_d, ntiles, eps_fill, (double*)rec_fill,
-                                    (double*)eps_t_fill));
-        else
-            CG_TRY(bin_rank<float>(g, n, (const float*)pos_d, ntiles, eps_fill, (float*)rec_fill,
-                                   (float*)eps_t_fill));
-        g->n_binned = n;
-        g->vol_valid = true;
-        g->hint_n = n;
-        return CG_OK;
+        if (g->fp64) CG_TRY(bin_rank<double>(g, n, (const double*)pos_d));
+        else CG_TRY(bin_rank<float>(g, n, (const float*)pos_d));
+    } else {
+        for (int p = 0; p < g->npasses; ++p)
+            if (((long long)ntiles << g->pass_bits[p]) > g->hist_cap) return CG_ERR_OUT_OF_RANGE;
+        if (g->fp64) CG_TRY(bin_passes<double>(g, n, (const double*)pos_d, ntiles, m0));
+        else CG_TRY(bin_passes<float>(g, n, (const float*)pos_d, ntiles, m0));
     }
-    for (int p = 0; p < g->npasses; ++p)
-        if (((long long)ntiles << g->pass_bits[p]) > g->hist_cap) return CG_ERR_OUT_OF_RANGE;
-
-    if (g->fp64)
-        CG_TRY(bin_passes<double>(g, n, (const double*)pos_d, ntiles, m0, eps_fill, (double*)rec_fill,
-                                  (double*)eps_t_fill));
-    else
-        CG_TRY(bin_passes<float>(g, n, (const float*)pos_d, ntiles, m0, eps_fill, (float*)rec_fill,
-                                 (float*)eps_t_fill));
     g->n_binned = n;
-    g->vol_valid = true;
     g->hint_n = n;
     return CG_OK;
 }

@@ -117,12 +117,13 @@ struct GridDev {
     float xhif[3];      // (float)xhi
     float invHf[3];     // (float)(1/H)
     float ax0f[3];      // |x0 / H| (filter margin term)
+    float vch, vcl;     // pi / (6 V_B) as float-float: a sphere's volume over V_B is this times d^3
+    double vcd57;       // 2^57 pi / (6 V_B)
     float x0h[3], x0l[3];   // x0 as float-float
     float ihh[3], ihl[3];   // 1/H as float-float
     float xbh[3], xbl[3];   // -(x0 / H + 1/2) as float-float: the lattice coordinate is x / H + xb
     float invVBf, VBf, Vff;
     float VBh, VBl, Vfh, Vfl;   // V_B, V_f as float-float
-    float ivBh, ivBl;           // 1 / V_B as float-float
     // physics
     int law, interp;
     double rho_f, mu_f, rho_p, eps_switch, eps_min, g[3];
@@ -183,8 +184,8 @@ struct cg_grids {
     void* vol = nullptr;           // [cap] T particle diameter, caller order (for the volume deposit)
     void* vol_sorted = nullptr;    // [cap] T particle diameter, sorted order
     void* Fs = nullptr;            // [cap] T4 drag force, sorted order
-    bool vol_valid = false;        // vol_sorted matches the binned positions
-    bool key_valid = false;        // key holds the binning's caller-order cells (see ensure_keys)
+    bool key_valid = false;        // key holds the binning's caller-order cells (see copy_cells)
+    bool inv_valid = false;        // inv_perm holds the binning's inverse (see ensure_inverse)
     // incremental rebinning (rebin.cu): a binning of hint_n particles held in
     // perm / key_sorted / cell_start is where the next binning of the same
     // count starts; hint_ident is the particle array the last sorted step
@@ -193,9 +194,9 @@ struct cg_grids {
     const void* hint_ident = nullptr;
     int32_t* rb_rid = nullptr;     // [cap] per old slot: its particle id (the caller's order kept)
     int32_t* rb_rkn = nullptr;     // [cap] per old slot: the new cell, complemented for a mover
-    int2* rb_mov = nullptr;        // [rb_nblk * kRebinTile] movers, each block of old slots its own part: (id, cell | rank << 22)
-    int2* rb_arr = nullptr;        // [cap] arrivals grouped by cell: (id, cell)
-    int32_t* rb_small = nullptr;   // new counts / starts, arrivals, departures per cell; block movers; counters
+    int4* rb_mov = nullptr;        // [rb_nblk * kRebinTile] movers, each block of old slots its own part:
+                                   // (id, new cell, next mover of that cell + 1, arrival rank)
+    int32_t* rb_small = nullptr;   // per-cell and per-block counts, starts, list heads; counters (rebin_ptrs)
     long long rb_nblk = 0;
     int32_t* hist = nullptr;       // [2^digit * ntiles]
     int32_t* scan_part = nullptr;  // scan block partials
@@ -205,6 +206,7 @@ struct cg_grids {
     int32_t* cell_start = nullptr; // [nbulk + 1]
     void* bulk4 = nullptr;         // [nbulk] T4: eps, u_x, u_y, u_z
     void* eps_t = nullptr;         // [nbulk] T: porosity in the path precision
+    unsigned long long* vol_acc = nullptr;   // [nbulk][2] volume accumulators, then [nbulk] double (see EpsOut)
     void* partials = nullptr;      // conservation-sum block partials: (s, c) pairs of T
     long long part_off[cg::PS_NREG] = {0, 0, 0};
     long long part_blocks[cg::PS_NREG] = {0, 0, 0};
@@ -295,15 +297,14 @@ void prof_end(cg_grids* g, int slot, int ev);
 // ----------------------------------------------------------------------
 // Step launchers (one .cu each)
 // ----------------------------------------------------------------------
-// Up to three independent arrays are scanned by one pair of launches: blocks
-// [0, n0) cover array 0, blocks [n0, n0 + n1) array 1, and so on.
-constexpr int kScanArrays = 3;
+// Up to two independent arrays are scanned by one pair of launches: blocks
+// [0, n0) cover array 0, the others array 1.
+constexpr int kScanArrays = 2;
 struct ScanJob {
     const int32_t* in[kScanArrays] = {};
     int32_t* out[kScanArrays] = {};
     long long m[kScanArrays] = {};
     long long nblk[kScanArrays] = {};
-    const int32_t* skip = nullptr;   // device flag: when 0, the outputs already hold the scans and nothing runs
 };
 
 // Column map of the conservation-sum reduction: sum k merges cnt[k]
@@ -314,43 +315,55 @@ struct SumsMap {
 };
 
 cg_status ensure_particle_capacity(cg_grids* g, long long n);
-// Exclusive scans of up to kScanArrays int32 arrays (in[a] nullable: skipped).
-cg_status scan_exclusive(cg_grids* g, int count, const int32_t* const* in, int32_t* const* out, const long long* m,
-                         const int32_t* skip = nullptr);
-// Placement and per-cell sort of the per-cell binning sort from the cell
-// starts cs; with run_if set they do nothing unless *run_if != 0.
-cg_status launch_cellsort_tail(cg_grids* g, long long n, const int32_t* cs, const int32_t* run_if);
+// The per-cell sort of the ids placed in val1 from the cell starts cs, as the
+// fallback of the incremental rebinning (does nothing but copy cs to cs_copy
+// unless *run_if != 0).
+cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, const int32_t* run_if, int32_t* cs_copy,
+                                   int32_t* inv_perm);
 // Incremental rebinning (rebin.cu).
 constexpr int kRebinThreads = 256;
 constexpr int kRebinItems = 4;
 constexpr int kRebinTile = kRebinThreads * kRebinItems;   // old slots per block
-constexpr int kRebinMaxArrivals = 256;                     // arrivals per cell before the fallback
+constexpr int kRebinScan = 1024;                           // elements per block of its scans
+constexpr int kRebinMaxArrivals = 32;                      // arrivals per cell before the fallback
+constexpr long long kRebinMaxParticles = 1LL << 30;        // the porosity accumulators' limit (a longer list is sorted)
 constexpr int kRebinCounters = 8;
-// The small rebinning arrays (three of n_b + 1 ints, one of nblk + 1, the
-// counters) each start on a 256-byte boundary: the scan reads them as int4.
+// The small rebinning arrays each start on a 256-byte boundary (the scan reads
+// them as int4): the counts (n_b + 1), the departures per block (nblk + 1), the
+// arrivals with the list heads (2 (n_b + 1)), the departures per cell, the
+// counters, the scans' block totals.
 inline long long rebin_pad(long long ints) { return (ints + 63) / 64 * 64; }
+inline long long rebin_tiles(long long m) { return (m + kRebinScan - 1) / kRebinScan; }
 inline long long rebin_small_ints(long long nbulk, long long nblk) {
-    return 3 * rebin_pad(nbulk + 1) + rebin_pad(nblk + 1) + kRebinCounters;
+    return 4 * rebin_pad(nbulk + 1) + rebin_pad(nblk + 1) + rebin_pad(kRebinCounters) + 2 * rebin_tiles(nbulk + 1) +
+           rebin_tiles(nblk + 1);
 }
+// Where a step wants its porosity (EpsOut), formed while binning when the
+// binning is incremental; sums: also the deposited volume's partials.
+struct StepEps {
+    double* eps = nullptr;
+    void* rec = nullptr;
+    void* eps_t = nullptr;
+    void* S = nullptr;
+    bool sums = false;
+    bool formed = false;             // set by the binning when it formed the porosity
+    cudaEvent_t ready = nullptr;     // recorded (nullable) once the porosity is formed
+};
 // The binning of n particles from the handle's last binning of n; ident:
 // the particles are that binning's sorted output (particle i at old slot i).
-cg_status launch_rebin(cg_grids* g, long long n, const void* pos_d, bool ident, double* eps_fill, void* rec_fill,
-                       void* eps_t_fill);
-// g->key of the last binning (an identity-hint rebinning leaves it to be
-// formed from its records on demand).
-cg_status ensure_keys(cg_grids* g, long long n);
+cg_status launch_rebin(cg_grids* g, long long n, const void* pos_d, bool ident, StepEps* eps);
+// The caller-order cells of the last binning into cell_out.
+cg_status copy_cells(cg_grids* g, long long n, int32_t* cell_out);
+// inv_perm of the last binning (the identity-hint rebinning leaves it out).
+cg_status ensure_inverse(cg_grids* g, long long n);
 cg_status ensure_partials(cg_grids* g, long long n);
 
-// eps_fill (nullable): also set this [n_b] porosity to 1 (when n > 0), and
-// likewise the porosity of the drag record rec_fill and of eps_t_fill (T).
-cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, double* eps_fill = nullptr,
-                     void* rec_fill = nullptr, void* eps_t_fill = nullptr);
-// prefilled: eps already holds 1 for every cell (the binning set it);
-// rec / eps_t (nullable, sorted-diameter path only): also write the porosity
-// of occupied cells into the drag record and its T copy.
-cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, double* eps, bool sums,
-                                bool prefilled = false, void* rec = nullptr, void* eps_t = nullptr);
-cg_status launch_deposit_sorted_force(cg_grids* g, long long n, void* S_bulk);
+cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps = nullptr);
+// Porosity of the binned particles: from the sorted diameters of a binning
+// from scratch (pos_d null), or gathered from pos_d [n] T4.
+cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, StepEps* eps);
+// cleared: S_bulk is zero already.
+cg_status launch_deposit_sorted_force(cg_grids* g, long long n, void* S_bulk, bool cleared);
 // Gather the particle records into the binned order (cg_reorder_particles).
 cg_status launch_reorder(cg_grids* g, long long n, const void* pos_d, const void* vel, void* pos_out, void* vel_out);
 // Semi-implicit coefficients [4][n_b] (A, b) from the drag's sorted (beta, beta u) records.
@@ -361,13 +374,14 @@ cg_status launch_average(cg_grids* g, const void* u_fine, void* u_bulk, void* va
 cg_status launch_pack(cg_grids* g, const double* eps, const void* u_bulk, bool want_eps_t);
 // pos_out, vel_out (nullable, needs S_bulk): the particles, advanced when
 // dt > 0, are written to these arrays in the order of the binning.
+// S_cleared: S_bulk is zero already.
 cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* vel, void* force, void* S_bulk,
-                      bool sums, double dt, void* coef_bulk = nullptr, void* pos_out = nullptr,
+                      bool sums, double dt, bool S_cleared = false, void* coef_bulk = nullptr, void* pos_out = nullptr,
                       void* vel_out = nullptr);
 // Learned drag (FP32 only): bulk4 must hold (phi of this step, stale u).
 cg_status launch_drag_learned(cg_grids* g, const cg_mlp* m, long long n, void* pos_d, void* vel,
                               const void* var_stale, const void* u_fine, int32_t age, void* force, void* S_bulk,
-                              double dt);
+                              double dt, bool S_cleared = false);
 cg_status grow_buf(DevBuf& b, size_t bytes);
 // The closure's feature box (CG_MLP_NFEAT values each).
 cg_status mlp_feature_box(const cg_mlp* m, float* lo, float* hi);
@@ -431,46 +445,6 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
     s = a + b;
     T z = s - a;
     e = (a - (s - z)) + (b - z);
-}
-
-// A float's exact value as a double, assembled from its bits with integer
-// operations (sign, exponent rebiased by 1023 - 127, mantissa shifted to the
-// double's 52 bits), so that no conversion instruction lands on the FP64
-// pipe; subnormal floats (below 2^-126) take the ordinary conversion.
-__device__ __forceinline__ double f32_exact_f64(float f) {
-    const unsigned u = __float_as_uint(f);
-    const unsigned e = (u >> 23) & 0xffu;
-    if (e == 0u && (u & 0x7fffffu)) return (double)f;
-    const unsigned long long sign = (unsigned long long)(u >> 31) << 63;
-    const unsigned long long ex = e == 0u ? 0ull : e == 255u ? 0x7ffull << 52 : (unsigned long long)(e + 896u) << 52;
-    const unsigned long long man = (unsigned long long)(u & 0x7fffffu) << 29;
-    return __longlong_as_double((long long)(sign | ex | man));
-}
-
-// Porosity 1 - V / V_B of a bulk cell from its compensated volume sum
-// V = s + c: as a double (the output) and in the working precision (the
-// drag's record and the porosity projection).  FP32 path: the product with
-// 1 / V_B and the difference in float-float (relative error about 2^-46 of
-// V / V_B, the accuracy of the volume sum itself), then one FP64 addition
-// of the exact pair (GB300 issues FP64 at 1/64 of the FP32 rate, and this
-// runs wherever a lane of the warp closes a cell); FP64 path: plain double
-// arithmetic.
-__device__ __forceinline__ void cell_porosity(float s, float c, const GridDev& g, double& e, float& et) {
-    const float ph = s * g.ivBh;
-    float pl = fmaf(s, g.ivBh, -ph);   // s / V_B = ph + pl to second order
-    pl = fmaf(s, g.ivBl, pl);
-    pl = fmaf(c, g.ivBh, pl);
-    float eh, el;
-    two_sum(1.0f, -ph, eh, el);
-    el -= pl;
-    float hi, lo;
-    two_sum(eh, el, hi, lo);
-    e = f32_exact_f64(hi) + f32_exact_f64(lo);
-    et = hi;
-}
-__device__ __forceinline__ void cell_porosity(double s, double c, const GridDev& g, double& e, double& et) {
-    e = 1.0 - (s + c) * g.invVB;
-    et = e;
 }
 
 // Compensated accumulator (TwoSum cascade, Neumaier-equivalent).
@@ -604,9 +578,25 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 // (a0) bin index, shared by the binning and the cell-value gather.
 // ----------------------------------------------------------------------
 // ----------------------------------------------------------------------
-__device__ __forceinline__ int bin_axis_exact(double x, double x0, double H, int nb, int& outside) {
-    double q = __ddiv_rn(__dsub_rn(x, x0), H);
-    int i;
+// a / b correctly rounded, from y = 1 / b correctly rounded: q1 is within one
+// unit in the last place of a / b, so its remainder is exact and q1 + r y
+// rounds to the quotient (Markstein's theorem).  Six FP64 operations on a GPU
+// that issues FP64 at 1/64 of the FP32 rate, about half of a division.  Where
+// a product could leave the exponent range (or a is not finite) it divides.
+__device__ __forceinline__ double quotient_rn(double a, double b, double y) {
+    const double q0 = __dmul_rn(a, y);
+    const double q1 = __fma_rn(__fma_rn(-q0, b, a), y, q0);
+    const double q = __fma_rn(__fma_rn(-q1, b, a), y, q1);
+    // exponents of a within 2^-767 .. 2^752 and of b within 2^-511 .. 2^496; or a = +0
+    const unsigned ea = (unsigned)__double2hiint(a) & 0x7ff00000u, eb = (unsigned)__double2hiint(b) & 0x7ff00000u;
+    const bool zero = ((unsigned)__double2hiint(a) | (unsigned)__double2loint(a)) == 0u;
+    return (ea - 0x10000000u < 0x5f000000u || zero) && eb - 0x20000000u < 0x3f000000u ? q : __ddiv_rn(a, b);
+}
+
+__device__ __forceinline__ int bin_axis_exact(double x, double x0, double H, double invH, int nb, int& outside) {
+    const double q = quotient_rn(__dsub_rn(x, x0), H, invH);
+    int i = __double2int_rd(q);
+    if (__double2hiint(q) >= 0 && (unsigned)i < (unsigned)nb) return i;   // the quotient is not negative, nor NaN with i in range
     if (!(q >= 0.0)) i = 0;
     else if (q >= (double)nb) i = nb - 1;
     else i = (int)floor(q);
@@ -615,41 +605,54 @@ __device__ __forceinline__ int bin_axis_exact(double x, double x0, double H, int
 }
 
 // |q32 - q64| <= 4 u (|q| + |x0/H|), u = 2^-24, for
-// q32 = (x - fl(x0)) * fl(1/H) in round-to-nearest float; the margin below
-// is twice that bound.  Outside the margin floor(q32) == floor(q64).
-__device__ __forceinline__ int bin_axis_f32(float x, const GridDev& g, int a, int& outside) {
-    float q = __fmul_rn(__fsub_rn(x, g.x0f[a]), g.invHf[a]);
-    float fl = floorf(q);
-    float m = (fabsf(q) + g.ax0f[a]) * 4.76837158203125e-7f + 1e-30f;
-    if ((q - fl > m) && (fl + 1.0f - q > m)) {
-        int i = (int)fl;
-        if (i < 0) { outside = 1; return 0; }
-        if (i >= g.nb[a]) { outside = 1; return g.nb[a] - 1; }
-        return i;
-    }
-    return bin_axis_exact((double)x, g.x0[a], g.H[a], g.nb[a], outside);
+// q32 = (x - fl(x0)) * fl(1/H) in round-to-nearest float, and <= 5 u (|q| +
+// |x0/H|) when x is a double cut to float; the margin below is 8 u (|q| +
+// |x0/H|).  Outside the margin floor(q32) == floor(q64).  True when the cell
+// is decided and inside the grid.
+__device__ __forceinline__ bool bin_axis_fast(float x, const GridDev& g, int a, int& i) {
+    const float q = __fmul_rn(__fsub_rn(x, g.x0f[a]), g.invHf[a]);
+    const float fl = floorf(q), fr = q - fl;
+    const float m = (fabsf(q) + g.ax0f[a]) * 4.76837158203125e-7f + 1e-30f;
+    i = (int)fl;
+    return fminf(fr, 1.0f - fr) > m && (unsigned)i < (unsigned)g.nb[a];
 }
 
-__device__ __forceinline__ int cell_of(const V4<float>& v, const GridDev& g, int& outside) {
-    int i = bin_axis_f32(v.x, g, 0, outside);
-    int j = bin_axis_f32(v.y, g, 1, outside);
-    int k = bin_axis_f32(v.z, g, 2, outside);
-    return i + g.nb[0] * (j + g.nb[1] * k);
+// A double cut (toward zero) to float with integer operations: no conversion
+// on the FP64 pipe, which GB300 runs at 1/64 of the FP32 rate.  Below 2^-126: 0,
+// from 2^128 on, infinities and NaN: an infinity, which no fast path takes.
+__device__ __forceinline__ float f64_cut_f32(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+    if (e < 897u) return __uint_as_float(sign);
+    if (e > 1150u) return __uint_as_float(sign | 0x7f800000u);
+    return __uint_as_float(sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
 }
-__device__ __forceinline__ int cell_of(const V4<double>& v, const GridDev& g, int& outside) {
-    int i = bin_axis_exact(v.x, g.x0[0], g.H[0], g.nb[0], outside);
-    int j = bin_axis_exact(v.y, g.x0[1], g.H[1], g.nb[1], outside);
-    int k = bin_axis_exact(v.z, g.x0[2], g.H[2], g.nb[2], outside);
+__device__ __forceinline__ float bin_float(float x) { return x; }
+__device__ __forceinline__ float bin_float(double x) { return f64_cut_f32(x); }
+
+// Bulk cell of a point by the exact rule (bin_axis_exact), decided in float
+// away from the cell faces.
+template <typename T>
+__device__ __forceinline__ int cell_of(const V4<T>& v, const GridDev& g, int& outside, int& nonfinite) {
+    int i, j, k;
+    const bool a = bin_axis_fast(bin_float(v.x), g, 0, i), b = bin_axis_fast(bin_float(v.y), g, 1, j);
+    const bool c = bin_axis_fast(bin_float(v.z), g, 2, k);
+    if (!(a && b && c)) {   // near a face, outside, or not finite
+        if (!a) i = bin_axis_exact((double)v.x, g.x0[0], g.H[0], g.invH[0], g.nb[0], outside);
+        if (!b) j = bin_axis_exact((double)v.y, g.x0[1], g.H[1], g.invH[1], g.nb[1], outside);
+        if (!c) k = bin_axis_exact((double)v.z, g.x0[2], g.H[2], g.invH[2], g.nb[2], outside);
+        if (!(isfinite(v.x) && isfinite(v.y) && isfinite(v.z))) nonfinite = 1;
+    }
     return i + g.nb[0] * (j + g.nb[1] * k);
 }
 
 __device__ __forceinline__ int cell_of_f(float x, float y, float z, const GridDev& g) {
-    int o = 0;
-    return cell_of(V4<float>{x, y, z, 0.f}, g, o);
+    int o = 0, f = 0;
+    return cell_of(V4<float>{x, y, z, 0.f}, g, o, f);
 }
 __device__ __forceinline__ int cell_of_d(double x, double y, double z, const GridDev& g) {
-    int o = 0;
-    return cell_of(V4<double>{x, y, z, 0.0}, g, o);
+    int o = 0, f = 0;
+    return cell_of(V4<double>{x, y, z, 0.0}, g, o, f);
 }
 
 // ----------------------------------------------------------------------
@@ -660,11 +663,9 @@ __device__ __forceinline__ int cell_of_d(double x, double y, double z, const Gri
 // finish its last segment, so every segment is reduced by exactly one warp
 // and the work follows the particles, not the cells (a dense bed occupying
 // a few percent of the cells still spreads over every SM).  The warp reduces
-// its range in rounds: 32 slots a round, one per lane, with a segmented
-// shuffle scan (seg_rounds: the reaction), or 256 slots a round, 8
-// consecutive ones per lane (seg_seq: the porosity).  The rounds start at the
-// range's first slot, so the summation order depends only on the chunk's
-// slots, never on the launch shape.
+// its range in rounds of 32 slots, one per lane, with a segmented shuffle
+// scan.  The rounds start at the range's first slot, so the summation order
+// depends only on the chunk's slots, never on the launch shape.
 // ----------------------------------------------------------------------
 constexpr int kSegChunk = 256;
 
@@ -777,130 +778,6 @@ __device__ __forceinline__ void seg_rounds(long long s, long long t, const int32
     }
 }
 
-// Segmented sums over the slots [s, t) of one chunk, 256 slots per round.
-// Lane l walks its own 8 consecutive slots r0 + 8l .. r0 + 8l + 7 in order
-// with compensated sums: runs that start and end inside the lane are
-// emitted at once; the open first and last runs of the lanes are joined by
-// one segmented scan over the lanes (compensated merges, lower slots
-// first), and the round's last run is carried into the next round.  With
-// EXACT every addition is compensated; otherwise a lane adds its own (at
-// most 8) slots plainly and only the joins are compensated.  load(i, v)
-// fills slot i's K compensated values; emit(key, tot) receives each
-// segment's total (on one lane, once).  The summation order depends only on
-// the chunk's slots, not on the launch.
-template <typename T, int K, bool EXACT, typename Load, typename Emit>
-__device__ __forceinline__ void seg_seq(long long s, long long t, const int32_t* __restrict__ key_sorted,
-                                        Load load, Emit emit) {
-    constexpr int P = 8;
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    CSum<T> carry[K];
-    int carry_key = -1;
-    for (long long r0 = s; r0 < t; r0 += 32 * P) {
-        const long long b0 = r0 + (long long)P * lane;
-        int key[P];
-        CSum<T> v[P][K];
-#pragma unroll
-        for (int j = 0; j < P; ++j) {
-            key[j] = -1;
-            if (b0 + j < t) {
-                key[j] = __ldg(key_sorted + b0 + j);
-                load(b0 + j, v[j]);
-            }
-        }
-        const int nk = (r0 + 32 * P < t) ? __ldg(key_sorted + r0 + 32 * P) : -1;   // first key after the round
-        // the lane's own slots: head run, complete middle runs, open tail run
-        const int head_key = key[0];
-        int cur = key[0];
-        int nruns = key[0] >= 0 ? 1 : 0;
-        CSum<T> acc[K], head[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] = v[0][k];
-#pragma unroll
-        for (int j = 1; j < P; ++j) {
-            if (key[j] < 0) break;
-            if (key[j] != cur) {
-                if (nruns == 1) {
-#pragma unroll
-                    for (int k = 0; k < K; ++k) head[k] = acc[k];
-                } else {
-                    emit(cur, acc);
-                }
-                ++nruns;
-                cur = key[j];
-#pragma unroll
-                for (int k = 0; k < K; ++k) acc[k] = v[j][k];
-            } else {
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    if (EXACT) acc[k].merge(v[j][k]);
-                    else acc[k].s += v[j][k].s;
-                }
-            }
-        }
-        const int tail_key = nruns ? cur : -2;
-        // lane 0 continues the run carried from the previous round
-        if (lane == 0 && nruns == 1 && head_key == carry_key)
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                CSum<T> c0 = carry[k];
-                c0.merge(acc[k]);
-                acc[k] = c0;
-            }
-        // segmented inclusive scan of the tail runs over the lanes: a lane
-        // holding one run of the previous lane's tail key continues it
-        const int prev_tail = __shfl_up_sync(full, tail_key, 1);
-        bool fl = lane == 0 || nruns != 1 || head_key != prev_tail;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const bool ofl = __shfl_up_sync(full, fl, off);
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                CSum<T> o;
-                o.s = __shfl_up_sync(full, acc[k].s, off);
-                o.c = __shfl_up_sync(full, acc[k].c, off);
-                if (lane >= off && !fl) {
-                    o.merge(acc[k]);
-                    acc[k] = o;
-                }
-            }
-            if (lane >= off && !fl) fl = ofl;
-        }
-        // head runs that end inside a lane take the chain before them
-        CSum<T> before[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            before[k].s = __shfl_up_sync(full, acc[k].s, 1);
-            before[k].c = __shfl_up_sync(full, acc[k].c, 1);
-        }
-        if (nruns > 1) {
-            CSum<T> tot[K];
-            const bool cont = lane == 0 ? head_key == carry_key : head_key == prev_tail;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                tot[k] = cont ? (lane == 0 ? carry[k] : before[k]) : CSum<T>();
-                tot[k].merge(head[k]);
-            }
-            emit(head_key, tot);
-        }
-        // tail runs that end at the lane's end
-        int next = __shfl_down_sync(full, head_key, 1);
-        if (lane == 31) next = nk;
-        const int last = (int)min((long long)31, (t - r0 - 1) / P);   // last lane holding slots
-        if (lane == last) next = nk;
-        if (nruns > 0 && next != tail_key) emit(tail_key, acc);
-        // carry the round's last run into the next round
-        const int lk = __shfl_sync(full, tail_key, last);
-        const bool goes_on = nk >= 0 && nk == lk;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            carry[k].s = __shfl_sync(full, acc[k].s, last);
-            carry[k].c = __shfl_sync(full, acc[k].c, last);
-        }
-        carry_key = goes_on ? lk : -1;
-    }
-}
-
 // Component k of the reaction of one cell from its force sum: S_B =
 // -(1/V_B) sum F (Eq. UFP: F_fpi is the fluid-side reaction to F_drag), written
 // to S ([3][n_b]).  The conservation sum of S_B V_B is formed by the
@@ -910,47 +787,188 @@ __device__ __forceinline__ void reaction_emit(const GridDev& g, T* __restrict__ 
     S[k * g.nbulk + key] = -sum * (sizeof(T) == 4 ? (T)g.invVBf : (T)g.invVB);
 }
 
-// Sphere volume pi d^3 / 6 as an unevaluated pair hi + lo: exact products
-// by FMA in FP32 (relative error ~2^-46), the plain product in FP64.
-__device__ __forceinline__ void sphere_volume_pair(float d, float& hi, float& lo) {
-    const float p = d * d;
-    const float pe = fmaf(d, d, -p);             // d^2 = p + pe exactly
-    const float q = p * d;
-    const float qe = fmaf(p, d, -q);             // p d = q + qe exactly
-    const float r = fmaf(pe, d, qe);             // d^3 = q + r (to 2^-48)
-    const float ch = 0.5235987901687622f;        // pi / 6 = ch + cl
-    const float cl = -1.457046305830545e-08f;
-    hi = ch * q;
-    const float he = fmaf(ch, q, -hi);
-    lo = fmaf(ch, r, fmaf(cl, q, he));
+// ----------------------------------------------------------------------
+// Porosity (Table 1: sum of the particle volumes of a cell over V_B).
+//
+// Each sphere's volume over V_B is rounded once to a multiple of 2^-57 and the
+// cells add whole numbers, so the sum is exact and the same in any order:
+// particles can be added where their cell is first known, with one pair of
+// atomics per run of equal cells in a warp, and every path (binning from
+// scratch, incremental, batched) gives the same bits.  A cell's accumulator
+// is two 64-bit words: the multiples of 2^-30 in acc[2 c + 1], what is left,
+// below 2^-30 per particle, in acc[2 c] (so neither can overflow for 2^30
+// particles), and, for spheres of 2^32 V_B and more and for non-finite ones,
+// a double in big[c], marked by bit 62 of acc[2 c].  The accumulators are
+// zero between steps: whoever forms the porosity of a cell clears them.
+// ----------------------------------------------------------------------
+// 2^57 pi d^3 / (6 V_B) rounded; false when it is not in [0, 2^57) (the slow
+// path's).  FP32: the product as a pair by FMA (relative error about 2^-46);
+// its upper part is cut into the integer with shifts, since the conversions
+// to 64-bit integers issue on the FP64 pipe at 1/64 of the FP32 rate (two of
+// them per row of 32 particles took over half of the marking kernel's time).
+__device__ __forceinline__ bool sphere_fraction57(float d, const GridDev& g, long long& t) {
+    const float p = __fmul_rn(d, d), pe = __fmaf_rn(d, d, -p);   // d^2 = p + pe exactly
+    const float q = __fmul_rn(p, d), qe = __fmaf_rn(p, d, -q);   // p d = q + qe exactly
+    const float r = __fmaf_rn(pe, d, qe);                        // d^3 = q + r (to 2^-48)
+    const float hi = __fmul_rn(g.vch, q);
+    const float lo = __fmaf_rn(g.vch, r, __fmaf_rn(g.vcl, q, __fmaf_rn(g.vch, q, -hi)));
+    // hi = m 2^(E - 150) with a 24-bit m: 2^57 hi = m 2^(E - 93), E <= 126 below 1 (smaller than 2^-57: 0);
+    // lo is below 2^-24 hi and rounded to 2^-54
+    const unsigned u = __float_as_uint(hi);
+    const int E = (int)(u >> 23);
+    const unsigned long long m = (unsigned long long)((u & 0x7fffffu) | 0x800000u) << 33;
+    t = (long long)(E > 63 ? m >> ((126 - E) & 63) : 0ull) + ((long long)__float2int_rn(lo * 18014398509481984.0f) << 3);
+    return u < 0x3f800000u;   // 0 <= hi < 1, not NaN
 }
-__device__ __forceinline__ void sphere_volume_pair(double d, double& hi, double& lo) {
-    hi = 0.52359877559829887308 * d * d * d;
-    lo = 0.0;
+__device__ __forceinline__ bool sphere_fraction57(double d, const GridDev& g, long long& t) {
+    const double v = __dmul_rn(__dmul_rn(__dmul_rn(g.vcd57, d), d), d);
+    t = __double2ll_rn(v);
+    return (unsigned)__double2hiint(v) < 0x43800000u;   // 0 <= v < 2^57, compared as integers
 }
 
-// Inclusive segmented scan of K compensated sums over the lanes, keyed by
-// `key`; lane i ends with the sum of its segment's lanes <= i.
-template <typename T, int K>
-__device__ __forceinline__ void warp_seg_scan(CSum<T> (&v)[K], int key) {
+// One sphere outside that range: a large one, or a diameter that is negative
+// or not finite.
+static __device__ __noinline__ void volume_add_slow(double d, int cell, double vcd57, unsigned long long* __restrict__ acc,
+                                                    double* __restrict__ big) {
+    const double t = vcd57 * 6.938893903907228e-18 * d * d * d;   // 2^-57
+    if (fabs(t) < 4294967296.0) {
+        const double x = t * 1073741824.0, f = floor(x);
+        atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)__double2ull_rn((x - f) * 134217728.0));
+        atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)(long long)f);
+    } else {
+        atomicAdd(big + cell, isfinite(t) ? t : __longlong_as_double(0x7ff8000000000000LL));
+        atomicOr(acc + 2 * (size_t)cell, 1ULL << 62);
+    }
+}
+
+// Add 32 spheres, one per lane (valid lanes), to their cells: equal cells on
+// consecutive lanes are summed first.  One or two runs by warp reductions,
+// more by a segmented scan (two 27-bit pieces, which cannot overflow 32 bits
+// over 32 lanes).  Called by the whole warp.
+template <typename T>
+__device__ __forceinline__ void volume_add_row(bool valid, int cell, T d, const GridDev& g,
+                                               unsigned long long* __restrict__ acc, double* __restrict__ big) {
+    const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int ko = __shfl_up_sync(0xffffffffu, key, off);
-        const bool take = lane >= off && ko == key;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            CSum<T> o;
-            o.s = __shfl_up_sync(0xffffffffu, v[k].s, off);
-            o.c = __shfl_up_sync(0xffffffffu, v[k].c, off);
-            if (take) {
-                // earlier lanes first: result = o (+) v
-                CSum<T> r = o;
-                r.merge(v[k]);
-                v[k] = r;
-            }
+    long long t = 0;
+    const bool fast = sphere_fraction57(d, g, t);
+    unsigned w0 = (unsigned)t & 0x7ffffffu, w1 = (unsigned)(t >> 27);
+    const bool use = valid && fast && w1 < (1u << 27);   // below 1/8
+    if (valid && !use) {
+        if (fast) {
+            atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)w0);
+            atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)w1);
+        } else {
+            volume_add_slow((double)d, cell, g.vcd57, acc, big);
         }
     }
+    if (!use) w0 = w1 = 0u;
+    const int c = valid ? cell : -1;
+    const int prev = __shfl_up_sync(full, c, 1);
+    const unsigned heads = __ballot_sync(full, lane == 0 || prev != c);
+    bool owner;
+    if (__popc(heads) <= 2) {
+        const unsigned later = heads & ~1u;
+        const bool first = lane < (later ? __ffs(later) - 1 : 32);   // of the first run, or of the second
+        const unsigned a0 = __reduce_add_sync(full, first ? w0 : 0u), a1 = __reduce_add_sync(full, first ? w1 : 0u);
+        if (later) {
+            w0 = __reduce_add_sync(full, first ? 0u : w0);
+            w1 = __reduce_add_sync(full, first ? 0u : w1);
+        }
+        if (first) {
+            w0 = a0;
+            w1 = a1;
+        }
+        owner = heads >> lane & 1u;
+    } else {
+        const int head = 31 - __clz(heads & ((2u << lane) - 1u));
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned x0 = __shfl_up_sync(full, w0, off), x1 = __shfl_up_sync(full, w1, off);
+            if (lane - off >= head) {
+                w0 += x0;
+                w1 += x1;
+            }
+        }
+        owner = lane == 31 || (heads >> (lane + 1) & 1u);
+    }
+    if (owner && valid) {
+        atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)w0);
+        atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)w1);
+    }
+}
+
+// Where a step's porosity goes: double, and (nullable) the porosity of the
+// drag's record, its copy in the path precision, and the reaction source to
+// clear (cells without particles keep the zero).
+template <typename T>
+struct EpsOut {
+    unsigned long long* acc;
+    double* big;
+    double* eps;
+    T* rec;
+    T* eps_t;
+    T* S;
+};
+
+// The accumulators of the handle with a step's (or no) outputs.
+template <typename T>
+inline EpsOut<T> eps_out(cg_grids* g, const StepEps* e) {
+    return {g->vol_acc, (double*)(g->vol_acc + 2 * g->gd.nbulk), e ? e->eps : nullptr, e ? (T*)e->rec : nullptr,
+            e ? (T*)e->eps_t : nullptr, e ? (T*)e->S : nullptr};
+}
+
+__device__ __forceinline__ void eps_round(long long e57, double, float& et) {
+    et = __ll2float_rn(e57) * 6.938893903907228e-18f;
+}
+__device__ __forceinline__ void eps_round(long long, double e, double& et) { et = e; }
+__device__ __forceinline__ void deposited_volume(long long p57, const GridDev& g, CSum<float>& tot) {
+    const float ph = __ll2float_rn(p57);
+    const float pl = __ll2float_rn(p57 - __float2ll_rn(ph)) * 6.938893903907228e-18f;
+    const float p = ph * 6.938893903907228e-18f;
+    const float hi = p * g.VBh;
+    const float lo = fmaf(pl, g.VBh, fmaf(p, g.VBl, fmaf(p, g.VBh, -hi)));
+    tot.add(hi);
+    tot.c += lo;
+}
+__device__ __forceinline__ void deposited_volume(long long p57, const GridDev& g, CSum<double>& tot) {
+    tot.add((double)p57 * 6.938893903907228e-18 * g.VB);
+}
+
+// The porosity of one cell from its accumulator, which is cleared; its
+// deposited volume goes into tot with SUMS.
+template <typename T, bool SUMS>
+__device__ __forceinline__ void eps_finish(long long c, const GridDev& g, const EpsOut<T>& o, CSum<T>& tot) {
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(o.acc + 2 * c);
+    double e = 1.0;
+    T et = T(1);
+    if (a.x | a.y) {
+        *reinterpret_cast<ulonglong2*>(o.acc + 2 * c) = make_ulonglong2(0, 0);
+        const unsigned long long low = a.x & ~(1ULL << 62);
+        const long long h = (long long)a.y + (long long)(low >> 27);
+        const unsigned l = (unsigned)low & 0x7ffffffu;
+        if (low == a.x && h >= 0 && h < (1LL << 33)) {
+            const long long p57 = (h << 27) | l, e57 = (1LL << 57) - p57;   // 1 - sum, exactly
+            e = __ll2double_rn(e57) * 6.938893903907228e-18;
+            eps_round(e57, e, et);
+            if (SUMS) deposited_volume(p57, g, tot);
+        } else {
+            double phi = (double)h * 9.313225746154785e-10 + (double)l * 6.938893903907228e-18;   // 2^-30, 2^-57
+            if (low != a.x) {
+                phi += o.big[c];
+                o.big[c] = 0.0;
+            }
+            e = 1.0 - phi;
+            et = (T)e;
+            if (SUMS) tot.add((T)(phi * g.VB));
+        }
+    }
+    o.eps[c] = e;
+    if (o.rec) o.rec[4 * c] = et;
+    if (o.eps_t) o.eps_t[c] = et;
+    if (o.S)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) o.S[k * g.nbulk + c] = T(0);
 }
 
 }  // namespace cg

@@ -372,7 +372,7 @@ int batch_drag_occupancy() {
 }
 
 cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* vel, void* force, void* S_bulk,
-                      bool sums, double dt, void* coef_bulk, void* pos_out, void* vel_out) {
+                      bool sums, double dt, bool S_cleared, void* coef_bulk, void* pos_out, void* vel_out) {
     const bool euler = dt > 0.0;
     void* part = part_ptr(g, PS_DRAG);
     // exactly the resident CTAs (the launch bounds' minimum per SM): a grid-stride
@@ -381,6 +381,7 @@ cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* v
     const unsigned nblk = (unsigned)std::max(1LL, std::min((n + 255) / 256, (long long)g->num_sms * per_sm));
     g->part_blocks[PS_DRAG] = sums ? (long long)nblk : -1;
     void* Fs = S_bulk ? g->Fs : nullptr;
+    if (Fs) CG_TRY(ensure_inverse(g, n));
     if (pos_out && !Fs) return CG_ERR_INVALID_ARG;   // the sorted slots come with the fused reaction
     void* Bs = nullptr;
     if (coef_bulk && n > 0) {
@@ -417,7 +418,7 @@ cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* v
         }
 #undef CG_DRAGP
     }
-    if (S_bulk) CG_TRY(launch_deposit_sorted_force(g, n, S_bulk));
+    if (S_bulk) CG_TRY(launch_deposit_sorted_force(g, n, S_bulk, S_cleared));
     if (coef_bulk) CG_TRY(launch_deposit_implicit(g, n, coef_bulk));
     return CG_OK;
 }

@@ -1202,12 +1202,13 @@ cg_status mlp_bound_inputs(const cg_mlp* m, const void** var_stale, const void**
 
 cg_status launch_drag_learned(cg_grids* g, const cg_mlp* m, long long n, void* pos_d, void* vel,
                               const void* var_stale, const void* u_fine, int32_t age, void* force, void* S_bulk,
-                              double dt) {
+                              double dt, bool S_cleared) {
     if (g->fp64 || !var_stale || !u_fine || age < 1) return CG_ERR_INVALID_ARG;
     if (n > 0 && ((uintptr_t)u_fine & 15u)) return CG_ERR_INVALID_ARG;
     CG_TRY(mlp_attrs());
     g->part_blocks[PS_DRAG] = -1;   // the drag diagnostics are not formed on this path
     void* Fs = S_bulk ? g->Fs : nullptr;
+    if (Fs) CG_TRY(ensure_inverse(g, n));
     if (n > 0) {
         const long long ntiles = (n + TILE - 1) / TILE;
         const unsigned grid = (unsigned)std::min(ntiles, (long long)4 * g->num_sms);
@@ -1217,7 +1218,7 @@ cg_status launch_drag_learned(cg_grids* g, const cg_mlp* m, long long n, void* p
                   (const WeightImage*)m->img, (float*)force, (float*)Fs, g->inv_perm, (float)dt, (float)age,
                   g->status);
     }
-    if (S_bulk) CG_TRY(launch_deposit_sorted_force(g, n, S_bulk));
+    if (S_bulk) CG_TRY(launch_deposit_sorted_force(g, n, S_bulk, S_cleared));
     return CG_OK;
 }
 

@@ -24,14 +24,19 @@
 //
 // Old slot s holds particle perm_old[s] when the caller kept its particle
 // order, or particle s when the particles are the sorted output of the last
-// step (cg_step_sorted; the identity hint).  When a cell receives more than
-// kRebinMaxArrivals movers (the movers' searches and counts grow with the
-// arrivals of their cell) the device falls back to the per-cell sort: both
-// paths are launched and
-// each kernel checks a device flag, so a captured CUDA graph takes the
-// right path on every replay.  The same holds when no particle changed its
-// cell: the scans return at once on a device count of the movers, and the
-// kernels after them keep the old bins.
+// step (cg_step_sorted; the identity hint).  The movers of a cell are a linked
+// list (its few entries are walked, in any order, to count the ids below
+// one).  When a cell receives more than kRebinMaxArrivals movers the walks
+// would grow with the square of the arrivals, and the device falls back to a
+// sort of every cell: the slots kernel then places the ids of each cell in any
+// order, and the last kernel sorts them; each kernel checks a device flag, so
+// a captured CUDA graph takes the right path on every replay.  When no
+// particle changed its cell the device leaves the scans out and keeps the bins.
+//
+// In a coupling step the kernels also form the porosity: the first one, which
+// has every particle's position and diameter in nearly sorted order, adds the
+// spheres to their cells' accumulators (volume_add_row), and the second one,
+// which goes over the cells, turns them into the porosity.
 #include <algorithm>
 
 #include "cg_internal.cuh"
@@ -41,39 +46,28 @@ namespace cg {
 namespace {
 
 enum { RB_FALLBACK = 0, RB_MOVERS = 1 };   // counters: fallback flag, movers
-constexpr int kCellBits = 22;   // a mover entry packs its new cell (< 2^22) and arrival rank (< 2^8)
 
 struct RebinPtrs {
     int32_t* cnt;       // [n_b + 1] new counts, then (scanned in place) new starts
-    int32_t* arr;       // [n_b + 1] arrivals per cell, then their starts
-    int32_t* dep;       // [n_b + 1] departures per cell
     int32_t* blk;       // [nblk + 1] departures per block of old slots, then their starts
-    int32_t* ctr;       // [kRebinCounters] movers, fallback flag
+    int2* arr;          // [n_b + 1] arrivals per cell, then their starts; first mover of the cell's list + 1 (0: none)
+    int32_t* dep;       // [n_b] departures per cell
+    int32_t* ctr;       // [kRebinCounters] fallback flag, movers
+    int32_t* part;      // block totals of the scans
+    size_t zero_bytes;  // arr .. ctr, to be cleared before the first kernel
 };
 
 RebinPtrs rebin_ptrs(cg_grids* g) {
     const long long nb1 = rebin_pad(g->gd.nbulk + 1);
     RebinPtrs r;
     r.cnt = g->rb_small;
-    r.arr = r.cnt + nb1;
-    r.dep = r.arr + nb1;
-    r.blk = r.dep + nb1;
-    r.ctr = r.blk + rebin_pad(g->rb_nblk + 1);
+    r.blk = r.cnt + nb1;
+    r.arr = (int2*)(r.blk + rebin_pad(g->rb_nblk + 1));
+    r.dep = (int32_t*)(r.arr + nb1);
+    r.ctr = r.dep + nb1;
+    r.part = r.ctr + rebin_pad(kRebinCounters);
+    r.zero_bytes = sizeof(int32_t) * (3 * nb1 + kRebinCounters);
     return r;
-}
-
-// Set every cell's porosity to 1 (and that of the drag record and of its
-// path-precision copy); the porosity deposit overwrites the occupied cells.
-template <typename T>
-__device__ __forceinline__ void eps_fill_cells(long long nbulk, double* __restrict__ eps_fill,
-                                               T* __restrict__ rec_fill, T* __restrict__ eps_t_fill) {
-    if (!eps_fill) return;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < nbulk;
-         c += (long long)gridDim.x * blockDim.x) {
-        eps_fill[c] = 1.0;
-        if (rec_fill) rec_fill[4 * c] = T(1);
-        if (eps_t_fill) eps_t_fill[c] = T(1);
-    }
 }
 
 __device__ __forceinline__ void add_status_counts(unsigned long long* st, int outside, int nonfin) {
@@ -87,486 +81,521 @@ __device__ __forceinline__ void add_status_counts(unsigned long long* st, int ou
     }
 }
 
-// Cell and diameter of particle p (caller order, record v), with the status counts.
-template <typename T>
-__device__ __forceinline__ int key_of(const V4<T>& v, long long p, const GridDev& g, int32_t* __restrict__ key,
-                                      T* __restrict__ vol, int& n_out, int& n_nf) {
-    int outside = 0;
-    if (!(isfinite(v.x) && isfinite(v.y) && isfinite(v.z))) n_nf++;
-    const int c = cell_of(v, g, outside);
-    n_out += outside;
-    key[p] = c;
-    vol[p] = v.w;   // the diameter: the porosity forms the volume as an exact pair
-    return c;
-}
-
-__device__ __forceinline__ void flush_status(unsigned long long* st, int n_out, int n_nf) {
-    n_out = __reduce_add_sync(0xffffffffu, n_out);
-    n_nf = __reduce_add_sync(0xffffffffu, n_nf);
-    if ((threadIdx.x & 31) == 0 && (n_out | n_nf)) add_status_counts(st, n_out, n_nf);
-}
-
 }  // namespace
 
-// Cells and diameters in the caller's order (the particles kept their order:
-// old slot s holds perm_old[s]).  FP32: six CTAs per SM (40 registers),
-// the loads of more warps in flight (measured faster than four).
-template <typename T>
-__global__ void __launch_bounds__(kRebinThreads, sizeof(T) == 4 ? 6 : 4)
-k_rebin_key(const T* __restrict__ pos, long long n, GridDev g, int32_t* __restrict__ key, T* __restrict__ vol,
-            unsigned long long* __restrict__ status, double* __restrict__ eps_fill, T* __restrict__ rec_fill,
-            T* __restrict__ eps_t_fill) {
-    pdl_wait();
-    int n_out = 0, n_nf = 0;
-    const long long base = (long long)blockIdx.x * kRebinTile;
-    V4<T> pv[kRebinItems];
-    // every load of the thread first, so that they are in flight together
-#pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long p = base + k * kRebinThreads + threadIdx.x;
-        if (p < n) pv[k] = ld4(pos, p);
-    }
-#pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long p = base + k * kRebinThreads + threadIdx.x;
-        if (p < n) key_of(pv[k], p, g, key, vol, n_out, n_nf);
-    }
-    flush_status(status, n_out, n_nf);
-    eps_fill_cells<T>(g.nbulk, eps_fill, rec_fill, eps_t_fill);
-}
-
 // Mark the movers, over the old slots (slot base + k * threads + t of
-// thread t, so every load and store of a row is coalesced): the new cell of
-// every old slot, complemented for a mover (rkn), and the old id (rid, only
-// when the particles kept the caller's order); per mover one departure
-// from its old cell, one arrival (with its rank) in its new cell and an
-// entry in the block's own part of the mover list (kRebinTile entries per
-// block: no atomic decides a position); the movers of each block.  IDENT: old slot s holds particle
-// s, whose cell and diameter are formed here.
-template <typename T, bool IDENT>
-__global__ void __launch_bounds__(kRebinThreads)
-k_rebin_mark(const T* __restrict__ pos, long long n, GridDev g, const int32_t* __restrict__ perm_old,
-             const int32_t* __restrict__ ks_old, int32_t* __restrict__ key, T* __restrict__ vol,
-             int32_t* __restrict__ rid, int32_t* __restrict__ rkn, int32_t* __restrict__ arr,
-             int32_t* __restrict__ dep, int2* __restrict__ mov, int32_t* __restrict__ blk_dep,
-             int32_t* __restrict__ ctr, unsigned long long* __restrict__ status, double* __restrict__ eps_fill,
-             T* __restrict__ rec_fill, T* __restrict__ eps_t_fill) {
+// thread t): the new cell of every old slot, complemented for a mover (rkn),
+// and the old id (rid, only when the particles kept the caller's order, whose
+// records are gathered through the old permutation: neighbours of a cell, so
+// the cells come out nearly sorted in either case); per mover one departure
+// from its old cell, one arrival (with its rank) in its new cell, and an entry
+// at the head of that cell's list, in the block's own part of the mover array
+// (no atomic decides a position).  VOL: the spheres are added to their new
+// cells' volumes.  IDENT: old slot s holds particle s.
+//
+// Bound by HBM in the sorted step (20 bytes read, 4 written per particle) and
+// by instruction issue with VOL (about 200 warp instructions per 32 slots);
+// 32M particles 213 us, where marking and the porosity as kernels of their
+// own took 201 + 148.  In the caller's order it replaces a key kernel over the
+// particles as well: 4M packed 31 + 19 + 25 -> 54 us.
+template <typename T, bool IDENT, bool VOL>
+__global__ void __launch_bounds__(kRebinThreads, sizeof(T) == 4 ? (IDENT ? 5 : 4) : 3)
+k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restrict__ perm_old,
+             const int32_t* __restrict__ ks_old, int32_t* __restrict__ rid, int32_t* __restrict__ rkn,
+             int2* __restrict__ arr, int32_t* __restrict__ dep, int4* __restrict__ mov, int32_t* __restrict__ blk_dep, int32_t* __restrict__ ctr,
+             unsigned long long* __restrict__ status, unsigned long long* __restrict__ acc, double* __restrict__ big) {
     pdl_wait();
     constexpr int W = kRebinThreads / 32;
     __shared__ int s_cnt[W];
-    __shared__ int s_base[W];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long base = (long long)blockIdx.x * kRebinTile;
+    const int nblk = (n + kRebinTile - 1) / kRebinTile;   // n < 2^30
     int n_out = 0, n_nf = 0;
-    int idk[kRebinItems], cnk[kRebinItems], cok[kRebinItems];
-    V4<T> pv[kRebinItems];
-    // every load of the thread first, so that they are in flight together
+    int idk[kRebinItems], cok[kRebinItems];
+    auto fetch = [&](int b) {   // ids and old cells of a block of old slots
 #pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long s = base + k * kRebinThreads + threadIdx.x;
-        idk[k] = -1;
-        cnk[k] = cok[k] = 0;
-        if (s < n) {
-            idk[k] = IDENT ? (int)s : __ldg(perm_old + s);
-            cok[k] = __ldg(ks_old + s);
-            if (IDENT) pv[k] = ld4(pos, s);
+        for (int k = 0; k < kRebinItems; ++k) {
+            const int s = b * kRebinTile + k * kRebinThreads + threadIdx.x;
+            const bool valid = b < nblk && s < n;
+            idk[k] = IDENT ? s : valid ? __ldg(perm_old + s) : 0;
+            cok[k] = valid ? __ldg(ks_old + s) : 0;
         }
-    }
+    };
+    fetch(blockIdx.x);
+    for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
+        const int base = b * kRebinTile;
+        int id[kRebinItems], co[kRebinItems], cn[kRebinItems];
+        V4<T> pv[kRebinItems];
+        // every load of the thread first, so that they are in flight together
 #pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long s = base + k * kRebinThreads + threadIdx.x;
-        if (s >= n) continue;
-        if (IDENT) {
-            // the cell itself is kept only in rkn below (key is formed from it on demand)
-            int outside = 0;
-            const V4<T>& v = pv[k];
-            if (!(isfinite(v.x) && isfinite(v.y) && isfinite(v.z))) n_nf++;
-            cnk[k] = cell_of(v, g, outside);
-            n_out += outside;
-            vol[s] = v.w;   // the diameter: the porosity forms the volume as an exact pair
-        } else {
-            cnk[k] = __ldg(key + idk[k]);
+        for (int k = 0; k < kRebinItems; ++k) {
+            const int s = base + k * kRebinThreads + threadIdx.x;
+            id[k] = idk[k];
+            co[k] = cok[k];
+            pv[k] = {T(0), T(0), T(0), T(0)};
+            if (s < n) pv[k] = ld4(pos, id[k]);
         }
-    }
-    unsigned mb[kRebinItems];
-    int wc = 0;
+        if (!IDENT) fetch(b + gridDim.x);
+        unsigned mb[kRebinItems];
+        int wc = 0;
 #pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long s = base + k * kRebinThreads + threadIdx.x;
-        const bool valid = s < n;
-        const bool moved = valid && cnk[k] != cok[k];
-        mb[k] = __ballot_sync(full, moved);
-        wc += __popc(mb[k]);
-        if (valid) {
-            rkn[s] = moved ? ~cnk[k] : cnk[k];
-            if (!IDENT) rid[s] = idk[k];
+        for (int k = 0; k < kRebinItems; ++k) {
+            const int s = base + k * kRebinThreads + threadIdx.x;
+            const bool valid = s < n;
+            cn[k] = 0;
+            if (valid) {
+                int outside = 0, nonfinite = 0;
+                cn[k] = cell_of(pv[k], g, outside, nonfinite);
+                n_out += outside;
+                n_nf += nonfinite;
+            }
+            const bool moved = valid && cn[k] != co[k];
+            mb[k] = __ballot_sync(full, moved);
+            wc += __popc(mb[k]);
+            if (valid) {
+                rkn[s] = moved ? ~cn[k] : cn[k];
+                if (!IDENT) rid[s] = id[k];
+            }
+            if (VOL) volume_add_row<T>(valid, cn[k], pv[k].w, g, acc, big);
         }
-    }
-    if (lane == 0) s_cnt[warp] = wc;
-    if (IDENT) flush_status(status, n_out, n_nf);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t = 0;
+        if (lane == 0) s_cnt[warp] = wc;
+        __syncthreads();
+        // each warp its own prefix over the warps' counts
+        int before = 0, total = 0;
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            s_base[w] = t;
-            t += s_cnt[w];
+            const int c = s_cnt[w];
+            if (w < warp) before += c;
+            total += c;
         }
-        blk_dep[blockIdx.x] = t;
-        if (t) atomicAdd(&ctr[RB_MOVERS], t);
+        if (threadIdx.x == 0) {
+            blk_dep[b] = total;
+            if (total) atomicAdd(&ctr[RB_MOVERS], total);
+        }
+        if (wc) {
+            int idx = base + before;
+#pragma unroll
+            for (int k = 0; k < kRebinItems; ++k) {
+                if (mb[k] >> lane & 1u) {
+                    const int j = idx + __popc(mb[k] & lanemask_lt());
+                    atomicAdd(&dep[co[k]], 1);
+                    const int r = atomicAdd(&arr[cn[k]].x, 1);
+                    const int next = atomicExch(&arr[cn[k]].y, j + 1);
+                    mov[j] = make_int4(id[k], cn[k], next, r);
+                    if (r >= kRebinMaxArrivals) ctr[RB_FALLBACK] = 1;
+                }
+                idx += __popc(mb[k]);
+            }
+        }
+        if (IDENT) break;   // one block of old slots per CTA
+        __syncthreads();
+    }
+    n_out = __reduce_add_sync(full, n_out);
+    n_nf = __reduce_add_sync(full, n_nf);
+    if (lane == 0 && (n_out | n_nf)) add_status_counts(status, n_out, n_nf);
+}
+
+// Over the cells: the new count of every cell, the block totals of the scans
+// (of the counts, the arrivals, and the departures per block of old slots),
+// and the porosity of every cell.  When no particle changed its cell the new
+// starts are the old ones, written in their scanned form, and the scans are
+// left out.
+template <typename T, bool EPS, bool SUMS>
+__global__ void __launch_bounds__(256)
+k_rebin_cells(const int32_t* __restrict__ cs_old, GridDev g, const int32_t* __restrict__ dep,
+              const int2* __restrict__ arr, int32_t* __restrict__ cnt, const int32_t* __restrict__ blk, long long nblk, const int32_t* __restrict__ ctr, int32_t* __restrict__ part, long long tiles,
+              EpsOut<T> eps, T* __restrict__ vpart) {
+    pdl_wait();
+    __shared__ int sh[2][8];
+    const bool moved = ctr[RB_MOVERS] != 0;
+    const long long nbulk = g.nbulk, b = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int s0 = 0, s1 = 0;
+    CSum<T> tot[1];
+    if (b < tiles) {
+#pragma unroll
+        for (int j = 0; j < kRebinScan / 256; ++j) {
+            const long long c = b * kRebinScan + j * 256 + threadIdx.x;
+            if (c < nbulk) {
+                const int start = __ldg(cs_old + c);
+                if (moved) {
+                    const int a = __ldg(&arr[c].x), v = __ldg(cs_old + c + 1) - start - __ldg(dep + c) + a;
+                    cnt[c] = v;
+                    s0 += v;
+                    s1 += a;
+                } else {
+                    cnt[c] = start;
+                }
+                if (EPS) eps_finish<T, SUMS>(c, g, eps, tot[0]);
+            } else if (c == nbulk) {
+                cnt[c] = moved ? 0 : __ldg(cs_old + c);
+            }
+        }
+        if (SUMS) block_sums<T, 1>(tot, vpart, tiles, b);
+    } else if (moved) {
+#pragma unroll
+        for (int j = 0; j < kRebinScan / 256; ++j) {
+            const long long i = (b - tiles) * kRebinScan + j * 256 + threadIdx.x;
+            if (i < nblk) s0 += __ldg(blk + i);
+        }
+    }
+    if (!moved) return;
+    s0 = __reduce_add_sync(0xffffffffu, s0);
+    s1 = __reduce_add_sync(0xffffffffu, s1);
+    if (lane == 0) {
+        sh[0][warp] = s0;
+        sh[1][warp] = s1;
     }
     __syncthreads();
-    if (wc) {
-        long long idx = base + s_base[warp];
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) {
-            if (mb[k] >> lane & 1u) {
-                const long long j = idx + __popc(mb[k] & lanemask_lt());
-                atomicAdd(&dep[cok[k]], 1);
-                const int r = atomicAdd(&arr[cnk[k]], 1);
-                if (r < kRebinMaxArrivals) mov[j] = make_int2(idk[k], cnk[k] | (r << kCellBits));
-                else ctr[RB_FALLBACK] = 1;
-            }
-            idx += __popc(mb[k]);
+    if (threadIdx.x == 0) {
+        int t0 = 0, t1 = 0;
+        for (int w = 0; w < 8; ++w) {
+            t0 += sh[0][w];
+            t1 += sh[1][w];
         }
-    }
-    if (IDENT) eps_fill_cells<T>(g.nbulk, eps_fill, rec_fill, eps_t_fill);
-}
-
-// The new count of every cell (the new starts themselves when no particle
-// changed its cell: the scans are then left out); or, when the device falls back to the
-// per-cell sort, that sort's per-cell counts and arrival ranks (consecutive
-// lanes on consecutive particles, one atomic per run of equal cells), from
-// the cells already formed (IDENT: from rkn, whose cells are written to key
-// here for the sort's placement).
-template <bool IDENT>
-__global__ void __launch_bounds__(kRebinThreads)
-k_rebin_cells(const int32_t* __restrict__ cs_old, long long nbulk, const int32_t* __restrict__ dep,
-              const int32_t* __restrict__ arr, int32_t* __restrict__ cnt, const int32_t* __restrict__ ctr,
-              int32_t* __restrict__ key, const int32_t* __restrict__ rkn, long long n, int32_t* __restrict__ arrival) {
-    pdl_wait();
-    if (!ctr[RB_FALLBACK]) {
-        if (ctr[RB_MOVERS] == 0) {
-            // no particle changed its cell: the new starts are the old ones,
-            // written in their scanned form (the scans are left out; the
-            // arrivals and departures, all zero, are their own scans)
-            for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c <= nbulk;
-                 c += (long long)gridDim.x * blockDim.x)
-                cnt[c] = __ldg(cs_old + c);
-            return;
-        }
-        for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < nbulk;
-             c += (long long)gridDim.x * blockDim.x)
-            cnt[c] = __ldg(cs_old + c + 1) - __ldg(cs_old + c) - __ldg(dep + c) + __ldg(arr + c);
-        return;
-    }
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    for (long long base = (long long)blockIdx.x * kRebinTile; base < n; base += (long long)gridDim.x * kRebinTile) {
-        int ck[kRebinItems], lk[kRebinItems], old[kRebinItems];
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) {
-            const long long p = base + k * kRebinThreads + threadIdx.x;
-            const bool valid = p < n;
-            ck[k] = -1;
-            if (valid) {
-                if (IDENT) {
-                    const int r = __ldg(rkn + p);
-                    ck[k] = r >= 0 ? r : ~r;
-                    key[p] = ck[k];
-                } else {
-                    ck[k] = __ldg(key + p);
-                }
-            }
-            lk[k] = run_head_length(ck[k], valid);
-        }
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) old[k] = lk[k] ? atomicAdd(&cnt[ck[k]], lk[k]) : 0;
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) {
-            const long long p = base + k * kRebinThreads + threadIdx.x;
-            const unsigned heads = __ballot_sync(full, lk[k] != 0);
-            const int head = 31 - __clz(heads & ((2u << lane) - 1u));
-            const int o = __shfl_sync(full, old[k], head < 0 ? 0 : head);
-            if (p < n) arrival[p] = o + lane - head;
-        }
+        part[b < tiles ? b : tiles + b] = t0;   // counts, then (after the arrivals) the blocks' departures
+        if (b < tiles) part[tiles + b] = t1;
     }
 }
 
-// The caller-order cells of an identity-hint binning, from the records
-// (a caller asks for them, or the handle needs them).
-__global__ void __launch_bounds__(256) k_rebin_keys(const int32_t* __restrict__ rkn, long long n,
-                                                    int32_t* __restrict__ key) {
-    pdl_wait();
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        const int r = __ldg(rkn + p);
-        key[p] = r >= 0 ? r : ~r;
+// Exclusive scan of one tile of 1024 elements, four consecutive ones per
+// thread; `before` is the sum of the tiles before it.
+__device__ __forceinline__ void scan4(int (&v)[4], int before, int* sh) {
+    int total;
+    int e = before + block_exclusive_scan(v[0] + v[1] + v[2] + v[3], sh, total);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int x = v[j];
+        v[j] = e;
+        e += x;
     }
 }
+__device__ __forceinline__ void scan_tile(int32_t* __restrict__ a, long long first, long long m, int before, int* sh) {
+    const long long i = first + 4 * threadIdx.x;
+    int v[4] = {0, 0, 0, 0};
+    const bool whole = i + 4 <= m;
+    if (whole) {
+        const int4 q = *reinterpret_cast<const int4*>(a + i);
+        v[0] = q.x;
+        v[1] = q.y;
+        v[2] = q.z;
+        v[3] = q.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j < m) v[j] = a[i + j];
+    }
+    scan4(v, before, sh);
+    if (whole) {
+        *reinterpret_cast<int4*>(a + i) = make_int4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j < m) a[i + j] = v[j];
+    }
+}
+__device__ __forceinline__ void scan_tile_x(int2* __restrict__ a, long long first, long long m, int before, int* sh) {
+    const long long i = first + 4 * threadIdx.x;
+    int2 q[4];
+    int v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        q[j] = i + j < m ? a[i + j] : make_int2(0, 0);
+        v[j] = q[j].x;
+    }
+    scan4(v, before, sh);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (i + j < m) a[i + j] = make_int2(v[j], q[j].y);
+}
 
-// Each mover into the arrival list of its new cell, at its arrival rank:
-// one warp per block of old slots walks that block's movers.
+// Starts from the counts and the block totals: the cells' counts and
+// arrivals, and the departures per block of old slots.
 __global__ void __launch_bounds__(256)
-k_rebin_place(const int2* __restrict__ mov, const int32_t* __restrict__ blk_start, long long nblk,
-              const int32_t* __restrict__ arr_start, int2* __restrict__ arr_list, const int32_t* __restrict__ ctr) {
+k_rebin_scan(int32_t* __restrict__ cnt, int2* __restrict__ arr, long long ncell, int32_t* __restrict__ blk,
+             long long nblk, const int32_t* __restrict__ part, long long tiles, const int32_t* __restrict__ ctr) {
     pdl_wait();
-    if (ctr[RB_FALLBACK]) return;
-    const int lane = threadIdx.x & 31;
-    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long b = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < nblk; b += nw) {
-        const int cnt = __ldg(blk_start + b + 1) - __ldg(blk_start + b);
-        for (int j = lane; j < cnt; j += 32) {
-            const int2 m = mov[b * kRebinTile + j];
-            const int c = m.y & ((1 << kCellBits) - 1), r = m.y >> kCellBits;
-            arr_list[__ldg(arr_start + c) + r] = make_int2(m.x, c);
-        }
+    __shared__ int sh[32];
+    if (ctr[RB_MOVERS] == 0) return;
+    const bool cells = blockIdx.x < tiles;
+    const long long b = cells ? blockIdx.x : blockIdx.x - tiles;
+    const int32_t* p0 = cells ? part : part + 2 * tiles;
+    int a0 = 0, a1 = 0;
+    for (long long i = threadIdx.x; i < b; i += blockDim.x) {
+        a0 += __ldg(p0 + i);
+        if (cells) a1 += __ldg(part + tiles + i);
+    }
+    int t0, t1 = 0;
+    block_exclusive_scan(a0, sh, t0);
+    if (cells) {
+        block_exclusive_scan(a1, sh, t1);
+        scan_tile(cnt, b * kRebinScan, ncell, t0, sh);
+        scan_tile_x(arr, b * kRebinScan, ncell, t1, sh);
+    } else {
+        scan_tile(blk, b * kRebinScan, nblk + 1, t0, sh);
     }
 }
 
-// Arrivals in the list [a0, a1) with an id below i.
-__device__ __forceinline__ int arrivals_below(const int2* __restrict__ arr_list, int a0, int a1, int i) {
+// Movers of the list starting at h with an id below i.
+__device__ __forceinline__ int movers_below(const int4* __restrict__ mov, int h, int i) {
     int a = 0;
-    for (int q = a0; q < a1; ++q) a += __ldg(&arr_list[q].x) < i;
+    while (h) {
+        const int4 m = __ldg(mov + ((unsigned)h - 1u));
+        a += m.x < i;
+        h = m.z;
+    }
     return a;
 }
 
-template <typename T>
-__device__ __forceinline__ void emit(long long n, long long ns, int i, int c, int32_t* __restrict__ perm,
-                                     int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-                                     const T* __restrict__ vol, T* __restrict__ vol_sorted) {
-    if ((unsigned long long)ns >= (unsigned long long)n) return;   // never for a valid binning
-    perm[ns] = i;
-    key_sorted[ns] = c;
-    inv_perm[i] = (int)ns;
-    vol_sorted[ns] = __ldg(vol + i);
-}
-
-// Stayers, over the old slots in the layout of the mark kernel (coalesced
-// rows).  Departures before a slot: the block's start (scan of the block
-// totals), the rows and warps before it in the block (a table of warp
-// counts), and the lanes before it (ballot).
-template <typename T, bool IDENT>
+// New slots of the stayers, in the layout of the mark kernel (coalesced
+// rows), one block of old slots at a time; the records of the next one are
+// loaded while this one's gathers (the arrivals before its cell and its cell's
+// list) are under way.  Departures before a slot: the block's start (scan of
+// the block totals), the rows and warps before it in the block (a table of
+// warp counts), and the lanes before it (ballot).
+template <bool IDENT>
 __device__ __forceinline__ void rebin_stay_body(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn,
-                                                long long n, const int32_t* __restrict__ blk_start,
-                                                const int32_t* __restrict__ arr_start, const int2* __restrict__ arr_list,
-                                                const T* __restrict__ vol, int32_t* __restrict__ perm,
-                                                int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-                                                T* __restrict__ vol_sorted, long long bid, long long nblk) {
-    const long long base0 = bid * kRebinTile;
-    if (__ldg(blk_start + nblk) == 0) {
-        // no particle changed its cell (the scanned departures sum to zero):
-        // slot s keeps its particle and cell, so key_sorted stands, and in the
-        // caller's order perm and inv_perm stand too; the diameters are read
-        // afresh (a particle may have changed its size)
-        int ik[kRebinItems];
-        T dk[kRebinItems];
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) {
-            const long long s = base0 + k * kRebinThreads + threadIdx.x;
-            ik[k] = IDENT ? (int)s : (s < n ? __ldg(rid + s) : 0);
-        }
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) {
-            const long long s = base0 + k * kRebinThreads + threadIdx.x;
-            if (s < n) dk[k] = __ldg(vol + ik[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < kRebinItems; ++k) {
-            const long long s = base0 + k * kRebinThreads + threadIdx.x;
-            if (s >= n) continue;
-            vol_sorted[s] = dk[k];
-            if (IDENT) {
-                perm[s] = ik[k];
-                inv_perm[ik[k]] = (int)s;
-            }
-        }
-        return;
-    }
+                                                int n, const int32_t* __restrict__ blk_start,
+                                                const int2* __restrict__ arr, const int4* __restrict__ mov,
+                                                int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted,
+                                                int32_t* __restrict__ inv_perm, int32_t* __restrict__ place,
+                                                int nblk, int bid, int nb) {
     constexpr int W = kRebinThreads / 32;
-    __shared__ int s_tab[kRebinItems * W];
+    __shared__ int s_tab[2][kRebinItems * W];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long base = base0;
-    int kn[kRebinItems], id[kRebinItems], a0[kRebinItems], a1[kRebinItems];
-    T d[kRebinItems];
-    unsigned db[kRebinItems];
+    int kn[kRebinItems], id[kRebinItems];
+    auto fetch = [&](int b) {
 #pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long s = base + k * kRebinThreads + threadIdx.x;
-        kn[k] = s < n ? __ldg(rkn + s) : -1;
-        id[k] = IDENT ? (int)s : (s < n ? __ldg(rid + s) : 0);
-    }
-    // the gathers of each stayer (its cell's arrivals, its diameter) go out
-    // before the block waits for the departure table
-#pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long s = base + k * kRebinThreads + threadIdx.x;
-        a0[k] = a1[k] = 0;
-        if (s < n && kn[k] >= 0) {
-            a0[k] = __ldg(arr_start + kn[k]);
-            a1[k] = __ldg(arr_start + kn[k] + 1);
-            d[k] = __ldg(vol + id[k]);
+        for (int k = 0; k < kRebinItems; ++k) {
+            const int s = b * kRebinTile + k * kRebinThreads + threadIdx.x;
+            const bool valid = b < nblk && s < n;
+            kn[k] = valid ? __ldg(rkn + s) : -1;
+            id[k] = IDENT ? s : (valid ? __ldg(rid + s) : 0);
         }
-        db[k] = __ballot_sync(full, s < n && kn[k] < 0);
-        if (lane == 0) s_tab[k * W + warp] = __popc(db[k]);
-    }
-    __syncthreads();
-    static_assert(kRebinItems * W == 32, "one lane per (row, warp) entry");
-    if (warp == 0) {   // exclusive prefix over (row, warp) in slot order: one shuffle scan
-        const int c = s_tab[lane];
-        int incl = c;
+    };
+    fetch(bid);
+    int turn = 0;
+    for (int b = bid; b < nblk; b += nb, turn ^= 1) {
+        const int base = b * kRebinTile;
+        int2 ah[kRebinItems];
+        int c[kRebinItems], i[kRebinItems];
+        unsigned db[kRebinItems];
+        int* tab = s_tab[turn];
+#pragma unroll
+        for (int k = 0; k < kRebinItems; ++k) {
+            const int s = base + k * kRebinThreads + threadIdx.x;
+            c[k] = kn[k];
+            i[k] = id[k];
+            ah[k] = make_int2(0, 0);
+            if (c[k] >= 0) ah[k] = __ldg(arr + c[k]);
+            db[k] = __ballot_sync(full, s < n && c[k] < 0);
+            if (lane == 0) tab[k * W + warp] = __popc(db[k]);
+        }
+        fetch(b + nb);
+        __syncthreads();
+        static_assert(kRebinItems * W == 32, "one lane per (row, warp) entry");
+        // exclusive prefix over (row, warp) in slot order: every warp its own shuffle scan
+        const int mine = tab[lane];
+        int incl = mine;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const int o = __shfl_up_sync(full, incl, off);
             if (lane >= off) incl += o;
         }
-        s_tab[lane] = __ldg(blk_start + bid) + incl - c;
-    }
-    __syncthreads();
+        incl += __ldg(blk_start + b) - mine;
 #pragma unroll
-    for (int k = 0; k < kRebinItems; ++k) {
-        const long long s = base + k * kRebinThreads + threadIdx.x;
-        if (s >= n || kn[k] < 0) continue;
-        const int D = s_tab[k * W + warp] + __popc(db[k] & lanemask_lt());
-        const int c = kn[k], i = id[k];
-        const long long ns = s - D + a0[k] + (a1[k] > a0[k] ? arrivals_below(arr_list, a0[k], a1[k], i) : 0);
-        if ((unsigned long long)ns >= (unsigned long long)n) continue;   // never for a valid binning
-        perm[ns] = i;
-        key_sorted[ns] = c;
-        inv_perm[i] = (int)ns;
-        vol_sorted[ns] = d[k];
+        for (int k = 0; k < kRebinItems; ++k) {
+            const int s = base + k * kRebinThreads + threadIdx.x;
+            const int D = __shfl_sync(full, incl, k * W + warp) + __popc(db[k] & lanemask_lt());
+            if (c[k] < 0) continue;
+            int ns = s - D + ah[k].x;
+            if (ah[k].y && !place) ns += movers_below(mov, ah[k].y, i[k]);
+            if ((unsigned)ns >= (unsigned)n) continue;   // never for a valid binning
+            if (place) {
+                place[ns] = i[k];
+                continue;
+            }
+            perm[ns] = i[k];
+            key_sorted[ns] = c[k];
+            if (!IDENT) inv_perm[i[k]] = ns;
+        }
     }
 }
 
-// Movers: the stayers of the new cell with an id below the mover's (a binary
-// search over the old segment, whose ids ascend, then a count of the
-// stayers before that point) and the arrivals with an id below it.
-template <typename T, bool IDENT>
+// Movers, one warp per block of old slots: the stayers of the new cell with
+// an id below the mover's (a binary search over the old segment, whose ids
+// ascend, then a count of the stayers before that point) and the movers of
+// its list with an id below it.
+template <bool IDENT>
 __device__ __forceinline__ void rebin_movers_body(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn,
-                                                  long long n, const int32_t* __restrict__ cs_old,
+                                                  long long n, const int32_t* __restrict__ blk_start,
+                                                  const int32_t* __restrict__ cs_old,
                                                   const int32_t* __restrict__ cs_new,
-                                                  const int32_t* __restrict__ arr_start,
-                                                  const int2* __restrict__ arr_list, long long nbulk,
-                                                  const T* __restrict__ vol, int32_t* __restrict__ perm,
-                                                  int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-                                                  T* __restrict__ vol_sorted, long long bid, long long nb) {
-    const long long nm = __ldg(arr_start + nbulk);   // all arrivals
-    for (long long q = bid * blockDim.x + threadIdx.x; q < nm; q += nb * blockDim.x) {
-        const int2 m = arr_list[q];
-        const int i = m.x, c = m.y;
-        const int o0 = __ldg(cs_old + c), o1 = __ldg(cs_old + c + 1);
-        int lo = o0, hi = o1;
-        if (IDENT) {
-            lo = i < o0 ? o0 : (i > o1 ? o1 : i);   // the old ids of the segment are its slots
-        } else {
-            while (lo < hi) {
-                const int mid = lo + ((hi - lo) >> 1);
-                if (__ldg(rid + mid) < i) lo = mid + 1;
-                else hi = mid;
+                                                  const int2* __restrict__ arr, const int4* __restrict__ mov,
+                                                  int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted,
+                                                  int32_t* __restrict__ inv_perm, int32_t* __restrict__ place,
+                                                  long long nblk, long long bid, long long nb) {
+    const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+    for (long long b = bid * W + (threadIdx.x >> 5); b < nblk; b += nb * W) {
+        const int cntb = __ldg(blk_start + b + 1) - __ldg(blk_start + b);
+        for (int j = lane; j < cntb; j += 32) {
+            const int4 m = __ldg(mov + b * kRebinTile + j);
+            const int i = m.x, c = m.y;
+            long long ns;
+            if (place) {
+                // after the cell's stayers, in the order of arrival
+                ns = (long long)__ldg(cs_new + c + 1) - (__ldg(&arr[c + 1].x) - __ldg(&arr[c].x)) + m.w;
+            } else {
+                const int o0 = __ldg(cs_old + c), o1 = __ldg(cs_old + c + 1);
+                int lo = o0, hi = o1;
+                if (IDENT) {
+                    lo = i < o0 ? o0 : (i > o1 ? o1 : i);   // the old ids of the segment are its slots
+                } else {
+                    while (lo < hi) {
+                        const int mid = lo + ((hi - lo) >> 1);
+                        if (__ldg(rid + mid) < i) lo = mid + 1;
+                        else hi = mid;
+                    }
+                }
+                int stay = 0;
+                for (int p = o0; p < lo; ++p) stay += __ldg(rkn + p) >= 0;
+                ns = (long long)__ldg(cs_new + c) + stay + movers_below(mov, __ldg(&arr[c].y), i);
             }
+            if ((unsigned long long)ns >= (unsigned long long)n) continue;   // never for a valid binning
+            if (place) {
+                place[ns] = i;
+                continue;
+            }
+            perm[ns] = i;
+            key_sorted[ns] = c;
+            if (!IDENT) inv_perm[i] = (int)ns;
         }
-        int stay = 0;
-        for (int p = o0; p < lo; ++p) stay += __ldg(rkn + p) >= 0;
-        const int a0 = __ldg(arr_start + c), a1 = __ldg(arr_start + c + 1);
-        const long long ns = (long long)__ldg(cs_new + c) + stay + arrivals_below(arr_list, a0, a1, i);
-        emit<T>(n, ns, i, c, perm, key_sorted, inv_perm, vol, vol_sorted);
     }
 }
 
 // Every particle's new slot in one launch: blocks [0, mgrid) place the
-// movers (first, so that their searches run beside the stayers), blocks
-// [mgrid, mgrid + nblk) the stayers of one block of old slots each.
-template <typename T, bool IDENT>
-__global__ void __launch_bounds__(kRebinThreads)
+// movers (first, so that their searches run beside the stayers), the other
+// blocks the stayers.  In the fallback both put the ids into their cells'
+// places of `place` in any order.  Bound by HBM and by the latency of the
+// gather behind each record: 32M particles 105 us, against 207 for one
+// block of old slots per CTA with the diameters and the inverse carried along.
+template <bool IDENT>
+__global__ void __launch_bounds__(kRebinThreads, 6)
 k_rebin_slots(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn, long long n,
               const int32_t* __restrict__ blk_start, const int32_t* __restrict__ cs_old,
-              const int32_t* __restrict__ cs_new, const int32_t* __restrict__ arr_start,
-              const int2* __restrict__ arr_list, long long nbulk, const T* __restrict__ vol,
+              const int32_t* __restrict__ cs_new, const int2* __restrict__ arr, const int4* __restrict__ mov,
               int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-              T* __restrict__ vol_sorted, const int32_t* __restrict__ ctr, long long nblk, long long mgrid) {
+              int32_t* __restrict__ place, const int32_t* __restrict__ ctr, long long nblk, long long mgrid) {
     pdl_wait();
-    if (ctr[RB_FALLBACK]) return;
+    int32_t* const where = ctr[RB_FALLBACK] ? place : nullptr;
+    if (ctr[RB_MOVERS] == 0) {
+        // slot s keeps its particle and cell; with the identity hint the
+        // particles are renumbered to their slots
+        if (IDENT)
+            for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x)
+                perm[s] = (int)s;
+        return;
+    }
     if ((long long)blockIdx.x < mgrid)
-        rebin_movers_body<T, IDENT>(rid, rkn, n, cs_old, cs_new, arr_start, arr_list, nbulk, vol, perm, key_sorted,
-                                    inv_perm, vol_sorted, blockIdx.x, mgrid);
+        rebin_movers_body<IDENT>(rid, rkn, n, blk_start, cs_old, cs_new, arr, mov, perm, key_sorted, inv_perm, where,
+                                 nblk, blockIdx.x, mgrid);
     else
-        rebin_stay_body<T, IDENT>(rid, rkn, n, blk_start, arr_start, arr_list, vol, perm, key_sorted, inv_perm,
-                                  vol_sorted, blockIdx.x - mgrid, nblk);
+        rebin_stay_body<IDENT>(rid, rkn, (int)n, blk_start, arr, mov, perm, key_sorted, inv_perm, where, (int)nblk,
+                               (int)(blockIdx.x - mgrid), (int)(gridDim.x - mgrid));
 }
 
 template <typename T>
-static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, double* eps_fill, T* rec_fill,
-                            T* eps_t_fill) {
+static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, StepEps* eps) {
     const long long nbulk = g->gd.nbulk;
     const RebinPtrs R = rebin_ptrs(g);
     const long long nblk = (n + kRebinTile - 1) / kRebinTile;
     if (nblk > g->rb_nblk) return CG_ERR_OUT_OF_RANGE;
-    CG_CUDA(cudaMemsetAsync(g->rb_small, 0, sizeof(int32_t) * rebin_small_ints(nbulk, g->rb_nblk), g->stream));
-    if (!ident)
-        CG_LAUNCH(g, "rebin_key", k_rebin_key<T>, (unsigned)nblk, kRebinThreads, 0, pos, n, g->gd, g->key, (T*)g->vol,
-                  g->status, eps_fill, rec_fill, eps_t_fill);
-    if (ident)
-        CG_LAUNCH(g, "rebin_mark", (k_rebin_mark<T, true>), (unsigned)nblk, kRebinThreads, 0, pos, n, g->gd,
-                  (const int32_t*)nullptr, (const int32_t*)g->key_sorted, g->key, (T*)g->vol, g->rb_rid, g->rb_rkn,
-                  R.arr, R.dep, g->rb_mov, R.blk, R.ctr, g->status, eps_fill, rec_fill, eps_t_fill);
-    else
-        CG_LAUNCH(g, "rebin_mark", (k_rebin_mark<T, false>), (unsigned)nblk, kRebinThreads, 0, pos, n, g->gd,
-                  (const int32_t*)g->perm, (const int32_t*)g->key_sorted, g->key, (T*)g->vol, g->rb_rid, g->rb_rkn,
-                  R.arr, R.dep, g->rb_mov, R.blk, R.ctr, g->status, (double*)nullptr, (T*)nullptr, (T*)nullptr);
-    const unsigned cgrid = (unsigned)std::max<long long>(1, std::min<long long>(std::max((nbulk + 255) / 256, nblk),
-                                                                               (long long)g->num_sms * 8));
-    if (ident)
-        CG_LAUNCH(g, "rebin_cells", k_rebin_cells<true>, cgrid, kRebinThreads, 0, (const int32_t*)g->cell_start,
-                  nbulk, (const int32_t*)R.dep, (const int32_t*)R.arr, R.cnt, (const int32_t*)R.ctr, g->key,
-                  (const int32_t*)g->rb_rkn, n, g->key2);
-    else
-        CG_LAUNCH(g, "rebin_cells", k_rebin_cells<false>, cgrid, kRebinThreads, 0, (const int32_t*)g->cell_start,
-                  nbulk, (const int32_t*)R.dep, (const int32_t*)R.arr, R.cnt, (const int32_t*)R.ctr, g->key,
-                  (const int32_t*)g->rb_rkn, n, g->key2);
-    {
-        const int32_t* in[3] = {R.cnt, R.arr, R.blk};
-        int32_t* out[3] = {R.cnt, R.arr, R.blk};
-        const long long m[3] = {nbulk + 1, nbulk + 1, nblk + 1};
-        CG_TRY(scan_exclusive(g, 3, in, out, m, R.ctr + RB_MOVERS));
-    }
-    const unsigned pgrid = (unsigned)std::max<long long>(1, std::min<long long>((nblk + 7) / 8, (long long)g->num_sms * 8));
-    CG_LAUNCH(g, "rebin_place", k_rebin_place, pgrid, 256, 0, (const int2*)g->rb_mov, (const int32_t*)R.blk, nblk,
-              (const int32_t*)R.arr, g->rb_arr, (const int32_t*)R.ctr);
-    const long long mgrid = (long long)g->num_sms * 8;
-#define CG_REBIN_SLOTS(ID)                                                                                        \
-    CG_LAUNCH(g, "rebin_slots", (k_rebin_slots<T, ID>), (unsigned)(mgrid + nblk), kRebinThreads, 0,                 \
-              (const int32_t*)g->rb_rid, (const int32_t*)g->rb_rkn, n, (const int32_t*)R.blk,                      \
-              (const int32_t*)g->cell_start, (const int32_t*)R.cnt, (const int32_t*)R.arr, (const int2*)g->rb_arr,   \
-              nbulk, (const T*)g->vol, g->perm, g->key_sorted, g->inv_perm, (T*)g->vol_sorted,                      \
-              (const int32_t*)R.ctr, nblk, mgrid)
+    const EpsOut<T> eo = eps_out<T>(g, eps);
+    CG_CUDA(cudaMemsetAsync(R.arr, 0, R.zero_bytes, g->stream));
+    // the caller's order: resident CTAs that walk the blocks of old slots, the
+    // next block's ids and cells loaded ahead of the gather they lead to
+    const long long walk = (long long)g->num_sms * (sizeof(T) == 4 ? 4 : 3);
+#define CG_REBIN_MARK(ID, VOL)                                                                                     \
+    CG_LAUNCH(g, "rebin_mark", (k_rebin_mark<T, ID, VOL>), (unsigned)(ID ? nblk : std::min(nblk, walk)), kRebinThreads, 0, pos, (int)n, g->gd,    \
+              (const int32_t*)g->perm, (const int32_t*)g->key_sorted, g->rb_rid, g->rb_rkn, R.arr, R.dep,           \
+              g->rb_mov, R.blk, R.ctr, g->status, eo.acc, eo.big)
     if (ident) {
-        CG_REBIN_SLOTS(true);
+        if (eps) CG_REBIN_MARK(true, true);
+        else CG_REBIN_MARK(true, false);
     } else {
-        CG_REBIN_SLOTS(false);
+        if (eps) CG_REBIN_MARK(false, true);
+        else CG_REBIN_MARK(false, false);
     }
+#undef CG_REBIN_MARK
+    const long long tiles = rebin_tiles(nbulk + 1), btiles = rebin_tiles(nblk + 1);
+    T* vpart = (T*)part_ptr(g, PS_VOL);
+#define CG_REBIN_CELLS(EPS, SUMS)                                                                                  \
+    CG_LAUNCH(g, "rebin_cells", (k_rebin_cells<T, EPS, SUMS>), (unsigned)(tiles + btiles), 256, 0,                  \
+              (const int32_t*)g->cell_start, g->gd, (const int32_t*)R.dep, (const int2*)R.arr, R.cnt,               \
+              (const int32_t*)R.blk, nblk, (const int32_t*)R.ctr, R.part, tiles, eo, vpart)
+    if (eps && eps->sums) CG_REBIN_CELLS(true, true);
+    else if (eps) CG_REBIN_CELLS(true, false);
+    else CG_REBIN_CELLS(false, false);
+#undef CG_REBIN_CELLS
+    if (eps) {
+        g->part_blocks[PS_VOL] = eps->sums ? tiles : -1;
+        eps->formed = true;
+        if (eps->ready) CG_CUDA(cudaEventRecord(eps->ready, g->stream));
+    }
+    CG_LAUNCH(g, "rebin_scan", k_rebin_scan, (unsigned)(tiles + btiles), 256, 0, R.cnt, R.arr, nbulk + 1, R.blk, nblk,
+              (const int32_t*)R.part, tiles, (const int32_t*)R.ctr);
+    const long long mgrid = std::min<long long>((nblk + 7) / 8, (long long)g->num_sms * 8);
+    // resident blocks that walk the old slots (the sorted step), or, where the
+    // scattered stores of a caller's random order dominate, a block per 1024
+    // slots (4M particles: 42 us against 50)
+    const long long sgrid = ident ? std::min<long long>(nblk, (long long)g->num_sms * 6) : nblk;
+#define CG_REBIN_SLOTS(ID)                                                                                        \
+    CG_LAUNCH(g, "rebin_slots", (k_rebin_slots<ID>), (unsigned)(mgrid + sgrid), kRebinThreads, 0,                   \
+              (const int32_t*)g->rb_rid, (const int32_t*)g->rb_rkn, n, (const int32_t*)R.blk,                      \
+              (const int32_t*)g->cell_start, (const int32_t*)R.cnt, (const int2*)R.arr, (const int4*)g->rb_mov,      \
+              g->perm, g->key_sorted, g->inv_perm, g->val1, (const int32_t*)R.ctr, nblk, mgrid)
+    if (ident) CG_REBIN_SLOTS(true);
+    else CG_REBIN_SLOTS(false);
 #undef CG_REBIN_SLOTS
-    // fallback: placement and per-cell sort from the scanned counts
-    CG_TRY(launch_cellsort_tail(g, n, R.cnt, R.ctr + RB_FALLBACK));
-    CG_CUDA(cudaMemcpyAsync(g->cell_start, R.cnt, sizeof(int32_t) * (nbulk + 1), cudaMemcpyDeviceToDevice, g->stream));
-    return CG_OK;
+    // the starts to their place; in the fallback also the sort of every cell
+    return launch_cellsort_fallback(g, R.cnt, R.ctr + RB_FALLBACK, g->cell_start, ident ? nullptr : g->inv_perm);
 }
 
-// The caller-order cells of the last binning (g->key), formed from the
-// mover records when an identity-hint binning left them out.
-cg_status ensure_keys(cg_grids* g, long long n) {
-    if (g->key_valid || n <= 0) return CG_OK;
+// Caller-order values of the binning's slots: the cell of every particle, or
+// its slot.
+__global__ void __launch_bounds__(256)
+k_scatter_bins(const int32_t* __restrict__ perm, const int32_t* __restrict__ key_sorted, long long n,
+               int32_t* __restrict__ out) {
+    pdl_wait();
+    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x)
+        out[__ldg(perm + s)] = key_sorted ? __ldg(key_sorted + s) : (int)s;
+}
+
+cg_status copy_cells(cg_grids* g, long long n, int32_t* cell_out) {
+    if (n <= 0) return CG_OK;
+    if (g->key_valid) {
+        CG_CUDA(cudaMemcpyAsync(cell_out, g->key, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, g->stream));
+        return CG_OK;
+    }
     const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)g->num_sms * 8);
-    CG_LAUNCH(g, "rebin_keys", k_rebin_keys, grid, 256, 0, (const int32_t*)g->rb_rkn, n, g->key);
-    g->key_valid = true;
+    CG_LAUNCH(g, "bin_cells", k_scatter_bins, grid, 256, 0, (const int32_t*)g->perm, (const int32_t*)g->key_sorted, n,
+              cell_out);
     return CG_OK;
 }
 
-cg_status launch_rebin(cg_grids* g, long long n, const void* pos_d, bool ident, double* eps_fill, void* rec_fill,
-                       void* eps_t_fill) {
-    if (g->fp64) return rebin_impl<double>(g, n, (const double*)pos_d, ident, eps_fill, (double*)rec_fill,
-                                           (double*)eps_t_fill);
-    return rebin_impl<float>(g, n, (const float*)pos_d, ident, eps_fill, (float*)rec_fill, (float*)eps_t_fill);
+cg_status ensure_inverse(cg_grids* g, long long n) {
+    if (g->inv_valid || n <= 0) return CG_OK;
+    const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)g->num_sms * 8);
+    CG_LAUNCH(g, "bin_inverse", k_scatter_bins, grid, 256, 0, (const int32_t*)g->perm, (const int32_t*)nullptr, n,
+              g->inv_perm);
+    g->inv_valid = true;
+    return CG_OK;
+}
+
+cg_status launch_rebin(cg_grids* g, long long n, const void* pos_d, bool ident, StepEps* eps) {
+    return g->fp64 ? rebin_impl<double>(g, n, (const double*)pos_d, ident, eps)
+                   : rebin_impl<float>(g, n, (const float*)pos_d, ident, eps);
 }
 
 }  // namespace cg
