@@ -79,8 +79,8 @@ enum {
 #define CG_SORT_CELLS_AUTO_DENSITY 32   /* particles per bulk cell */
 
 /* Stencil reads of the drag (cg_grid_desc.stencil). */
-#define CG_STENCIL_GATHER 0   /* the eight records of each particle's stencil from global memory */
-#define CG_STENCIL_WINDOW 1   /* in the sorted step, each warp's stencil window staged in shared memory */
+#define CG_STENCIL_GATHER 0
+#define CG_STENCIL_WINDOW 1
 
 /* Number of counters returned by cg_sync_status. */
 #define CG_NCOUNTS 5
@@ -110,18 +110,13 @@ enum {
  *                 below 2^20 bulk cells, up to 8 from 2^20 on; an instance of
  *                 a batch (cg_batch_create) takes the digit sort unless its
  *                 descriptor asks for CG_SORT_CELLS
- *   stencil     how the drag reads the bulk records of each particle's
- *               trilinear stencil (both give the same bits):
- *               CG_STENCIL_GATHER (0): eight 16-byte loads per particle,
- *                 served by L1 and L2 (the bulk record of a 2^22-cell grid
- *                 is 64 MB, inside the 129 MB L2); the faster choice;
- *               CG_STENCIL_WINDOW (1): in cg_step_sorted on the FP32
- *                 trilinear path, each warp stages the bounding box of its
- *                 32 particles' stencils (with the +1 halo) in shared memory
- *                 and reads the corners there; a box of more than 64
- *                 records takes the global gather (measured slower, see
- *                 the design notes: the kernel is bound by instruction
- *                 issue, and the window costs instructions)
+ *   stencil     CG_STENCIL_GATHER (0) or CG_STENCIL_WINDOW (1); both give
+ *               the same bits, and both now run the same kernels:
+ *               cg_step_sorted on the FP32 trilinear path stages the bulk
+ *               records around a run of cells in shared memory for each
+ *               warp, every other drag reads the eight 16-byte records of a
+ *               particle's stencil through L1 and L2 (the bulk record of a
+ *               2^22-cell grid is 64 MB, inside the 129 MB L2)
  * Limits: fine_n[a] % ratio == 0, bulk cells >= 2 per axis, at most 2^22
  * bulk cells and 2^31 - 1 fine cells. */
 typedef struct {

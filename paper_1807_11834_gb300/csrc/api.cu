@@ -341,6 +341,7 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
         gd.invH[a] = 1.0 / gd.H[a];
         gd.x0f[a] = (float)d.origin[a];
         gd.xhif[a] = (float)gd.xhi[a];
+        gd.topf[a] = (float)(nb[a] - 2);
         gd.invHf[a] = (float)gd.invH[a];
         gd.ax0f[a] = (float)fabs(d.origin[a] * gd.invH[a]);
         split_ff(d.origin[a], gd.x0h[a], gd.x0l[a]);
@@ -576,7 +577,7 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     CG_TRY(launch_bin(g, n, p->pos_d, &eps));
     // sorted diameters of this binning
     if (!eps.formed) CG_TRY(launch_deposit_volume(g, n, nullptr, &eps));
-    CG_TRY(copy_bins(g, n, o->cell, o->perm, o->cell_start));
+    CG_TRY(copy_bins(g, n, o->cell, sorted_out ? nullptr : o->perm, o->cell_start));   // the sorted drag writes perm
     if (!fused) {
         CG_CUDA(cudaStreamWaitEvent(g->stream, g->ev_avg, 0));
         CG_TRY(launch_pack(g, o->eps_bulk, o->u_bulk, o->eps_fine != nullptr));
@@ -595,7 +596,8 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
                                    dt, true));
     else
         CG_TRY(launch_drag(g, n, p->pos_d, p->vel, o->force, o->S_bulk, true, dt, true, o->implicit_bulk,
-                           sorted_out ? sorted_out->pos_d : nullptr, sorted_out ? sorted_out->vel : nullptr));
+                           sorted_out ? sorted_out->pos_d : nullptr, sorted_out ? sorted_out->vel : nullptr,
+                           sorted_out ? o->perm : nullptr));
     // the binning above lists the sorted output's particle i at slot i
     if (sorted_out && g->n_binned == n) g->hint_ident = sorted_out->pos_d;
     const size_t bs = (size_t)g->gd.nbulk * g->tsize, fs = (size_t)g->gd.nfine * g->tsize;

@@ -178,7 +178,7 @@ cg_status plan(cg_batch* b) {
         // virtual blocks per phase
         long long* B = &blocks[(size_t)i];
         auto set = [&](int ph, long long v) { B[(size_t)ph * ni] = v; };
-        const long long chunks = cdiv(n, kSegChunk);
+        const long long chunks = cdiv(n, seg_chunk(n));
         const long long seg = std::max(1LL, cdiv(chunks, 8LL * c.seg_chunks));
         const long long cellb = cdiv(nb, 256);
         set(BP_ZERO, cdiv(nb + 1, 1024));

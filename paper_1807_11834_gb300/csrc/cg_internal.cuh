@@ -122,6 +122,7 @@ struct GridDev {
     float x0h[3], x0l[3];   // x0 as float-float
     float ihh[3], ihl[3];   // 1/H as float-float
     float xbh[3], xbl[3];   // -(x0 / H + 1/2) as float-float: the lattice coordinate is x / H + xb
+    float topf[3];      // n_b - 2
     float invVBf, VBf, Vff;
     float VBh, VBl, Vfh, Vfl;   // V_B, V_f as float-float
     // physics
@@ -362,6 +363,14 @@ cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps =
 // Porosity of the binned particles: from the sorted diameters of a binning
 // from scratch (pos_d null), or gathered from pos_d [n] T4.
 cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, StepEps* eps);
+// Slots per chunk of the segmented sums.
+__host__ __device__ inline int seg_chunk(long long) { return 256; }
+// Threads per block of the kernels over chunks: few chunks take smaller blocks, so that
+// they reach every SM (10,000 particles, FP64, blocks of 256 -> 32: 47 -> 19 us).
+inline unsigned seg_threads(const cg_grids* g, long long n) {
+    const long long per_sm = (n + seg_chunk(n) - 1) / seg_chunk(n) / g->num_sms;
+    return per_sm < 8 ? 32 : per_sm < 16 ? 64 : per_sm < 32 ? 128 : 256;
+}
 // cleared: S_bulk is zero already.
 cg_status launch_deposit_sorted_force(cg_grids* g, long long n, void* S_bulk, bool cleared);
 // Gather the particle records into the binned order (cg_reorder_particles).
@@ -374,10 +383,11 @@ cg_status launch_average(cg_grids* g, const void* u_fine, void* u_bulk, void* va
 cg_status launch_pack(cg_grids* g, const double* eps, const void* u_bulk, bool want_eps_t);
 // pos_out, vel_out (nullable, needs S_bulk): the particles, advanced when
 // dt > 0, are written to these arrays in the order of the binning.
-// S_cleared: S_bulk is zero already.
+// perm_out (nullable): also gets the binning's permutation.  S_cleared: S_bulk
+// is zero already.
 cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* vel, void* force, void* S_bulk,
                       bool sums, double dt, bool S_cleared = false, void* coef_bulk = nullptr, void* pos_out = nullptr,
-                      void* vel_out = nullptr);
+                      void* vel_out = nullptr, int32_t* perm_out = nullptr);
 // Learned drag (FP32 only): bulk4 must hold (phi of this step, stale u).
 cg_status launch_drag_learned(cg_grids* g, const cg_mlp* m, long long n, void* pos_d, void* vel,
                               const void* var_stale, const void* u_fine, int32_t age, void* force, void* S_bulk,
@@ -658,7 +668,7 @@ __device__ __forceinline__ int cell_of_d(double x, double y, double z, const Gri
 // ----------------------------------------------------------------------
 // Segmented reductions over the sorted particle order.
 //
-// The sorted order is cut into chunks of kSegChunk slots; warp w owns the
+// The sorted order is cut into chunks of seg_chunk(n) slots; warp w owns the
 // segments (cells) that START in its chunks and runs past a chunk's end to
 // finish its last segment, so every segment is reduced by exactly one warp
 // and the work follows the particles, not the cells (a dense bed occupying
@@ -667,12 +677,11 @@ __device__ __forceinline__ int cell_of_d(double x, double y, double z, const Gri
 // scan.  The rounds start at the range's first slot, so the summation order
 // depends only on the chunk's slots, never on the launch shape.
 // ----------------------------------------------------------------------
-constexpr int kSegChunk = 256;
-
 // Range [s, t) of sorted slots owned by the chunk starting at `base`.
 __device__ __forceinline__ void seg_chunk_range(long long base, long long n, const int32_t* __restrict__ key_sorted,
                                                 const int32_t* __restrict__ cs, long long& s, long long& t) {
-    const long long last = (base + kSegChunk < n ? base + kSegChunk : n) - 1;
+    const int len = seg_chunk(n);
+    const long long last = (base + len < n ? base + len : n) - 1;
     s = base;
     if (base > 0) {
         const int k0 = __ldg(key_sorted + base);

@@ -91,7 +91,7 @@ __device__ __forceinline__ void deposit_sorted_force_body(const T* __restrict__ 
                                                           T* __restrict__ S, Blk b) {
     const long long wg = b.id * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = b.n * (blockDim.x >> 5);
-    for (long long base = wg * kSegChunk; base < n; base += nw * kSegChunk) {
+    for (long long base = wg * seg_chunk(n); base < n; base += nw * seg_chunk(n)) {
         long long s, t;
         seg_chunk_range(base, n, key_sorted, cs, s, t);
         seg_rounds<T, 3>(
@@ -116,7 +116,7 @@ __device__ __forceinline__ void deposit_implicit_body(const T* __restrict__ Bs, 
                                                       T* __restrict__ coef, Blk b) {
     const long long wg = b.id * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = b.n * (blockDim.x >> 5);
-    for (long long base = wg * kSegChunk; base < n; base += nw * kSegChunk) {
+    for (long long base = wg * seg_chunk(n); base < n; base += nw * seg_chunk(n)) {
         long long s, t;
         seg_chunk_range(base, n, key_sorted, cs, s, t);
         seg_rounds<T, 4>(
@@ -163,7 +163,7 @@ k_deposit_momentum(const T* __restrict__ F, long long n, const int32_t* __restri
     pdl_wait();
     const long long wg = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long base = wg * kSegChunk; base < n; base += nw * kSegChunk) {
+    for (long long base = wg * seg_chunk(n); base < n; base += nw * seg_chunk(n)) {
         long long s, t;
         seg_chunk_range(base, n, key_sorted, cs, s, t);
         seg_rounds<T, 3>(
@@ -323,13 +323,10 @@ static inline unsigned blocks_for(long long n, int per) { return (unsigned)((n +
 
 // Grid of the segmented deposits: at most one chunk per warp, and no more
 // CTAs than are resident at once (the reaction's 48 registers allow five per
-// SM, 64 four), so the grid-stride loop runs without a second, partial wave.  Few chunks take
-// blocks of one warp, so that they reach as many SMs as there are chunks
-// (10,000 particles, FP64: 40 chunks, 47 -> 19 us).
-static unsigned seg_threads(cg_grids* g, long long n) { return n <= (long long)g->num_sms * 8 * kSegChunk ? 32 : 256; }
+// SM, 64 four), so the grid-stride loop runs without a second, partial wave.
 static unsigned seg_blocks(cg_grids* g, long long n, int per_sm = 4) {
-    const long long chunks = (n + kSegChunk - 1) / kSegChunk, per = seg_threads(g, n) / 32;
-    return (unsigned)std::max(1LL, std::min((chunks + per - 1) / per, (long long)g->num_sms * (per == 1 ? 8 : per_sm)));
+    const long long chunks = (n + seg_chunk(n) - 1) / seg_chunk(n), per = seg_threads(g, n) / 32;
+    return (unsigned)std::max(1LL, std::min((chunks + per - 1) / per, (long long)g->num_sms * per_sm * 8 / per));
 }
 
 template <typename T>

@@ -18,8 +18,9 @@
 // carry only the final float rounding even at |xi| ~ 100; the correlations
 // run in float with explicitly rounded operations, their powers, logarithm,
 // roots and reciprocals on the special-function unit (drag_law.cuh).
-// On request (CG_STENCIL_WINDOW) the sorted step stages each warp's stencil
-// window in shared memory instead of gathering from L2 (window_gather).
+// The sorted step's kernel (k_drag_sorted) takes the particles in cell order,
+// stages the bulk records around a run of cells in shared memory and sums the
+// reaction itself.
 #include <algorithm>
 
 #include "cg_internal.cuh"
@@ -80,18 +81,24 @@ __device__ __forceinline__ DragOne<T> drag_from(const V4<T>& x, const V4<T>& v, 
     r.u[2] = v.z;
     if (EULER) {
         const T inv_m = X::rcp_(r.m);   // one reciprocal for the three components
+        bool out = false;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            T ua = X::fma_(dt, X::fma_(r.f[a], inv_m, P.g[a]), r.u[a]);
-            T xa = X::fma_(dt, ua, r.x[a]);
+            r.u[a] = X::fma_(dt, X::fma_(r.f[a], inv_m, P.g[a]), r.u[a]);
+            r.x[a] = X::fma_(dt, r.u[a], r.x[a]);
             // the FP32 path reads the bounds' float copies (no conversion in the loop)
             const T lo = sizeof(T) == 4 ? (T)g.x0f[a] : (T)g.x0[a];
             const T hi = sizeof(T) == 4 ? (T)g.xhif[a] : (T)g.xhi[a];
-            if (xa < lo) { xa = X::sub(X::mul(T(2), lo), xa); ua = -ua; }
-            else if (xa > hi) { xa = X::sub(X::mul(T(2), hi), xa); ua = -ua; }
-            r.x[a] = xa;
-            r.u[a] = ua;
+            out = out || r.x[a] < lo || r.x[a] > hi;
         }
+        if (out)   // specular walls: rare, so one branch for the three axes
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const T lo = sizeof(T) == 4 ? (T)g.x0f[a] : (T)g.x0[a];
+                const T hi = sizeof(T) == 4 ? (T)g.xhif[a] : (T)g.xhi[a];
+                if (r.x[a] < lo) { r.x[a] = X::sub(X::mul(T(2), lo), r.x[a]); r.u[a] = -r.u[a]; }
+                else if (r.x[a] > hi) { r.x[a] = X::sub(X::mul(T(2), hi), r.x[a]); r.u[a] = -r.u[a]; }
+            }
     }
     return r;
 }
@@ -100,73 +107,6 @@ template <typename T, bool EULER>
 __device__ __forceinline__ DragOne<T> drag_one(const V4<T>& x, const V4<T>& v, const GridDev& g, const Phys<T>& P,
                                                const T* __restrict__ bulk4, T dt) {
     return drag_from<T, EULER>(x, v, gather(bulk4, x.x, x.y, x.z, g), g, P, dt);
-}
-
-// Stencil window of a warp (particles in cell order): the bounding box of
-// the 32 particles' stencil base cells, grown by the +1 halo on each axis,
-// staged from the bulk record into the warp's slice of shared memory with
-// one 16-byte load per record (x rows contiguous), and each particle's
-// eight corners read from there.  A box of more than kWinRecs records (the
-// particles far apart: not in cell order) takes the gather from global
-// memory.  Both give the same value (interp8).  All lanes of the warp call
-// it together (valid: the lane holds a particle).
-constexpr int kWinRecs = 64;
-__device__ __forceinline__ void st_win(V4<float>* q, const V4<float>& v) {
-    *reinterpret_cast<float4*>(q) = make_float4(v.x, v.y, v.z, v.w);
-}
-__device__ __forceinline__ void st_win(V4<double>* q, const V4<double>& v) {
-    reinterpret_cast<double2*>(q)[0] = make_double2(v.x, v.y);
-    reinterpret_cast<double2*>(q)[1] = make_double2(v.z, v.w);
-}
-__device__ __forceinline__ V4<float> ld_win(const V4<float>* q) {
-    const float4 v = *reinterpret_cast<const float4*>(q);
-    return {v.x, v.y, v.z, v.w};
-}
-__device__ __forceinline__ V4<double> ld_win(const V4<double>* q) {
-    const double2 a = reinterpret_cast<const double2*>(q)[0], b = reinterpret_cast<const double2*>(q)[1];
-    return {a.x, a.y, b.x, b.y};
-}
-template <typename T>
-__device__ __forceinline__ V4<T> window_gather(const T* __restrict__ bulk4, const V4<T>& x, bool valid,
-                                               const GridDev& g, V4<T>* __restrict__ win) {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    int i0 = 0, j0 = 0, k0 = 0;
-    T tx = T(0), ty = T(0), tz = T(0);
-    if (valid) {
-        axis_weight(x.x, g, 0, i0, tx);
-        axis_weight(x.y, g, 1, j0, ty);
-        axis_weight(x.z, g, 2, k0, tz);
-    }
-    const int big = 0x7fffffff;
-    const int imin = __reduce_min_sync(full, valid ? i0 : big), imax = __reduce_max_sync(full, valid ? i0 : -1);
-    const int jmin = __reduce_min_sync(full, valid ? j0 : big), jmax = __reduce_max_sync(full, valid ? j0 : -1);
-    const int kmin = __reduce_min_sync(full, valid ? k0 : big), kmax = __reduce_max_sync(full, valid ? k0 : -1);
-    const int nx = imax - imin + 2, ny = jmax - jmin + 2, nz = kmax - kmin + 2;
-    const int sy = g.nb[0], sz = g.nb[0] * g.nb[1];
-    const V4<T>* rec = reinterpret_cast<const V4<T>*>(bulk4);
-    V4<T> out = {T(0), T(0), T(0), T(0)};
-    // the box is small only if every extent is (no product of large extents)
-    if (nx <= kWinRecs && ny <= kWinRecs && nz <= kWinRecs && nx * ny * nz <= kWinRecs) {
-        const int W = nx * ny * nz;
-        // record r = wx + nx (wy + ny wz); (r + 1/2) / n never rounds across an integer for r < 2^11
-        const float inx = 1.0f / (float)nx, iny = 1.0f / (float)ny;
-        for (int r = lane; r < W; r += 32) {
-            const int q = (int)(((float)r + 0.5f) * inx);
-            const int wx = r - q * nx;
-            const int wz = (int)(((float)q + 0.5f) * iny);
-            const int wy = q - wz * ny;
-            st_win(win + r, ldv4(rec + (imin + wx) + sy * (jmin + wy) + sz * (kmin + wz)));
-        }
-        __syncwarp();
-        if (valid)
-            out = interp8<T>(win + (i0 - imin) + nx * ((j0 - jmin) + ny * (k0 - kmin)), nx, nx * ny, tx, ty, tz,
-                             [](const V4<T>* q) { return ld_win(q); });
-        __syncwarp();   // the next call restages the slice
-    } else if (valid) {
-        out = interp8<T>(rec + (i0 + sy * j0 + sz * k0), sy, sz, tx, ty, tz, [](const V4<T>* q) { return ldv4(q); });
-    }
-    return out;
 }
 
 // Per-lane diagnostics: V_p, F (3), |F|, m u (3) after the advance, clamped.
@@ -191,16 +131,12 @@ __device__ __forceinline__ void drag_lane_sums(T (&ls)[kDragSums], const DragOne
 // ----------------------------------------------------------------------
 // Bs (nullable): the semi-implicit record (beta, beta u_p) of each particle,
 // written to its sorted slot beside the force record.
-// pos_out, vel_out (nullable, with Fs): the particle records, advanced when
-// EULER, are written to their sorted slot of these arrays instead of in
-// place (the sorted step: the particles leave in this binning's order).
 template <typename T, bool EULER, bool PREFETCH = true>
 __device__ __forceinline__ void drag_body(T* pos, T* vel, long long n, const GridDev& g, const Phys<T>& P,
                                           const T* __restrict__ bulk4, T* __restrict__ F, T* __restrict__ Fs,
                                           const int32_t* __restrict__ inv_perm, T dt, T* __restrict__ part,
                                           long long pstride, int do_sums, unsigned long long* __restrict__ status,
-                                          Blk b, T* __restrict__ Bs = nullptr, T* __restrict__ pos_out = nullptr,
-                                          T* __restrict__ vel_out = nullptr) {
+                                          Blk b, T* __restrict__ Bs = nullptr) {
     T lane_sums[kDragSums];
 #pragma unroll
     for (int k = 0; k < kDragSums; ++k) lane_sums[k] = T(0);
@@ -237,10 +173,7 @@ __device__ __forceinline__ void drag_body(T* pos, T* vel, long long n, const Gri
         F[2 * n + p] = r.f[2];
         if (Fs) st4(Fs, slot, r.f[0], r.f[1], r.f[2], T(0));
         if (Bs) st4(Bs, slot, r.beta, r.beta * v.x, r.beta * v.y, r.beta * v.z);
-        if (pos_out) {
-            st4(pos_out, slot, r.x[0], r.x[1], r.x[2], x.w);
-            st4(vel_out, slot, r.u[0], r.u[1], r.u[2], v.w);
-        } else if (EULER) {
+        if (EULER) {
             st4(pos, p, r.x[0], r.x[1], r.x[2], x.w);
             st4(vel, p, r.u[0], r.u[1], r.u[2], v.w);
         }
@@ -261,88 +194,262 @@ __device__ __forceinline__ void drag_body(T* pos, T* vel, long long n, const Gri
     }
 }
 
-// The drag of particles in cell order (the sorted step) with the stencil
-// window of each warp (window_gather); otherwise as drag_body, whose
-// results it reproduces bit for bit.  The loop runs warp by warp (every
-// lane of a warp takes the same number of turns).
 template <typename T, bool EULER>
-__device__ __forceinline__ void drag_body_win(T* pos, T* vel, long long n, const GridDev& g, const Phys<T>& P,
-                                              const T* __restrict__ bulk4, T* __restrict__ F, T* __restrict__ Fs,
-                                              const int32_t* __restrict__ inv_perm, T dt, T* __restrict__ part,
-                                              long long pstride, int do_sums, unsigned long long* __restrict__ status,
-                                              Blk b, T* __restrict__ pos_out, T* __restrict__ vel_out,
-                                              V4<T>* __restrict__ win) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
+k_drag(T* pos, T* vel, long long n, GridDev g, Phys<T> P, const T* __restrict__ bulk4,
+       T* __restrict__ F, T* __restrict__ Fs, const int32_t* __restrict__ inv_perm, T dt,
+       T* __restrict__ part, long long pstride, int do_sums, unsigned long long* __restrict__ status,
+       T* __restrict__ Bs) {
+    pdl_wait();
+    drag_body<T, EULER>(pos, vel, n, g, P, bulk4, F, Fs, inv_perm, dt, part, pstride, do_sums, status,
+                        launch_blk(), Bs);
+}
+
+// Window of bulk records in a warp's shared memory (FP32): the stencils of
+// the particles of up to kWinCells consecutive cells of one x row reach from
+// the cell before to the cell after, in three rows of three layers.  The
+// strides are 2 and 4 modulo 8 records (of 16 bytes; eight cover the 32
+// banks), so that the eight stencils of one cell's octants lie in eight
+// different bank groups.
+constexpr int kWinX = 16, kWinCells = kWinX - 2, kWinRow = 18, kWinLayer = 60;
+constexpr int kWinRecs = 2 * kWinLayer + 2 * kWinRow + kWinX;
+struct Window {
+    int begin = 0, end = -1;   // cells covered (linear; none at first)
+    int I, J, K;               // position of the first one
+};
+// Make the window cover the cells [first, last]; false when they are not in
+// one row or too many.  Called by the whole warp with uniform arguments.
+__device__ __forceinline__ bool window_cover(Window& w, int first, int last, const V4<float>* __restrict__ rec,
+                                             const GridDev& g, V4<float>* __restrict__ win) {
+    if (first >= w.begin && last <= w.end) return true;
+    const int nbx = g.nb[0], nby = g.nb[1], nbz = g.nb[2];
+    const int row = (int)((unsigned)first / (unsigned)nbx);
+    const int end = min(first + kWinCells, (row + 1) * nbx) - 1;
+    if (last > end) return false;
+    w.begin = first;
+    w.end = end;
+    w.K = (int)((unsigned)row / (unsigned)nby);
+    w.J = row - w.K * nby;
+    w.I = first - row * nbx;
+    const int lane = threadIdx.x & 31, x = lane & (kWinX - 1);
+    const int cx = min(max(w.I - 1 + x, 0), nbx - 1);
+    __syncwarp();   // every lane has read the window before
+#pragma unroll
+    for (int p = 0; p < 5; ++p) {
+        const int q = 2 * p + (lane >> 4);   // row of the window, three per layer
+        const int z = (q * 11) >> 5, y = q - 3 * z;
+        if (q < 9) {
+            const int cy = min(max(w.J - 1 + y, 0), nby - 1), cz = min(max(w.K - 1 + z, 0), nbz - 1);
+            const V4<float> v = ldv4(rec + cx + nbx * (cy + nby * cz));
+            *reinterpret_cast<float4*>(win + x + kWinRow * y + kWinLayer * z) = make_float4(v.x, v.y, v.z, v.w);
+        }
+    }
+    __syncwarp();
+    return true;
+}
+__device__ __forceinline__ Pair2 ld_win(const V4<float>* q) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(q);
+    return {v.x, v.y};
+}
+// (eps, u) at a point of a covered cell.
+__device__ __forceinline__ V4<float> window_gather(const Window& w, const V4<float>* __restrict__ win,
+                                                   const float* __restrict__ bulk4, const V4<float>& x,
+                                                   const GridDev& g) {
+    int i, j, k;
+    float tx, ty, tz;
+    axis_weight(x.x, g, 0, i, tx);
+    axis_weight(x.y, g, 1, j, ty);
+    axis_weight(x.z, g, 2, k, tz);
+    const int lx = i - w.I + 1, ly = j - w.J + 1, lz = k - w.K + 1;
+    // a stencil begins at its cell or at the one before it
+    if ((unsigned)lx <= (unsigned)(kWinX - 2) && (unsigned)ly <= 1u && (unsigned)lz <= 1u)
+    {
+        // interp8 in pairs
+        const V4<float>* c = win + lx + kWinRow * ly + kWinLayer * lz;
+        const unsigned long long t = f2_pack(tx, tx), u = f2_pack(ty, ty), w2 = f2_pack(tz, tz);
+        const Pair2 a00 = lerp_pairs(ld_win(c), ld_win(c + 1), t);
+        const Pair2 a10 = lerp_pairs(ld_win(c + kWinRow), ld_win(c + kWinRow + 1), t);
+        const Pair2 a01 = lerp_pairs(ld_win(c + kWinLayer), ld_win(c + kWinLayer + 1), t);
+        const Pair2 a11 = lerp_pairs(ld_win(c + kWinLayer + kWinRow), ld_win(c + kWinLayer + kWinRow + 1), t);
+        const Pair2 r = lerp_pairs(lerp_pairs(a00, a10, u), lerp_pairs(a01, a11, u), w2);
+        V4<float> o;
+        f2_unpack(r.a, o.x, o.y);
+        f2_unpack(r.b, o.z, o.w);
+        return o;
+    }
+    return gather(bulk4, x.x, x.y, x.z, g);
+}
+
+// The drag of the sorted step, in the order of the binning: lane l of a warp
+// takes slot r + l, the particle perm[r + l] (nearly r + l, since the particles
+// come in the last step's cell order), and its record, advanced when EULER,
+// leaves at that slot.  The force goes to the particle's own index, and its
+// reaction is summed right here, in the rounds of the segmented sum (seg_round)
+// over the chunks that k_deposit_sorted_force would take: the same additions
+// in the same order, without the 16-byte force record per particle written and
+// read back.  A block's warps take neighbouring chunks (they share the bulk
+// records in L1); a warp walks the rounds of its chunks as one sequence, with
+// the ids loaded two rounds ahead and the records one.
+//
+// 84 bytes per particle instead of 96 and another 20 for the reaction; 32M
+// particles 710 us, against 607 + 172 + 50 for the drag in the particles'
+// order, the reaction as a kernel of its own and the inverse permutation it
+// needs.  Bound by instruction issue (about 530 a round, 60 to 70% of the
+// slots) and the load / store unit (40 to 48%; 69% with the eight gathers of a
+// stencil from L1 in place of the window, 725 us).  Three CTAs per SM: two 795,
+// four (spilling) 789.  Neighbouring chunks per block rather than a run of
+// chunks per warp: 714 against 855 (L1 misses).
+template <typename T, bool EULER, bool WIN>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n, GridDev g, Phys<T> P,
+              const T* __restrict__ bulk4, T* __restrict__ F, const int32_t* __restrict__ perm,
+              const int32_t* __restrict__ key_sorted, const int32_t* __restrict__ cs, T* __restrict__ S, T dt,
+              T* __restrict__ part, long long pstride, int do_sums, unsigned long long* __restrict__ status,
+              T* __restrict__ Bs, T* __restrict__ pos_out, T* __restrict__ vel_out, int32_t* __restrict__ perm_out) {
+    extern __shared__ __align__(16) V4<float> s_win[];   // WIN: kWinRecs per warp
+    pdl_wait();
+    const unsigned full = 0xffffffffu;
+    const unsigned lane = threadIdx.x & 31;
+    V4<float>* win = s_win + (threadIdx.x >> 5) * kWinRecs;
+    Window wd;
     T lane_sums[kDragSums];
 #pragma unroll
     for (int k = 0; k < kDragSums; ++k) lane_sums[k] = T(0);
     int clamped_total = 0;
-    const long long stride = b.n * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    V4<T> xn = {T(0), T(0), T(0), T(0)}, vn = xn;
-    int slot_n = 0;
-    long long p = b.id * blockDim.x + threadIdx.x;
-    if (p < n) {
-        xn = EULER ? ld4_plain(pos, p) : ld4((const T*)pos, p);
-        vn = EULER ? ld4_plain(vel, p) : ld4((const T*)vel, p);
-        slot_n = __ldg(inv_perm + p);
-    }
-    for (; p - lane < n; p += stride) {
-        const bool valid = p < n;
-        const V4<T> x = xn, v = vn;
-        const int slot = slot_n;
-        if (p + stride < n) {
-            xn = EULER ? ld4_plain(pos, p + stride) : ld4((const T*)pos, p + stride);
-            vn = EULER ? ld4_plain(vel, p + stride) : ld4((const T*)vel, p + stride);
-            slot_n = __ldg(inv_perm + p + stride);
+    // slots as 32-bit unsigned (n < 2^31); tt = 0 after the last round
+    const unsigned un = (unsigned)n;
+    const unsigned long long step = (unsigned long long)gridDim.x * (blockDim.x >> 5) * seg_chunk(n);
+    unsigned long long base = ((unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * seg_chunk(n);
+    auto chunk = [&](unsigned& rr, unsigned& tt) {   // the first round from the chunk at `base` on
+        for (; base < un; base += step) {
+            long long s, e;
+            seg_chunk_range((long long)base, n, key_sorted, cs, s, e);
+            if (s < e) {
+                rr = (unsigned)s;
+                tt = (unsigned)e;
+                base += step;
+                return;
+            }
         }
-        const V4<T> bv = window_gather(bulk4, x, valid, g, win);
-        if (valid) {
-            const DragOne<T> r = drag_from<T, EULER>(x, v, bv, g, P, dt);
-            clamped_total += r.cl;
-            F[p] = r.f[0];
-            F[n + p] = r.f[1];
-            F[2 * n + p] = r.f[2];
-            st4(Fs, slot, r.f[0], r.f[1], r.f[2], T(0));
-            st4(pos_out, slot, r.x[0], r.x[1], r.x[2], x.w);
-            st4(vel_out, slot, r.u[0], r.u[1], r.u[2], v.w);
-            drag_lane_sums(lane_sums, r);
+        tt = 0u;
+    };
+    unsigned r = 0, t = 0;
+    chunk(r, t);
+    if (t) {
+        int id = 0, key = -1, id1 = 0, key1 = -1;
+        V4<T> x = {T(0), T(0), T(0), T(0)}, v = x;
+        auto ids = [&](unsigned rr, unsigned tt, int& i, int& k) {
+            k = -1;
+            if (rr + lane < tt) {
+                i = __ldg(perm + rr + lane);
+                k = __ldg(key_sorted + rr + lane);
+            }
+        };
+        auto advance = [&](unsigned& rr, unsigned& tt) {
+            rr += 32;
+            if (rr >= tt) chunk(rr, tt);
+        };
+        ids(r, t, id, key);
+        if (key >= 0) {
+            x = ld4(pos, id);
+            v = ld4(vel, id);
         }
-    }
-    int wsum = clamped_total;
+        unsigned r1 = r, t1 = t;
+        advance(r1, t1);
+        ids(r1, t1, id1, key1);
+        SegCarry<T, 3> carry;
+        for (;;) {
+            V4<T> x1 = {T(0), T(0), T(0), T(0)}, v1 = x1;
+            if (key1 >= 0) {
+                x1 = ld4(pos, id1);
+                v1 = ld4(vel, id1);
+            }
+            unsigned r2 = r1, t2 = t1;
+            int id2 = 0, key2 = -1;
+            if (t1) {
+                advance(r2, t2);
+                ids(r2, t2, id2, key2);
+            }
+            bool in_win = false;
+            if constexpr (WIN) {
+                const unsigned left = t - r;   // slots of this round: min(left, 32), at least one
+                const int c0 = __shfl_sync(full, key, 0), c1 = __shfl_sync(full, key, left < 32u ? left - 1u : 31u);
+                in_win = window_cover(wd, c0, c1, reinterpret_cast<const V4<float>*>(bulk4), g, win);
+            }
+            T f[3] = {T(0), T(0), T(0)};
+            if (key >= 0) {
+                V4<T> b;
+                if constexpr (WIN) b = in_win ? window_gather(wd, win, bulk4, x, g) : gather(bulk4, x.x, x.y, x.z, g);
+                else b = gather(bulk4, x.x, x.y, x.z, g);
+                const DragOne<T> d = drag_from<T, EULER>(x, v, b, g, P, dt);
+                clamped_total += d.cl;
+                const unsigned slot = r + lane;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
-    if ((threadIdx.x & 31) == 0 && wsum) {
-        atomicAdd(&status[ST_CLAMPED], (unsigned long long)wsum);
+                for (int k = 0; k < 3; ++k) {
+                    f[k] = d.f[k];
+                    F[k * n + id] = f[k];
+                }
+                if (Bs) st4(Bs, slot, d.beta, d.beta * v.x, d.beta * v.y, d.beta * v.z);
+                st4(pos_out, slot, d.x[0], d.x[1], d.x[2], x.w);
+                st4(vel_out, slot, d.u[0], d.u[1], d.u[2], v.w);
+                if (perm_out) perm_out[slot] = id;
+                drag_lane_sums(lane_sums, d);
+            }
+            const int next31 = __shfl_sync(full, key1, 0);
+            seg_round<T, 3>(f, key, r + 32 >= t ? -1 : next31, carry,
+                            [&](int c, int k, T sum) { reaction_emit<T>(g, S, c, k, sum); });
+            if (!t1) break;
+            r = r1;
+            t = t1;
+            id = id1;
+            key = key1;
+            x = x1;
+            v = v1;
+            r1 = r2;
+            t1 = t2;
+            id1 = id2;
+            key1 = key2;
+        }
+    }
+    clamped_total = __reduce_add_sync(full, clamped_total);
+    if (lane == 0 && clamped_total) {
+        atomicAdd(&status[ST_CLAMPED], (unsigned long long)clamped_total);
         atomicOr(&status[ST_FLAGS], (unsigned long long)CG_FLAG_EPS_CLAMPED);
     }
     if (do_sums) {
         CSum<T> acc[kDragSums];
 #pragma unroll
         for (int k = 0; k < kDragSums; ++k) acc[k].add(lane_sums[k]);
-        block_sums<T, kDragSums>(acc, part, pstride, b.id);
+        block_sums<T, kDragSums>(acc, part, pstride, blockIdx.x);
     }
 }
 
-template <typename T, bool EULER>
-__global__ void __launch_bounds__(256, 4)
-k_drag_win(T* pos, T* vel, long long n, GridDev g, Phys<T> P, const T* __restrict__ bulk4, T* __restrict__ F,
-           T* __restrict__ Fs, const int32_t* __restrict__ inv_perm, T dt, T* __restrict__ part, long long pstride,
-           int do_sums, unsigned long long* __restrict__ status, T* __restrict__ pos_out, T* __restrict__ vel_out) {
-    __shared__ __align__(16) V4<T> win[256 / 32][kWinRecs];
-    pdl_wait();
-    drag_body_win<T, EULER>(pos, vel, n, g, P, bulk4, F, Fs, inv_perm, dt, part, pstride, do_sums, status,
-                            launch_blk(), pos_out, vel_out, win[threadIdx.x >> 5]);
-}
-
-template <typename T, bool EULER>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-k_drag(T* pos, T* vel, long long n, GridDev g, Phys<T> P, const T* __restrict__ bulk4,
-       T* __restrict__ F, T* __restrict__ Fs, const int32_t* __restrict__ inv_perm, T dt,
-       T* __restrict__ part, long long pstride, int do_sums, unsigned long long* __restrict__ status,
-       T* __restrict__ Bs, T* __restrict__ pos_out, T* __restrict__ vel_out) {
-    pdl_wait();
-    drag_body<T, EULER>(pos, vel, n, g, P, bulk4, F, Fs, inv_perm, dt, part, pstride, do_sums, status,
-                        launch_blk(), Bs, pos_out, vel_out);
+template <typename T>
+static cg_status launch_drag_sorted(cg_grids* g, long long n, const T* pos, const T* vel, T* force, T* S, bool sums,
+                                    double dt, T* Bs, T* pos_out, T* vel_out, int32_t* perm_out) {
+    // at most the resident CTAs
+    const long long chunks = (n + seg_chunk(n) - 1) / seg_chunk(n);
+    const int bs = (int)seg_threads(g, n), warps = bs / 32;
+    const long long nblk = std::min((chunks + warps - 1) / warps, (long long)g->num_sms * (sizeof(T) == 4 ? 24 : 16) / warps);
+    T* part = (T*)part_ptr(g, PS_DRAG);
+    g->part_blocks[PS_DRAG] = sums ? nblk : -1;
+#define CG_DRAGS(E, W)                                                                                          \
+    CG_LAUNCH(g, "drag", (k_drag_sorted<T, E, W>), (unsigned)nblk, bs, W ? warps * kWinRecs * sizeof(V4<float>) : 0, pos,  \
+              vel, n, g->gd, phys_of<T>(g->gd),                                                                 \
+              (const T*)g->bulk4, force, (const int32_t*)g->perm, (const int32_t*)g->key_sorted,                  \
+              (const int32_t*)g->cell_start, S, (T)dt, part, nblk, (int)sums, g->status, Bs, pos_out, vel_out,      \
+              perm_out)
+    if constexpr (sizeof(T) == 4) {
+        if (g->gd.interp != CG_INTERP_CELL) {
+            if (dt > 0.0) CG_DRAGS(true, true);
+            else CG_DRAGS(false, true);
+            return CG_OK;
+        }
+    }
+    if (dt > 0.0) CG_DRAGS(true, false);
+    else CG_DRAGS(false, false);
+#undef CG_DRAGS
+    return CG_OK;
 }
 
 // Batched drag with the fused sorted-order force record (FP32 instances).
@@ -372,7 +479,8 @@ int batch_drag_occupancy() {
 }
 
 cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* vel, void* force, void* S_bulk,
-                      bool sums, double dt, bool S_cleared, void* coef_bulk, void* pos_out, void* vel_out) {
+                      bool sums, double dt, bool S_cleared, void* coef_bulk, void* pos_out, void* vel_out,
+                      int32_t* perm_out) {
     const bool euler = dt > 0.0;
     void* part = part_ptr(g, PS_DRAG);
     // exactly the resident CTAs (the launch bounds' minimum per SM): a grid-stride
@@ -380,36 +488,35 @@ cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* v
     const long long per_sm = g->fp64 ? 2 : 4;
     const unsigned nblk = (unsigned)std::max(1LL, std::min((n + 255) / 256, (long long)g->num_sms * per_sm));
     g->part_blocks[PS_DRAG] = sums ? (long long)nblk : -1;
-    void* Fs = S_bulk ? g->Fs : nullptr;
-    if (Fs) CG_TRY(ensure_inverse(g, n));
-    if (pos_out && !Fs) return CG_ERR_INVALID_ARG;   // the sorted slots come with the fused reaction
     void* Bs = nullptr;
     if (coef_bulk && n > 0) {
         // sized by the step before its first launch
         if (g->Bs.bytes < 4 * g->tsize * (size_t)n) return CG_ERR_INVALID_ARG;
         Bs = g->Bs.p;
     }
+    if (pos_out && !S_bulk) return CG_ERR_INVALID_ARG;   // the sorted slots come with the fused reaction
+    if (pos_out && n > 0) {
+        if (!S_cleared) CG_CUDA(cudaMemsetAsync(S_bulk, 0, 3 * g->tsize * (size_t)g->gd.nbulk, g->stream));
+        if (g->fp64)
+            CG_TRY(launch_drag_sorted<double>(g, n, (const double*)pos_d, (const double*)vel, (double*)force,
+                                              (double*)S_bulk, sums, dt, (double*)Bs, (double*)pos_out,
+                                              (double*)vel_out, perm_out));
+        else
+            CG_TRY(launch_drag_sorted<float>(g, n, (const float*)pos_d, (const float*)vel, (float*)force, (float*)S_bulk,
+                                             sums, dt, (float*)Bs, (float*)pos_out, (float*)vel_out, perm_out));
+        if (coef_bulk) CG_TRY(launch_deposit_implicit(g, n, coef_bulk));
+        return CG_OK;
+    }
+    if (perm_out && n > 0)
+        CG_CUDA(cudaMemcpyAsync(perm_out, g->perm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, g->stream));
+    void* Fs = S_bulk ? g->Fs : nullptr;
+    if (Fs) CG_TRY(ensure_inverse(g, n));
     if (n > 0 || sums) {
 #define CG_DRAGP(T, E)                                                                                      \
     CG_LAUNCH(g, "drag", (k_drag<T, E>), nblk, 256, 0, (T*)pos_d, (T*)vel, n, g->gd, phys_of<T>(g->gd),          \
               (const T*)g->bulk4, (T*)force, (T*)Fs, g->inv_perm, (T)dt, (T*)part, (long long)nblk, (int)sums,   \
-              g->status, (T*)Bs, (T*)pos_out, (T*)vel_out)
-        // on request, the sorted step (its particles come in nearly in cell
-        // order) stages each warp's stencil window on the FP32 trilinear path
-        const bool win = g->desc.stencil == CG_STENCIL_WINDOW && pos_out && !g->fp64 && !Bs &&
-                         g->gd.interp != CG_INTERP_CELL;
-        if (win) {
-            if (euler)
-                CG_LAUNCH(g, "drag", (k_drag_win<float, true>), nblk, 256, 0, (float*)pos_d, (float*)vel, n, g->gd,
-                          phys_of<float>(g->gd), (const float*)g->bulk4, (float*)force, (float*)Fs, g->inv_perm,
-                          (float)dt, (float*)part, (long long)nblk, (int)sums, g->status, (float*)pos_out,
-                          (float*)vel_out);
-            else
-                CG_LAUNCH(g, "drag", (k_drag_win<float, false>), nblk, 256, 0, (float*)pos_d, (float*)vel, n, g->gd,
-                          phys_of<float>(g->gd), (const float*)g->bulk4, (float*)force, (float*)Fs, g->inv_perm,
-                          (float)dt, (float*)part, (long long)nblk, (int)sums, g->status, (float*)pos_out,
-                          (float*)vel_out);
-        } else if (g->fp64) {
+              g->status, (T*)Bs)
+        if (g->fp64) {
             if (euler) CG_DRAGP(double, true);
             else CG_DRAGP(double, false);
         } else {

@@ -167,3 +167,43 @@ def test_porosity_after_a_bad_diameter(cuda_lib, bad):
     other = torch.arange(g.n_bulk, device="cuda") != c
     assert torch.equal(eps[1][other], eps[0][other]) and torch.equal(eps[2], eps[0])
     g.close()
+
+
+@pytest.mark.parametrize("fp64,interp,law", [(False, 0, 0), (False, 0, 1), (False, 1, 0), (True, 0, 1)])
+@pytest.mark.parametrize("n,nb", [(1, (2, 2, 2)), (33, (2, 3, 2)), (5_000, (3, 2, 5)), (20_000, (40, 20, 24)),
+                                  (60_001, (17, 9, 13)), (400_003, (33, 16, 12))])
+def test_sorted_drag_equals_the_drag_in_the_callers_order(cuda_lib, n, nb, fp64, interp, law):
+    """The sorted step's fused drag and reaction over grids from two cells per
+    axis on, a particle in many cells to thousands in one, rows shorter and
+    longer than a staged window: every field, force and record as cg_step's,
+    bit for bit, with and without advancing."""
+    import torch
+    cg = cuda_lib
+    r = 2
+    desc = synth.make_desc((-0.3, 0.0, 0.1), (1.0, 0.7, 0.9), [r * m for m in nb], r, fp64=fp64, law=law, interp=interp,
+                           gravity=(0.0, 1.0, -9.0))
+    rng = synth.rng_for(n, 11)
+    T = np.float64 if fp64 else np.float32
+    pos = np.empty((n, 4), T)
+    pos[:, :3] = np.array(desc["origin"]) + rng.random((n, 3)) * np.array(desc["extent"])
+    pos[:, 3] = 0.002
+    vel = (0.05 * rng.standard_normal((n, 4))).astype(T)
+    g, f = cg.Grids(desc), cg.Grids(desc)
+    u = to_dev((0.5 + 0.02 * rng.standard_normal((3, g.n_fine))).astype(T))
+    pi, vi = to_dev(pos), to_dev(vel)
+    oa = g.alloc_outputs(n, eps_fine=True, bins=True, implicit=True)
+    ob = f.alloc_outputs(n, eps_fine=True, bins=True, implicit=True)
+    for dt in (0.0, 1e-4, 1e-4, 0.0):
+        po, vo = torch.empty_like(pi), torch.empty_like(vi)
+        pr, vr = pi.clone(), vi.clone()
+        g.cg_step_sorted(pi, vi, po, vo, u, oa, dt=dt)
+        f.cg_step(pr, vr, u, ob, dt=dt)
+        torch.cuda.synchronize()
+        perm = oa["perm"].long()
+        assert torch.equal(po, pr[perm]) and torch.equal(vo, vr[perm])
+        for k in FIELDS + ("cell", "perm", "cell_start", "implicit_bulk"):
+            assert torch.equal(oa[k], ob[k]), (dt, k)
+        pi, vi = po, vo
+    assert g.cg_sync_status()[:2] == f.cg_sync_status()[:2]
+    g.close()
+    f.close()
