@@ -96,7 +96,8 @@ enum { ST_FLAGS = 0, ST_OUTSIDE = 1, ST_NONFINITE = 2, ST_CLAMPED = 3, ST_TIMEOU
 // The projection's region holds six columns: sum S_f V_f (3), then sum S_B
 // V_B (3) of the source it reads.
 enum { PS_VOL = 0, PS_DRAG = 1, PS_PROJ = 2, PS_NREG = 3 };
-constexpr int kDragSums = 9;   // V_p, F(3), |F|, m u (3), clamped count
+constexpr int kDragLaneSums = 8;              // V_p, F(3), |F|, m u (3)
+constexpr int kDragSums = kDragLaneSums + 1;   // + the clamped count
 constexpr int kDragCellSums = kDragSums + 3;   // + S_B V_B (3) in the cell-order drag
 
 // ----------------------------------------------------------------------
@@ -363,8 +364,14 @@ cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps =
 // Porosity of the binned particles: from the sorted diameters of a binning
 // from scratch (pos_d null), or gathered from pos_d [n] T4.
 cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, StepEps* eps);
-// Slots per chunk of the segmented sums.
-__host__ __device__ inline int seg_chunk(long long) { return 256; }
+// Slots per chunk of the segmented sums: 256, and fewer for small particle
+// counts, whose few chunks would be a chain of eight rounds on a few SMs
+// (10,000 particles, FP64: the reaction 18 -> 10 us; at 500,000 a chunk of
+// 128 gains nothing, 256 is faster).  By the particle count alone, so that
+// every path over the same particles cuts them alike and gives the same sums.
+__host__ __device__ inline int seg_chunk(long long n) {
+    return n >= (1 << 17) ? 256 : n >= (1 << 16) ? 128 : n >= (1 << 15) ? 64 : 32;
+}
 // Threads per block of the kernels over chunks: few chunks take smaller blocks, so that
 // they reach every SM (10,000 particles, FP64, blocks of 256 -> 32: 47 -> 19 us).
 inline unsigned seg_threads(const cg_grids* g, long long n) {
@@ -496,22 +503,53 @@ struct Blk {
 };
 __device__ __forceinline__ Blk launch_blk() { return {(long long)blockIdx.x, (long long)gridDim.x}; }
 
-// Block-level deterministic reduction of K compensated sums.  Thread 0..K-1
-// writes the pair (s, c) of sum k to part[2 * (k * stride + bid)]:
-// partials stay in the path precision as compensated pairs, so no FP64
-// arithmetic runs per block (GB300's FP64 rate is a small fraction of FP32).
+// Warp sums of K (a power of two) values in one pass over the lanes: at each
+// of the first log2 K steps a lane hands half of its sums to its partner and
+// keeps the others, so a step merges K/2, K/4, ... sums instead of K (for eight
+// values 9 merges instead of 40, of 8 FP64 operations each: the drag's were
+// an eighth of its FP64 time over 1M particles, half over 10,000).  Value k ends
+// on lane 32 / K * k, in a fixed order.
+template <typename T, int K>
+__device__ __forceinline__ CSum<T> warp_reduce_many(CSum<T> (&v)[K]) {
+    static_assert(K == 1 || K == 2 || K == 4 || K == 8, "a power of two");
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int m = K / 2; m > 0; m >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int j = 0; j < m; ++j) {
+            const CSum<T> a = up ? v[m + j] : v[j], b = up ? v[j] : v[m + j];
+            CSum<T> o;
+            o.s = __shfl_xor_sync(0xffffffffu, b.s, off);
+            o.c = __shfl_xor_sync(0xffffffffu, b.c, off);
+            v[j] = a;
+            v[j].merge(o);
+        }
+    }
+    for (; off > 0; off >>= 1) {
+        CSum<T> o;
+        o.s = __shfl_xor_sync(0xffffffffu, v[0].s, off);
+        o.c = __shfl_xor_sync(0xffffffffu, v[0].c, off);
+        v[0].merge(o);
+    }
+    return v[0];
+}
+
+// Block-level deterministic reduction of K compensated sums.  The pair (s, c)
+// of sum k goes to part[2 * (k * stride + bid)]: partials stay in the path
+// precision as compensated pairs, so no FP64 arithmetic runs per block (GB300's
+// FP64 rate is a small fraction of FP32).
 template <typename T, int K>
 __device__ __forceinline__ void block_sums(CSum<T> (&v)[K], T* __restrict__ part, long long stride, long long bid) {
     __shared__ T sh_s[K][32];
     __shared__ T sh_c[K][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        CSum<T> r = warp_reduce(v[k]);
-        if (lane == 0) {
-            sh_s[k][warp] = r.s;
-            sh_c[k][warp] = r.c;
-        }
+    const CSum<T> r = warp_reduce_many<T, K>(v);
+    if ((lane & (32 / K - 1)) == 0) {
+        const int k = lane / (32 / K);
+        sh_s[k][warp] = r.s;
+        sh_c[k][warp] = r.c;
     }
     __syncthreads();
     if (threadIdx.x < K) {
@@ -528,6 +566,20 @@ __device__ __forceinline__ void block_sums(CSum<T> (&v)[K], T* __restrict__ part
         T* dst = part + 2 * ((long long)k * stride + bid);
         dst[0] = a.s;
         dst[1] = a.c;
+    }
+}
+
+// The block's sum of a count held once per warp (on every lane), as such a pair.
+template <typename T>
+__device__ __forceinline__ void block_count(int warp_count, T* __restrict__ dst) {
+    __shared__ int sh[32];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = warp_count;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        long long c = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) c += sh[w];
+        dst[0] = (T)c;
+        dst[1] = (T)(c - (long long)dst[0]);
     }
 }
 

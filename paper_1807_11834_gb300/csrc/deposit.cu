@@ -211,6 +211,7 @@ template <typename T>
 __device__ __forceinline__ void sums_body(const T* __restrict__ part, const SumsMap& map, double* __restrict__ sums,
                                           Blk b) {
     __shared__ T sh_s[8], sh_c[8];
+    const int nw = blockDim.x >> 5;
     const int k = (int)b.id;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     CSum<T> a;
@@ -231,7 +232,7 @@ __device__ __forceinline__ void sums_body(const T* __restrict__ part, const Sums
         CSum<T> t;
         t.s = sh_s[0];
         t.c = sh_c[0];
-        for (int w = 1; w < 8; ++w) {
+        for (int w = 1; w < nw; ++w) {
             CSum<T> o;
             o.s = sh_s[w];
             o.c = sh_c[w];
@@ -433,8 +434,12 @@ SumsMap sums_map(const long long* part_off, const long long* part_blocks) {
 
 cg_status launch_sums(cg_grids* g, double* sums) {
     const SumsMap m = sums_map(g->part_off, g->part_blocks);
+    // FP64: two warps for the few partials of a small grid, whose time is the
+    // warps' trees (10,000 particles, 512 cells: 7 -> 5 us)
+    long long most = 0;
+    for (int k = 0; k < CG_NSUMS; ++k) most = std::max(most, m.cnt[k]);
     if (g->fp64)
-        CG_LAUNCH(g, "sums", k_sums<double>, CG_NSUMS, 256, 0, (const double*)g->partials, m, sums);
+        CG_LAUNCH(g, "sums", k_sums<double>, CG_NSUMS, most <= 2048 ? 64 : 256, 0, (const double*)g->partials, m, sums);
     else
         CG_LAUNCH(g, "sums", k_sums<float>, CG_NSUMS, 256, 0, (const float*)g->partials, m, sums);
     return CG_OK;

@@ -109,9 +109,9 @@ __device__ __forceinline__ DragOne<T> drag_one(const V4<T>& x, const V4<T>& v, c
     return drag_from<T, EULER>(x, v, gather(bulk4, x.x, x.y, x.z, g), g, P, dt);
 }
 
-// Per-lane diagnostics: V_p, F (3), |F|, m u (3) after the advance, clamped.
+// Per-lane diagnostics: V_p, F (3), |F|, m u (3) after the advance.
 template <typename T>
-__device__ __forceinline__ void drag_lane_sums(T (&ls)[kDragSums], const DragOne<T>& r) {
+__device__ __forceinline__ void drag_lane_sums(T (&ls)[kDragLaneSums], const DragOne<T>& r) {
     using X = M<T>;
     ls[0] = X::add(ls[0], r.vp);
     ls[1] = X::add(ls[1], r.f[0]);
@@ -121,7 +121,26 @@ __device__ __forceinline__ void drag_lane_sums(T (&ls)[kDragSums], const DragOne
     ls[5] = X::fma_(r.m, r.u[0], ls[5]);
     ls[6] = X::fma_(r.m, r.u[1], ls[6]);
     ls[7] = X::fma_(r.m, r.u[2], ls[7]);
-    ls[8] = X::add(ls[8], (T)r.cl);
+}
+
+// The end of a drag kernel: the block's clamped particles to the status, its
+// diagnostics to the partials.
+template <typename T>
+__device__ __forceinline__ void drag_totals(int clamped, const T (&lane_sums)[kDragLaneSums], T* __restrict__ part,
+                                            long long pstride, int do_sums, unsigned long long* __restrict__ status,
+                                            long long bid) {
+    clamped = __reduce_add_sync(0xffffffffu, clamped);
+    if ((threadIdx.x & 31) == 0 && clamped) {
+        atomicAdd(&status[ST_CLAMPED], (unsigned long long)clamped);
+        atomicOr(&status[ST_FLAGS], (unsigned long long)CG_FLAG_EPS_CLAMPED);
+    }
+    if (do_sums) {
+        CSum<T> acc[kDragLaneSums];
+#pragma unroll
+        for (int k = 0; k < kDragLaneSums; ++k) acc[k].s = lane_sums[k];
+        block_sums<T, kDragLaneSums>(acc, part, pstride, bid);
+        block_count<T>(clamped, part + 2 * (kDragLaneSums * pstride + bid));
+    }
 }
 
 // ----------------------------------------------------------------------
@@ -137,9 +156,9 @@ __device__ __forceinline__ void drag_body(T* pos, T* vel, long long n, const Gri
                                           const int32_t* __restrict__ inv_perm, T dt, T* __restrict__ part,
                                           long long pstride, int do_sums, unsigned long long* __restrict__ status,
                                           Blk b, T* __restrict__ Bs = nullptr) {
-    T lane_sums[kDragSums];
+    T lane_sums[kDragLaneSums];
 #pragma unroll
-    for (int k = 0; k < kDragSums; ++k) lane_sums[k] = T(0);
+    for (int k = 0; k < kDragLaneSums; ++k) lane_sums[k] = T(0);
     int clamped_total = 0;
     const long long stride = b.n * blockDim.x;
     // PREFETCH: the next particle's record is loaded while this one's
@@ -179,19 +198,7 @@ __device__ __forceinline__ void drag_body(T* pos, T* vel, long long n, const Gri
         }
         drag_lane_sums(lane_sums, r);
     }
-    int wsum = clamped_total;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
-    if ((threadIdx.x & 31) == 0 && wsum) {
-        atomicAdd(&status[ST_CLAMPED], (unsigned long long)wsum);
-        atomicOr(&status[ST_FLAGS], (unsigned long long)CG_FLAG_EPS_CLAMPED);
-    }
-    if (do_sums) {
-        CSum<T> acc[kDragSums];
-#pragma unroll
-        for (int k = 0; k < kDragSums; ++k) acc[k].add(lane_sums[k]);
-        block_sums<T, kDragSums>(acc, part, pstride, b.id);
-    }
+    drag_totals<T>(clamped_total, lane_sums, part, pstride, do_sums, status, b.id);
 }
 
 template <typename T, bool EULER>
@@ -312,9 +319,9 @@ k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n,
     const unsigned lane = threadIdx.x & 31;
     V4<float>* win = s_win + (threadIdx.x >> 5) * kWinRecs;
     Window wd;
-    T lane_sums[kDragSums];
+    T lane_sums[kDragLaneSums];
 #pragma unroll
-    for (int k = 0; k < kDragSums; ++k) lane_sums[k] = T(0);
+    for (int k = 0; k < kDragLaneSums; ++k) lane_sums[k] = T(0);
     int clamped_total = 0;
     // slots as 32-bit unsigned (n < 2^31); tt = 0 after the last round
     const unsigned un = (unsigned)n;
@@ -411,17 +418,7 @@ k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n,
             key1 = key2;
         }
     }
-    clamped_total = __reduce_add_sync(full, clamped_total);
-    if (lane == 0 && clamped_total) {
-        atomicAdd(&status[ST_CLAMPED], (unsigned long long)clamped_total);
-        atomicOr(&status[ST_FLAGS], (unsigned long long)CG_FLAG_EPS_CLAMPED);
-    }
-    if (do_sums) {
-        CSum<T> acc[kDragSums];
-#pragma unroll
-        for (int k = 0; k < kDragSums; ++k) acc[k].add(lane_sums[k]);
-        block_sums<T, kDragSums>(acc, part, pstride, blockIdx.x);
-    }
+    drag_totals<T>(clamped_total, lane_sums, part, pstride, do_sums, status, blockIdx.x);
 }
 
 template <typename T>
@@ -485,8 +482,11 @@ cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* v
     void* part = part_ptr(g, PS_DRAG);
     // exactly the resident CTAs (the launch bounds' minimum per SM): a grid-stride
     // loop with no second, partial wave of blocks
+    // (of 256 threads); small counts take smaller blocks, so that they reach every SM
     const long long per_sm = g->fp64 ? 2 : 4;
-    const unsigned nblk = (unsigned)std::max(1LL, std::min((n + 255) / 256, (long long)g->num_sms * per_sm));
+    int bs = 32;
+    while (bs < 256 && n > 8LL * g->num_sms * bs) bs *= 2;
+    const unsigned nblk = (unsigned)std::max(1LL, std::min((n + bs - 1) / bs, (long long)g->num_sms * per_sm * 256 / bs));
     g->part_blocks[PS_DRAG] = sums ? (long long)nblk : -1;
     void* Bs = nullptr;
     if (coef_bulk && n > 0) {
@@ -513,7 +513,7 @@ cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* v
     if (Fs) CG_TRY(ensure_inverse(g, n));
     if (n > 0 || sums) {
 #define CG_DRAGP(T, E)                                                                                      \
-    CG_LAUNCH(g, "drag", (k_drag<T, E>), nblk, 256, 0, (T*)pos_d, (T*)vel, n, g->gd, phys_of<T>(g->gd),          \
+    CG_LAUNCH(g, "drag", (k_drag<T, E>), nblk, bs, 0, (T*)pos_d, (T*)vel, n, g->gd, phys_of<T>(g->gd),          \
               (const T*)g->bulk4, (T*)force, (T*)Fs, g->inv_perm, (T)dt, (T*)part, (long long)nblk, (int)sums,   \
               g->status, (T*)Bs)
         if (g->fp64) {
