@@ -13,13 +13,13 @@
 // compressed-row table per axis and direction (bulk index -> overlapping
 // fine indices and overlap lengths, and fine -> bulk), built once on the
 // host in double and kept on the device; the 3-D weight of a pair is the
-// product of its three axis entries.  Average: one thread per bulk cell
-// walks its fine box (consecutive threads read consecutive fine runs);
-// projection: when no fine cell overlaps more than two bulk cells along an
-// axis (fine cells no larger than bulk cells) a fixed 2 x 2 x 2 stencil,
-// one CTA per fine row with the bulk rows it reaches collapsed over y and z
-// in shared memory first; else one thread per fine cell through the
-// compressed rows.
+// product of its three axis entries.  Average: a thread per fine x index of a
+// bulk row sums its fine column over y and z, and the block combines the
+// columns along x in shared memory.  Projection: when no fine cell overlaps
+// more than two bulk cells along an axis (fine cells no larger than bulk
+// cells), a thread per fine column along z with the bulk planes collapsed over
+// x and y in registers; else one thread per fine cell through the compressed
+// rows.
 #include <math.h>
 #include <string.h>
 
@@ -43,6 +43,7 @@ struct cg_map {
     bool two = false;
     long long off_f2b[3], off_f2w0[3], off_f2w1[3];
     double Vf = 0.0;
+    int avg_tile = 0, avg_threads = 0;   // bulk x cells and threads per block of the average; 0: a cell per thread
 };
 
 namespace cg {
@@ -122,10 +123,130 @@ MapDev<T> dev_view(const cg_map* m) {
 
 constexpr int kMapMaxComp = 8;
 
-// Both kernels take cells in x-fastest order with 32-bit index arithmetic
-// (grids hold fewer than 2^31 cells): one division per cell splits the index
-// into the x index and the row (y, z), whose two axis ranges are looked up
-// once per cell.
+// Average, thread t of a block taking the t-th fine x index under a tile of bulk
+// x cells, over the fine rows of bulk row (J, K) for the K of a chunk: the
+// column's few y terms in plain FMAs, its planes (weighted by z) into a
+// compensated sum, then the x terms, compensated likewise, from shared memory.
+// A plane shared by the cells K and K + 1 is kept.  Every fine value is read
+// once from HBM, those of the rows shared by two bulk rows a second time from L2.
+// The loads are coalesced along x and copied asynchronously into shared memory
+// two planes ahead (in registers they cost half of the occupancy: 117 us).
+// Bound by instruction issue and latency (issue 53%).  A thread per bulk cell
+// (the form below, kept for a bulk cell over more than 256 fine x indices)
+// gathers runs of a few values per lane, four times the L1 wavefronts: 250 x 250
+// x 500 fine to 64 x 64 x 128 bulk cells, three components, FP32 127 -> 102 us.
+template <typename T>
+__device__ __forceinline__ void copy_async(T* dst, const T* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(sizeof(T))
+                 : "memory");
+}
+constexpr int kMapRows = 6, kMapStages = 2;   // rows of a plane in shared memory, planes in flight
+template <typename T, int NC>
+__global__ void __launch_bounds__(256) k_map_average_rows(MapDev<T> d, int tile, int ntiles, int depth,
+                                                          const T* __restrict__ in, T* __restrict__ out) {
+    pdl_wait();
+    constexpr int G = sizeof(T) == 4 ? kMapRows : kMapRows / 2;
+    __shared__ T sh[2][NC][256];
+    __shared__ T ring[kMapStages][G][NC][256];   // a thread copies and reads its own column only
+    const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
+    const size_t nbk = (size_t)nbx * nby * nbz;
+    const size_t nfx = d.nf[0], plane = nfx * d.nf[1], nfn = plane * d.nf[2];
+    in += blockIdx.y * (NC * nfn);
+    out += blockIdx.y * (NC * nbk);
+    unsigned b = blockIdx.x;
+    const int t = (int)(b % (unsigned)ntiles);
+    b /= (unsigned)ntiles;
+    const int J = (int)(b % (unsigned)nby);
+    const int K0 = (int)(b / (unsigned)nby) * depth, K1 = min(K0 + depth, nbz);
+    const int I0 = t * tile, I1 = min(I0 + tile, nbx);
+    const int p0 = __ldg(d.bptr[0] + I0), p1 = __ldg(d.bptr[0] + I1);
+    const int f0 = p1 > p0 ? __ldg(d.bidx[0] + p0) : 0;
+    const int span = p1 > p0 ? __ldg(d.bidx[0] + p1 - 1) - f0 + 1 : 0;
+    const int y0 = __ldg(d.bptr[1] + J), ny = __ldg(d.bptr[1] + J + 1) - y0;
+    const int zp0 = __ldg(d.bptr[2] + K0), zp1 = __ldg(d.bptr[2] + K1);
+    const bool on = (int)threadIdx.x < span && ny > 0 && zp1 > zp0;
+    // the overlapping indices of a row are consecutive
+    const T* wy = d.bw[1] + y0;
+    T w[G];
+#pragma unroll
+    for (int y = 0; y < G; ++y) w[y] = y < ny ? __ldg(wy + y) : T(0);
+    int fz = on ? __ldg(d.bidx[2] + zp0) : 0;   // the next plane to be added; ahead: to be copied
+    const int zlast = on ? __ldg(d.bidx[2] + zp1 - 1) : -1;
+    const T* ahead = in + (f0 + (int)threadIdx.x) + (on ? nfx * __ldg(d.bidx[1] + y0) : 0) + plane * fz;
+    int za = fz;
+    auto copy_plane = [&](int stage) {
+        if (za <= zlast) {
+            const T* q = ahead;
+#pragma unroll
+            for (int y = 0; y < G; ++y, q += nfx)
+                if (y < ny)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) copy_async(&ring[stage][y][c][threadIdx.x], q + c * nfn);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ahead += plane;
+        ++za;
+    };
+    int stage = 0;
+    if (on)
+#pragma unroll
+        for (int i = 0; i < kMapStages; ++i) copy_plane(i);
+    T rs[NC];
+    int have = -1;   // the plane that rs holds
+    for (int K = K0; K < K1; ++K) {
+        if (on) {
+            CSum<T> acc[NC];
+            const int z1 = __ldg(d.bptr[2] + K + 1);
+            for (int kz = __ldg(d.bptr[2] + K); kz < z1; ++kz) {
+                const int f = __ldg(d.bidx[2] + kz);
+                const T wz = __ldg(d.bw[2] + kz);
+                if (f != have) {   // then f is the next plane
+                    have = f;
+                    asm volatile("cp.async.wait_group %0;" ::"n"(kMapStages - 1) : "memory");
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) rs[c] = T(0);
+#pragma unroll
+                    for (int y = 0; y < G; ++y)
+                        if (y < ny)
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) rs[c] = fma(w[y], ring[stage][y][c][threadIdx.x], rs[c]);
+                    if (ny > G) {
+                        const T* q = ahead - kMapStages * plane + nfx * G;
+                        for (int y = G; y < ny; ++y, q += nfx)
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) rs[c] = fma(__ldg(wy + y), __ldg(q + c * nfn), rs[c]);
+                    }
+                    copy_plane(stage);
+                    stage = stage + 1 == kMapStages ? 0 : stage + 1;
+                }
+#pragma unroll
+                for (int c = 0; c < NC; ++c) acc[c].add(wz * rs[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) sh[K & 1][c][threadIdx.x] = acc[c].get();
+        }
+        __syncthreads();   // one per K: the next one writes the other half
+        const T wJK = __ldg(d.cov[1] + J) * __ldg(d.cov[2] + K);
+        const int m = I1 - I0;
+        for (int o = threadIdx.x; o < m * NC; o += blockDim.x) {
+            const int c = o / m, I = I0 + o - c * m;
+            const T W = __ldg(d.cov[0] + I) * wJK;
+            CSum<T> a;
+            if (W > T(0)) {
+                const int x0 = __ldg(d.bptr[0] + I), x1 = __ldg(d.bptr[0] + I + 1);
+                const T* v = sh[K & 1][c] + (__ldg(d.bidx[0] + x0) - f0 - x0);
+                for (int kx = x0; kx < x1; ++kx) a.add(__ldg(d.bw[0] + kx) * v[kx]);
+            }
+            out[c * nbk + I + (size_t)nbx * (J + (size_t)nby * K)] = W > T(0) ? a.get() / W : T(0);
+        }
+    }
+}
+
+// The kernels over cells take them in x-fastest order with 32-bit index
+// arithmetic (grids hold fewer than 2^31 cells): one division per cell splits
+// the index into the x index and the row (y, z), whose two axis ranges are
+// looked up once per cell.
 template <typename T, int NC>
 __global__ void __launch_bounds__(256) k_map_average(MapDev<T> d, const T* __restrict__ in, T* __restrict__ out) {
     pdl_wait();
@@ -206,85 +327,55 @@ __global__ void __launch_bounds__(256) k_map_project(MapDev<T> d, const T* __res
     }
 }
 
-// Projection when every fine cell overlaps at most two bulk cells per axis:
-// a fixed 2 x 2 x 2 stencil (the second weight 0 where there is one), all
-// loads independent, as in the trilinear projection of nested grids.
+// Projection when every fine cell overlaps at most two bulk cells per axis (the
+// second weight 0 where there is one): a thread per fine column walks `depth`
+// fine planes along z with the two bulk planes around it, collapsed over x and
+// y, in registers, so that a plane costs one load of its z weights and two
+// operations and a store per component.  Bound by the HBM stores: 64 x 64 x 128
+// bulk to 250 x 250 x 500 fine cells, three components, FP32 78 us, against
+// 169 for a block per fine row with the bulk rows collapsed in shared memory.
 template <typename T, int NC>
-__global__ void __launch_bounds__(256) k_map_project2(MapDev<T> d, const T* __restrict__ in, T* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_map_project2(MapDev<T> d, unsigned colblk, int depth,
+                                                      const T* __restrict__ in, T* __restrict__ out) {
     pdl_wait();
     const unsigned nbx = (unsigned)d.nb[0], nby = (unsigned)d.nb[1], nbz = (unsigned)d.nb[2];
-    const size_t nbk = (size_t)nbx * nby * nbz;
-    const unsigned nfx = (unsigned)d.nf[0], nfy = (unsigned)d.nf[1];
-    const unsigned nfn = nfx * nfy * (unsigned)d.nf[2];
-    for (unsigned cf = blockIdx.x * blockDim.x + threadIdx.x; cf < nfn; cf += gridDim.x * blockDim.x) {
-        const unsigned row = cf / nfx;
-        const unsigned i = cf - row * nfx;
-        const unsigned j = row % nfy, k = row / nfy;
-        const unsigned bx = (unsigned)__ldg(d.f2b[0] + i), by = (unsigned)__ldg(d.f2b[1] + j);
+    const size_t bplane = (size_t)nbx * nby, nbk = bplane * nbz;
+    const unsigned nfx = (unsigned)d.nf[0], plane = nfx * (unsigned)d.nf[1];
+    const size_t nfn = (size_t)plane * (unsigned)d.nf[2];
+    const unsigned chunk = blockIdx.x / colblk;
+    const unsigned q = (blockIdx.x - chunk * colblk) * blockDim.x + threadIdx.x;
+    if (q >= plane) return;
+    const unsigned j = q / nfx, i = q - j * nfx;
+    const unsigned bx = (unsigned)__ldg(d.f2b[0] + i), by = (unsigned)__ldg(d.f2b[1] + j);
+    const T wx0 = __ldg(d.f2w0[0] + i), wx1 = __ldg(d.f2w1[0] + i);
+    const T wy0 = __ldg(d.f2w0[1] + j), wy1 = __ldg(d.f2w1[1] + j);
+    // the second neighbour stays inside the grid (its weight is 0 at the edge)
+    const unsigned dx = bx + 1 < nbx ? 1u : 0u, dy = by + 1 < nby ? nbx : 0u;
+    const T* s0 = in + bx + (size_t)nbx * by;
+    T lo[NC], hi[NC];
+    auto collapse = [&](unsigned bz, T (&v)[NC]) {
+        const T* s = s0 + bplane * bz;
+#pragma unroll
+        for (int c = 0; c < NC; ++c, s += nbk)
+            v[c] = wy0 * fma(wx1, __ldg(s + dx), wx0 * __ldg(s)) + wy1 * fma(wx1, __ldg(s + dy + dx), wx0 * __ldg(s + dy));
+    };
+    const unsigned k0 = chunk * (unsigned)depth, k1 = min(k0 + (unsigned)depth, (unsigned)d.nf[2]);
+    unsigned have = ~0u;   // the bulk plane that lo holds
+    T* o = out + q + (size_t)plane * k0;
+    for (unsigned k = k0; k < k1; ++k, o += plane) {
         const unsigned bz = (unsigned)__ldg(d.f2b[2] + k);
-        const T wx[2] = {__ldg(d.f2w0[0] + i), __ldg(d.f2w1[0] + i)};
-        const T wy[2] = {__ldg(d.f2w0[1] + j), __ldg(d.f2w1[1] + j)};
-        const T wz[2] = {__ldg(d.f2w0[2] + k), __ldg(d.f2w1[2] + k)};
-        // the second neighbour stays inside the grid (its weight is 0 at the edge)
-        const unsigned dx = bx + 1 < nbx ? 1u : 0u, dy = by + 1 < nby ? nbx : 0u;
-        const size_t dz = bz + 1 < nbz ? (size_t)nbx * nby : 0;
-        const size_t b0 = bx + (size_t)nbx * (by + (size_t)nby * bz);
+        if (bz != have) {
+            if (have + 1 == bz && have != ~0u)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const T* s = in + c * nbk + b0;
-            const T v000 = __ldg(s), v001 = __ldg(s + dx), v010 = __ldg(s + dy), v011 = __ldg(s + dy + dx);
-            const T v100 = __ldg(s + dz), v101 = __ldg(s + dz + dx), v110 = __ldg(s + dz + dy);
-            const T v111 = __ldg(s + dz + dy + dx);
-            const T y0 = wy[0] * fma(wx[1], v001, wx[0] * v000) + wy[1] * fma(wx[1], v011, wx[0] * v010);
-            const T y1 = wy[0] * fma(wx[1], v101, wx[0] * v100) + wy[1] * fma(wx[1], v111, wx[0] * v110);
-            out[(size_t)c * nfn + cf] = (wz[0] * y0 + wz[1] * y1) * d.inv_Vf;
+                for (int c = 0; c < NC; ++c) lo[c] = hi[c];
+            else
+                collapse(bz, lo);
+            collapse(bz + 1 < nbz ? bz + 1 : bz, hi);
+            have = bz;
         }
-    }
-}
-
-// Row-tiled projection (the default for the two-point stencil when its
-// shared memory, NC x (bulk cells per x row) values, fits).  (A row-tiled
-// average that collapsed the fine rows of each bulk row first read the fine
-// field about 1.6 times over, and ran slower than the cell kernel above.)
-// Projection with the two-point stencil: the CTA takes fine row (j, k); it
-// first collapses the (at most 2 x 2) bulk rows over y and z for every bulk
-// x index the row reaches, into shared memory, then thread i combines the
-// two x neighbours of its fine cell.
-template <typename T, int NC>
-__global__ void __launch_bounds__(256) k_map_project2_rows(MapDev<T> d, const T* __restrict__ in, T* __restrict__ out) {
-    pdl_wait();
-    extern __shared__ unsigned char smem_raw[];
-    T* v = reinterpret_cast<T*>(smem_raw);   // [NC][nbx]
-    const unsigned nbx = (unsigned)d.nb[0], nby = (unsigned)d.nb[1], nbz = (unsigned)d.nb[2];
-    const size_t nbk = (size_t)nbx * nby * nbz;
-    const unsigned nfx = (unsigned)d.nf[0], nfy = (unsigned)d.nf[1];
-    const unsigned nfn = nfx * nfy * (unsigned)d.nf[2];
-    const unsigned rows = nfy * (unsigned)d.nf[2];
-    for (unsigned r = blockIdx.x; r < rows; r += gridDim.x) {
-        const unsigned j = r % nfy, k = r / nfy;
-        const unsigned by = (unsigned)__ldg(d.f2b[1] + j), bz = (unsigned)__ldg(d.f2b[2] + k);
-        const T wy0 = __ldg(d.f2w0[1] + j), wy1 = __ldg(d.f2w1[1] + j);
         const T wz0 = __ldg(d.f2w0[2] + k), wz1 = __ldg(d.f2w1[2] + k);
-        const size_t dy = by + 1 < nby ? nbx : 0, dz = bz + 1 < nbz ? (size_t)nbx * nby : 0;
-        const size_t b0 = (size_t)nbx * (by + (size_t)nby * bz);
-        for (unsigned X = threadIdx.x; X < nbx; X += blockDim.x) {
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const T* s = in + c * nbk + b0 + X;
-                v[c * nbx + X] = wz0 * fma(wy1, __ldg(s + dy), wy0 * __ldg(s)) +
-                                 wz1 * fma(wy1, __ldg(s + dz + dy), wy0 * __ldg(s + dz));
-            }
-        }
-        __syncthreads();
-        for (unsigned i = threadIdx.x; i < nfx; i += blockDim.x) {
-            const unsigned bx = (unsigned)__ldg(d.f2b[0] + i);
-            const unsigned bx1 = bx + 1 < nbx ? bx + 1 : bx;
-            const T wx0 = __ldg(d.f2w0[0] + i), wx1 = __ldg(d.f2w1[0] + i);
-            const unsigned cf = i + nfx * r;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) out[(size_t)c * nfn + cf] = fma(wx1, v[c * nbx + bx1], wx0 * v[c * nbx + bx]) * d.inv_Vf;
-        }
-        __syncthreads();
+        for (int c = 0; c < NC; ++c) o[c * nfn] = fma(wz1, hi[c], wz0 * lo[c]) * d.inv_Vf;
     }
 }
 
@@ -369,6 +460,29 @@ extern "C" cg_status cg_map_create(const cg_box_grid* bulk, const cg_box_grid* f
         m->off_fw[a] = put_t(fw[a]);
         m->off_cov[a] = put_t(cov[a]);
     }
+    // the widest tile of bulk x cells whose fine indices fit a block's 256 threads
+    auto span = [&](int tile) {
+        int most = 0;
+        for (int i = 0; i < bulk->n[0]; i += tile) {
+            const int p0 = bp[0][i], p1 = bp[0][std::min(i + tile, bulk->n[0])];
+            if (p1 > p0) most = std::max(most, bi[0][p1 - 1] - bi[0][p0] + 1);
+        }
+        return most;
+    };
+    // (for rows that are runs of consecutive indices, one after the other, which
+    // rounding could break only for cells below the resolution of their coordinates)
+    bool runs = true;
+    for (int a = 0; a < 3; ++a)
+        for (size_t k = 1; k < bi[a].size(); ++k) {
+            const int step = bi[a][k] - bi[a][k - 1];
+            runs = runs && (step == 0 || step == 1);
+        }
+    for (int parts = 1; parts <= bulk->n[0] && runs && !m->avg_tile; ++parts) {
+        const int tile = (bulk->n[0] + parts - 1) / parts, w = span(tile);
+        if (w > 256) continue;
+        m->avg_tile = tile;
+        m->avg_threads = std::max(32, (w + 31) / 32 * 32);
+    }
     if (cudaMalloc(&m->dev, std::max<size_t>(host.size(), 16)) != cudaSuccess) {
         cudaGetLastError();
         delete m;
@@ -396,13 +510,13 @@ extern "C" cg_status cg_map_destroy(cg_map* m) {
 // The map's launches go through CG_LAUNCH's counterpart without a handle:
 // a programmatic dependent launch on the map's stream.
 template <typename K, typename... Args>
-static cg_status map_launch(cg_map* m, K kernel, long long work, Args... args) {
+static cg_status map_launch(cg_map* m, K kernel, dim3 grid, int block, Args... args) {
     cudaLaunchAttribute a[1];
     a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(grid_for(work));
-    c.blockDim = dim3(256);
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)block);
     c.stream = m->stream;
     c.attrs = a;
     c.numAttrs = 1;
@@ -411,49 +525,36 @@ static cg_status map_launch(cg_map* m, K kernel, long long work, Args... args) {
     return e == cudaSuccess ? CG_OK : CG_ERR_CUDA;
 }
 
-constexpr size_t kMapRowSmem = 96 * 1024;   // shared memory of a row-tiled CTA at most
-
-template <typename K>
-static cg_status row_attr(K kernel, size_t smem) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMapRowSmem) != cudaSuccess) {
-        cudaGetLastError();
-        return CG_ERR_CUDA;
-    }
-    return CG_OK;
-}
-
-// One CTA per row (grid-stride over the rows), with dynamic shared memory.
-template <typename K, typename... Args>
-static cg_status map_launch_rows(cg_map* m, K kernel, long long rows, size_t smem, Args... args) {
-    cudaLaunchAttribute a[1];
-    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3((unsigned)std::max(1LL, std::min(rows, 65535LL)));
-    c.blockDim = dim3(256);
-    c.dynamicSmemBytes = smem;
-    c.stream = m->stream;
-    c.attrs = a;
-    c.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&c, kernel, args...);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    return e == cudaSuccess ? CG_OK : CG_ERR_CUDA;
+// z planes per thread: as many as leave `fill` threads for each of the chip's
+// (152 SMs of 2048), since the start of a walk is work of its own; at most 64.
+// Average: fill 1 102, 2 104, 4 106 us at the size above; projection: 81, 87, 78.
+static int map_depth(long long columns, long long nz, int fill) {
+    const long long chunks = (fill * 152LL * 2048 + columns - 1) / columns;
+    return (int)std::max(1LL, std::min((nz + chunks - 1) / chunks, 64LL));
 }
 
 template <typename T, int NC>
 static cg_status map_apply(cg_map* m, bool avg, const void* in, void* out) {
-    if (avg) return map_launch(m, k_map_average<T, NC>, m->nbulk, dev_view<T>(m), (const T*)in, (T*)out);
-    if (m->two) {
-        const size_t smem = (size_t)NC * m->bulk.n[0] * sizeof(T);
-        if (smem <= kMapRowSmem) {
-            CG_TRY(row_attr(k_map_project2_rows<T, NC>, smem));
-            return map_launch_rows(m, k_map_project2_rows<T, NC>, (long long)m->fine.n[1] * m->fine.n[2], smem,
-                                   dev_view<T>(m), (const T*)in, (T*)out);
+    const MapDev<T> d = dev_view<T>(m);
+    if (avg) {
+        if (m->avg_tile) {
+            // components per block: what shared memory holds
+            constexpr int NB = NC % 3 == 0 ? 3 : NC % 2 == 0 ? 2 : 1;
+            const long long tiles = (m->bulk.n[0] + m->avg_tile - 1) / m->avg_tile, rows = tiles * m->bulk.n[1];
+            const int depth = map_depth(rows * m->avg_threads * (NC / NB), m->bulk.n[2], 1);
+            return map_launch(m, k_map_average_rows<T, NB>,
+                              dim3((unsigned)(rows * ((m->bulk.n[2] + depth - 1) / depth)), NC / NB), m->avg_threads, d,
+                              m->avg_tile, (int)tiles, depth, (const T*)in, (T*)out);
         }
-        return map_launch(m, k_map_project2<T, NC>, m->nfine, dev_view<T>(m), (const T*)in, (T*)out);
+        return map_launch(m, k_map_average<T, NC>, grid_for(m->nbulk), 256, d, (const T*)in, (T*)out);
     }
-    return map_launch(m, k_map_project<T, NC>, m->nfine, dev_view<T>(m), (const T*)in, (T*)out);
+    if (m->two) {
+        const long long columns = (long long)m->fine.n[0] * m->fine.n[1], colblk = (columns + 255) / 256;
+        const int depth = map_depth(columns, m->fine.n[2], 4);
+        return map_launch(m, k_map_project2<T, NC>, dim3((unsigned)(colblk * ((m->fine.n[2] + depth - 1) / depth))), 256, d, (unsigned)colblk,
+                          depth, (const T*)in, (T*)out);
+    }
+    return map_launch(m, k_map_project<T, NC>, grid_for(m->nfine), 256, d, (const T*)in, (T*)out);
 }
 
 template <typename T>
