@@ -119,7 +119,10 @@ cg_status plan(cg_batch* b) {
         I.cellsort = g->desc.sort_digits == CG_SORT_CELLS ? 1 : 0;
         const int bits = std::max(1, ceil_log2_ll(nb));
         if (!I.cellsort && bits > 2 * c.digit_bits) return CG_ERR_OUT_OF_RANGE;
-        I.npasses = I.cellsort ? 0 : bits <= c.digit_bits ? 1 : 2;
+        // one pass up to 9 bits: with 11, the warps' counters of a scatter tile take the
+        // shared memory of a whole SM and outnumber its particles eight to
+        // one (16 instances, 4.3M particles: scatters 162 -> 124 us, the second histogram 8 -> 13)
+        I.npasses = I.cellsort ? 0 : bits <= std::min(c.digit_bits, 9) ? 1 : 2;
         I.b0 = I.cellsort ? 0 : I.npasses == 1 ? bits : (bits + 1) / 2;
         I.b1 = I.npasses == 2 ? bits - I.b0 : 0;
         I.pos = (float*)it.particles.pos_d;
@@ -157,14 +160,13 @@ cg_status plan(cg_batch* b) {
         const long long m1 = (long long)I.ntiles << I.b1;
         const long long hist_m = std::max(m0, I.npasses == 2 ? m1 : 0LL);
         CG_TRY(dev_alloc(b, (void**)&I.hist, sizeof(int32_t) * hist_m));
-        I.scan0.in[0] = I.count;
-        I.scan0.out[0] = I.count;
-        I.scan0.m[0] = nb + 1;
-        I.scan0.in[1] = I.hist;
-        I.scan0.out[1] = I.hist;
-        I.scan0.m[1] = m0;
-        I.scan0.nblk[0] = cdiv(nb + 1, kScanItems);
-        I.scan0.nblk[1] = cdiv(m0, kScanItems);
+        I.scan0.in[0] = I.scan0.out[0] = I.cellsort ? I.count : I.hist;
+        I.scan0.m[0] = I.cellsort ? nb + 1 : m0;
+        I.scan0.nblk[0] = cdiv(I.scan0.m[0], kScanItems);
+        I.scan0.in[1] = nullptr;
+        I.scan0.out[1] = nullptr;
+        I.scan0.m[1] = 0;
+        I.scan0.nblk[1] = 0;
         I.scan1.in[0] = I.hist;
         I.scan1.out[0] = I.hist;
         I.scan1.m[0] = I.npasses == 2 ? m1 : 0;
@@ -173,7 +175,7 @@ cg_status plan(cg_batch* b) {
         I.scan1.out[1] = nullptr;
         I.scan1.m[1] = 0;
         I.scan1.nblk[1] = 0;
-        const long long scan_blocks = std::max(I.scan0.nblk[0] + I.scan0.nblk[1], I.scan1.nblk[0]);
+        const long long scan_blocks = std::max(I.scan0.nblk[0], I.scan1.nblk[0]);
         CG_TRY(dev_alloc(b, (void**)&I.scan_part, sizeof(int32_t) * scan_blocks));
         // virtual blocks per phase
         long long* B = &blocks[(size_t)i];
@@ -181,15 +183,16 @@ cg_status plan(cg_batch* b) {
         const long long chunks = cdiv(n, seg_chunk(n));
         const long long seg = std::max(1LL, cdiv(chunks, 8LL * c.seg_chunks));
         const long long cellb = cdiv(nb, 256);
-        set(BP_ZERO, cdiv(nb + 1, 1024));
+        set(BP_ZERO, I.cellsort ? cdiv(nb + 1, 1024) : 0);
         set(BP_KEY, I.cellsort ? cdiv(n, (long long)kSortThreads * kKeyItems) : I.ntiles);
-        set(BP_SCAN0_R, I.scan0.nblk[0] + I.scan0.nblk[1]);
-        set(BP_SCAN0_D, I.scan0.nblk[0] + I.scan0.nblk[1]);
+        set(BP_SCAN0_R, I.scan0.nblk[0]);
+        set(BP_SCAN0_D, I.scan0.nblk[0]);
         set(BP_SCAT0, I.cellsort ? 0 : I.ntiles);
         set(BP_HIST1, I.npasses == 2 ? I.ntiles : 0);
         set(BP_SCAN1_R, I.scan1.nblk[0]);
         set(BP_SCAN1_D, I.scan1.nblk[0]);
         set(BP_SCAT1, I.npasses == 2 ? I.ntiles : 0);
+        set(BP_STARTS, I.cellsort ? 0 : cdiv(nb + 1, 256));
         set(BP_PLACE, I.cellsort ? cdiv(n, 512LL * kPlaceItems) : 0);
         set(BP_SEGSORT, I.cellsort ? cdiv(nb, (long long)kGroupCells * kSegSortWarps) : 0);
         set(BP_DEPV, std::max(1LL, cdiv(n, 1024LL * c.seg_chunks)));
@@ -239,7 +242,8 @@ cg_status plan(cg_batch* b) {
         int occ = 1;
         switch (ph) {
             case BP_KEY: case BP_SCAN0_R: case BP_SCAN0_D: case BP_SCAT0:
-            case BP_HIST1: case BP_SCAN1_R: case BP_SCAN1_D: case BP_SCAT1: case BP_PLACE: case BP_SEGSORT:
+            case BP_HIST1: case BP_SCAN1_R: case BP_SCAN1_D: case BP_SCAT1: case BP_STARTS: case BP_PLACE:
+            case BP_SEGSORT:
                 occ = batch_bin_occupancy(ph, b->smem[ph]);
                 break;
             case BP_AVG: case BP_PROJ: case BP_PROJE: occ = batch_fine_occupancy(ph); break;

@@ -39,7 +39,7 @@ struct BInst {
     double* sums;
     // scratch of the instance's handle and of the batch
     int32_t* key;
-    int32_t* count;        // cell counts, then cell_start after the scan
+    int32_t* count;        // cell_start (per-cell sort: the counts until their scan)
     int32_t* hist;
     int32_t* key1;         // digit sort: keys after pass 1; per-cell sort: second id buffer
     int32_t* val1;         // digit sort: ids after pass 1; per-cell sort: placed ids
@@ -64,7 +64,7 @@ struct BInst {
 // Phases of a batched step, in launch order.
 enum BPhase {
     BP_ZERO = 0, BP_KEY, BP_SCAN0_R, BP_SCAN0_D, BP_SCAT0, BP_HIST1, BP_SCAN1_R, BP_SCAN1_D, BP_SCAT1,
-    BP_PLACE, BP_SEGSORT, BP_DEPV, BP_AVG, BP_PACK, BP_DRAG, BP_DEPM, BP_PROJ, BP_PROJE, BP_SUMS, BP_COUNT
+    BP_STARTS, BP_PLACE, BP_SEGSORT, BP_DEPV, BP_AVG, BP_PACK, BP_DRAG, BP_DEPM, BP_PROJ, BP_PROJE, BP_SUMS, BP_COUNT
 };
 
 // One batched launch: virtual-block prefix over the instances (device).

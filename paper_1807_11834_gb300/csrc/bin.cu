@@ -24,8 +24,7 @@
 // memory, so the rank of a particle within its digit group follows its
 // index.  Tile histograms are scanned digit-major across tiles, which makes
 // the whole pass stable and fully deterministic (no atomics decide any
-// position).  Per-cell counts use integer atomics (order-independent), then
-// a scan.
+// position).  The cells' starts are searched in the sorted keys.
 #include <algorithm>
 
 #include "cg_internal.cuh"
@@ -46,13 +45,16 @@ __device__ __forceinline__ void add_status(unsigned long long* st, int outside, 
 }
 
 // ----------------------------------------------------------------------
-// Key kernel: cell per particle, per-cell counts, tile histogram of digit 0
+// Key kernel: cell per particle, tile histogram of digit 0.  The cells' starts
+// come from the sorted keys (k_cell_starts): a count atomic per particle, in
+// random order, cost more than everything else here (4.3M particles in 16
+// instances 128 -> 36 us).
 // ----------------------------------------------------------------------
 
 template <typename T>
 __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long long n, const GridDev& g,
-                                             int32_t* __restrict__ key, int32_t* __restrict__ count,
-                                             int32_t* __restrict__ hist, int ntiles, int bits0, T* __restrict__ vol,
+                                             int32_t* __restrict__ key, int32_t* __restrict__ hist, int ntiles,
+                                             int bits0, T* __restrict__ vol,
                                              unsigned long long* __restrict__ status, int* sh, Blk blk) {
     __shared__ int s_cnt[2];
     const int R = 1 << bits0;
@@ -82,13 +84,10 @@ __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long lon
             key[p] = c;
             vol[p] = v.w;   // the diameter: the porosity forms the volume as an exact pair
         }
-        // counts: one integer atomic per run of equal cells in the warp
-        // (spatially ordered input has runs of several particles)
+        // one atomic per run of equal cells in the warp (spatially ordered
+        // input has runs of several particles)
         const int len = run_head_length(c, valid);
-        if (len) {
-            atomicAdd(&count[c], len);
-            atomicAdd(&sh[c & (R - 1)], len);
-        }
+        if (len) atomicAdd(&sh[c & (R - 1)], len);
     }
     if (n_out) atomicAdd(&s_cnt[0], n_out);
     if (n_nf) atomicAdd(&s_cnt[1], n_nf);
@@ -100,11 +99,33 @@ __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long lon
 template <typename T>
 __global__ void __launch_bounds__(kSortThreads)
 k_bin_key(const T* __restrict__ pos, long long n, GridDev g, int32_t* __restrict__ key,
-          int32_t* __restrict__ count, int32_t* __restrict__ hist, int ntiles, int bits0,
-          T* __restrict__ vol, unsigned long long* __restrict__ status) {
+          int32_t* __restrict__ hist, int ntiles, int bits0, T* __restrict__ vol, unsigned long long* __restrict__ status) {
     pdl_wait();
     extern __shared__ int sh[];
-    bin_key_body<T>(pos, n, g, key, count, hist, ntiles, bits0, vol, status, sh, launch_blk());
+    bin_key_body<T>(pos, n, g, key, hist, ntiles, bits0, vol, status, sh, launch_blk());
+}
+
+// The cells' starts from the sorted keys: a thread per cell (and one past the
+// last) searches the first slot whose key is not below it.  About 20 dependent
+// loads, from L2, all cells at once; nothing depends on how many particles or
+// empty cells come together.
+__device__ __forceinline__ void cell_starts_body(const int32_t* __restrict__ key_sorted, long long n, long long nbulk,
+                                                 int32_t* __restrict__ cs, Blk b) {
+    for (long long c = b.id * blockDim.x + threadIdx.x; c <= nbulk; c += b.n * blockDim.x) {
+        long long lo = 0, hi = n;
+        while (lo < hi) {
+            const long long mid = (lo + hi) >> 1;
+            if (__ldg(key_sorted + mid) < c) lo = mid + 1;
+            else hi = mid;
+        }
+        cs[c] = (int32_t)lo;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_cell_starts(const int32_t* __restrict__ key_sorted, long long n, long long nbulk, int32_t* __restrict__ cs) {
+    pdl_wait();
+    cell_starts_body(key_sorted, n, nbulk, cs, launch_blk());
 }
 
 // Key kernel of the per-cell sort: cell, diameter and arrival rank of every
@@ -827,8 +848,8 @@ static cg_status bin_passes(cg_grids* g, long long n, const T* pos, int ntiles, 
     const int np = g->npasses;
     const int b0 = g->pass_bits[0];
     CG_LAUNCH(g, "bin_key", k_bin_key<T>, ntiles, kSortThreads, sizeof(int) << b0, pos, n, g->gd, g->key,
-              g->cell_start, g->hist, ntiles, b0, (T*)g->vol, g->status);
-    CG_TRY(scan_exclusive2(g, g->cell_start, g->cell_start, nbulk + 1, g->hist, g->hist, m0));
+              g->hist, ntiles, b0, (T*)g->vol, g->status);
+    CG_TRY(scan_exclusive2(g, g->hist, g->hist, m0, nullptr, nullptr, 0));
     // pass p reads (keys, ids) from in[p] and writes them to in[p + 1]; the
     // last pass writes the final order
     int32_t* ks[kMaxPasses + 1] = {g->key, g->key1, g->key2, nullptr};
@@ -862,6 +883,8 @@ static cg_status bin_passes(cg_grids* g, long long n, const T* pos, int ntiles, 
                       (const T*)nullptr, (T*)nullptr);
         shift += bits;
     }
+    CG_LAUNCH(g, "cell_starts", k_cell_starts, (unsigned)((nbulk + 256) / 256), 256, 0, (const int32_t*)g->key_sorted, n,
+              nbulk, g->cell_start);
     return CG_OK;
 }
 
@@ -926,13 +949,13 @@ cg_status launch_reorder(cg_grids* g, long long n, const void* pos_d, const void
 // ----------------------------------------------------------------------
 // Batched binning phases (FP32 instances)
 // ----------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads) kb_bin_key(BLaunch L) {
+__global__ void __launch_bounds__(kSortThreads, 2) kb_bin_key(BLaunch L) {
     extern __shared__ int sh[];
     batch_loop(L, [&](const BInst& I, Blk b) {
         if (I.cellsort)
             bin_key_rank_body<float>(I.pos, I.n, I.gd, I.key, I.count, I.vol, I.status, I.arrival, b);
         else
-            bin_key_body<float>(I.pos, I.n, I.gd, I.key, I.count, I.hist, I.ntiles, I.b0, I.vol, I.status, sh, b);
+            bin_key_body<float>(I.pos, I.n, I.gd, I.key, I.hist, I.ntiles, I.b0, I.vol, I.status, sh, b);
     });
 }
 
@@ -966,6 +989,10 @@ __global__ void __launch_bounds__(kSortThreads, 2) kb_bin_scatter(BLaunch L, int
                                                  nullptr, nullptr, nullptr, (const float*)nullptr, (float*)nullptr,
                                                  cnt, b);
     });
+}
+
+__global__ void __launch_bounds__(256) kb_cell_starts(BLaunch L) {
+    batch_loop(L, [&](const BInst& I, Blk b) { cell_starts_body(I.key_sorted, I.n, I.gd.nbulk, I.count, b); });
 }
 
 __global__ void __launch_bounds__(256) kb_scan_reduce(BLaunch L, int pass) {
@@ -1002,6 +1029,7 @@ cg_status launch_batch_bin(int phase, const BLaunch& L, unsigned grid, size_t sm
         case BP_SCAN1_R: kb_scan_reduce<<<grid, 256, 0, s>>>(L, 1); break;
         case BP_SCAN1_D: kb_scan_down<<<grid, 256, 0, s>>>(L, 1); break;
         case BP_SCAT1: kb_bin_scatter<<<grid, kSortThreads, smem, s>>>(L, 1); break;
+        case BP_STARTS: kb_cell_starts<<<grid, 256, 0, s>>>(L); break;
         case BP_PLACE: kb_bin_place<<<grid, 512, 0, s>>>(L); break;
         case BP_SEGSORT: kb_seg_sort<<<grid, kSegSortWarps * 32, 0, s>>>(L); break;
         default: return CG_ERR_INVALID_ARG;
@@ -1021,6 +1049,7 @@ int batch_bin_occupancy(int phase, size_t smem) {
         case BP_SCAT1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_bin_scatter, kSortThreads, smem); break;
         case BP_SCAN0_R:
         case BP_SCAN1_R: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_scan_reduce, 256, 0); break;
+        case BP_STARTS: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_cell_starts, 256, 0); break;
         case BP_PLACE: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_bin_place, 512, 0); break;
         case BP_SEGSORT:
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_seg_sort, kSegSortWarps * 32, 0);
@@ -1056,15 +1085,17 @@ cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps) 
         return CG_OK;
     }
     g->key_valid = g->inv_valid = true;
-    // count[] lives in cell_start; the exclusive scan turns it into starts
-    CG_CUDA(cudaMemsetAsync(g->cell_start, 0, sizeof(int32_t) * (nbulk + 1), g->stream));
+    // the per-cell sort counts in cell_start; the exclusive scan turns it into starts
+    const bool cells = use_cell_sort(g->desc.sort_digits, n, nbulk);
+    if (cells || n == 0)
+        CG_CUDA(cudaMemsetAsync(g->cell_start, 0, sizeof(int32_t) * (nbulk + 1), g->stream));
     if (n == 0) {
         g->n_binned = 0;
         return CG_OK;
     }
     const int ntiles = (int)((n + kSortTile - 1) / kSortTile);
     const long long m0 = (long long)ntiles << g->pass_bits[0];
-    if (use_cell_sort(g->desc.sort_digits, n, nbulk)) {
+    if (cells) {
         if (g->fp64) CG_TRY(bin_rank<double>(g, n, (const double*)pos_d));
         else CG_TRY(bin_rank<float>(g, n, (const float*)pos_d));
     } else {
