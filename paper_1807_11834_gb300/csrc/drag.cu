@@ -312,7 +312,8 @@ k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n,
               const T* __restrict__ bulk4, T* __restrict__ F, const int32_t* __restrict__ perm,
               const int32_t* __restrict__ key_sorted, const int32_t* __restrict__ cs, T* __restrict__ S, T dt,
               T* __restrict__ part, long long pstride, int do_sums, unsigned long long* __restrict__ status,
-              T* __restrict__ Bs, T* __restrict__ pos_out, T* __restrict__ vel_out, int32_t* __restrict__ perm_out) {
+              T* __restrict__ Bs, T* __restrict__ pos_out, T* __restrict__ vel_out, int32_t* __restrict__ perm_out,
+              T* __restrict__ Fs) {
     extern __shared__ __align__(16) V4<float> s_win[];   // WIN: kWinRecs per warp
     pdl_wait();
     const unsigned full = 0xffffffffu;
@@ -392,10 +393,11 @@ k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n,
                 clamped_total += d.cl;
                 const unsigned slot = r + lane;
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    f[k] = d.f[k];
-                    F[k * n + id] = f[k];
-                }
+                for (int k = 0; k < 3; ++k) f[k] = d.f[k];
+                if (Fs) st4(Fs, slot, f[0], f[1], f[2], T(0));
+                else
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) F[k * n + id] = f[k];
                 if (Bs) st4(Bs, slot, d.beta, d.beta * v.x, d.beta * v.y, d.beta * v.z);
                 st4(pos_out, slot, d.x[0], d.x[1], d.x[2], x.w);
                 st4(vel_out, slot, d.u[0], d.u[1], d.u[2], v.w);
@@ -421,9 +423,27 @@ k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n,
     drag_totals<T>(clamped_total, lane_sums, part, pstride, do_sums, status, blockIdx.x);
 }
 
+// The forces from the binned order into the particles' own.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_unsort_force(const T* __restrict__ Fs, const int32_t* __restrict__ inv_perm, long long n, T* __restrict__ F) {
+    pdl_wait();
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
+        const V4<T> f = ld4(Fs, __ldg(inv_perm + p));
+        F[p] = f.x;
+        F[n + p] = f.y;
+        F[2 * n + p] = f.z;
+    }
+}
+
 template <typename T>
 static cg_status launch_drag_sorted(cg_grids* g, long long n, const T* pos, const T* vel, T* force, T* S, bool sums,
                                     double dt, T* Bs, T* pos_out, T* vel_out, int32_t* perm_out) {
+    // Particles that come in any order (the binning was not the identity-hint
+    // one): their forces leave in the order of the binning and are gathered from
+    // there, instead of three scattered 4-byte stores each (32M in random order,
+    // the first step: 4390 -> 2480 us)
+    T* Fs = g->inv_valid ? (T*)g->Fs : nullptr;
     // at most the resident CTAs
     const long long chunks = (n + seg_chunk(n) - 1) / seg_chunk(n);
     const int bs = (int)seg_threads(g, n), warps = bs / 32;
@@ -435,17 +455,18 @@ static cg_status launch_drag_sorted(cg_grids* g, long long n, const T* pos, cons
               vel, n, g->gd, phys_of<T>(g->gd),                                                                 \
               (const T*)g->bulk4, force, (const int32_t*)g->perm, (const int32_t*)g->key_sorted,                  \
               (const int32_t*)g->cell_start, S, (T)dt, part, nblk, (int)sums, g->status, Bs, pos_out, vel_out,      \
-              perm_out)
+              perm_out, Fs)
+    const bool win = sizeof(T) == 4 && g->gd.interp != CG_INTERP_CELL;
     if constexpr (sizeof(T) == 4) {
-        if (g->gd.interp != CG_INTERP_CELL) {
-            if (dt > 0.0) CG_DRAGS(true, true);
-            else CG_DRAGS(false, true);
-            return CG_OK;
-        }
+        if (win && dt > 0.0) CG_DRAGS(true, true);
+        else if (win) CG_DRAGS(false, true);
     }
-    if (dt > 0.0) CG_DRAGS(true, false);
-    else CG_DRAGS(false, false);
+    if (!win && dt > 0.0) CG_DRAGS(true, false);
+    else if (!win) CG_DRAGS(false, false);
 #undef CG_DRAGS
+    if (Fs)
+        CG_LAUNCH(g, "unsort_force", k_unsort_force<T>, (unsigned)std::min((n + 255) / 256, (long long)g->num_sms * 16), 256, 0,
+                  (const T*)Fs, (const int32_t*)g->inv_perm, n, force);
     return CG_OK;
 }
 
