@@ -249,7 +249,6 @@ static void free_all(cg_grids* g) {
     dfree(g->eps_t);
     dfree(g->vol_acc);
     dfree(g->partials);
-    dfree(g->sums_scratch);
     dfree(g->status);
     for (HostStage& S : g->hs) {
         DevBuf* st[] = {&S.pos, &S.vel, &S.ufine, &S.eps, &S.ub, &S.var, &S.Sb,
@@ -378,7 +377,6 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     if (st == CG_OK) st = dalloc(&g->vol_acc, 3 * sizeof(unsigned long long) * nbulk);
     if (st == CG_OK && cudaMemsetAsync(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk, g->stream) != cudaSuccess)
         st = CG_ERR_CUDA;
-    if (st == CG_OK) st = dalloc(&g->sums_scratch, sizeof(double) * CG_NSUMS);
     if (st == CG_OK) st = dalloc(&g->status, sizeof(unsigned long long) * kNumSlots);
     if (st == CG_OK && cudaMemset(g->status, 0, sizeof(unsigned long long) * kNumSlots) != cudaSuccess)
         st = CG_ERR_CUDA;
@@ -556,6 +554,9 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     if (o->implicit_bulk && mlp) return CG_ERR_INVALID_ARG;   // no drag factor in the learned form
     if (o->implicit_bulk && n > 0) CG_TRY(grow_buf(g->Bs, 4 * g->tsize * (size_t)g->cap));
     for (int r = 0; r < PS_NREG; ++r) g->part_blocks[r] = -1;
+    // without a place for them the conservation sums are not formed: one launch at
+    // the end of the chain less (4 to 5 us), and the kernels before it form no partials
+    const bool sums = o->sums != nullptr;
     cudaStream_t side = g->prof ? g->stream : g->aux;
     CG_CUDA(cudaEventRecord(g->ev_fork, g->stream));
     CG_CUDA(cudaStreamWaitEvent(side, g->ev_fork, 0));
@@ -572,7 +573,7 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     eps.S = o->S_bulk;
     eps.rec = fused ? g->bulk4 : nullptr;
     eps.eps_t = fused && o->eps_fine ? g->eps_t : nullptr;
-    eps.sums = true;
+    eps.sums = sums;
     eps.ready = eps.eps_t ? g->ev_pack : nullptr;
     CG_TRY(launch_bin(g, n, p->pos_d, &eps));
     // sorted diameters of this binning
@@ -595,7 +596,7 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
         CG_TRY(launch_drag_learned(g, mlp, n, p->pos_d, p->vel, o->var_bulk, u_fine, age, o->force, o->S_bulk,
                                    dt, true));
     else
-        CG_TRY(launch_drag(g, n, p->pos_d, p->vel, o->force, o->S_bulk, true, dt, true, o->implicit_bulk,
+        CG_TRY(launch_drag(g, n, p->pos_d, p->vel, o->force, o->S_bulk, sums, dt, true, o->implicit_bulk,
                            sorted_out ? sorted_out->pos_d : nullptr, sorted_out ? sorted_out->vel : nullptr,
                            sorted_out ? o->perm : nullptr));
     // the binning above lists the sorted output's particle i at slot i
@@ -603,7 +604,7 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     const size_t bs = (size_t)g->gd.nbulk * g->tsize, fs = (size_t)g->gd.nfine * g->tsize;
     const void* in[4] = {o->S_bulk, (const char*)o->S_bulk + bs, (const char*)o->S_bulk + 2 * bs, nullptr};
     void* out[4] = {o->S_fine, (char*)o->S_fine + fs, (char*)o->S_fine + 2 * fs, nullptr};
-    CG_TRY(launch_project(g, 3, in, out, true));
+    CG_TRY(launch_project(g, 3, in, out, sums));
     if (o->implicit_fine) {
         const void* ci[4];
         void* co[4];
@@ -614,7 +615,7 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
         CG_TRY(launch_project(g, 4, ci, co, false));
     }
     CG_CUDA(cudaStreamWaitEvent(g->stream, g->ev_epsf, 0));
-    CG_TRY(launch_sums(g, o->sums ? o->sums : g->sums_scratch));
+    if (sums) CG_TRY(launch_sums(g, o->sums));
     return CG_OK;
 }
 

@@ -134,7 +134,7 @@ cg_status plan(cg_batch* b) {
         I.force = (float*)it.out.force;
         I.S_fine = (float*)it.out.S_fine;
         I.eps_fine = (float*)it.out.eps_fine;
-        I.sums = it.out.sums ? it.out.sums : g->sums_scratch;
+        I.sums = it.out.sums;   // null: the instance's sums are not formed
         I.key = g->key;
         I.count = g->cell_start;
         I.key1 = g->key1;
@@ -205,7 +205,7 @@ cg_status plan(cg_batch* b) {
         const long long projb = cdiv(project_threads(g->gd, I.depth), 256);
         set(BP_PROJ, 3 * projb);
         set(BP_PROJE, I.eps_fine ? cdiv(project_threads(g->gd, I.depth_eps), 256) : 0);
-        set(BP_SUMS, CG_NSUMS);
+        set(BP_SUMS, I.sums ? CG_NSUMS : 0);
         // partial regions (pairs): volume 1 column, projection 6 (S_f V_f, S_B V_B), drag 9
         I.part_blocks[PS_VOL] = cellb;
         I.part_blocks[PS_PROJ] = projb;
@@ -246,7 +246,7 @@ cg_status plan(cg_batch* b) {
             case BP_SEGSORT:
                 occ = batch_bin_occupancy(ph, b->smem[ph]);
                 break;
-            case BP_AVG: case BP_PROJ: case BP_PROJE: occ = batch_fine_occupancy(ph); break;
+            case BP_AVG: case BP_PROJ: case BP_PROJE: occ = batch_fine_occupancy(ph, b->total[BP_SUMS] > 0); break;
             case BP_DRAG: occ = batch_drag_occupancy(); break;
             default: occ = batch_deposit_occupancy(ph); break;
         }
@@ -276,6 +276,7 @@ cg_status enqueue(cg_batch* b, double dt) {
         l.start = b->d_start + (size_t)ph * (ni + 1);
         l.ninst = ni;
         l.total = b->total[ph];
+        l.sums = b->total[BP_SUMS] > 0;
         return l;
     };
     cudaStream_t s = b->stream;

@@ -73,6 +73,7 @@ struct BLaunch {
     const long long* start;   // [ninst + 1]
     int ninst;
     long long total;
+    bool sums;                // some instance wants its conservation sums
 };
 
 // Instance owning virtual block v (start is non-decreasing, start[0] = 0,
@@ -108,7 +109,7 @@ cg_status launch_batch_drag(const BLaunch& L, unsigned grid, float dt, cudaStrea
 // Resident CTAs per SM of a phase's kernel.
 int batch_bin_occupancy(int phase, size_t smem);
 int batch_deposit_occupancy(int phase);
-int batch_fine_occupancy(int phase);
+int batch_fine_occupancy(int phase, bool sums);
 int batch_drag_occupancy();
 
 }  // namespace cg

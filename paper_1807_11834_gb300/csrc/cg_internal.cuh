@@ -213,7 +213,6 @@ struct cg_grids {
     long long part_off[cg::PS_NREG] = {0, 0, 0};
     long long part_blocks[cg::PS_NREG] = {0, 0, 0};
     long long part_cap = 0;
-    double* sums_scratch = nullptr;   // [CG_NSUMS] when the caller gives none
     unsigned long long* status = nullptr;   // [kNumSlots]
 
     // host-buffer entries: two staging sets used in turn, and the copy

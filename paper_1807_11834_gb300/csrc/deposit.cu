@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(256) kb_pack(BLaunch L) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) I.bulk4[4 * c + 1 + k] = __ldg(I.u_bulk + k * g.nbulk + c);
         }
-        block_sums<float, 1>(tot, I.part + 2 * I.part_off[PS_VOL], I.part_blocks[PS_VOL], b.id);
+        if (I.sums) block_sums<float, 1>(tot, I.part + 2 * I.part_off[PS_VOL], I.part_blocks[PS_VOL], b.id);
     });
 }
 

@@ -196,7 +196,7 @@ __device__ __forceinline__ void drag_body(T* pos, T* vel, long long n, const Gri
             st4(pos, p, r.x[0], r.x[1], r.x[2], x.w);
             st4(vel, p, r.u[0], r.u[1], r.u[2], v.w);
         }
-        drag_lane_sums(lane_sums, r);
+        if (do_sums) drag_lane_sums(lane_sums, r);
     }
     drag_totals<T>(clamped_total, lane_sums, part, pstride, do_sums, status, b.id);
 }
@@ -402,7 +402,7 @@ k_drag_sorted(const T* __restrict__ pos, const T* __restrict__ vel, long long n,
                 st4(pos_out, slot, d.x[0], d.x[1], d.x[2], x.w);
                 st4(vel_out, slot, d.u[0], d.u[1], d.u[2], v.w);
                 if (perm_out) perm_out[slot] = id;
-                drag_lane_sums(lane_sums, d);
+                if (do_sums) drag_lane_sums(lane_sums, d);
             }
             const int next31 = __shfl_sync(full, key1, 0);
             seg_round<T, 3>(f, key, r + 32 >= t ? -1 : next31, carry,
@@ -475,7 +475,7 @@ template <bool EULER>
 __global__ void __launch_bounds__(256) kb_drag(BLaunch L, float dt) {
     batch_loop(L, [&](const BInst& I, Blk b) {
         drag_body<float, EULER, false>(I.pos, I.vel, I.n, I.gd, I.P, I.bulk4, I.force, I.Fs, I.inv_perm, dt,
-                                I.part + 2 * I.part_off[PS_DRAG], I.part_blocks[PS_DRAG], 1, I.status, b);
+                                I.part + 2 * I.part_off[PS_DRAG], I.part_blocks[PS_DRAG], I.sums != nullptr, I.status, b);
     });
 }
 

@@ -588,8 +588,9 @@ __global__ void __launch_bounds__(256, 2) kb_average(BLaunch L) {
 }
 
 // eps: project the porosity (one component, no sums) instead of the source
-// (three components, a third of the instance's blocks each)
-template <int EPS>
+// (three components, a third of the instance's blocks each); SUMS: some
+// instance of the batch wants its conservation sums
+template <bool EPS, bool SUMS>
 __global__ void __launch_bounds__(256) kb_project(BLaunch L) {
     batch_loop(L, [&](const BInst& I, Blk b) {
         const long long nb = I.gd.nbulk, nf = I.gd.nfine;
@@ -601,9 +602,9 @@ __global__ void __launch_bounds__(256) kb_project(BLaunch L) {
         const Blk bb = {b.id - c * per, per};
         const int depth = EPS ? I.depth_eps : I.depth;
         switch (I.gd.r) {
-            case 2: project_body<float, 2, !EPS>(in, out, I.gd, depth, part, per, c, bb); break;
-            case 4: project_body<float, 4, !EPS>(in, out, I.gd, depth, part, per, c, bb); break;
-            default: project_body<float, 8, !EPS>(in, out, I.gd, depth, part, per, c, bb); break;
+            case 2: project_body<float, 2, SUMS>(in, out, I.gd, depth, part, per, c, bb); break;
+            case 4: project_body<float, 4, SUMS>(in, out, I.gd, depth, part, per, c, bb); break;
+            default: project_body<float, 8, SUMS>(in, out, I.gd, depth, part, per, c, bb); break;
         }
     });
 }
@@ -612,19 +613,24 @@ cg_status launch_batch_fine(int phase, const BLaunch& L, unsigned grid, cudaStre
     if (L.total == 0 || grid == 0) return CG_OK;
     switch (phase) {
         case BP_AVG: kb_average<<<grid, 256, 0, s>>>(L); break;
-        case BP_PROJ: kb_project<0><<<grid, 256, 0, s>>>(L); break;
-        case BP_PROJE: kb_project<1><<<grid, 256, 0, s>>>(L); break;
+        case BP_PROJ:
+            if (L.sums) kb_project<false, true><<<grid, 256, 0, s>>>(L);
+            else kb_project<false, false><<<grid, 256, 0, s>>>(L);
+            break;
+        case BP_PROJE: kb_project<true, false><<<grid, 256, 0, s>>>(L); break;
         default: return CG_ERR_INVALID_ARG;
     }
     CG_CUDA(cudaGetLastError());
     return CG_OK;
 }
 
-int batch_fine_occupancy(int phase) {
+int batch_fine_occupancy(int phase, bool sums) {
     int occ = 0;
-    cudaError_t e = phase == BP_AVG    ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_average, 256, 0)
-                    : phase == BP_PROJ ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_project<0>, 256, 0)
-                                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kb_project<1>, 256, 0);
+    auto of = [&](auto k) { return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, 256, 0); };
+    const cudaError_t e = phase == BP_AVG     ? of(kb_average)
+                          : phase == BP_PROJE ? of(kb_project<true, false>)
+                          : sums              ? of(kb_project<false, true>)
+                                              : of(kb_project<false, false>);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 1;

@@ -60,3 +60,40 @@ def test_sums_on_both_sides_of_every_size(cuda_lib, n, fp64, ordered):
     assert np.all(np.abs(sums[2:5] - tot) <= tol * tm)
     assert sums[15] == g.cg_sync_status()[2][2]
     g.close()
+
+
+@pytest.mark.parametrize("r", [2, 3, 5])
+@pytest.mark.parametrize("fp64,ordered", [(False, False), (False, True), (True, False)])
+def test_fields_without_the_sums_are_the_same(cuda_lib, r, fp64, ordered):
+    """A step that is given no place for its sums forms none: every other
+    output keeps its bits, and so does the clamped count."""
+    import torch
+    cg = cuda_lib
+    nb, n = (6, 5, 7), 20_011
+    desc = synth.make_desc((0.0, 0.0, 0.0), (0.6, 0.5, 0.7), [r * m for m in nb], r, fp64=fp64, law=1, interp=0,
+                           gravity=(0.0, 0.0, 0.0))
+    rng = synth.rng_for(n, 6)
+    T = np.float64 if fp64 else np.float32
+    pos = np.empty((n, 4), T)
+    pos[:, :3] = np.array(desc["extent"]) * rng.random((n, 3)) * 0.999
+    pos[:, 3] = 0.012
+    vel = (0.05 * rng.standard_normal((n, 4))).astype(T)
+    got = []
+    for sums in (True, False):
+        g = cg.Grids(desc)
+        u = to_dev((0.5 + 0.02 * synth.rng_for(n, 7).standard_normal((3, g.n_fine))).astype(T))
+        p, v = to_dev(pos), to_dev(vel)
+        out = g.alloc_outputs(n, eps_fine=True, bins=True)
+        if not sums:
+            out["sums"] = None
+        for _ in range(2):
+            if ordered:
+                g.cg_step_sorted(p, v, torch.empty_like(p), torch.empty_like(v), u, out)
+            else:
+                g.cg_step(p, v, u, out)
+        torch.cuda.synchronize()
+        got.append(({k: t.clone() for k, t in out.items() if t is not None and k != "sums"}, g.cg_sync_status()))
+        g.close()
+    assert got[0][1] == got[1][1]
+    for k in got[1][0]:
+        assert torch.equal(got[0][0][k], got[1][0][k]), k
