@@ -335,6 +335,15 @@ constexpr int kRebinCounters = 8;
 // counters, the scans' block totals.
 inline long long rebin_pad(long long ints) { return (ints + 63) / 64 * 64; }
 inline long long rebin_tiles(long long m) { return (m + kRebinScan - 1) / kRebinScan; }
+// Cells per thread of the pass over the cells: one, the shortest chain, except
+// on larger FP64 grids, where the block's compensated sum costs more than the
+// cells (128,000 cells: 17 us against 23).  Its blocks (with the end of the
+// last cell).
+inline int cell_items(long long nbulk, bool fp64) { return fp64 && nbulk >= (1 << 16) ? kRebinScan / 256 : 1; }
+inline long long cell_blocks(long long nbulk, bool fp64) {
+    const long long per = 256LL * cell_items(nbulk, fp64);
+    return (nbulk + per) / per;
+}
 inline long long rebin_small_ints(long long nbulk, long long nblk) {
     return 4 * rebin_pad(nbulk + 1) + rebin_pad(nblk + 1) + rebin_pad(kRebinCounters) + 2 * rebin_tiles(nbulk + 1) +
            rebin_tiles(nblk + 1);
@@ -365,9 +374,11 @@ cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps =
 cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, StepEps* eps);
 // Slots per chunk of the segmented sums: 256, and fewer for small particle
 // counts, whose few chunks would be a chain of eight rounds on a few SMs
-// (10,000 particles, FP64: the reaction 18 -> 10 us; at 500,000 a chunk of
-// 128 gains nothing, 256 is faster).  By the particle count alone, so that
-// every path over the same particles cuts them alike and gives the same sums.
+// (10,000 particles, FP64: the reaction 18 -> 10 us).  Chunks of 160 at 500,000
+// particles would take 2 us of 23 off the sorted drag, and add a quarter to the
+// reaction of a batch of such instances (52 -> 65 us).  By the particle count
+// alone, so that every path over the same particles cuts them alike and gives
+// the same sums.
 __host__ __device__ inline int seg_chunk(long long n) {
     return n >= (1 << 17) ? 256 : n >= (1 << 16) ? 128 : n >= (1 << 15) ? 64 : 32;
 }

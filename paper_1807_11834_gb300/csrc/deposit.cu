@@ -70,14 +70,13 @@ k_volume_rows(const T* __restrict__ d, long long n, const int32_t* __restrict__ 
 }
 
 template <typename T, bool SUMS>
-__global__ void __launch_bounds__(256) k_eps_finish(GridDev g, EpsOut<T> o, T* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_eps_finish(GridDev g, int items, EpsOut<T> o, T* __restrict__ part) {
     pdl_wait();
     // the cells of a block as in the incremental binning's pass over them, so
     // that the sums come out the same
     CSum<T> tot[1];
-#pragma unroll
-    for (int j = 0; j < kRebinScan / 256; ++j) {
-        const long long c = (long long)blockIdx.x * kRebinScan + j * 256 + threadIdx.x;
+    for (int j = 0; j < items; ++j) {
+        const long long c = ((long long)blockIdx.x * items + j) * 256 + threadIdx.x;
         if (c < g.nbulk) eps_finish<T, SUMS>(c, g, o, tot[0]);
     }
     if (SUMS) block_sums<T, 1>(tot, part, gridDim.x, blockIdx.x);
@@ -342,11 +341,12 @@ static cg_status deposit_volume_impl(cg_grids* g, long long n, const T* pos_d, S
             CG_LAUNCH(g, "deposit_volume", (k_volume_rows<T, false>), nblk, 256, 0, (const T*)g->vol_sorted, n,
                       (const int32_t*)g->perm, (const int32_t*)g->key_sorted, g->gd, o);
     }
-    const unsigned fblk = (unsigned)rebin_tiles(g->gd.nbulk + 1);
+    const unsigned fblk = (unsigned)cell_blocks(g->gd.nbulk, sizeof(T) == 8);
+    const int items = cell_items(g->gd.nbulk, sizeof(T) == 8);
     T* part = (T*)part_ptr(g, PS_VOL);
     g->part_blocks[PS_VOL] = e->sums ? (long long)fblk : -1;
-    if (e->sums) CG_LAUNCH(g, "deposit_volume", (k_eps_finish<T, true>), fblk, 256, 0, g->gd, o, part);
-    else CG_LAUNCH(g, "deposit_volume", (k_eps_finish<T, false>), fblk, 256, 0, g->gd, o, part);
+    if (e->sums) CG_LAUNCH(g, "deposit_volume", (k_eps_finish<T, true>), fblk, 256, 0, g->gd, items, o, part);
+    else CG_LAUNCH(g, "deposit_volume", (k_eps_finish<T, false>), fblk, 256, 0, g->gd, items, o, part);
     e->formed = true;
     if (e->ready) CG_CUDA(cudaEventRecord(e->ready, g->stream));
     return CG_OK;
