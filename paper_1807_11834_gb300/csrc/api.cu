@@ -342,7 +342,7 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
         gd.xhif[a] = (float)gd.xhi[a];
         gd.topf[a] = (float)(nb[a] - 2);
         gd.invHf[a] = (float)gd.invH[a];
-        gd.ax0f[a] = (float)fabs(d.origin[a] * gd.invH[a]);
+        gd.binh[a] = (float)(0.5 - ldexp(fabs(d.origin[a] * gd.invH[a]), -21) - ldexp(1.0, -24));
         split_ff(d.origin[a], gd.x0h[a], gd.x0l[a]);
         split_ff(gd.invH[a], gd.ihh[a], gd.ihl[a]);
         split_ff(-(d.origin[a] / gd.H[a] + 0.5), gd.xbh[a], gd.xbl[a]);

@@ -77,10 +77,7 @@ __device__ __forceinline__ void bin_key_body(const T* __restrict__ pos, long lon
         int c = -1;
         if (valid) {
             const V4<T>& v = pv[k];
-            int outside = 0, nonfinite = 0;
-            c = cell_of(v, g, outside, nonfinite);
-            n_out += outside;
-            n_nf += nonfinite;
+            c = cell_of(v, g, n_out, n_nf);
             key[p] = c;
             vol[p] = v.w;   // the diameter: the porosity forms the volume as an exact pair
         }
@@ -158,10 +155,7 @@ __device__ __forceinline__ void bin_key_rank_body(const T* __restrict__ pos, lon
         int c = -1;
         if (valid) {
             const V4<T>& v = pv[k];
-            int outside = 0, nonfinite = 0;
-            c = cell_of(v, g, outside, nonfinite);
-            n_out += outside;
-            n_nf += nonfinite;
+            c = cell_of(v, g, n_out, n_nf);
             key[p] = c;
             vol[p] = v.w;   // the diameter: the porosity forms the volume as an exact pair
         }

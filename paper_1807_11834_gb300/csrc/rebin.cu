@@ -95,8 +95,8 @@ __device__ __forceinline__ void add_status_counts(unsigned long long* st, int ou
 // cells' volumes.  IDENT: old slot s holds particle s.
 //
 // Bound by HBM in the sorted step (20 bytes read, 4 written per particle) and
-// by instruction issue with VOL (about 200 warp instructions per 32 slots);
-// 32M particles 213 us, where marking and the porosity as kernels of their
+// by instruction issue with VOL (about 190 warp instructions per 32 slots);
+// 32M particles 209 us, where marking and the porosity as kernels of their
 // own took 201 + 148.  In the caller's order it replaces a key kernel over the
 // particles as well: 4M packed 31 + 19 + 25 -> 54 us.
 template <typename T, bool IDENT, bool VOL>
@@ -145,10 +145,7 @@ k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restr
             const bool valid = s < n;
             cn[k] = 0;
             if (valid) {
-                int outside = 0, nonfinite = 0;
-                cn[k] = cell_of(pv[k], g, outside, nonfinite);
-                n_out += outside;
-                n_nf += nonfinite;
+                cn[k] = cell_of(pv[k], g, n_out, n_nf);
             }
             const bool moved = valid && cn[k] != co[k];
             mb[k] = __ballot_sync(full, moved);

@@ -135,7 +135,7 @@ extern "C" cg_status cg_bin_particles_static(const cg_grid_desc* desc, int64_t n
         gd.invH[a] = 1.0 / gd.H[a];
         gd.x0f[a] = (float)d.origin[a];
         gd.invHf[a] = (float)gd.invH[a];
-        gd.ax0f[a] = (float)fabs(d.origin[a] * gd.invH[a]);
+        gd.binh[a] = (float)(0.5 - ldexp(fabs(d.origin[a] * gd.invH[a]), -21) - ldexp(1.0, -24));
     }
     int bits = 0;
     while ((1LL << bits) < nbulk) ++bits;
