@@ -763,11 +763,13 @@ __device__ __forceinline__ void seg_chunk_range(long long base, long long n, con
 
 // One round of the segmented sum of K (<= 4) values per slot over a chunk's
 // slots: 32 consecutive slots, one per lane (key -1: none), with `next31` the key
-// of the next round's first slot (-1 past the chunk's end).  A plain inclusive shuffle scan inside the round
-// (at most five roundings); the segment that goes on from round to round is a
-// compensated sum.  That sum is held once per warp, value k on lane k, so that
-// its additions cost one instruction for all K values (held by every lane,
-// they were 40% of the reaction's FP32 and two thirds of its FP64
+// of the next round's first slot (-1 past the chunk's end).  Inside the round a
+// plain inclusive shuffle scan, or, where the round holds one cell, a tree (at
+// most five roundings either way; the tree: FP64, 1M packed particles, 62 ->
+// 53 us, the sorted drag of 32M 710 -> 701); the segment that goes on from
+// round to round is a compensated sum.  That sum is held once per warp, value k
+// on lane k, so that its additions cost one instruction for all K values (held
+// by every lane, they were 40% of the reaction's FP32 and two thirds of its FP64
 // instructions: FP64, 1M particles 137 -> 68 us; FP32, which the shuffles bound,
 // 4M particles 32 -> 29, 32M 190 -> 170).
 // emit(key, k, total) is called once per segment and value, each value by
@@ -784,6 +786,30 @@ __device__ __forceinline__ void seg_round(T (&v)[K], int key, int next31, SegCar
     const int lane = threadIdx.x & 31;
     const int prev = __shfl_up_sync(full, key, 1);
     const unsigned heads = __ballot_sync(full, lane == 0 || prev != key);
+    if (heads == 1u) {
+        // one cell: a tree over the lanes in which a lane hands half of its values
+        // on at the first two steps (six additions for up to four values)
+        const int first = __shfl_sync(full, key, 0);
+        T w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = k < K ? v[k < K ? k : 0] : T(0);
+        const bool up = lane & 16, up2 = lane & 8;
+        const T a0 = (up ? w[2] : w[0]) + __shfl_xor_sync(full, up ? w[0] : w[2], 16);
+        const T a1 = (up ? w[3] : w[1]) + __shfl_xor_sync(full, up ? w[1] : w[3], 16);
+        T x = (up2 ? a1 : a0) + __shfl_xor_sync(full, up2 ? a0 : a1, 8);
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) x += __shfl_xor_sync(full, x, off);
+        x = __shfl_sync(full, x, (lane & 2) * 8 + (lane & 1) * 8);   // value k on lane k
+        if (first == carry.key) {
+            carry.a.add(x);
+        } else {
+            carry.a = CSum<T>();
+            carry.a.s = x;
+            carry.key = first;
+        }
+        if (first >= 0 && next31 != first && lane < K) emit(first, lane, carry.a.get());
+        return;
+    }
     const int head = 31 - __clz(heads & ((2u << lane) - 1u));   // first lane of this lane's segment
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {

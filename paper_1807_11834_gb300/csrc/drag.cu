@@ -51,6 +51,20 @@ struct DragOne {
     int cl;
 };
 
+// Whether x may lie outside [lo, hi]; exact in FP32.  FP64 compares the upper words
+// as integers (their order for equal signs, reversed for negative ones), off the FP64
+// pipe; x within 2^-20 of a bound counts as outside, which the caller then
+// decides exactly.
+__device__ __forceinline__ bool outside_of(float x, float lo, float hi) { return x < lo || x > hi; }
+__device__ __forceinline__ int ordered_hi(double x) {
+    const int h = __double2hiint(x);
+    return h ^ ((h >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ bool outside_of(double x, double lo, double hi) {
+    const int h = ordered_hi(x);
+    return h <= ordered_hi(lo) || h >= ordered_hi(hi);
+}
+
 template <typename T, bool EULER>
 __device__ __forceinline__ DragOne<T> drag_from(const V4<T>& x, const V4<T>& v, const V4<T>& b, const GridDev& g,
                                                 const Phys<T>& P, T dt) {
@@ -89,7 +103,7 @@ __device__ __forceinline__ DragOne<T> drag_from(const V4<T>& x, const V4<T>& v, 
             // the FP32 path reads the bounds' float copies (no conversion in the loop)
             const T lo = sizeof(T) == 4 ? (T)g.x0f[a] : (T)g.x0[a];
             const T hi = sizeof(T) == 4 ? (T)g.xhif[a] : (T)g.xhi[a];
-            out = out || r.x[a] < lo || r.x[a] > hi;
+            out = out || outside_of(r.x[a], lo, hi);
         }
         if (out)   // specular walls: rare, so one branch for the three axes
 #pragma unroll
