@@ -375,11 +375,12 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     if (st == CG_OK) st = dalloc(&g->bulk4, 4 * g->tsize * nbulk);
     if (st == CG_OK) st = dalloc(&g->eps_t, g->tsize * nbulk);
     if (st == CG_OK) st = dalloc(&g->vol_acc, 3 * sizeof(unsigned long long) * nbulk);
-    if (st == CG_OK && cudaMemsetAsync(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk, g->stream) != cudaSuccess)
-        st = CG_ERR_CUDA;
+    if (st == CG_OK && cudaMemset(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk) != cudaSuccess) st = CG_ERR_CUDA;
     if (st == CG_OK) st = dalloc(&g->status, sizeof(unsigned long long) * kNumSlots);
     if (st == CG_OK && cudaMemset(g->status, 0, sizeof(unsigned long long) * kNumSlots) != cudaSuccess)
         st = CG_ERR_CUDA;
+    // both zeroes are there before a step on any stream (cg_set_stream, a batch) adds to them
+    if (st == CG_OK && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) st = CG_ERR_CUDA;
     if (st == CG_OK && cudaStreamCreateWithFlags(&g->aux, cudaStreamNonBlocking) != cudaSuccess) st = CG_ERR_CUDA;
     cudaEvent_t* evs[] = {&g->ev_fork, &g->ev_avg, &g->ev_pack, &g->ev_epsf};
     for (cudaEvent_t* e : evs)
