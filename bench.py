@@ -44,12 +44,12 @@ UNIT = "particle-steps/s"
 # dram__bytes_write.sum), keyed by kernel, valid only while the kernel's
 # source files are byte-identical to the ones profiled (sha256 prefixes).
 NCU_TRAFFIC = {
-    # packed bed, one warm launch of k_average<float,4>: 405.5 MB read + 8.1 MB written
-    ("packed_bed", "average"): {"files": {"fine.cu": "b5357b772279f4b1"}, "bytes": 413.6e6},
-    # clustered-bed recipe at 16M particles, a warm sorted step of k_drag<float,1>:
-    # 578.7 MB read + 904.7 MB written, times 2 for the 32M bed (traffic per particle)
-    ("clustered_bed", "drag"): {"files": {"drag.cu": "96408310edce01e8", "drag_law.cuh": "e2f8745533c61039"},
-                                "bytes": 2.967e9},
+    # packed bed, one warm launch of k_average<float, 4>: 404.9 MB read + 6.8 MB written
+    ("packed_bed", "average"): {"files": {"fine.cu": "e49b8f73f42fa649"}, "bytes": 411.7e6},
+    # clustered-bed recipe at 16M particles, a warm sorted step of k_drag_sorted<float, 1, 1> (the
+    # reaction with it): 668.4 MB read + 661.3 MB written, times 2 for the 32M bed (traffic per particle)
+    ("clustered_bed", "drag"): {"files": {"drag.cu": "cc7422222cbf8a04", "drag_law.cuh": "fc474a5902a1ea4d"},
+                                "bytes": 2.659e9},
 }
 
 
@@ -251,9 +251,14 @@ def algorithmic_bytes(g, n, eps_fine=True, implicit=False, euler=False, sorted_s
         "bin_hist": n * 4,
         "bin_place": n * (4 + 4 + 4),                     # key, rank read; id written at its slot
         "bin_seg_sort": n * (4 + 4 + 16),                 # placed id, diameter read; perm, key, inverse, diameter written
-        "deposit_volume": (nbx * 8 + n * 8 + nbx * 8) // 2,   # fill eps; read sorted volume + key; write eps
+        "cell_starts": nbx * 4,                           # digit sort: the starts searched in the sorted cells
+        # two launches (mean): diameter + cell read; accumulator read, eps, its copies and the cleared source written
+        "deposit_volume": (n * 8 + nbx * (16 + 28)) // 2,
         "pack": nbx * (8 + 12 + 16 + 4),
-        "drag": n * (16 + 16 + 4 + 12 + 16),              # pos, vel, slot read; F and sorted F written
+        # caller order: pos, vel, slot read; F and sorted F written; sorted step (the
+        # reaction with it): pos, vel, id, cell read; F, pos, vel written
+        "drag": n * (16 + 16 + 8 + 12 + 32) if sorted_step else n * (16 + 16 + 4 + 12 + 16),
+        "unsort_force": n * (4 + 16 + 12),                # slot, sorted F read; F written
         "deposit_momentum": n * (16 + 4) + nbx * 12,
         "project": nf * 12 + nbx * 12,                    # S_f written, S_B read
         "project_eps": nf * 4 + nbx * 4,                  # eps_f written, eps_B read
@@ -261,18 +266,19 @@ def algorithmic_bytes(g, n, eps_fine=True, implicit=False, euler=False, sorted_s
         "deposit_implicit": n * (16 + 4) + nbx * 16,      # sorted (beta, beta u) + key read; A, b written
         "project_implicit": nf * 16 + nbx * 16,           # A_f, b_f written, A, b read
         # incremental rebinning (the movers' placement and the idle fallback not counted)
-        "rebin_key": n * (16 + 4 + 4),                    # pos read; key, diameter written
-        "rebin_mark": n * ((16 + 4 + 4 + 4) if sorted_step else (4 + 4 + 4 + 8)),
-        # sorted input: pos, old cell read; diameter, record written;
-        # else old id, old cell, new cell (gathered) read; record, old id written
-        "rebin_cells": nbx * 16,                          # old starts, departures, arrivals read; counts written
-        "rebin_slots": n * (4 + 4 + 16 + (0 if sorted_step else 4)),
-        # stayers (the movers beside them not counted): record, diameter (and
-        # in caller order the old id) read; perm, cell, inverse, diameter written
+        "rebin_mark": n * ((16 + 4 + 4) if sorted_step else (4 + 4 + 16 + 4 + 4)),
+        # pos, old cell (in caller order the old id) read; record (old id) written
+        "rebin_cells": nbx * (16 + 4 + 16 + 28),
+        # old starts, departures, arrivals read, counts written; accumulator read, eps, its copies and
+        # the cleared source written
+        "rebin_slots": n * ((4 + 8) if sorted_step else (8 + 12)),
+        # stayers (the movers beside them not counted): record (and old id) read; perm, cell (and inverse) written
+        "rebin_starts": nbx * 8,
     }
     step = n * 48 + nf * (24 + (4 if eps_fine else 0)) + nb * 40
     if euler:
-        per["drag"] += n * 24                             # x and u_p written back
+        if not sorted_step:
+            per["drag"] += n * 24                         # x and u_p written back
         step += n * 24
     if implicit:
         per["drag"] += n * 16                             # the sorted (beta, beta u) record

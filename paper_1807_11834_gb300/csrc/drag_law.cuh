@@ -12,7 +12,7 @@ namespace cg {
 // Euler advance is written with explicitly rounded operations (mul, add,
 // sub, div, and fma where a fused product is meant), so the compiler cannot
 // fuse a product into an addition in one kernel and not in another: every
-// kernel built from this code (plain, windowed, batched, learned) gives the
+// kernel built from this code (caller order, sorted, batched, learned) gives the
 // same bits for the same particle.
 template <typename T> struct M;
 template <> struct M<float> {
