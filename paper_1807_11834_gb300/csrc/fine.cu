@@ -649,7 +649,12 @@ static cg_status average_launch(cg_grids* g, const void* u_fine, void* u_bulk, v
     constexpr bool warp = RC == 2 || RC == 4 || RC == 8;
     const int bs = warp && g->gd.nbulk >= 64LL * g->num_sms ? 256 : 64;
     const long long need = (g->gd.nbulk + average_cells<RC, sizeof(T) == 8>(bs) - 1) / average_cells<RC, sizeof(T) == 8>(bs);
-    const unsigned nblk = (unsigned)std::min(need, (long long)g->num_sms * (bs == 256 ? (RC == 2 ? 4 : 2) : 32));
+    // FP64: a block per group of cells.  The busiest SM's arithmetic is its time, and two
+    // resident blocks per SM, placed beside the particle kernels that have
+    // started first, fall unevenly on the SMs (1M particles, 128,000 cells: the
+    // step 1026 -> 939 us)
+    const unsigned nblk =
+        (unsigned)std::min(need, (long long)g->num_sms * (bs == 256 && sizeof(T) == 4 ? (RC == 2 ? 4 : 2) : 32));
     CG_LAUNCH(g, "average", (k_average<T, RC>), nblk, bs, 0, (const T*)u_fine, g->gd, (T*)u_bulk, (T*)var_bulk, (T*)rec);
     return CG_OK;
 }
