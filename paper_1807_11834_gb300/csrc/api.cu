@@ -197,7 +197,10 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     CG_TRY(dalloc(&g->rb_rid, sizeof(int32_t) * cap));
     CG_TRY(dalloc(&g->rb_rkn, sizeof(int32_t) * cap));
     CG_TRY(dalloc(&g->rb_mov, sizeof(int4) * g->rb_nblk * kRebinTile));
-    CG_TRY(dalloc(&g->rb_small, sizeof(int32_t) * rebin_small_ints(g->gd.nbulk, g->rb_nblk)));
+    const size_t small = sizeof(int32_t) * rebin_small_ints(g->gd.nbulk, g->rb_nblk);
+    CG_TRY(dalloc(&g->rb_small, small));
+    CG_CUDA(cudaMemsetAsync(g->rb_small, 0, small, g->stream));   // the rebinning leaves its counters zero
+    g->rb_dirty = false;
     const long long cells_blk = (g->gd.nbulk + 1 + kScanItems - 1) / kScanItems;
     g->scan_cap = (g->hist_cap + kScanItems - 1) / kScanItems + cells_blk;
     CG_TRY(dalloc(&g->scan_part, sizeof(int32_t) * g->scan_cap));

@@ -804,15 +804,27 @@ k_seg_sort(const int32_t* __restrict__ cell_start, long long nbulk, int32_t* tmp
 }
 
 // The last kernel of an incremental rebinning: the new starts to their
-// place, and in the fallback (run_if) the sort of every cell.
+// place, the arrays that the next rebinning counts in to zero (they are, when
+// nothing moved), and in the fallback the sort of every cell.  The block that
+// finishes last clears the counters, which every block has read by then.
 __global__ void __launch_bounds__(kSegSortWarps * 32, 4)
 k_seg_sort_fallback(const int32_t* __restrict__ cs, long long nbulk, int32_t* tmp, int32_t* alt,
                     int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-                    const int32_t* __restrict__ run_if, int32_t* __restrict__ cs_copy) {
+                    int32_t* ctr, int32_t* __restrict__ cs_copy, RebinClear z) {
     pdl_wait();
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c <= nbulk; c += (long long)gridDim.x * blockDim.x)
-        cs_copy[c] = __ldg(cs + c);
-    if (*run_if == 0) return;
+    const bool fallback = ctr[RB_FALLBACK] != 0, moved = ctr[RB_MOVERS] != 0;
+    const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    for (long long c = i0; c <= nbulk; c += step) cs_copy[c] = __ldg(cs + c);
+    if (moved) {
+        for (long long c = i0; c < z.na; c += step) z.a[c] = make_int4(0, 0, 0, 0);
+        for (long long c = i0; c < z.npart; c += step) z.part[c] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(ctr + RB_DONE, 1) == (int)gridDim.x - 1) ctr[RB_FALLBACK] = ctr[RB_MOVERS] = ctr[RB_DONE] = 0;
+    }
+    if (!fallback) return;
     seg_sort_body<float>(cs, nbulk, tmp, alt, perm, key_sorted, inv_perm, nullptr, nullptr, launch_blk());
 }
 
@@ -900,11 +912,11 @@ static cg_status bin_rank(cg_grids* g, long long n, const T* pos) {
     return CG_OK;
 }
 
-cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, const int32_t* run_if, int32_t* cs_copy,
-                                   int32_t* inv_perm) {
-    // usually only the copy: one grid-stride CTA per SM keeps the launch short
+cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, int32_t* ctr, int32_t* cs_copy, int32_t* inv_perm,
+                                   const RebinClear& clear) {
+    // usually only the copy and the clear: one grid-stride CTA per SM keeps the launch short
     CG_LAUNCH(g, "rebin_starts", k_seg_sort_fallback, (unsigned)g->num_sms, kSegSortWarps * 32, 0, cs, g->gd.nbulk,
-              g->val1, g->key1, g->perm, g->key_sorted, inv_perm, run_if, cs_copy);
+              g->val1, g->key1, g->perm, g->key_sorted, inv_perm, ctr, cs_copy, clear);
     return CG_OK;
 }
 

@@ -199,6 +199,7 @@ struct cg_grids {
     int4* rb_mov = nullptr;        // [rb_nblk * kRebinTile] movers, each block of old slots its own part:
                                    // (id, new cell, next mover of that cell + 1, arrival rank)
     int32_t* rb_small = nullptr;   // per-cell and per-block counts, starts, list heads; counters (rebin_ptrs)
+    bool rb_dirty = false;         // a rebinning was not launched to its end: its counters are not zero
     long long rb_nblk = 0;
     int32_t* hist = nullptr;       // [2^digit * ntiles]
     int32_t* scan_part = nullptr;  // scan block partials
@@ -319,9 +320,18 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n);
 // The per-cell sort of the ids placed in val1 from the cell starts cs, as the
 // fallback of the incremental rebinning (does nothing but copy cs to cs_copy
 // unless *run_if != 0).
-cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, const int32_t* run_if, int32_t* cs_copy,
-                                   int32_t* inv_perm);
+// What the last kernel of a rebinning clears for the next one: the per-cell
+// arrays (in int4) and the tile totals.
+struct RebinClear {
+    int4* a;
+    long long na;
+    int32_t* part;
+    long long npart;
+};
+cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, int32_t* ctr, int32_t* cs_copy, int32_t* inv_perm,
+                                   const RebinClear& clear);
 // Incremental rebinning (rebin.cu).
+enum { RB_FALLBACK = 0, RB_MOVERS = 1, RB_DONE = 2 };   // counters: fallback flag, movers, finished blocks of the last kernel
 constexpr int kRebinThreads = 256;
 constexpr int kRebinItems = 4;
 constexpr int kRebinTile = kRebinThreads * kRebinItems;   // old slots per block

@@ -45,16 +45,14 @@ namespace cg {
 
 namespace {
 
-enum { RB_FALLBACK = 0, RB_MOVERS = 1 };   // counters: fallback flag, movers
-
 struct RebinPtrs {
     int32_t* cnt;       // [n_b + 1] new counts, then (scanned in place) new starts
     int32_t* blk;       // [nblk + 1] departures per block of old slots, then their starts
     int2* arr;          // [n_b + 1] arrivals per cell, then their starts; first mover of the cell's list + 1 (0: none)
     int32_t* dep;       // [n_b] departures per cell
-    int32_t* ctr;       // [kRebinCounters] fallback flag, movers
+    int32_t* ctr;       // [kRebinCounters]
     int32_t* part;      // block totals of the scans
-    size_t zero_bytes;  // arr .. ctr, to be cleared before the first kernel
+    size_t zero_bytes;  // arr .. part: zero before the first kernel
 };
 
 RebinPtrs rebin_ptrs(cg_grids* g) {
@@ -508,7 +506,10 @@ static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, 
     const long long nblk = (n + kRebinTile - 1) / kRebinTile;
     if (nblk > g->rb_nblk) return CG_ERR_OUT_OF_RANGE;
     const EpsOut<T> eo = eps_out<T>(g, eps);
-    CG_CUDA(cudaMemsetAsync(R.arr, 0, R.zero_bytes, g->stream));
+    // the last kernel clears what the next rebinning counts in (a clear of its own
+    // at the head of the chain costs 2 to 3 us)
+    if (g->rb_dirty) CG_CUDA(cudaMemsetAsync(R.arr, 0, R.zero_bytes, g->stream));
+    g->rb_dirty = true;
     // the caller's order: resident CTAs that walk the blocks of old slots, the
     // next block's ids and cells loaded ahead of the gather they lead to
     const long long walk = (long long)g->num_sms * (sizeof(T) == 4 ? 4 : 3);
@@ -556,8 +557,12 @@ static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, 
     if (ident) CG_REBIN_SLOTS(true);
     else CG_REBIN_SLOTS(false);
 #undef CG_REBIN_SLOTS
-    // the starts to their place; in the fallback also the sort of every cell
-    return launch_cellsort_fallback(g, R.cnt, R.ctr + RB_FALLBACK, g->cell_start, ident ? nullptr : g->inv_perm);
+    // the starts to their place, the counters to zero; in the fallback also the sort of every cell
+    const long long nb1 = rebin_pad(nbulk + 1);
+    CG_TRY(launch_cellsort_fallback(g, R.cnt, R.ctr, g->cell_start, ident ? nullptr : g->inv_perm,
+                                    {(int4*)R.arr, 3 * nb1 / 4, R.part, 2 * tiles + btiles}));
+    g->rb_dirty = false;
+    return CG_OK;
 }
 
 // Caller-order values of the binning's slots: the cell of every particle, or
