@@ -506,6 +506,7 @@ cg_status cg_drag(cg_grids* g, int64_t n, const void* pos_d, const void* vel, co
     }
     CG_TRY(ensure_particle_capacity(g, n));
     CG_TRY(launch_pack(g, eps_bulk, u_bulk, false));
+    if (S_bulk_out) CG_TRY(ensure_inverse(g, n));
     if (mlp)
         return launch_drag_learned(g, mlp, n, const_cast<void*>(pos_d), const_cast<void*>(vel), var_stale, u_fine,
                                    age, force_out, S_bulk_out, 0.0);
@@ -580,6 +581,8 @@ static cg_status step_impl(cg_grids* g, const cg_particles* p, const void* u_fin
     eps.sums = sums;
     eps.ready = eps.eps_t ? g->ev_pack : nullptr;
     CG_TRY(launch_bin(g, n, p->pos_d, &eps));
+    // every other binning of this call left the inverse valid
+    if (g->bin_ident && !sorted_out) CG_TRY(ensure_inverse(g, n));
     // sorted diameters of this binning
     if (!eps.formed) CG_TRY(launch_deposit_volume(g, n, nullptr, &eps));
     CG_TRY(copy_bins(g, n, o->cell, sorted_out ? nullptr : o->perm, o->cell_start));   // the sorted drag writes perm

@@ -822,7 +822,10 @@ k_seg_sort_fallback(const int32_t* __restrict__ cs, long long nbulk, int32_t* tm
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(ctr + RB_DONE, 1) == (int)gridDim.x - 1) ctr[RB_FALLBACK] = ctr[RB_MOVERS] = ctr[RB_DONE] = 0;
+        if (atomicAdd(ctr + RB_DONE, 1) == (int)gridDim.x - 1) {
+            ctr[RB_FALLBACK] = ctr[RB_MOVERS] = ctr[RB_DONE] = 0;
+            ctr[RB_INV_STALE] = inv_perm == nullptr;
+        }
     }
     if (!fallback) return;
     seg_sort_body<float>(cs, nbulk, tmp, alt, perm, key_sorted, inv_perm, nullptr, nullptr, launch_blk());
@@ -1077,8 +1080,8 @@ cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps) 
     const bool rebin = n > 0 && n < kRebinMaxParticles && g->rb_rkn && g->hint_n == n && n <= g->cap &&
                        (g->desc.sort_digits == CG_SORT_AUTO || g->desc.sort_digits == CG_SORT_CELLS);
     const bool ident = rebin && pos_d == g->hint_ident;
-    // a binning that finds no mover leaves perm and inv_perm as they are
-    if (rebin && !ident) CG_TRY(ensure_inverse(g, n));
+    g->bin_ident = ident;
+    g->ident_seen = g->ident_seen || ident;
     g->hint_n = -1;
     g->hint_ident = nullptr;
     g->n_binned = -1;
@@ -1086,11 +1089,10 @@ cg_status launch_bin(cg_grids* g, long long n, const void* pos_d, StepEps* eps) 
         CG_TRY(launch_rebin(g, n, pos_d, ident, eps));
         g->n_binned = n;
         g->key_valid = false;
-        g->inv_valid = !ident;
         g->hint_n = n;
         return CG_OK;
     }
-    g->key_valid = g->inv_valid = true;
+    g->key_valid = true;
     // the per-cell sort counts in cell_start; the exclusive scan turns it into starts
     const bool cells = use_cell_sort(g->desc.sort_digits, n, nbulk);
     if (cells || n == 0)

@@ -187,7 +187,8 @@ struct cg_grids {
     void* vol_sorted = nullptr;    // [cap] T particle diameter, sorted order
     void* Fs = nullptr;            // [cap] T4 drag force, sorted order
     bool key_valid = false;        // key holds the binning's caller-order cells (see copy_cells)
-    bool inv_valid = false;        // inv_perm holds the binning's inverse (see ensure_inverse)
+    bool bin_ident = false;        // the binning of this call took the identity hint, which leaves inv_perm out
+    bool ident_seen = false;       // some binning of this handle did, called or captured (see ensure_inverse)
     // incremental rebinning (rebin.cu): a binning of hint_n particles held in
     // perm / key_sorted / cell_start is where the next binning of the same
     // count starts; hint_ident is the particle array the last sorted step
@@ -331,7 +332,10 @@ struct RebinClear {
 cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, int32_t* ctr, int32_t* cs_copy, int32_t* inv_perm,
                                    const RebinClear& clear);
 // Incremental rebinning (rebin.cu).
-enum { RB_FALLBACK = 0, RB_MOVERS = 1, RB_DONE = 2 };   // counters: fallback flag, movers, finished blocks of the last kernel
+// Counters: fallback flag, movers, finished blocks of the last kernel, which
+// clears these three; whether inv_perm is not the inverse of perm, and the
+// finished blocks of the kernel that makes it so.
+enum { RB_FALLBACK = 0, RB_MOVERS = 1, RB_DONE = 2, RB_INV_STALE = 3, RB_INV_DONE = 4 };
 constexpr int kRebinThreads = 256;
 constexpr int kRebinItems = 4;
 constexpr int kRebinTile = kRebinThreads * kRebinItems;   // old slots per block
@@ -374,7 +378,10 @@ struct StepEps {
 cg_status launch_rebin(cg_grids* g, long long n, const void* pos_d, bool ident, StepEps* eps);
 // The caller-order cells of the last binning into cell_out.
 cg_status copy_cells(cg_grids* g, long long n, int32_t* cell_out);
-// inv_perm of the last binning (the identity-hint rebinning leaves it out).
+// inv_perm of the last binning.  The identity-hint rebinning leaves it out, and
+// whether it did is a word on the device: what ran last may have been a
+// replayed graph, which the host does not see.  A handle that never took that
+// path, by a call or a capture, launches nothing.
 cg_status ensure_inverse(cg_grids* g, long long n);
 cg_status ensure_partials(cg_grids* g, long long n);
 
@@ -411,11 +418,11 @@ cg_status launch_pack(cg_grids* g, const double* eps, const void* u_bulk, bool w
 // pos_out, vel_out (nullable, needs S_bulk): the particles, advanced when
 // dt > 0, are written to these arrays in the order of the binning.
 // perm_out (nullable): also gets the binning's permutation.  S_cleared: S_bulk
-// is zero already.
+// is zero already.  Without pos_out, S_bulk needs inv_perm (ensure_inverse).
 cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* vel, void* force, void* S_bulk,
                       bool sums, double dt, bool S_cleared = false, void* coef_bulk = nullptr, void* pos_out = nullptr,
                       void* vel_out = nullptr, int32_t* perm_out = nullptr);
-// Learned drag (FP32 only): bulk4 must hold (phi of this step, stale u).
+// Learned drag (FP32 only): bulk4 must hold (phi of this step, stale u); S_bulk needs inv_perm.
 cg_status launch_drag_learned(cg_grids* g, const cg_mlp* m, long long n, void* pos_d, void* vel,
                               const void* var_stale, const void* u_fine, int32_t age, void* force, void* S_bulk,
                               double dt, bool S_cleared = false);

@@ -457,7 +457,7 @@ static cg_status launch_drag_sorted(cg_grids* g, long long n, const T* pos, cons
     // one): their forces leave in the order of the binning and are gathered from
     // there, instead of three scattered 4-byte stores each (32M in random order,
     // the first step: 4390 -> 2480 us)
-    T* Fs = g->inv_valid ? (T*)g->Fs : nullptr;
+    T* Fs = g->bin_ident ? nullptr : (T*)g->Fs;
     // at most the resident CTAs
     const long long chunks = (n + seg_chunk(n) - 1) / seg_chunk(n);
     const int bs = (int)seg_threads(g, n), warps = bs / 32;
@@ -545,7 +545,6 @@ cg_status launch_drag(cg_grids* g, long long n, const void* pos_d, const void* v
     if (perm_out && n > 0)
         CG_CUDA(cudaMemcpyAsync(perm_out, g->perm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, g->stream));
     void* Fs = S_bulk ? g->Fs : nullptr;
-    if (Fs) CG_TRY(ensure_inverse(g, n));
     if (n > 0 || sums) {
 #define CG_DRAGP(T, E)                                                                                      \
     CG_LAUNCH(g, "drag", (k_drag<T, E>), nblk, bs, 0, (T*)pos_d, (T*)vel, n, g->gd, phys_of<T>(g->gd),          \

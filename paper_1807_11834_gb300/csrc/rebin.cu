@@ -485,10 +485,14 @@ k_rebin_slots(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn, 
     int32_t* const where = ctr[RB_FALLBACK] ? place : nullptr;
     if (ctr[RB_MOVERS] == 0) {
         // slot s keeps its particle and cell; with the identity hint the
-        // particles are renumbered to their slots
-        if (IDENT)
-            for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x)
-                perm[s] = (int)s;
+        // particles are renumbered to their slots, without it the inverse is
+        // made where the steps before left it out
+        const bool stale = !IDENT && ctr[RB_INV_STALE];
+        if (IDENT || stale)
+            for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
+                if (IDENT) perm[s] = (int)s;
+                else inv_perm[__ldg(perm + s)] = (int)s;
+            }
         return;
     }
     if ((long long)blockIdx.x < mgrid)
@@ -565,14 +569,28 @@ static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, 
     return CG_OK;
 }
 
-// Caller-order values of the binning's slots: the cell of every particle, or
-// its slot.
+// Caller-order cells of the binning's slots.
 __global__ void __launch_bounds__(256)
-k_scatter_bins(const int32_t* __restrict__ perm, const int32_t* __restrict__ key_sorted, long long n,
-               int32_t* __restrict__ out) {
+k_scatter_cells(const int32_t* __restrict__ perm, const int32_t* __restrict__ key_sorted, long long n,
+                int32_t* __restrict__ out) {
     pdl_wait();
     for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x)
-        out[__ldg(perm + s)] = key_sorted ? __ldg(key_sorted + s) : (int)s;
+        out[__ldg(perm + s)] = __ldg(key_sorted + s);
+}
+
+// The inverse of perm, where it is out of date; the block that finishes last
+// marks it valid, when every block has read the mark.
+__global__ void __launch_bounds__(256)
+k_inverse(const int32_t* __restrict__ perm, long long n, int32_t* __restrict__ inv_perm, int32_t* ctr) {
+    pdl_wait();
+    if (ctr[RB_INV_STALE] == 0) return;
+    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x)
+        inv_perm[__ldg(perm + s)] = (int)s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(ctr + RB_INV_DONE, 1) == (int)gridDim.x - 1) ctr[RB_INV_STALE] = ctr[RB_INV_DONE] = 0;
+    }
 }
 
 cg_status copy_cells(cg_grids* g, long long n, int32_t* cell_out) {
@@ -582,17 +600,15 @@ cg_status copy_cells(cg_grids* g, long long n, int32_t* cell_out) {
         return CG_OK;
     }
     const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)g->num_sms * 8);
-    CG_LAUNCH(g, "bin_cells", k_scatter_bins, grid, 256, 0, (const int32_t*)g->perm, (const int32_t*)g->key_sorted, n,
+    CG_LAUNCH(g, "bin_cells", k_scatter_cells, grid, 256, 0, (const int32_t*)g->perm, (const int32_t*)g->key_sorted, n,
               cell_out);
     return CG_OK;
 }
 
 cg_status ensure_inverse(cg_grids* g, long long n) {
-    if (g->inv_valid || n <= 0) return CG_OK;
+    if (!g->ident_seen || n <= 0) return CG_OK;
     const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, (long long)g->num_sms * 8);
-    CG_LAUNCH(g, "bin_inverse", k_scatter_bins, grid, 256, 0, (const int32_t*)g->perm, (const int32_t*)nullptr, n,
-              g->inv_perm);
-    g->inv_valid = true;
+    CG_LAUNCH(g, "bin_inverse", k_inverse, grid, 256, 0, (const int32_t*)g->perm, n, g->inv_perm, rebin_ptrs(g).ctr);
     return CG_OK;
 }
 
