@@ -199,7 +199,11 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     CG_TRY(dalloc(&g->rb_mov, sizeof(int4) * g->rb_nblk * kRebinTile));
     const size_t small = sizeof(int32_t) * rebin_small_ints(g->gd.nbulk, g->rb_nblk);
     CG_TRY(dalloc(&g->rb_small, small));
-    CG_CUDA(cudaMemsetAsync(g->rb_small, 0, small, g->stream));   // the rebinning leaves its counters zero
+    // The rebinning leaves its counters zero; their first zeroes are there before
+    // this returns, on whatever stream the next call runs (the handle's own side
+    // stream has nothing of the caller's to wait for).
+    CG_CUDA(cudaMemsetAsync(g->rb_small, 0, small, g->aux));
+    CG_CUDA(cudaStreamSynchronize(g->aux));
     g->rb_dirty = false;
     const long long cells_blk = (g->gd.nbulk + 1 + kScanItems - 1) / kScanItems;
     g->scan_cap = (g->hist_cap + kScanItems - 1) / kScanItems + cells_blk;
@@ -378,13 +382,14 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     if (st == CG_OK) st = dalloc(&g->bulk4, 4 * g->tsize * nbulk);
     if (st == CG_OK) st = dalloc(&g->eps_t, g->tsize * nbulk);
     if (st == CG_OK) st = dalloc(&g->vol_acc, 3 * sizeof(unsigned long long) * nbulk);
-    if (st == CG_OK && cudaMemset(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk) != cudaSuccess) st = CG_ERR_CUDA;
     if (st == CG_OK) st = dalloc(&g->status, sizeof(unsigned long long) * kNumSlots);
-    if (st == CG_OK && cudaMemset(g->status, 0, sizeof(unsigned long long) * kNumSlots) != cudaSuccess)
-        st = CG_ERR_CUDA;
-    // both zeroes are there before a step on any stream (cg_set_stream, a batch) adds to them
-    if (st == CG_OK && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) st = CG_ERR_CUDA;
+    // zero before a step on any stream (cg_set_stream, a batch) adds to them:
+    // ensure_particle_capacity below waits for this stream
     if (st == CG_OK && cudaStreamCreateWithFlags(&g->aux, cudaStreamNonBlocking) != cudaSuccess) st = CG_ERR_CUDA;
+    if (st == CG_OK &&
+        (cudaMemsetAsync(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk, g->aux) != cudaSuccess ||
+         cudaMemsetAsync(g->status, 0, sizeof(unsigned long long) * kNumSlots, g->aux) != cudaSuccess))
+        st = CG_ERR_CUDA;
     cudaEvent_t* evs[] = {&g->ev_fork, &g->ev_avg, &g->ev_pack, &g->ev_epsf};
     for (cudaEvent_t* e : evs)
         if (st == CG_OK && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) st = CG_ERR_CUDA;
