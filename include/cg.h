@@ -210,6 +210,13 @@ cg_status cg_destroy_grids(cg_grids* g);
  * valid and allocates again on its next call. */
 cg_status cg_debug_fail_alloc_after(int64_t k);
 
+/* The same for the kernel launches of the coupling handles and of the phases
+ * of a batched step: the next k succeed and the one after is left out, as if
+ * the runtime had refused it, so that its call returns CG_ERR_CUDA with the
+ * launches before it enqueued.  Nothing of such a call is left in the sums of
+ * the next one. */
+cg_status cg_debug_fail_launch_after(int64_t k);
+
 /* Change the stream later calls are enqueued on. */
 cg_status cg_set_stream(cg_grids* g, void* cuda_stream);
 

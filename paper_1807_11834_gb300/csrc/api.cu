@@ -17,16 +17,18 @@ bool finite3(const double* v) { return isfinite(v[0]) && isfinite(v[1]) && isfin
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// Host-side fault injection (cg_debug_fail_alloc_after): the number of
-// handle-owned allocations still allowed before one fails; -1 = none fails.
-std::atomic<long long> g_alloc_fail_after{-1};
+// Host-side fault injection (cg_debug_fail_alloc_after, cg_debug_fail_launch_after):
+// the number of handle-owned allocations, or launches, still allowed before one
+// fails; -1 = none fails.
+std::atomic<long long> g_alloc_fail_after{-1}, g_launch_fail_after{-1};
 
-bool injected_alloc_failure() {
-    long long k = g_alloc_fail_after.load();
+bool injected_failure(std::atomic<long long>& after) {
+    long long k = after.load(std::memory_order_relaxed);
     while (k >= 0)
-        if (g_alloc_fail_after.compare_exchange_weak(k, k - 1)) return k == 0;   // after the failure: -1
+        if (after.compare_exchange_weak(k, k - 1)) return k == 0;   // after the failure: -1
     return false;
 }
+bool injected_alloc_failure() { return injected_failure(g_alloc_fail_after); }
 
 template <typename P>
 cg_status dalloc(P** p, size_t bytes) {
@@ -103,6 +105,8 @@ static void prof_drain(cg_grids* g) {
     g->pending.clear();
     g->ev_used = 0;
 }
+
+bool injected_launch_failure() { return injected_failure(g_launch_fail_after); }
 
 void prof_begin(cg_grids* g, int slot, int* ev) {
     (void)slot;
@@ -204,7 +208,6 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     // stream has nothing of the caller's to wait for).
     CG_CUDA(cudaMemsetAsync(g->rb_small, 0, small, g->aux));
     CG_CUDA(cudaStreamSynchronize(g->aux));
-    g->rb_dirty = false;
     const long long cells_blk = (g->gd.nbulk + 1 + kScanItems - 1) / kScanItems;
     g->scan_cap = (g->hist_cap + kScanItems - 1) / kScanItems + cells_blk;
     CG_TRY(dalloc(&g->scan_part, sizeof(int32_t) * g->scan_cap));
@@ -381,13 +384,13 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     if (st == CG_OK) st = dalloc(&g->cell_start, sizeof(int32_t) * (nbulk + 1));
     if (st == CG_OK) st = dalloc(&g->bulk4, 4 * g->tsize * nbulk);
     if (st == CG_OK) st = dalloc(&g->eps_t, g->tsize * nbulk);
-    if (st == CG_OK) st = dalloc(&g->vol_acc, 3 * sizeof(unsigned long long) * nbulk);
+    if (st == CG_OK) st = dalloc(&g->vol_acc, vol_acc_bytes(nbulk));
     if (st == CG_OK) st = dalloc(&g->status, sizeof(unsigned long long) * kNumSlots);
     // zero before a step on any stream (cg_set_stream, a batch) adds to them:
     // ensure_particle_capacity below waits for this stream
     if (st == CG_OK && cudaStreamCreateWithFlags(&g->aux, cudaStreamNonBlocking) != cudaSuccess) st = CG_ERR_CUDA;
     if (st == CG_OK &&
-        (cudaMemsetAsync(g->vol_acc, 0, 3 * sizeof(unsigned long long) * nbulk, g->aux) != cudaSuccess ||
+        (clear_volumes(g, g->aux) != cudaSuccess ||
          cudaMemsetAsync(g->status, 0, sizeof(unsigned long long) * kNumSlots, g->aux) != cudaSuccess))
         st = CG_ERR_CUDA;
     cudaEvent_t* evs[] = {&g->ev_fork, &g->ev_avg, &g->ev_pack, &g->ev_epsf};
@@ -406,6 +409,12 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
 cg_status cg_debug_fail_alloc_after(int64_t k) {
     if (k < -1) return CG_ERR_INVALID_ARG;
     g_alloc_fail_after.store(k);
+    return CG_OK;
+}
+
+cg_status cg_debug_fail_launch_after(int64_t k) {
+    if (k < -1) return CG_ERR_INVALID_ARG;
+    g_launch_fail_after.store(k);
     return CG_OK;
 }
 

@@ -282,19 +282,26 @@ cg_status enqueue(cg_batch* b, double dt) {
     cudaStream_t s = b->stream;
     for (int ph = 0; ph < BP_COUNT; ++ph) {
         if (b->total[ph] == 0) continue;
-        switch (ph) {
+        cg_status st = injected_launch_failure() ? CG_ERR_CUDA : CG_OK;
+        if (st == CG_OK) switch (ph) {
             case BP_ZERO: case BP_DEPV: case BP_PACK: case BP_DEPM: case BP_SUMS:
-                CG_TRY(launch_batch_deposit(ph, L(ph), b->grid[ph], s));
+                st = launch_batch_deposit(ph, L(ph), b->grid[ph], s);
                 break;
             case BP_AVG: case BP_PROJ: case BP_PROJE:
-                CG_TRY(launch_batch_fine(ph, L(ph), b->grid[ph], s));
+                st = launch_batch_fine(ph, L(ph), b->grid[ph], s);
                 break;
             case BP_DRAG:
-                CG_TRY(launch_batch_drag(L(ph), b->grid[ph], (float)dt, s));
+                st = launch_batch_drag(L(ph), b->grid[ph], (float)dt, s);
                 break;
             default:
-                CG_TRY(launch_batch_bin(ph, L(ph), b->grid[ph], b->smem[ph], s));
+                st = launch_batch_bin(ph, L(ph), b->grid[ph], b->smem[ph], s);
                 break;
+        }
+        if (st != CG_OK) {
+            // the spheres of BP_DEPV that BP_PACK has not taken
+            for (cg_grids* g : b->h) clear_volumes(g, s);
+            cudaGetLastError();
+            return st;
         }
         b->launches++;
     }

@@ -200,7 +200,6 @@ struct cg_grids {
     int4* rb_mov = nullptr;        // [rb_nblk * kRebinTile] movers, each block of old slots its own part:
                                    // (id, new cell, next mover of that cell + 1, arrival rank)
     int32_t* rb_small = nullptr;   // per-cell and per-block counts, starts, list heads; counters (rebin_ptrs)
-    bool rb_dirty = false;         // a rebinning was not launched to its end: its counters are not zero
     long long rb_nblk = 0;
     int32_t* hist = nullptr;       // [2^digit * ntiles]
     int32_t* scan_part = nullptr;  // scan block partials
@@ -253,6 +252,7 @@ namespace cg {
 int prof_slot(cg_grids* g, const char* name);
 void prof_begin(cg_grids* g, int slot, int* ev);
 void prof_end(cg_grids* g, int slot, int ev);
+bool injected_launch_failure();   // cg_debug_fail_launch_after
 
 // Launch a kernel on the handle's stream, count it, time it when profiling,
 // and turn a launch error into CG_ERR_CUDA.
@@ -278,7 +278,8 @@ void prof_end(cg_grids* g, int slot, int ev);
         c_.stream = (g)->stream;                                                 \
         c_.attrs = a_;                                                           \
         c_.numAttrs = 1;                                                         \
-        cudaError_t e_ = cudaLaunchKernelEx(&c_, kernel, __VA_ARGS__);           \
+        cudaError_t e_ = cg::injected_launch_failure() ? cudaErrorLaunchFailure  \
+                                                       : cudaLaunchKernelEx(&c_, kernel, __VA_ARGS__); \
         (g)->launches++;                                                         \
         if (e_ == cudaSuccess) e_ = cudaGetLastError();                          \
         if ((g)->prof) cg::prof_end((g), slot_, ev_);                            \
@@ -1032,6 +1033,13 @@ struct EpsOut {
     T* eps_t;
     T* S;
 };
+
+// Accumulators of n_b cells, and zeroes into them on stream s: of a new handle,
+// and after a launch between the spheres and the cells' porosity failed.
+inline size_t vol_acc_bytes(long long nbulk) { return 3 * sizeof(unsigned long long) * nbulk; }
+inline cudaError_t clear_volumes(cg_grids* g, cudaStream_t s) {
+    return cudaMemsetAsync(g->vol_acc, 0, vol_acc_bytes(g->gd.nbulk), s);
+}
 
 // The accumulators of the handle with a step's (or no) outputs.
 template <typename T>

@@ -330,7 +330,7 @@ static unsigned seg_blocks(cg_grids* g, long long n, int per_sm = 4) {
 }
 
 template <typename T>
-static cg_status deposit_volume_impl(cg_grids* g, long long n, const T* pos_d, StepEps* e) {
+static cg_status deposit_volume_launches(cg_grids* g, long long n, const T* pos_d, StepEps* e) {
     const EpsOut<T> o = eps_out<T>(g, e);
     if (n > 0) {
         const unsigned nblk = (unsigned)std::min<long long>((n + 1023) / 1024, (long long)g->num_sms * 8);
@@ -353,8 +353,13 @@ static cg_status deposit_volume_impl(cg_grids* g, long long n, const T* pos_d, S
 }
 
 cg_status launch_deposit_volume(cg_grids* g, long long n, const void* pos_d, StepEps* e) {
-    return g->fp64 ? deposit_volume_impl<double>(g, n, (const double*)pos_d, e)
-                   : deposit_volume_impl<float>(g, n, (const float*)pos_d, e);
+    const cg_status st = g->fp64 ? deposit_volume_launches<double>(g, n, (const double*)pos_d, e)
+                                 : deposit_volume_launches<float>(g, n, (const float*)pos_d, e);
+    if (st != CG_OK) {
+        clear_volumes(g, g->stream);
+        cudaGetLastError();
+    }
+    return st;
 }
 
 cg_status launch_deposit_sorted_force(cg_grids* g, long long n, void* S_bulk, bool cleared) {

@@ -504,16 +504,11 @@ k_rebin_slots(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn, 
 }
 
 template <typename T>
-static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, StepEps* eps) {
+static cg_status rebin_launches(cg_grids* g, long long n, const T* pos, bool ident, StepEps* eps) {
     const long long nbulk = g->gd.nbulk;
     const RebinPtrs R = rebin_ptrs(g);
     const long long nblk = (n + kRebinTile - 1) / kRebinTile;
-    if (nblk > g->rb_nblk) return CG_ERR_OUT_OF_RANGE;
     const EpsOut<T> eo = eps_out<T>(g, eps);
-    // the last kernel clears what the next rebinning counts in (a clear of its own
-    // at the head of the chain costs 2 to 3 us)
-    if (g->rb_dirty) CG_CUDA(cudaMemsetAsync(R.arr, 0, R.zero_bytes, g->stream));
-    g->rb_dirty = true;
     // the caller's order: resident CTAs that walk the blocks of old slots, the
     // next block's ids and cells loaded ahead of the gather they lead to
     const long long walk = (long long)g->num_sms * (sizeof(T) == 4 ? 4 : 3);
@@ -565,8 +560,23 @@ static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, 
     const long long nb1 = rebin_pad(nbulk + 1);
     CG_TRY(launch_cellsort_fallback(g, R.cnt, R.ctr, g->cell_start, ident ? nullptr : g->inv_perm,
                                     {(int4*)R.arr, 3 * nb1 / 4, R.part, 2 * tiles + btiles}));
-    g->rb_dirty = false;
     return CG_OK;
+}
+
+// The last kernel clears what the next rebinning counts in (a clear of its own
+// at the head of the chain costs 2 to 3 us); a launch that fails before it leaves
+// that to this, with the volumes that no pass over the cells has taken.
+template <typename T>
+static cg_status rebin_impl(cg_grids* g, long long n, const T* pos, bool ident, StepEps* eps) {
+    if ((n + kRebinTile - 1) / kRebinTile > g->rb_nblk) return CG_ERR_OUT_OF_RANGE;
+    const cg_status st = rebin_launches<T>(g, n, pos, ident, eps);
+    if (st == CG_OK) return CG_OK;
+    const RebinPtrs R = rebin_ptrs(g);
+    cudaMemsetAsync(R.arr, 0, R.zero_bytes, g->stream);
+    cudaMemsetAsync(R.ctr + RB_INV_STALE, 0xff, sizeof(int32_t), g->stream);
+    if (eps) clear_volumes(g, g->stream);
+    cudaGetLastError();
+    return st;
 }
 
 // Caller-order cells of the binning's slots.

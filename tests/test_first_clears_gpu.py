@@ -1,5 +1,6 @@
-"""What a new handle counts in is zero before its first step, on whatever
-stream that runs, and making a handle waits for none of the caller's work."""
+"""What a handle counts in is zero before a step: the first one, on whatever
+stream that runs, and one after a step that failed halfway.  Making a handle
+waits for none of the caller's work."""
 import pytest
 
 import synth
@@ -62,3 +63,61 @@ def test_first_steps_on_another_stream(cuda_lib, fp64):
             assert torch.equal(got[name], ref[name]), (k, name)
     assert g.cg_sync_status()[:2] == (0, 0)
     g.close()
+
+
+NAMES = ("eps_bulk", "u_bulk", "var_bulk", "force", "S_bulk", "S_fine", "eps_fine", "sums")
+
+
+@pytest.mark.parametrize("form", ["scratch", "incremental", "sorted", "batch"])
+def test_a_step_after_one_whose_launch_failed(cuda_lib, form):
+    """Each launch of a step is left out in turn (on the host): the step says
+    so, and the next one is a fresh handle's bit for bit."""
+    import torch
+    cg = cuda_lib
+    w = synth.tiny(seed=5, n=20_000, fp64=False)
+    pos, vel, uf = inputs(w)
+
+    def fresh():
+        if form == "batch":
+            f = cg.Grids(w.desc)
+            out = f.alloc_outputs(w.n, eps_fine=True)
+            f.close()
+            h = cg.Batch([(w.desc, pos, vel, uf, out)])
+            return h, out, [h.step]
+        h = cg.Grids(w.desc)
+        out = h.alloc_outputs(w.n, eps_fine=True)
+        if form == "sorted":
+            ab = pos.clone(), vel.clone(), torch.empty_like(pos), torch.empty_like(vel)
+            return h, out, [lambda: h.cg_step_sorted(*ab, uf, out), lambda: h.cg_step_sorted(ab[2], ab[3], ab[0], ab[1], uf, out)]
+        return h, out, [lambda: h.cg_step(pos, vel, uf, out)] * (2 if form == "incremental" else 1)
+
+    h, out, calls = fresh()
+    for c in calls:
+        c()
+    torch.cuda.synchronize()
+    want = {k: out[k].clone() for k in NAMES}
+    h.close()
+    try:
+        failed = 0
+        while True:
+            h, out, calls = fresh()
+            for c in calls[:-1]:
+                c()
+            assert cg.lib().cg_debug_fail_launch_after(failed) == 0
+            try:
+                calls[-1]()
+            except cg.CgError as e:
+                assert e.code == 2
+            else:
+                break
+            calls[-1]()
+            torch.cuda.synchronize()
+            for k in NAMES:
+                assert torch.equal(out[k], want[k]), (failed, k)
+            h.close()
+            failed += 1
+            assert failed < 60
+        assert failed >= 8
+        h.close()
+    finally:
+        cg.lib().cg_debug_fail_launch_after(-1)
