@@ -365,9 +365,8 @@ cg_status cg_create_grids(const cg_grid_desc* desc, void* cuda_stream, cg_grids*
     gd.Vff = (float)gd.Vf;
     split_ff(gd.VB, gd.VBh, gd.VBl);
     split_ff(gd.Vf, gd.Vfh, gd.Vfl);
-    const double vc = 0.52359877559829887308 * gd.invVB;
-    split_ff(vc, gd.vch, gd.vcl);
-    gd.vcd57 = ldexp(vc, 57);
+    gd.vcd = 0.52359877559829887308 * gd.invVB;
+    split_ff(gd.vcd, gd.vch, gd.vcl);
     gd.law = d.law;
     gd.interp = d.interp;
     gd.rho_f = d.rho_f;

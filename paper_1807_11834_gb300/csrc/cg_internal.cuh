@@ -119,7 +119,7 @@ struct GridDev {
     float invHf[3];     // (float)(1/H)
     float binh[3];      // 1/2 - 2^-21 |x0 / H| - 2^-24: how near a cell's middle the float bin rule decides (bin_axis_fast)
     float vch, vcl;     // pi / (6 V_B) as float-float: a sphere's volume over V_B is this times d^3
-    double vcd57;       // 2^57 pi / (6 V_B)
+    double vcd;         // pi / (6 V_B)
     float x0h[3], x0l[3];   // x0 as float-float
     float ihh[3], ihl[3];   // 1/H as float-float
     float xbh[3], xbl[3];   // -(x0 / H + 1/2) as float-float: the lattice coordinate is x / H + xb
@@ -209,7 +209,7 @@ struct cg_grids {
     int32_t* cell_start = nullptr; // [nbulk + 1]
     void* bulk4 = nullptr;         // [nbulk] T4: eps, u_x, u_y, u_z
     void* eps_t = nullptr;         // [nbulk] T: porosity in the path precision
-    unsigned long long* vol_acc = nullptr;   // [nbulk][2] volume accumulators, then [nbulk] double (see EpsOut)
+    unsigned long long* vol_acc = nullptr;   // [5 nbulk] volume accumulators (see volume_add_row)
     void* partials = nullptr;      // conservation-sum block partials: (s, c) pairs of T
     long long part_off[cg::PS_NREG] = {0, 0, 0};
     long long part_blocks[cg::PS_NREG] = {0, 0, 0};
@@ -342,7 +342,7 @@ constexpr int kRebinItems = 4;
 constexpr int kRebinTile = kRebinThreads * kRebinItems;   // old slots per block
 constexpr int kRebinScan = 1024;                           // elements per block of its scans
 constexpr int kRebinMaxArrivals = 32;                      // arrivals per cell before the fallback
-constexpr long long kRebinMaxParticles = 1LL << 30;        // the porosity accumulators' limit (a longer list is sorted)
+constexpr long long kRebinMaxParticles = 1LL << 30;        // the marking kernel's 32-bit slots (a longer list is sorted)
 constexpr int kRebinCounters = 8;
 // The small rebinning arrays each start on a 256-byte boundary (the scan reads
 // them as int4): the counts (n_b + 1), the departures per block (nblk + 1), the
@@ -913,111 +913,226 @@ __device__ __forceinline__ void reaction_emit(const GridDev& g, T* __restrict__ 
 // ----------------------------------------------------------------------
 // Porosity (Table 1: sum of the particle volumes of a cell over V_B).
 //
-// Each sphere's volume over V_B is rounded once to a multiple of 2^-57 and the
+// Each sphere's volume over V_B is rounded once to a multiple of 2^-84 and the
 // cells add whole numbers, so the sum is exact and the same in any order:
-// particles can be added where their cell is first known, with one pair of
+// particles can be added where their cell is first known, with one set of
 // atomics per run of equal cells in a warp, and every path (binning from
-// scratch, incremental, batched) gives the same bits.  A cell's accumulator
-// is two 64-bit words: the multiples of 2^-30 in acc[2 c + 1], what is left,
-// below 2^-30 per particle, in acc[2 c] (so neither can overflow for 2^30
-// particles), and, for spheres of 2^32 V_B and more and for non-finite ones,
-// a double in big[c], marked by bit 62 of acc[2 c].  The accumulators are
-// zero between steps: whoever forms the porosity of a cell clears them.
+// scratch, incremental, batched) gives the same bits.
+//
+// A volume is cut into 27-bit pieces: w[0] the multiples of 2^-57 below 2^-30,
+// w[1] the multiples of 2^-30, w[2] those of 2^-84 below 2^-57.  The last one
+// keeps small spheres as exact as large ones (their sums against the sums of
+// their volumes: with 2^-57 alone a sphere of 0.001 H was off by up to 6e-9,
+// and spheres below 2e-6 H were not deposited).  FP32 volumes have 46 bits, so
+// they do without from 2^-12 of a cell (0.08 H) on, and rows of such spheres skip
+// it; FP64 volumes have 53 and nearly always fill it.
+//
+// A cell's accumulator: acc[2 c] the sum of the w[0], acc[2 c + 1] of the w[1],
+// acc[2 n_b + c] of the w[2].  Spheres of 2 V_B and more also add the multiples
+// of 2 V_B to acc[3 n_b + c], those of 2^32 V_B and more, and non-finite ones, go
+// into a double at acc[4 n_b + c]; bit 62 of acc[2 c] marks either, and, in FP32,
+// bit 61 the third pieces (most cells have none and save the read).  Each sphere
+// adds less than 2^31 to a word, so 2^31 spheres do not overflow one.  The
+// accumulators are zero between steps: whoever forms the porosity of a cell
+// clears them.
 // ----------------------------------------------------------------------
-// 2^57 pi d^3 / (6 V_B) rounded; false when it is not in [0, 2^57) (the slow
-// path's).  FP32: the product as a pair by FMA (relative error about 2^-46);
-// its upper part is cut into the integer with shifts, since the conversions
-// to 64-bit integers issue on the FP64 pipe at 1/64 of the FP32 rate (two of
-// them per row of 32 particles took over half of the marking kernel's time).
-__device__ __forceinline__ bool sphere_fraction57(float d, const GridDev& g, long long& t) {
+constexpr unsigned kVolMask = (1u << 27) - 1u;
+constexpr unsigned long long kVolMark = 1ULL << 62, kVolThird = 1ULL << 61;
+
+// The pieces of m 2^(s - 84), m below 2^53 and the result below 1, rounded.
+__device__ __forceinline__ void volume_pieces(unsigned long long m, int s, unsigned (&w)[3]) {
+    if (s < 0) {   // below 2^-31
+        m = s > -64 ? (m + (1ULL << (-s - 1))) >> -s : 0ULL;
+        s = 0;
+    }
+    const unsigned long long low = m << s;
+    w[2] = (unsigned)low & kVolMask;
+    w[0] = (unsigned)(low >> 27) & kVolMask;
+    w[1] = (unsigned)(m >> (54 - s));
+}
+
+// Pieces of pi d^3 / (6 V_B); false when it is not in [0, 1) (the slow path's).
+// FP32: the product as a pair hi + lo by FMA (relative error about 2^-46), put
+// into one integer with shifts: the conversions to 64-bit integers issue on the
+// FP64 pipe at 1/64 of the FP32 rate (two of them per row of 32 particles took
+// over half of the marking kernel's time).
+__device__ __forceinline__ void sphere_pair(float d, const GridDev& g, float& hi, float& lo) {
     const float p = __fmul_rn(d, d), pe = __fmaf_rn(d, d, -p);   // d^2 = p + pe exactly
     const float q = __fmul_rn(p, d), qe = __fmaf_rn(p, d, -q);   // p d = q + qe exactly
     const float r = __fmaf_rn(pe, d, qe);                        // d^3 = q + r (to 2^-48)
-    const float hi = __fmul_rn(g.vch, q);
-    const float lo = __fmaf_rn(g.vch, r, __fmaf_rn(g.vcl, q, __fmaf_rn(g.vch, q, -hi)));
-    // hi = m 2^(E - 150) with a 24-bit m: 2^57 hi = m 2^(E - 93), E <= 126 below 1 (smaller than 2^-57: 0);
-    // lo is below 2^-24 hi and rounded to 2^-54
+    hi = __fmul_rn(g.vch, q);
+    lo = __fmaf_rn(g.vch, r, __fmaf_rn(g.vcl, q, __fmaf_rn(g.vch, q, -hi)));
+}
+// The pair, hi = m 2^(E - 150) with a 24-bit m and lo below 2^-22 hi, as an
+// integer of 46 bits in units of 2^(E - 172).
+__device__ __forceinline__ unsigned long long sphere_int(float hi, float lo, float unit) {
+    const unsigned m = (__float_as_uint(hi) & 0x7fffffu) | 0x800000u;
+    return ((unsigned long long)m << 22) + (long long)__float2int_rn(__fmul_rn(lo, unit));
+}
+// Plain spheres, from 2^-12 of a cell (0.08 H) to 1/8: multiples of 2^-57, so the
+// third piece is zero.
+__device__ __forceinline__ bool sphere_plain(float hi) {
+    return __float_as_uint(hi) - (115u << 23) < (9u << 23);
+}
+__device__ __forceinline__ void sphere_pieces_plain(float hi, float lo, unsigned& w0, unsigned& w1) {
+    const unsigned e = __float_as_uint(hi) & 0x7f800000u;
+    const unsigned long long t = sphere_int(hi, lo, __uint_as_float((299u << 23) - e)) << ((e >> 23) - 115u & 63u);
+    w0 = (unsigned)t & kVolMask;
+    w1 = (unsigned)(t >> 27);
+}
+// Any other (2^(172 - E) is a float down to E = 45, a volume of 2^-82).
+__device__ __forceinline__ bool sphere_pieces_other(float hi, float lo, unsigned (&w)[3]) {
     const unsigned u = __float_as_uint(hi);
     const int E = (int)(u >> 23);
-    const unsigned long long m = (unsigned long long)((u & 0x7fffffu) | 0x800000u) << 33;
-    t = (long long)(E > 63 ? m >> ((126 - E) & 63) : 0ull) + ((long long)__float2int_rn(lo * 18014398509481984.0f) << 3);
-    return u < 0x3f800000u;   // 0 <= hi < 1, not NaN
+    const bool in = u < 0x3f800000u;   // 0 <= hi < 1, not NaN
+    volume_pieces(sphere_int(hi, lo, __uint_as_float(E >= 45 ? (unsigned)(299 - E) << 23 : 0u)), in ? E - 88 : -64, w);
+    return in;
 }
-__device__ __forceinline__ bool sphere_fraction57(double d, const GridDev& g, long long& t) {
-    const double v = __dmul_rn(__dmul_rn(__dmul_rn(g.vcd57, d), d), d);
-    t = __double2ll_rn(v);
-    return (unsigned)__double2hiint(v) < 0x43800000u;   // 0 <= v < 2^57, compared as integers
+__device__ __forceinline__ bool sphere_pieces(double d, const GridDev& g, unsigned (&w)[3]) {
+    const double v = __dmul_rn(__dmul_rn(__dmul_rn(g.vcd, d), d), d);   // m 2^(E - 1075)
+    const unsigned hi = (unsigned)__double2hiint(v);
+    const bool in = hi < 0x3ff00000u;   // 0 <= v < 1, compared as integers
+    const unsigned long long m = (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(v);
+    volume_pieces(m, in ? (int)(hi >> 20) - 991 : -64, w);
+    return in;
 }
 
 // One sphere outside that range: a large one, or a diameter that is negative
 // or not finite.
-static __device__ __noinline__ void volume_add_slow(double d, int cell, double vcd57, unsigned long long* __restrict__ acc,
-                                                    double* __restrict__ big) {
-    const double t = vcd57 * 6.938893903907228e-18 * d * d * d;   // 2^-57
+__device__ __forceinline__ void volume_add_third(unsigned long long w2, int cell, long long nbulk, bool fp32,
+                                                 unsigned long long* __restrict__ acc) {
+    atomicAdd(acc + 2 * nbulk + cell, w2);
+    if (fp32) atomicOr(acc + 2 * (size_t)cell, kVolThird);
+}
+static __device__ __noinline__ void volume_add_slow(double d, int cell, const double vcd, long long nbulk,
+                                                    unsigned long long* __restrict__ acc) {
+    const double t = vcd * d * d * d;
     if (fabs(t) < 4294967296.0) {
-        const double x = t * 1073741824.0, f = floor(x);
-        atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)__double2ull_rn((x - f) * 134217728.0));
-        atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)(long long)f);
+        const double x = t * 1073741824.0, f = floor(x);                        // 2^30
+        const double y = (x - f) * 134217728.0, e = floor(y);                   // 2^27
+        const long long h = (long long)f;
+        atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)e);
+        atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)(h & 0x7fffffffLL));
+        volume_add_third(__double2ull_rn((y - e) * 134217728.0), cell, nbulk, true, acc);
+        if (h >> 31) {
+            atomicAdd(acc + 3 * nbulk + cell, (unsigned long long)(h >> 31));
+            atomicOr(acc + 2 * (size_t)cell, kVolMark);
+        }
     } else {
-        atomicAdd(big + cell, isfinite(t) ? t : __longlong_as_double(0x7ff8000000000000LL));
-        atomicOr(acc + 2 * (size_t)cell, 1ULL << 62);
+        atomicAdd((double*)(acc + 4 * nbulk) + cell, isfinite(t) ? t : __longlong_as_double(0x7ff8000000000000LL));
+        atomicOr(acc + 2 * (size_t)cell, kVolMark);
     }
 }
 
-// Add 32 spheres, one per lane (valid lanes), to their cells: equal cells on
-// consecutive lanes are summed first.  One or two runs by warp reductions,
-// more by a segmented scan (two 27-bit pieces, which cannot overflow 32 bits
-// over 32 lanes).  Called by the whole warp.
-template <typename T>
-__device__ __forceinline__ void volume_add_row(bool valid, int cell, T d, const GridDev& g,
-                                               unsigned long long* __restrict__ acc, double* __restrict__ big) {
+// The first lanes of the runs of equal cells among a row's valid lanes.
+__device__ __forceinline__ unsigned run_heads(bool valid, int cell) {
+    const int c = valid ? cell : -1;
+    const int prev = __shfl_up_sync(0xffffffffu, c, 1);
+    return __ballot_sync(0xffffffffu, (threadIdx.x & 31) == 0 || prev != c);
+}
+// Sums of N values (of at most 27 bits, which cannot overflow 32 bits over 32
+// lanes) over the runs that begin at the lanes `heads`: one or two runs by
+// warp reductions, more by a segmented scan.  True on the lane that holds its
+// run's sums.
+template <int N>
+__device__ __forceinline__ bool volume_runs(unsigned* w, unsigned heads) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    long long t = 0;
-    const bool fast = sphere_fraction57(d, g, t);
-    unsigned w0 = (unsigned)t & 0x7ffffffu, w1 = (unsigned)(t >> 27);
-    const bool use = valid && fast && w1 < (1u << 27);   // below 1/8
-    if (valid && !use) {
-        if (fast) {
-            atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)w0);
-            atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)w1);
-        } else {
-            volume_add_slow((double)d, cell, g.vcd57, acc, big);
-        }
-    }
-    if (!use) w0 = w1 = 0u;
-    const int c = valid ? cell : -1;
-    const int prev = __shfl_up_sync(full, c, 1);
-    const unsigned heads = __ballot_sync(full, lane == 0 || prev != c);
-    bool owner;
     if (__popc(heads) <= 2) {
         const unsigned later = heads & ~1u;
         const bool first = lane < (later ? __ffs(later) - 1 : 32);   // of the first run, or of the second
-        const unsigned a0 = __reduce_add_sync(full, first ? w0 : 0u), a1 = __reduce_add_sync(full, first ? w1 : 0u);
-        if (later) {
-            w0 = __reduce_add_sync(full, first ? 0u : w0);
-            w1 = __reduce_add_sync(full, first ? 0u : w1);
-        }
-        if (first) {
-            w0 = a0;
-            w1 = a1;
-        }
-        owner = heads >> lane & 1u;
-    } else {
-        const int head = 31 - __clz(heads & ((2u << lane) - 1u));
+        unsigned a[N];
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned x0 = __shfl_up_sync(full, w0, off), x1 = __shfl_up_sync(full, w1, off);
-            if (lane - off >= head) {
-                w0 += x0;
-                w1 += x1;
-            }
-        }
-        owner = lane == 31 || (heads >> (lane + 1) & 1u);
+        for (int k = 0; k < N; ++k) a[k] = __reduce_add_sync(full, first ? w[k] : 0u);
+        if (later)
+#pragma unroll
+            for (int k = 0; k < N; ++k) w[k] = __reduce_add_sync(full, first ? 0u : w[k]);
+        if (first)
+#pragma unroll
+            for (int k = 0; k < N; ++k) w[k] = a[k];
+        return heads >> lane & 1u;
     }
-    if (owner && valid) {
-        atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)w0);
-        atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)w1);
+    const int head = 31 - __clz(heads & ((2u << lane) - 1u));
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        unsigned x[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) x[k] = __shfl_up_sync(full, w[k], off);
+        if (lane - off >= head)
+#pragma unroll
+            for (int k = 0; k < N; ++k) w[k] += x[k];
+    }
+    return lane == 31 || (heads >> (lane + 1) & 1u);
+}
+__device__ __forceinline__ void volume_atomics(unsigned w0, unsigned w1, int cell, unsigned long long* __restrict__ acc) {
+    atomicAdd(acc + 2 * (size_t)cell, (unsigned long long)w0);
+    atomicAdd(acc + 2 * (size_t)cell + 1, (unsigned long long)w1);
+}
+// A sphere that is not to go into its run's sums: one of 1/8 of a cell or more
+// (its pieces w, when it is in their range).
+__device__ __forceinline__ bool volume_alone(bool in, const unsigned (&w)[3], double d, int cell, double vcd, long long nbulk,
+                                             bool fp32, unsigned long long* __restrict__ acc) {
+    if (in && w[1] <= kVolMask) return false;
+    if (in) {
+        volume_atomics(w[0], w[1], cell, acc);
+        if (w[2]) volume_add_third(w[2], cell, nbulk, fp32, acc);
+    } else {
+        volume_add_slow(d, cell, vcd, nbulk, acc);
+    }
+    return true;
+}
+
+// FP32 rows with spheres that are not plain: the first two pieces of such a lane
+// for its run's sums (the second in the upper half; zero for one added alone);
+// the third pieces of up to four lanes go to their cells by themselves, those of
+// more through sums of their own.  Out of line, so that the marking kernel's
+// registers are those of the plain rows.  (32M log-normal spheres, of whose rows
+// 7% hold another sphere: 207 us; with the whole row in three pieces then 223,
+// with every such sphere added alone 230.  700,001 spheres of 0.08 H, some below
+// 2^-12: 16 us; as rows of other spheres 18.7.)
+static __device__ __noinline__ unsigned long long volume_other(bool other, int cell, float hi, float lo, float d, double vcd,
+                                                               long long nbulk, unsigned heads,
+                                                               unsigned long long* __restrict__ acc) {
+    unsigned w[3] = {0u, 0u, 0u};
+    if (other) {
+        const bool in = sphere_pieces_other(hi, lo, w);
+        if (volume_alone(in, w, (double)d, cell, vcd, nbulk, true, acc)) w[0] = w[1] = w[2] = 0u;
+    }
+    unsigned third = w[2];
+    const int lanes = __popc(__ballot_sync(0xffffffffu, third != 0u));
+    const bool sum = lanes <= 4 || volume_runs<1>(&third, heads);
+    if (sum && third) volume_add_third(third, cell, nbulk, true, acc);
+    return (unsigned long long)w[1] << 32 | w[0];
+}
+
+// Add 32 spheres, one per lane (valid lanes), to their cells: equal cells on
+// consecutive lanes are summed first.  Called by the whole warp.
+__device__ __forceinline__ void volume_add_row(bool valid, int cell, float d, const GridDev& g,
+                                               unsigned long long* __restrict__ acc) {
+    const unsigned heads = run_heads(valid, cell);
+    float hi, lo;
+    sphere_pair(d, g, hi, lo);
+    unsigned w[2];
+    sphere_pieces_plain(hi, lo, w[0], w[1]);
+    if (!valid) w[0] = w[1] = 0u;
+    const bool other = valid && !sphere_plain(hi);
+    if (__any_sync(0xffffffffu, other)) {
+        const unsigned long long o = volume_other(other, cell, hi, lo, d, g.vcd, g.nbulk, heads, acc);
+        if (other) {
+            w[0] = (unsigned)o;
+            w[1] = (unsigned)(o >> 32);
+        }
+    }
+    if (volume_runs<2>(w, heads) && valid) volume_atomics(w[0], w[1], cell, acc);
+}
+__device__ __forceinline__ void volume_add_row(bool valid, int cell, double d, const GridDev& g,
+                                               unsigned long long* __restrict__ acc) {
+    unsigned w[3];
+    const bool in = sphere_pieces(d, g, w);
+    if (!valid || volume_alone(in, w, d, cell, g.vcd, g.nbulk, false, acc)) w[0] = w[1] = w[2] = 0u;
+    if (volume_runs<3>(w, run_heads(valid, cell)) && valid) {
+        volume_atomics(w[0], w[1], cell, acc);
+        if (w[2]) volume_add_third(w[2], cell, g.nbulk, false, acc);
     }
 }
 
@@ -1027,7 +1142,6 @@ __device__ __forceinline__ void volume_add_row(bool valid, int cell, T d, const 
 template <typename T>
 struct EpsOut {
     unsigned long long* acc;
-    double* big;
     double* eps;
     T* rec;
     T* eps_t;
@@ -1036,7 +1150,7 @@ struct EpsOut {
 
 // Accumulators of n_b cells, and zeroes into them on stream s: of a new handle,
 // and after a launch between the spheres and the cells' porosity failed.
-inline size_t vol_acc_bytes(long long nbulk) { return 3 * sizeof(unsigned long long) * nbulk; }
+inline size_t vol_acc_bytes(long long nbulk) { return 5 * sizeof(unsigned long long) * nbulk; }
 inline cudaError_t clear_volumes(cg_grids* g, cudaStream_t s) {
     return cudaMemsetAsync(g->vol_acc, 0, vol_acc_bytes(g->gd.nbulk), s);
 }
@@ -1044,7 +1158,7 @@ inline cudaError_t clear_volumes(cg_grids* g, cudaStream_t s) {
 // The accumulators of the handle with a step's (or no) outputs.
 template <typename T>
 inline EpsOut<T> eps_out(cg_grids* g, const StepEps* e) {
-    return {g->vol_acc, (double*)(g->vol_acc + 2 * g->gd.nbulk), e ? e->eps : nullptr, e ? (T*)e->rec : nullptr,
+    return {g->vol_acc, e ? e->eps : nullptr, e ? (T*)e->rec : nullptr,
             e ? (T*)e->eps_t : nullptr, e ? (T*)e->S : nullptr};
 }
 
@@ -1052,17 +1166,34 @@ __device__ __forceinline__ void eps_round(long long e57, double, float& et) {
     et = __ll2float_rn(e57) * 6.938893903907228e-18f;
 }
 __device__ __forceinline__ void eps_round(long long, double e, double& et) { et = e; }
-__device__ __forceinline__ void deposited_volume(long long p57, const GridDev& g, CSum<float>& tot) {
+// A cell's volume (p57 2^-57 + r 2^-84) V_B into a sum.  FP32: a pair of 48 bits.
+__device__ __forceinline__ void deposited_volume(long long p57, unsigned r, const GridDev& g, CSum<float>& tot) {
     const float ph = __ll2float_rn(p57);
-    const float pl = __ll2float_rn(p57 - __float2ll_rn(ph)) * 6.938893903907228e-18f;
+    const float pl = __ll2float_rn((p57 - __float2ll_rn(ph)) * (1LL << 27) + r) * 5.1698788284564230e-26f;   // 2^-84
     const float p = ph * 6.938893903907228e-18f;
     const float hi = p * g.VBh;
     const float lo = fmaf(pl, g.VBh, fmaf(p, g.VBl, fmaf(p, g.VBh, -hi)));
     tot.add(hi);
     tot.c += lo;
 }
-__device__ __forceinline__ void deposited_volume(long long p57, const GridDev& g, CSum<double>& tot) {
-    tot.add((double)p57 * 6.938893903907228e-18 * g.VB);
+__device__ __forceinline__ void deposited_volume(long long p57, unsigned r, const GridDev& g, CSum<double>& tot) {
+    tot.add(fma((double)r, 5.1698788284564230e-26, (double)p57 * 6.938893903907228e-18) * g.VB);
+}
+
+// The volume (over V_B) of a cell beyond the ordinary range, or with a marked
+// accumulator (out of line: such cells are rare).
+static __device__ __noinline__ double volume_far(long long h, unsigned l, unsigned r, bool marked, unsigned long long* fine,
+                                                 long long nbulk) {
+    double phi = (double)h * 9.313225746154785e-10 +
+                 ((double)l * 6.938893903907228e-18 + (double)r * 5.1698788284564230e-26);   // 2^-30, 2^-57, 2^-84
+    if (marked) {
+        long long* const top = (long long*)fine + nbulk;
+        double* const big = (double*)fine + 2 * nbulk;
+        phi += 2.0 * (double)*top + *big;
+        *top = 0;
+        *big = 0.0;
+    }
+    return phi;
 }
 
 // The porosity of one cell from its accumulator, which is cleared; its
@@ -1070,24 +1201,25 @@ __device__ __forceinline__ void deposited_volume(long long p57, const GridDev& g
 template <typename T, bool SUMS>
 __device__ __forceinline__ void eps_finish(long long c, const GridDev& g, const EpsOut<T>& o, CSum<T>& tot) {
     const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(o.acc + 2 * c);
+    unsigned long long* const fine = o.acc + 2 * g.nbulk + c;
+    const unsigned long long b = sizeof(T) == 8 || (a.x & kVolThird) ? *fine : 0ULL;
     double e = 1.0;
     T et = T(1);
-    if (a.x | a.y) {
+    if (a.x | a.y | b) {
         *reinterpret_cast<ulonglong2*>(o.acc + 2 * c) = make_ulonglong2(0, 0);
-        const unsigned long long low = a.x & ~(1ULL << 62);
+        if (b) *fine = 0;
+        const bool marked = a.x & kVolMark;
+        const unsigned long long low = (a.x & ~(kVolMark | kVolThird)) + (b >> 27);
         const long long h = (long long)a.y + (long long)(low >> 27);
-        const unsigned l = (unsigned)low & 0x7ffffffu;
-        if (low == a.x && h >= 0 && h < (1LL << 33)) {
-            const long long p57 = (h << 27) | l, e57 = (1LL << 57) - p57;   // 1 - sum, exactly
+        const unsigned l = (unsigned)low & kVolMask, r = (unsigned)b & kVolMask;
+        if (!marked && h >= 0 && h < (1LL << 33)) {
+            const long long p57 = (h << 27) | l;
+            const long long e57 = (1LL << 57) - p57 - (r >> 26);   // 1 - sum, to 2^-58
             e = __ll2double_rn(e57) * 6.938893903907228e-18;
             eps_round(e57, e, et);
-            if (SUMS) deposited_volume(p57, g, tot);
+            if (SUMS) deposited_volume(p57, r, g, tot);
         } else {
-            double phi = (double)h * 9.313225746154785e-10 + (double)l * 6.938893903907228e-18;   // 2^-30, 2^-57
-            if (low != a.x) {
-                phi += o.big[c];
-                o.big[c] = 0.0;
-            }
+            const double phi = volume_far(h, l, r, marked, fine, g.nbulk);
             e = 1.0 - phi;
             et = (T)e;
             if (SUMS) tot.add((T)(phi * g.VB));

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kRebinThreads, sizeof(T) == 4 ? (IDENT ? 5 : 4
 k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restrict__ perm_old,
              const int32_t* __restrict__ ks_old, int32_t* __restrict__ rid, int32_t* __restrict__ rkn,
              int2* __restrict__ arr, int32_t* __restrict__ dep, int4* __restrict__ mov, int32_t* __restrict__ blk_dep, int32_t* __restrict__ ctr,
-             unsigned long long* __restrict__ status, unsigned long long* __restrict__ acc, double* __restrict__ big) {
+             unsigned long long* __restrict__ status, unsigned long long* __restrict__ acc) {
     pdl_wait();
     constexpr int W = kRebinThreads / 32;
     __shared__ int s_cnt[W];
@@ -152,7 +152,7 @@ k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restr
                 rkn[s] = moved ? ~cn[k] : cn[k];
                 if (!IDENT) rid[s] = id[k];
             }
-            if (VOL) volume_add_row<T>(valid, cn[k], pv[k].w, g, acc, big);
+            if (VOL) volume_add_row(valid, cn[k], pv[k].w, g, acc);
         }
         if (lane == 0) s_cnt[warp] = wc;
         __syncthreads();
@@ -197,9 +197,10 @@ k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restr
 // starts are the old ones, written in their scanned form, and the scans are
 // left out.  A cell per thread (cell_items): the chain of one cell's loads and of its few
 // FP64 operations bounds small grids (16,384 cells, four per thread 9.3 -> 4.9
-// us; 1M cells 25 -> 21).
+// us; 1M cells 25 -> 21).  FP32: five CTAs per SM (48 registers; at 56, four: 27
+// -> 31 us in the step of 32M particles).
 template <typename T, bool EPS, bool SUMS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4)
 k_rebin_cells(const int32_t* __restrict__ cs_old, GridDev g, const int32_t* __restrict__ dep,
               const int2* __restrict__ arr, int32_t* __restrict__ cnt, const int32_t* __restrict__ blk, long long nblk,
               const int32_t* __restrict__ ctr, int32_t* __restrict__ part, long long tiles, long long cblk,
@@ -515,7 +516,7 @@ static cg_status rebin_launches(cg_grids* g, long long n, const T* pos, bool ide
 #define CG_REBIN_MARK(ID, VOL)                                                                                     \
     CG_LAUNCH(g, "rebin_mark", (k_rebin_mark<T, ID, VOL>), (unsigned)(ID ? nblk : std::min(nblk, walk)), kRebinThreads, 0, pos, (int)n, g->gd,    \
               (const int32_t*)g->perm, (const int32_t*)g->key_sorted, g->rb_rid, g->rb_rkn, R.arr, R.dep,           \
-              g->rb_mov, R.blk, R.ctr, g->status, eo.acc, eo.big)
+              g->rb_mov, R.blk, R.ctr, g->status, eo.acc)
     if (ident) {
         if (eps) CG_REBIN_MARK(true, true);
         else CG_REBIN_MARK(true, false);
