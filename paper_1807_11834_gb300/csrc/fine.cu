@@ -204,10 +204,21 @@ __device__ __forceinline__ void average_warp(const T* __restrict__ u, const Grid
     if (var) var[cb] = m2 * invn;
 }
 
+// sum (u - ref) of n values from their compensated sum: (s - n ref) + c, the
+// n ref product split exactly.
+template <typename T>
+__device__ __forceinline__ T sum_of_shifted(const CSum<T>& s, T n, T ref) {
+    const T p = n * ref, pe = fma(n, ref, -p);
+    T d, e;
+    two_sum(s.s, -p, d, e);
+    return d + (e + (s.c - pe));
+}
+
 // (a2) r = 3: one thread per bulk cell holds a component's 27 values (their
-// loads in flight together), the shifted sum and then the squared deviations
-// from the mean, both compensated.  The any-ratio form below reads value by
-// value into one chain (39 us for 128,527 cells, 19 here).
+// loads in flight together), the sum of the values (not of their differences
+// to one of them, whose roundings a mean near zero would show) and then the
+// squared deviations from the mean, shifted, both compensated.  The any-ratio form
+// below reads value by value into one chain (39 us for 128,527 cells, 19 here).
 template <typename T>
 __device__ __forceinline__ void average_cell3(const T* __restrict__ u, const GridDev& g, T* __restrict__ ub,
                                               T* __restrict__ var, long long cb, T* __restrict__ rec) {
@@ -227,20 +238,18 @@ __device__ __forceinline__ void average_cell3(const T* __restrict__ u, const Gri
         const T ref = v[0];
         CSum<T> s;
 #pragma unroll
-        for (int i = 0; i < 27; ++i) {
-            v[i] -= ref;
-            s.add(v[i]);
-        }
-        const T dm = s.get() / T(27);
-        const T mean = ref + dm;
+        for (int i = 0; i < 27; ++i) s.add(v[i]);
+        const T mean = s.get() / T(27);
         ub[c * g.nbulk + cb] = mean;
         if (rec) rec[4 * cb + 1 + c] = mean;
-        if (var)
+        if (var) {
+            const T dm = sum_of_shifted(s, T(27), ref) / T(27);
 #pragma unroll
             for (int i = 0; i < 27; ++i) {
-                const T d = v[i] - dm;
+                const T d = (v[i] - ref) - dm;
                 m2.add(d * d);
             }
+        }
     }
     if (var) var[cb] = m2.get() / T(27);
 }
@@ -321,12 +330,7 @@ __device__ __forceinline__ void average_cell(const T* __restrict__ u, const Grid
         mean[c] = s[c].get() * invn;
         ub[c * g.nbulk + cb] = mean[c];
         if (var) {
-            // D_c = (s_hi - n ref) + s_lo, the n ref product split exactly
-            T p = n * ref[c];
-            T pe = fma(n, ref[c], -p);
-            T d1, e1;
-            two_sum(s[c].s, -p, d1, e1);
-            T D = d1 + (e1 + (s[c].c - pe));
+            const T D = sum_of_shifted(s[c], n, ref[c]);
             corr += D * D;
         }
     }
