@@ -44,6 +44,7 @@ struct cg_map {
     long long off_f2b[3], off_f2w0[3], off_f2w1[3];
     double Vf = 0.0;
     int avg_tile = 0, avg_threads = 0;   // bulk x cells and threads per block of the average; 0: a cell per thread
+    int avg_rows = 0;                    // most fine rows (y) under a bulk row
 };
 
 namespace cg {
@@ -125,8 +126,10 @@ constexpr int kMapMaxComp = 8;
 
 // Average, thread t of a block taking the t-th fine x index under a tile of bulk
 // x cells, over the fine rows of bulk row (J, K) for the K of a chunk: the
-// column's few y terms in plain FMAs, its planes (weighted by z) into a
-// compensated sum, then the x terms, compensated likewise, from shared memory.
+// column's y terms in plain FMAs (MANY, some bulk row over more than map_plain of
+// them: in chains of that length, compensated; as one chain 4096 rows were off by
+// 2e-6), its planes (weighted by z) into a compensated sum, then the x terms,
+// compensated likewise, from shared memory.
 // A plane shared by the cells K and K + 1 is kept.  Every fine value is read
 // once from HBM, those of the rows shared by two bulk rows a second time from L2.
 // The loads are coalesced along x and copied asynchronously into shared memory
@@ -142,11 +145,13 @@ __device__ __forceinline__ void copy_async(T* dst, const T* src) {
                  : "memory");
 }
 constexpr int kMapRows = 6, kMapStages = 2;   // rows of a plane in shared memory, planes in flight
-template <typename T, int NC>
+// Terms of a plain chain; more go chain by chain into a compensated sum.
+__host__ __device__ constexpr int map_plain(size_t tsize) { return tsize == 4 ? 8 : 16; }
+template <typename T, int NC, bool MANY>
 __global__ void __launch_bounds__(256) k_map_average_rows(MapDev<T> d, int tile, int ntiles, int depth,
                                                           const T* __restrict__ in, T* __restrict__ out) {
     pdl_wait();
-    constexpr int G = sizeof(T) == 4 ? kMapRows : kMapRows / 2;
+    constexpr int G = sizeof(T) == 4 ? kMapRows : kMapRows / 2, P = map_plain(sizeof(T));
     __shared__ T sh[2][NC][256];
     __shared__ T ring[kMapStages][G][NC][256];   // a thread copies and reads its own column only
     const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
@@ -213,9 +218,24 @@ __global__ void __launch_bounds__(256) k_map_average_rows(MapDev<T> d, int tile,
                             for (int c = 0; c < NC; ++c) rs[c] = fma(w[y], ring[stage][y][c][threadIdx.x], rs[c]);
                     if (ny > G) {
                         const T* q = ahead - kMapStages * plane + nfx * G;
-                        for (int y = G; y < ny; ++y, q += nfx)
+                        CSum<T> sum[NC];   // MANY: of these terms and then P by P
+                        for (int y = G; y < ny;) {
+                            if (MANY)
 #pragma unroll
-                            for (int c = 0; c < NC; ++c) rs[c] = fma(__ldg(wy + y), __ldg(q + c * nfn), rs[c]);
+                                for (int c = 0; c < NC; ++c) {
+                                    sum[c].add(rs[c]);
+                                    rs[c] = T(0);
+                                }
+                            for (const int end = MANY ? min(y + P, ny) : ny; y < end; ++y, q += nfx)
+#pragma unroll
+                                for (int c = 0; c < NC; ++c) rs[c] = fma(__ldg(wy + y), __ldg(q + c * nfn), rs[c]);
+                        }
+                        if (MANY)
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) {
+                                sum[c].add(rs[c]);
+                                rs[c] = sum[c].get();
+                            }
                     }
                     copy_plane(stage);
                     stage = stage + 1 == kMapStages ? 0 : stage + 1;
@@ -261,8 +281,9 @@ __global__ void __launch_bounds__(256) k_map_average(MapDev<T> d, const T* __res
         const int x0 = __ldg(d.bptr[0] + I), x1 = __ldg(d.bptr[0] + I + 1);
         const int y0 = __ldg(d.bptr[1] + J), y1 = __ldg(d.bptr[1] + J + 1);
         const int z0 = __ldg(d.bptr[2] + K), z1 = __ldg(d.bptr[2] + K + 1);
-        // each fine row's few x terms in plain FMAs, the row sums (weighted
+        // each fine row's x terms in plain FMAs (FP32: of up to 16), these sums (weighted
         // by y and z) into compensated sums
+        const int chain = sizeof(T) == 4 ? 16 : max(x1 - x0, 1);
         CSum<T> acc[NC];
         for (int kz = z0; kz < z1; ++kz) {
             const unsigned fz = (unsigned)__ldg(d.bidx[2] + kz);
@@ -271,17 +292,19 @@ __global__ void __launch_bounds__(256) k_map_average(MapDev<T> d, const T* __res
                 const unsigned fy = (unsigned)__ldg(d.bidx[1] + ky);
                 const T wyz = __ldg(d.bw[1] + ky) * wz;
                 const T* rowp = in + (size_t)nfx * (fy + nfy * fz);
-                T rs[NC];
+                for (int k0 = x0; k0 < x1; k0 += chain) {
+                    T rs[NC];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) rs[c] = T(0);
-                for (int kx = x0; kx < x1; ++kx) {
-                    const unsigned fx = (unsigned)__ldg(d.bidx[0] + kx);
-                    const T wx = __ldg(d.bw[0] + kx);
+                    for (int c = 0; c < NC; ++c) rs[c] = T(0);
+                    for (int kx = k0; kx < min(k0 + chain, x1); ++kx) {
+                        const unsigned fx = (unsigned)__ldg(d.bidx[0] + kx);
+                        const T wx = __ldg(d.bw[0] + kx);
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) rs[c] = fma(wx, __ldg(rowp + c * nfn + fx), rs[c]);
+                        for (int c = 0; c < NC; ++c) rs[c] = fma(wx, __ldg(rowp + c * nfn + fx), rs[c]);
+                    }
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) acc[c].add(wyz * rs[c]);
                 }
-#pragma unroll
-                for (int c = 0; c < NC; ++c) acc[c].add(wyz * rs[c]);
             }
         }
         const T W = __ldg(d.cov[0] + I) * __ldg(d.cov[1] + J) * __ldg(d.cov[2] + K);
@@ -477,6 +500,7 @@ extern "C" cg_status cg_map_create(const cg_box_grid* bulk, const cg_box_grid* f
             const int step = bi[a][k] - bi[a][k - 1];
             runs = runs && (step == 0 || step == 1);
         }
+    for (int j = 0; j < bulk->n[1]; ++j) m->avg_rows = std::max(m->avg_rows, (int)(bp[1][j + 1] - bp[1][j]));
     for (int parts = 1; parts <= bulk->n[0] && runs && !m->avg_tile; ++parts) {
         const int tile = (bulk->n[0] + parts - 1) / parts, w = span(tile);
         if (w > 256) continue;
@@ -542,7 +566,8 @@ static cg_status map_apply(cg_map* m, bool avg, const void* in, void* out) {
             constexpr int NB = NC % 3 == 0 ? 3 : NC % 2 == 0 ? 2 : 1;
             const long long tiles = (m->bulk.n[0] + m->avg_tile - 1) / m->avg_tile, rows = tiles * m->bulk.n[1];
             const int depth = map_depth(rows * m->avg_threads * (NC / NB), m->bulk.n[2], 1);
-            return map_launch(m, k_map_average_rows<T, NB>,
+            const auto kernel = m->avg_rows > map_plain(sizeof(T)) ? k_map_average_rows<T, NB, true> : k_map_average_rows<T, NB, false>;
+            return map_launch(m, kernel,
                               dim3((unsigned)(rows * ((m->bulk.n[2] + depth - 1) / depth)), NC / NB), m->avg_threads, d,
                               m->avg_tile, (int)tiles, depth, (const T*)in, (T*)out);
         }
