@@ -240,10 +240,9 @@ cg_status cg_grid_dims(const cg_grids* g, int32_t bulk_n[3], int64_t* n_bulk, in
  * the particle i of that binning (or, for the sorted output of
  * cg_step_sorted, the particle at its slot i).  The result is the same
  * stable order whatever the particles did (moved, resized or permuted);
- * any share of them may change cell, and when a cell receives more than
- * 32 in one call the device falls back to the per-cell sort.  When none
- * changed cell the bins are kept.  A descriptor with a digit width (6..11)
- * always sorts from scratch. */
+ * any share of them may change cell, and only the cells that receive many
+ * take longer.  When none changed cell the bins are kept.  A descriptor with a
+ * digit width (6..11) always sorts from scratch. */
 cg_status cg_bin_particles(cg_grids* g, int64_t n, const void* pos_d,
                            int32_t* cell_out, int32_t* perm_out, int32_t* cell_start_out);
 

@@ -319,9 +319,6 @@ struct SumsMap {
 };
 
 cg_status ensure_particle_capacity(cg_grids* g, long long n);
-// The per-cell sort of the ids placed in val1 from the cell starts cs, as the
-// fallback of the incremental rebinning (does nothing but copy cs to cs_copy
-// unless *run_if != 0).
 // What the last kernel of a rebinning clears for the next one: the per-cell
 // arrays (in int4) and the tile totals.
 struct RebinClear {
@@ -330,18 +327,25 @@ struct RebinClear {
     int32_t* part;
     long long npart;
 };
-cg_status launch_cellsort_fallback(cg_grids* g, const int32_t* cs, int32_t* ctr, int32_t* cs_copy, int32_t* inv_perm,
-                                   const RebinClear& clear);
+// The last kernel of a rebinning: the ids of the crowded cells, placed in val1
+// from the cell starts cs, in order; cs to cs_copy; the clear.
+cg_status launch_rebin_finish(cg_grids* g, const int32_t* cs, int32_t* ctr, const int4* crowd, int32_t* cs_copy,
+                              int32_t* inv_perm, const RebinClear& clear);
 // Incremental rebinning (rebin.cu).
-// Counters: fallback flag, movers, finished blocks of the last kernel, which
-// clears these three; whether inv_perm is not the inverse of perm, and the
+// Counters: entries of the crowded cells' list, movers, finished blocks of the last
+// kernel, which clears these three; whether inv_perm is not the inverse of perm, and the
 // finished blocks of the kernel that makes it so.
-enum { RB_FALLBACK = 0, RB_MOVERS = 1, RB_DONE = 2, RB_INV_STALE = 3, RB_INV_DONE = 4 };
+enum { RB_CROWD = 0, RB_MOVERS = 1, RB_DONE = 2, RB_INV_STALE = 3, RB_INV_DONE = 4 };
 constexpr int kRebinThreads = 256;
 constexpr int kRebinItems = 4;
 constexpr int kRebinTile = kRebinThreads * kRebinItems;   // old slots per block
 constexpr int kRebinScan = 1024;                           // elements per block of its scans
-constexpr int kRebinMaxArrivals = 32;                      // arrivals per cell before the fallback
+// Arrivals of a cell whose list is walked; a cell of more is crowded.  (The bed of
+// 977 per cell, 2% leaving: 4 293, 8 298, 16 312, 32 349 us; 500,000 particles in
+// another order 149, 180, 258, 382 with one warp for the movers of 1024 slots; few
+// movers per cell: no difference.)
+constexpr int kRebinMaxArrivals = 4;
+constexpr int kCrowdPart = 4096;                           // ids of a crowded cell that a warp merges
 constexpr long long kRebinMaxParticles = 1LL << 30;        // the marking kernel's 32-bit slots (a longer list is sorted)
 constexpr int kRebinCounters = 8;
 // The small rebinning arrays each start on a 256-byte boundary (the scan reads

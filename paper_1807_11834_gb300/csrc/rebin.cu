@@ -26,12 +26,13 @@
 // order, or particle s when the particles are the sorted output of the last
 // step (cg_step_sorted; the identity hint).  The movers of a cell are a linked
 // list (its few entries are walked, in any order, to count the ids below
-// one).  When a cell receives more than kRebinMaxArrivals movers the walks
-// would grow with the square of the arrivals, and the device falls back to a
-// sort of every cell: the slots kernel then places the ids of each cell in any
-// order, and the last kernel sorts them; each kernel checks a device flag, so
-// a captured CUDA graph takes the right path on every replay.  When no
-// particle changed its cell the device leaves the scans out and keeps the bins.
+// one).  In a cell that receives more than kRebinMaxArrivals movers, a crowded
+// one, the walks would grow with the square of the arrivals: the slots kernel
+// puts its stayers, in order, and then its movers into a second array, and the
+// last kernel sorts the movers and merges the two.  The scan makes the list of
+// the crowded cells on the device, so a captured CUDA graph takes the right path
+// on every replay.  When no particle changed its cell the device leaves the scans
+// out and keeps the bins.
 //
 // In a coupling step the kernels also form the porosity: the first one, which
 // has every particle's position and diameter in nearly sorted order, adds the
@@ -178,7 +179,6 @@ k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restr
                     const int r = atomicAdd(&arr[cn[k]].x, 1);
                     const int next = atomicExch(&arr[cn[k]].y, j + 1);
                     mov[j] = make_int4(id[k], cn[k], next, r);
-                    if (r >= kRebinMaxArrivals) ctr[RB_FALLBACK] = 1;
                 }
                 idx += __popc(mb[k]);
             }
@@ -265,7 +265,8 @@ __device__ __forceinline__ void scan4(int (&v)[4], int before, int* sh) {
         e += x;
     }
 }
-__device__ __forceinline__ void scan_tile(int32_t* __restrict__ a, long long first, long long m, int before, int* sh) {
+__device__ __forceinline__ void scan_tile(int32_t* __restrict__ a, long long first, long long m, int before, int* sh,
+                                          int (&raw)[4]) {
     const long long i = first + 4 * threadIdx.x;
     int v[4] = {0, 0, 0, 0};
     const bool whole = i + 4 <= m;
@@ -280,6 +281,8 @@ __device__ __forceinline__ void scan_tile(int32_t* __restrict__ a, long long fir
         for (int j = 0; j < 4; ++j)
             if (i + j < m) v[j] = a[i + j];
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) raw[j] = v[j];
     scan4(v, before, sh);
     if (whole) {
         *reinterpret_cast<int4*>(a + i) = make_int4(v[0], v[1], v[2], v[3]);
@@ -289,14 +292,15 @@ __device__ __forceinline__ void scan_tile(int32_t* __restrict__ a, long long fir
             if (i + j < m) a[i + j] = v[j];
     }
 }
-__device__ __forceinline__ void scan_tile_x(int2* __restrict__ a, long long first, long long m, int before, int* sh) {
+__device__ __forceinline__ void scan_tile_x(int2* __restrict__ a, long long first, long long m, int before, int* sh,
+                                            int (&raw)[4]) {
     const long long i = first + 4 * threadIdx.x;
     int2 q[4];
     int v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         q[j] = i + j < m ? a[i + j] : make_int2(0, 0);
-        v[j] = q[j].x;
+        raw[j] = v[j] = q[j].x;
     }
     scan4(v, before, sh);
 #pragma unroll
@@ -305,10 +309,13 @@ __device__ __forceinline__ void scan_tile_x(int2* __restrict__ a, long long firs
 }
 
 // Starts from the counts and the block totals: the cells' counts and
-// arrivals, and the departures per block of old slots.
+// arrivals, and the departures per block of old slots.  The cells of many
+// arrivals go on the list of the crowded ones, (cell, arrivals, part, parts),
+// an entry per part of kCrowdPart ids where the last kernel merges by parts; fewer
+// than n / 4 in all, which the list's place, an int per particle, holds.
 __global__ void __launch_bounds__(256)
 k_rebin_scan(int32_t* __restrict__ cnt, int2* __restrict__ arr, long long ncell, int32_t* __restrict__ blk,
-             long long nblk, const int32_t* __restrict__ part, long long tiles, const int32_t* __restrict__ ctr) {
+             long long nblk, const int32_t* __restrict__ part, long long tiles, int32_t* ctr, int4* __restrict__ crowd) {
     pdl_wait();
     __shared__ int sh[32];
     if (ctr[RB_MOVERS] == 0) return;
@@ -324,10 +331,34 @@ k_rebin_scan(int32_t* __restrict__ cnt, int2* __restrict__ arr, long long ncell,
     block_exclusive_scan(a0, sh, t0);
     if (cells) {
         block_exclusive_scan(a1, sh, t1);
-        scan_tile(cnt, b * kRebinScan, ncell, t0, sh);
-        scan_tile_x(arr, b * kRebinScan, ncell, t1, sh);
+        int count[4], in[4];
+        scan_tile(cnt, b * kRebinScan, ncell, t0, sh, count);
+        scan_tile_x(arr, b * kRebinScan, ncell, t1, sh, in);
+        int parts[4], mine = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            parts[j] = in[j] <= kRebinMaxArrivals ? 0 : in[j] <= kSegWarpMax ? (count[j] + kCrowdPart - 1) / kCrowdPart : 1;
+            mine += parts[j];
+        }
+        if (__any_sync(0xffffffffu, mine != 0)) {   // one atomic per warp
+            const int lane = threadIdx.x & 31;
+            int at = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, at, off);
+                if (lane >= off) at += o;
+            }
+            int base = 0;
+            if (lane == 31) base = atomicAdd(ctr + RB_CROWD, at);
+            at += __shfl_sync(0xffffffffu, base, 31) - mine;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                for (int p = 0; p < parts[j]; ++p)
+                    crowd[at++] = make_int4((int)(b * kRebinScan) + 4 * (int)threadIdx.x + j, in[j], p, parts[j]);
+        }
     } else {
-        scan_tile(blk, b * kRebinScan, nblk + 1, t0, sh);
+        int count[4];
+        scan_tile(blk, b * kRebinScan, nblk + 1, t0, sh, count);
     }
 }
 
@@ -405,9 +436,10 @@ __device__ __forceinline__ void rebin_stay_body(const int32_t* __restrict__ rid,
             const int D = __shfl_sync(full, incl, k * W + warp) + __popc(db[k] & lanemask_lt());
             if (c[k] < 0) continue;
             int ns = s - D + ah[k].x;
-            if (ah[k].y && !place) ns += movers_below(mov, ah[k].y, i[k]);
+            const bool crowded = place && ah[k].y && __ldg(&arr[c[k] + 1].x) - ah[k].x > kRebinMaxArrivals;
+            if (ah[k].y && !crowded) ns += movers_below(mov, ah[k].y, i[k]);
             if ((unsigned)ns >= (unsigned)n) continue;   // never for a valid binning
-            if (place) {
+            if (crowded) {
                 place[ns] = i[k];
                 continue;
             }
@@ -418,7 +450,7 @@ __device__ __forceinline__ void rebin_stay_body(const int32_t* __restrict__ rid,
     }
 }
 
-// Movers, one warp per block of old slots: the stayers of the new cell with
+// Movers, `warps` warps (1, 2, 4 or 8) per block of old slots: the stayers of the new cell with
 // an id below the mover's (a binary search over the old segment, whose ids
 // ascend, then a count of the stayers before that point) and the movers of
 // its list with an id below it.
@@ -430,17 +462,19 @@ __device__ __forceinline__ void rebin_movers_body(const int32_t* __restrict__ ri
                                                   const int2* __restrict__ arr, const int4* __restrict__ mov,
                                                   int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted,
                                                   int32_t* __restrict__ inv_perm, int32_t* __restrict__ place,
-                                                  long long nblk, long long bid, long long nb) {
-    const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
-    for (long long b = bid * W + (threadIdx.x >> 5); b < nblk; b += nb * W) {
+                                                  long long nblk, long long bid, long long nb, int warps) {
+    const int W = (blockDim.x >> 5) / warps, w = threadIdx.x >> 5;
+    for (long long b = bid * W + w / warps; b < nblk; b += nb * W) {
         const int cntb = __ldg(blk_start + b + 1) - __ldg(blk_start + b);
-        for (int j = lane; j < cntb; j += 32) {
+        for (int j = threadIdx.x % (32 * warps); j < cntb; j += 32 * warps) {
             const int4 m = __ldg(mov + b * kRebinTile + j);
             const int i = m.x, c = m.y;
             long long ns;
-            if (place) {
+            const int in = place ? __ldg(&arr[c + 1].x) - __ldg(&arr[c].x) : 0;
+            const bool crowded = in > kRebinMaxArrivals;
+            if (crowded) {
                 // after the cell's stayers, in the order of arrival
-                ns = (long long)__ldg(cs_new + c + 1) - (__ldg(&arr[c + 1].x) - __ldg(&arr[c].x)) + m.w;
+                ns = (long long)__ldg(cs_new + c + 1) - in + m.w;
             } else {
                 const int o0 = __ldg(cs_old + c), o1 = __ldg(cs_old + c + 1);
                 int lo = o0, hi = o1;
@@ -458,7 +492,7 @@ __device__ __forceinline__ void rebin_movers_body(const int32_t* __restrict__ ri
                 ns = (long long)__ldg(cs_new + c) + stay + movers_below(mov, __ldg(&arr[c].y), i);
             }
             if ((unsigned long long)ns >= (unsigned long long)n) continue;   // never for a valid binning
-            if (place) {
+            if (crowded) {
                 place[ns] = i;
                 continue;
             }
@@ -471,8 +505,8 @@ __device__ __forceinline__ void rebin_movers_body(const int32_t* __restrict__ ri
 
 // Every particle's new slot in one launch: blocks [0, mgrid) place the
 // movers (first, so that their searches run beside the stayers), the other
-// blocks the stayers.  In the fallback both put the ids into their cells'
-// places of `place` in any order.  Bound by HBM and by the latency of the
+// blocks the stayers.  The ids of crowded cells go to `place` instead, the
+// stayers in their order, then the movers in any.  Bound by HBM and by the latency of the
 // gather behind each record: 32M particles 105 us, against 207 for one
 // block of old slots per CTA with the diameters and the inverse carried along.
 template <bool IDENT>
@@ -481,9 +515,9 @@ k_rebin_slots(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn, 
               const int32_t* __restrict__ blk_start, const int32_t* __restrict__ cs_old,
               const int32_t* __restrict__ cs_new, const int2* __restrict__ arr, const int4* __restrict__ mov,
               int32_t* __restrict__ perm, int32_t* __restrict__ key_sorted, int32_t* __restrict__ inv_perm,
-              int32_t* __restrict__ place, const int32_t* __restrict__ ctr, long long nblk, long long mgrid) {
+              int32_t* __restrict__ place, const int32_t* __restrict__ ctr, long long nblk, long long mgrid, int mwarps) {
     pdl_wait();
-    int32_t* const where = ctr[RB_FALLBACK] ? place : nullptr;
+    int32_t* const where = ctr[RB_CROWD] ? place : nullptr;
     if (ctr[RB_MOVERS] == 0) {
         // slot s keeps its particle and cell; with the identity hint the
         // particles are renumbered to their slots, without it the inverse is
@@ -498,7 +532,7 @@ k_rebin_slots(const int32_t* __restrict__ rid, const int32_t* __restrict__ rkn, 
     }
     if ((long long)blockIdx.x < mgrid)
         rebin_movers_body<IDENT>(rid, rkn, n, blk_start, cs_old, cs_new, arr, mov, perm, key_sorted, inv_perm, where,
-                                 nblk, blockIdx.x, mgrid);
+                                 nblk, blockIdx.x, mgrid, mwarps);
     else
         rebin_stay_body<IDENT>(rid, rkn, (int)n, blk_start, arr, mov, perm, key_sorted, inv_perm, where, (int)nblk,
                                (int)(blockIdx.x - mgrid), (int)(gridDim.x - mgrid));
@@ -543,8 +577,12 @@ static cg_status rebin_launches(cg_grids* g, long long n, const T* pos, bool ide
         if (eps->ready) CG_CUDA(cudaEventRecord(eps->ready, g->stream));
     }
     CG_LAUNCH(g, "rebin_scan", k_rebin_scan, (unsigned)(tiles + btiles), 256, 0, R.cnt, R.arr, nbulk + 1, R.blk, nblk,
-              (const int32_t*)R.part, tiles, (const int32_t*)R.ctr);
-    const long long mgrid = std::min<long long>((nblk + 7) / 8, (long long)g->num_sms * 8);
+              (const int32_t*)R.part, tiles, R.ctr, (int4*)g->key);
+    // few blocks of old slots: several warps for the movers of each, since a bed of
+    // which every particle has moved is a chain of 32 rounds for one (500,000
+    // particles in another order: the step 180 -> 140 us)
+    const long long mgrid = std::max((nblk + 7) / 8, std::min<long long>(nblk, (long long)g->num_sms * 3));
+    const int mwarps = nblk <= mgrid ? 8 : nblk <= 2 * mgrid ? 4 : nblk <= 4 * mgrid ? 2 : 1;
     // resident blocks that walk the old slots (the sorted step), or, where the
     // scattered stores of a caller's random order dominate, a block per 1024
     // slots (4M particles: 42 us against 50)
@@ -553,14 +591,13 @@ static cg_status rebin_launches(cg_grids* g, long long n, const T* pos, bool ide
     CG_LAUNCH(g, "rebin_slots", (k_rebin_slots<ID>), (unsigned)(mgrid + sgrid), kRebinThreads, 0,                   \
               (const int32_t*)g->rb_rid, (const int32_t*)g->rb_rkn, n, (const int32_t*)R.blk,                      \
               (const int32_t*)g->cell_start, (const int32_t*)R.cnt, (const int2*)R.arr, (const int4*)g->rb_mov,      \
-              g->perm, g->key_sorted, g->inv_perm, g->val1, (const int32_t*)R.ctr, nblk, mgrid)
+              g->perm, g->key_sorted, g->inv_perm, g->val1, (const int32_t*)R.ctr, nblk, mgrid, mwarps)
     if (ident) CG_REBIN_SLOTS(true);
     else CG_REBIN_SLOTS(false);
 #undef CG_REBIN_SLOTS
-    // the starts to their place, the counters to zero; in the fallback also the sort of every cell
     const long long nb1 = rebin_pad(nbulk + 1);
-    CG_TRY(launch_cellsort_fallback(g, R.cnt, R.ctr, g->cell_start, ident ? nullptr : g->inv_perm,
-                                    {(int4*)R.arr, 3 * nb1 / 4, R.part, 2 * tiles + btiles}));
+    CG_TRY(launch_rebin_finish(g, R.cnt, R.ctr, (const int4*)g->key, g->cell_start, ident ? nullptr : g->inv_perm,
+                               {(int4*)R.arr, 3 * nb1 / 4, R.part, 2 * tiles + btiles}));
     return CG_OK;
 }
 
