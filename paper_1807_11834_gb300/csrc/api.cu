@@ -156,6 +156,7 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     CG_TRY(ensure_partials(g, n));
     if (n <= g->cap) return CG_OK;
     const long long cap = ((n + kSortTile - 1) / kSortTile) * kSortTile;
+    const bool fresh = !g->rb_small;
     dfree(g->key);
     dfree(g->key1);
     dfree(g->val1);
@@ -203,11 +204,12 @@ cg_status ensure_particle_capacity(cg_grids* g, long long n) {
     CG_TRY(dalloc(&g->rb_mov, sizeof(int4) * g->rb_nblk * kRebinTile));
     const size_t small = sizeof(int32_t) * rebin_small_ints(g->gd.nbulk, g->rb_nblk);
     CG_TRY(dalloc(&g->rb_small, small));
-    // The rebinning leaves its counters zero; their first zeroes are there before
-    // this returns, on whatever stream the next call runs (the handle's own side
-    // stream has nothing of the caller's to wait for).
-    CG_CUDA(cudaMemsetAsync(g->rb_small, 0, small, g->aux));
-    CG_CUDA(cudaStreamSynchronize(g->aux));
+    // The rebinning leaves its counters zero.  A new handle's first zeroes are there
+    // before this returns, on whatever stream its first call runs (its own side
+    // stream has nothing of the caller's to wait for); one that grows is in a call
+    // on its stream.
+    CG_CUDA(cudaMemsetAsync(g->rb_small, 0, small, fresh ? g->aux : g->stream));
+    if (fresh) CG_CUDA(cudaStreamSynchronize(g->aux));
     const long long cells_blk = (g->gd.nbulk + 1 + kScanItems - 1) / kScanItems;
     g->scan_cap = (g->hist_cap + kScanItems - 1) / kScanItems + cells_blk;
     CG_TRY(dalloc(&g->scan_part, sizeof(int32_t) * g->scan_cap));
