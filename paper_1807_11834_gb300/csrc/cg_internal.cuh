@@ -1139,6 +1139,34 @@ __device__ __forceinline__ void volume_add_row(bool valid, int cell, double d, c
         if (w[2]) volume_add_third(w[2], cell, g.nbulk, false, acc);
     }
 }
+// The same in line, for kernels with registers to spare: rows with other spheres
+// sum three pieces at once (16 instances, 4.3M mostly small spheres: 27 us against
+// 31 out of line).
+__device__ __forceinline__ void volume_add_row_wide(bool valid, int cell, float d, const GridDev& g,
+                                                    unsigned long long* __restrict__ acc) {
+    const unsigned heads = run_heads(valid, cell);
+    float hi, lo;
+    sphere_pair(d, g, hi, lo);
+    unsigned w[3];
+    sphere_pieces_plain(hi, lo, w[0], w[1]);
+    w[2] = 0u;
+    const bool other = valid && !sphere_plain(hi);
+    const bool mixed = __any_sync(0xffffffffu, other);
+    bool out = !valid;
+    if (other) {
+        const bool in = sphere_pieces_other(hi, lo, w);
+        out = volume_alone(in, w, (double)d, cell, g.vcd, g.nbulk, true, acc);
+    }
+    if (out) w[0] = w[1] = w[2] = 0u;
+    if ((mixed ? volume_runs<3>(w, heads) : volume_runs<2>(w, heads)) && valid) {
+        volume_atomics(w[0], w[1], cell, acc);
+        if (mixed && w[2]) volume_add_third(w[2], cell, g.nbulk, true, acc);
+    }
+}
+__device__ __forceinline__ void volume_add_row_wide(bool valid, int cell, double d, const GridDev& g,
+                                                    unsigned long long* __restrict__ acc) {
+    volume_add_row(valid, cell, d, g, acc);
+}
 
 // Where a step's porosity goes: double, and (nullable) the porosity of the
 // drag's record, its copy in the path precision, and the reaction source to

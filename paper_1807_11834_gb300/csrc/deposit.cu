@@ -56,7 +56,7 @@ __device__ __forceinline__ void volume_rows_body(const T* __restrict__ d, long l
 #pragma unroll
         for (int j = 0; j < B; ++j) {
             if (r0 + 32 * j >= n) break;   // warp-uniform
-            volume_add_row(key[j] >= 0, key[j], v[j], g, o.acc);
+            volume_add_row_wide(key[j] >= 0, key[j], v[j], g, o.acc);
         }
     }
 }
