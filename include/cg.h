@@ -534,10 +534,13 @@ typedef struct {
 
 /* Work decomposition (results do not depend on it). */
 typedef struct {
-    int32_t digit_bits;  /* widest radix digit of a binning pass, 8..11      */
+    int32_t digit_bits;  /* radix digits, 8..11: an instance of up to
+                            min(digit_bits, 9) bits of cells is binned in one
+                            pass, one of up to 2 digit_bits in two          */
     int32_t drag_items;  /* particles per thread of a drag block, 1..64      */
     int32_t avg_items;   /* bulk cells per thread of an average block, 1..64 */
-    int32_t seg_chunks;  /* 256-slot chunks per warp of the deposits, 1..64  */
+    int32_t seg_chunks;  /* chunks of the sorted order (32 to 256 slots, by the
+                            particle count) per warp of the deposits, 1..64 */
     int32_t grid_mult;   /* persistent CTAs = grid_mult x resident per SM x SMs, 1..8 */
 } cg_batch_config;
 

@@ -4,8 +4,8 @@
 // the work decomposition chosen by an autotuner.
 //
 // Decomposition knobs (cg_batch_config) change only how work is cut into
-// blocks, never the arithmetic: the segmented sums own fixed 256-slot
-// chunks of the sorted order, the sort is stable for any digit split, and
+// blocks, never the arithmetic: the segmented sums own fixed chunks of the
+// sorted order (seg_chunk, by the particle count), the sort is stable for any digit split, and
 // each cell or particle is computed by one thread in a fixed order, so every
 // field is bit-identical across configurations and to cg_step of the same
 // instance.  Only the FP64 conservation sums, merged from per-block
@@ -56,6 +56,8 @@ int ceil_log2_ll(long long v) {
 }
 
 long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
+
+constexpr int kBatchOneDigit = 9;   // widest key that is binned in one pass
 
 bool valid_config(const cg_batch_config& c) {
     return c.digit_bits >= 8 && c.digit_bits <= kMaxDigitBits && c.drag_items >= 1 && c.drag_items <= 64 &&
@@ -119,10 +121,10 @@ cg_status plan(cg_batch* b) {
         I.cellsort = g->desc.sort_digits == CG_SORT_CELLS ? 1 : 0;
         const int bits = std::max(1, ceil_log2_ll(nb));
         if (!I.cellsort && bits > 2 * c.digit_bits) return CG_ERR_OUT_OF_RANGE;
-        // one pass up to 9 bits: with 11, the warps' counters of a scatter tile take the
-        // shared memory of a whole SM and outnumber its particles eight to
+        // one pass up to kBatchOneDigit bits: with 11, the warps' counters of a scatter tile
+        // take the shared memory of a whole SM and outnumber its particles eight to
         // one (16 instances, 4.3M particles: scatters 162 -> 124 us, the second histogram 8 -> 13)
-        I.npasses = I.cellsort ? 0 : bits <= std::min(c.digit_bits, 9) ? 1 : 2;
+        I.npasses = I.cellsort ? 0 : bits <= std::min(c.digit_bits, kBatchOneDigit) ? 1 : 2;
         I.b0 = I.cellsort ? 0 : I.npasses == 1 ? bits : (bits + 1) / 2;
         I.b1 = I.npasses == 2 ? bits - I.b0 : 0;
         I.pos = (float*)it.particles.pos_d;
@@ -579,12 +581,13 @@ cg_status cg_batch_tune(cg_batch* b, int32_t reps, const char* cache_path, cg_ba
     cg_batch_config best = b->cfg;
     double best_t = 0.0;
     cg_status st = measure(best, best_t);
-    const int digit[] = {8, 9, 10, 11};
+    // from kBatchOneDigit on the widths differ only in the widest grid they accept
+    const int digit[] = {8, kMaxDigitBits};
     const int items[] = {1, 2, 4, 8};
     const int mult[] = {1, 2, 4};
     for (int knob = 0; knob < 5 && st == CG_OK; ++knob) {
         const int* vals = knob == 0 ? digit : knob == 4 ? mult : items;
-        const int nv = knob == 0 ? 4 : knob == 4 ? 3 : 4;
+        const int nv = knob == 0 ? 2 : knob == 4 ? 3 : 4;
         for (int v = 0; v < nv && st == CG_OK; ++v) {
             cg_batch_config c = best;
             int* field = knob == 0 ? &c.digit_bits : knob == 1 ? &c.drag_items : knob == 2 ? &c.avg_items
