@@ -137,7 +137,7 @@ void prof_end(cg_grids* g, int slot, int ev) {
 cg_status ensure_partials(cg_grids* g, long long n) {
     const long long bulk_blk = (g->gd.nbulk + 7) / 8;   // cell kernels run 8 cells (warps) per block
     (void)n;
-    const long long proj_blk = project_blocks(g->gd, 3, g->fp64);   // the projection of the source forms sums
+    const long long proj_blk = project_blocks(g->gd, 3, g->fp64, g->num_sms);   // the projection of the source forms sums
     const long long part_blk = std::max(bulk_blk, (long long)g->num_sms * 8);
     const long long need = part_blk * (1 + kDragCellSums) + proj_blk * 6;
     if (need > g->part_cap) {

@@ -446,9 +446,9 @@ __host__ __device__ constexpr int average_lanes(int r, bool fp64) {
 // Layers a thread of the projection walks, and its blocks of
 // project_block threads per component.
 int project_depth(const GridDev& g, int ncomp, bool fp64);
-int project_block(const GridDev& g, int ncomp, bool fp64);
+int project_block(const GridDev& g, int ncomp, bool fp64, int num_sms);
 long long project_threads(const GridDev& g, int depth);
-long long project_blocks(const GridDev& g, int ncomp, bool fp64);
+long long project_blocks(const GridDev& g, int ncomp, bool fp64, int num_sms);
 cg_status launch_sums(cg_grids* g, double* sums);
 // Sum columns of the partial regions (offsets in pairs; blocks < 0: region not formed).
 SumsMap sums_map(const long long* part_off, const long long* part_blocks);
@@ -670,7 +670,6 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 
 // ----------------------------------------------------------------------
 // (a0) bin index, shared by the binning and the cell-value gather.
-// ----------------------------------------------------------------------
 // ----------------------------------------------------------------------
 // a / b correctly rounded, from y = 1 / b correctly rounded: q1 is within one
 // unit in the last place of a / b, so its remainder is exact and q1 + r y

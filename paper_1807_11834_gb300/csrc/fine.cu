@@ -560,11 +560,11 @@ long long project_threads(const GridDev& g, int depth) {
 }
 // Small grids take small blocks, so that their few warps reach every SM; so
 // does FP64, whose time is the busiest SM's share of the arithmetic.
-int project_block(const GridDev& g, int ncomp, bool fp64) {
-    return project_threads(g, project_depth(g, ncomp, fp64)) * ncomp >= 152 * 512 ? (fp64 ? 64 : 256) : 32;
+int project_block(const GridDev& g, int ncomp, bool fp64, int num_sms) {
+    return project_threads(g, project_depth(g, ncomp, fp64)) * ncomp >= 512LL * num_sms ? (fp64 ? 64 : 256) : 32;
 }
-long long project_blocks(const GridDev& g, int ncomp, bool fp64) {
-    const int bs = project_block(g, ncomp, fp64);
+long long project_blocks(const GridDev& g, int ncomp, bool fp64, int num_sms) {
+    const int bs = project_block(g, ncomp, fp64, num_sms);
     return (project_threads(g, project_depth(g, ncomp, fp64)) + bs - 1) / bs;
 }
 
@@ -685,8 +685,8 @@ static cg_status project_launch(cg_grids* g, int ncomp, const void* const* in, v
         io.out[c] = (T*)out[c];
     }
     const bool fp64 = sizeof(T) == 8;
-    const int depth = project_depth(g->gd, ncomp, fp64), bs = project_block(g->gd, ncomp, fp64);
-    const long long nblk = project_blocks(g->gd, ncomp, fp64);
+    const int depth = project_depth(g->gd, ncomp, fp64), bs = project_block(g->gd, ncomp, fp64, g->num_sms);
+    const long long nblk = project_blocks(g->gd, ncomp, fp64, g->num_sms);
     // only the projection that forms the sums claims their partials (a later
     // projection without sums, of the porosity or the semi-implicit
     // coefficients, leaves them to it)

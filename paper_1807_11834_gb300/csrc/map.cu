@@ -34,6 +34,7 @@ struct cg_map {
     int fp64 = 0;
     size_t tsize = 4;
     cudaStream_t stream = nullptr;
+    int num_sms = 148;
     long long nbulk = 0, nfine = 0;
     // per axis: [ptr (n+1) int32][idx int32][w T], average (bulk rows) and projection (fine rows)
     void* dev = nullptr;
@@ -431,6 +432,8 @@ extern "C" cg_status cg_map_create(const cg_box_grid* bulk, const cg_box_grid* f
     m->fp64 = bulk->prec == CG_FP64;
     m->tsize = m->fp64 ? 8 : 4;
     m->stream = (cudaStream_t)cuda_stream;
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
     m->nbulk = (long long)bulk->n[0] * bulk->n[1] * bulk->n[2];
     m->nfine = (long long)fine->n[0] * fine->n[1] * fine->n[2];
     m->Vf = (fine->extent[0] / fine->n[0]) * (fine->extent[1] / fine->n[1]) * (fine->extent[2] / fine->n[2]);
@@ -550,10 +553,10 @@ static cg_status map_launch(cg_map* m, K kernel, dim3 grid, int block, Args... a
 }
 
 // z planes per thread: as many as leave `fill` threads for each of the chip's
-// (152 SMs of 2048), since the start of a walk is work of its own; at most 64.
+// (2048 per SM), since the start of a walk is work of its own; at most 64.
 // Average: fill 1 102, 2 104, 4 106 us at the size above; projection: 81, 87, 78.
-static int map_depth(long long columns, long long nz, int fill) {
-    const long long chunks = (fill * 152LL * 2048 + columns - 1) / columns;
+static int map_depth(const cg_map* m, long long columns, long long nz, int fill) {
+    const long long chunks = (fill * 2048LL * m->num_sms + columns - 1) / columns;
     return (int)std::max(1LL, std::min((nz + chunks - 1) / chunks, 64LL));
 }
 
@@ -565,7 +568,7 @@ static cg_status map_apply(cg_map* m, bool avg, const void* in, void* out) {
             // components per block: what shared memory holds
             constexpr int NB = NC % 3 == 0 ? 3 : NC % 2 == 0 ? 2 : 1;
             const long long tiles = (m->bulk.n[0] + m->avg_tile - 1) / m->avg_tile, rows = tiles * m->bulk.n[1];
-            const int depth = map_depth(rows * m->avg_threads * (NC / NB), m->bulk.n[2], 1);
+            const int depth = map_depth(m, rows * m->avg_threads * (NC / NB), m->bulk.n[2], 1);
             const auto kernel = m->avg_rows > map_plain(sizeof(T)) ? k_map_average_rows<T, NB, true> : k_map_average_rows<T, NB, false>;
             return map_launch(m, kernel,
                               dim3((unsigned)(rows * ((m->bulk.n[2] + depth - 1) / depth)), NC / NB), m->avg_threads, d,
@@ -575,7 +578,7 @@ static cg_status map_apply(cg_map* m, bool avg, const void* in, void* out) {
     }
     if (m->two) {
         const long long columns = (long long)m->fine.n[0] * m->fine.n[1], colblk = (columns + 255) / 256;
-        const int depth = map_depth(columns, m->fine.n[2], 4);
+        const int depth = map_depth(m, columns, m->fine.n[2], 4);
         return map_launch(m, k_map_project2<T, NC>, dim3((unsigned)(colblk * ((m->fine.n[2] + depth - 1) / depth))), 256, d, (unsigned)colblk,
                           depth, (const T*)in, (T*)out);
     }
