@@ -88,8 +88,8 @@ def parse():
                     help="the step timed: cg_step_sorted (particles left in cell order every step; the default "
                          "for an advancing workload) or cg_step (the caller's particle order kept)")
     ap.add_argument("--stencil", choices=("gather", "window"), default="gather",
-                    help="the drag's stencil reads: eight loads per particle from L1/L2, or each warp's stencil "
-                         "window staged in shared memory (sorted step only)")
+                    help="accepted and without effect: the sorted FP32 step always stages each warp's stencil "
+                         "window in shared memory, the other drags always gather")
     ap.add_argument("--implicit", action="store_true",
                     help="also form the semi-implicit exchange coefficients (bulk and fine) in every step "
                          "(device entry only: no e2e line)")
@@ -563,7 +563,6 @@ def run_gb300(args):
                        "l2": (f"inputs {input_bytes / 1e6:.0f} MB {'>' if input_bytes > 126e6 else '<'} L2 (126 MB) "
                               "per step, no flush"),
                        "step": "cg_step_sorted" if sorted_step else "cg_step",
-                       "stencil": args.stencil,
                        "timing": ("CUDA graph of one step, replayed K times" if not args.no_graph
                                   else "eager step calls") + (" (one graph per particle buffer, in turn)"
                                                               if sorted_step and not args.no_graph else ""),

@@ -78,7 +78,7 @@ enum {
 #define CG_SORT_CELLS_AUTO_MAX 8388608   /* 2^23 particles */
 #define CG_SORT_CELLS_AUTO_DENSITY 32   /* particles per bulk cell */
 
-/* Stencil reads of the drag (cg_grid_desc.stencil). */
+/* Stencil reads of the drag (cg_grid_desc.stencil); without effect. */
 #define CG_STENCIL_GATHER 0
 #define CG_STENCIL_WINDOW 1
 
@@ -110,13 +110,13 @@ enum {
  *                 below 2^20 bulk cells, up to 8 from 2^20 on; an instance of
  *                 a batch (cg_batch_create) takes the digit sort unless its
  *                 descriptor asks for CG_SORT_CELLS
- *   stencil     CG_STENCIL_GATHER (0) or CG_STENCIL_WINDOW (1); both give
- *               the same bits, and both now run the same kernels:
- *               cg_step_sorted on the FP32 trilinear path stages the bulk
- *               records around a run of cells in shared memory for each
- *               warp, every other drag reads the eight 16-byte records of a
- *               particle's stencil through L1 and L2 (the bulk record of a
- *               2^22-cell grid is 64 MB, inside the 129 MB L2)
+ *   stencil     CG_STENCIL_GATHER (0) or CG_STENCIL_WINDOW (1), checked and
+ *               otherwise without effect: cg_step_sorted on the FP32 trilinear
+ *               path always stages the bulk records around a run of cells in
+ *               shared memory for each warp, every other drag always reads the
+ *               eight 16-byte records of a particle's stencil through L1 and L2
+ *               (the bulk record of a 2^22-cell grid is 64 MB, inside the 129 MB
+ *               L2); both give the same bits
  * Limits: fine_n[a] % ratio == 0, bulk cells >= 2 per axis, at most 2^22
  * bulk cells and 2^31 - 1 fine cells. */
 typedef struct {

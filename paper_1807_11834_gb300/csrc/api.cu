@@ -139,7 +139,7 @@ cg_status ensure_partials(cg_grids* g, long long n) {
     (void)n;
     const long long proj_blk = project_blocks(g->gd, 3, g->fp64, g->num_sms);   // the projection of the source forms sums
     const long long part_blk = std::max(bulk_blk, (long long)g->num_sms * 8);
-    const long long need = part_blk * (1 + kDragCellSums) + proj_blk * 6;
+    const long long need = part_blk * (1 + kDragSums) + proj_blk * 6;
     if (need > g->part_cap) {
         dfree(g->partials);
         g->part_cap = 0;

@@ -98,7 +98,6 @@ enum { ST_FLAGS = 0, ST_OUTSIDE = 1, ST_NONFINITE = 2, ST_CLAMPED = 3, ST_TIMEOU
 enum { PS_VOL = 0, PS_DRAG = 1, PS_PROJ = 2, PS_NREG = 3 };
 constexpr int kDragLaneSums = 8;              // V_p, F(3), |F|, m u (3)
 constexpr int kDragSums = kDragLaneSums + 1;   // + the clamped count
-constexpr int kDragCellSums = kDragSums + 3;   // + S_B V_B (3) in the cell-order drag
 
 // ----------------------------------------------------------------------
 // Device-side view of the grid geometry (passed by value to kernels)
