@@ -255,9 +255,9 @@ __device__ __forceinline__ void average_cell3(const T* __restrict__ u, const Gri
 }
 
 // ----------------------------------------------------------------------
-// (a2) mean and variance of the r^3 fine cells of a bulk cell, any r: the odd
-// ratios but 3 and those above 8, which have no kernel of their own because no
-// workload here uses them (the projection has one for 5 besides).
+// (a2) mean and variance of the r^3 fine cells of a bulk cell, any r: the ratios
+// but 2, 3, 4 and 8, which have no form of their own because no workload here
+// uses them in earnest (the projection has one for 5 besides).
 // The variance uses a shift by the first fine value of the cell:
 // var = (Q - sum_c D_c^2 / n) / n with Q = sum (u - ref)^2 and
 // D_c = sum_f u_c - n ref_c, both compensated, which equals the two-pass
