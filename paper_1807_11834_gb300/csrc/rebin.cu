@@ -153,7 +153,10 @@ k_rebin_mark(const T* __restrict__ pos, int n, GridDev g, const int32_t* __restr
                 rkn[s] = moved ? ~cn[k] : cn[k];
                 if (!IDENT) rid[s] = id[k];
             }
-            if (VOL) volume_add_row(valid, cn[k], pv[k].w, g, acc);
+            if (VOL) {
+                if (IDENT) volume_add_row(valid, cn[k], pv[k].w, g, acc);
+                else volume_add_row_wide(valid, cn[k], pv[k].w, g, acc);
+            }
         }
         if (lane == 0) s_cnt[warp] = wc;
         __syncthreads();
