@@ -44,11 +44,11 @@ UNIT = "particle-steps/s"
 # dram__bytes_write.sum), keyed by kernel, valid only while the kernel's
 # source files are byte-identical to the ones profiled (sha256 prefixes).
 NCU_TRAFFIC = {
-    # packed bed, one warm launch of k_average<float, 4>: 404.8 MB read + 6.7 MB written
-    ("packed_bed", "average"): {"files": {"fine.cu": "421c8cff56ee4956"}, "bytes": 411.6e6},
+    # packed bed, one warm launch of k_average<float, 4>: 405.8 MB read + 7.8 MB written
+    ("packed_bed", "average"): {"files": {"fine.cu": "b468c31af5421e5d"}, "bytes": 413.7e6},
     # clustered-bed recipe at 16M particles, a warm sorted step of k_drag_sorted<float, 1, 1> (the
-    # reaction with it): 668.4 MB read + 661.3 MB written, times 2 for the 32M bed (traffic per particle)
-    ("clustered_bed", "drag"): {"files": {"drag.cu": "cc7422222cbf8a04", "drag_law.cuh": "fc474a5902a1ea4d"},
+    # reaction with it): 668.3 MB read + 661.1 MB written, times 2 for the 32M bed (traffic per particle)
+    ("clustered_bed", "drag"): {"files": {"drag.cu": "4ee80081749c4b5d", "drag_law.cuh": "fc474a5902a1ea4d"},
                                 "bytes": 2.659e9},
 }
 
@@ -265,7 +265,7 @@ def algorithmic_bytes(g, n, eps_fine=True, implicit=False, euler=False, sorted_s
         "average": nf * 12 + nbx * 16,                    # u_f read, u_B and var written
         "deposit_implicit": n * (16 + 4) + nbx * 16,      # sorted (beta, beta u) + key read; A, b written
         "project_implicit": nf * 16 + nbx * 16,           # A_f, b_f written, A, b read
-        # incremental rebinning (the movers' placement and the idle fallback not counted)
+        # incremental rebinning (the movers' placement and the crowded cells' merges not counted)
         "rebin_mark": n * ((16 + 4 + 4) if sorted_step else (4 + 4 + 16 + 4 + 4)),
         # pos, old cell (in caller order the old id) read; record (old id) written
         "rebin_cells": nbx * (16 + 4 + 16 + 28),
