@@ -119,5 +119,6 @@ def test_a_step_after_one_whose_launch_failed(cuda_lib, form):
             assert failed < 60
         assert failed >= 8
         h.close()
+        assert cg.lib().cg_debug_fail_launch_after(-2) == 1
     finally:
         cg.lib().cg_debug_fail_launch_after(-1)
